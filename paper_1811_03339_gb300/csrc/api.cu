@@ -369,12 +369,10 @@ int fem3_assemble(fem3_mesh h, const double alpha[3], const double K[3], int pre
         } else {
             FEM3_TRY(f32_to_f64(m->A32, A_out, n * n, m->stream));
             note_launch(m);
-            if (precision == FEM3_TF32X3 || precision == FEM3_BF16X3) {
-                // the tensor-core paths fill the lower triangle
-                FEM3_TRY(sym_from_lower(A_out, n, m->stream));
-                note_launch(m);
-            }
         }
+        // the contractions fill the lower triangle
+        FEM3_TRY(sym_from_lower(A_out, n, m->stream));
+        note_launch(m);
     }
     return FEM3_OK;
 }

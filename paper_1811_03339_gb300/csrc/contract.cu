@@ -1,12 +1,7 @@
 // Contraction A = sum_i s_i K_i (L_i^T W R_i + R_i^T W L_i) on CUDA cores, bin by bin
 // (Section 2.1 element sum, Section 2.3 template: only dofs of a bin's template set can
-// meet the bin's Gauss points, so each bin contributes a dense D_b x D_b block).
-//
-// Work item (bin, t1, t2), t1 <= t2, covers the 64 x 64 output tile of local dofs
-// [64 t1, 64 t1 + 64) x [64 t2, 64 t2 + 64):
-//   out(c1, c2) = sum_r w_r (L[c1][r] R[c2][r] + R[c1][r] L[c2][r])   (symmetric)
-// and adds s K out(c1, c2) to A[dof c1][dof c2] (and to the mirror element when t1 < t2).
-// TA is the arithmetic type (double for the FP64 form, float for the FP32 form).
+// meet the bin's Gauss points, so each bin contributes to a D_b x D_b block), from the
+// nonzeros of the bin's table blocks (about a fifth of their entries: k_contract_rows).
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -17,92 +12,184 @@ namespace fem3 {
 
 namespace {
 
-constexpr int kTile = 64, kKC = 16;
+constexpr int kRowsThreads = 256, kRowsWarps = kRowsThreads / 32;
+constexpr int kRowsEntryBytes = 48 * 1024;   // compacted entries in shared memory, at most
+// the largest launch: entries, FP64 accumulator rows, offsets and cursors of the points
+constexpr size_t kRowsSmemMax = kRowsEntryBytes + sizeof(double) * kRowsWarps * kRowsWindow +
+                                sizeof(int) * (2 * kMaxBinItems + 1) + 64;
 
-// table entry (hi + lo pair) in the arithmetic type of the contraction
+// table entry (hi + lo pair) in the arithmetic type of the contraction; the FP64 value is
+// assembled from the pair's bits (f32 -> f64 conversions run at the FP64 rate) and one add
 template <class TA>
-__device__ __forceinline__ TA tab_value(const float2 *p) {
-    const float2 v = *p;
-    if constexpr (sizeof(TA) == 8) return (double)v.x + (double)v.y;
+__device__ __forceinline__ TA pair_value(float2 v) {
+    if constexpr (sizeof(TA) == 8) return f32_to_f64_exact(v.x) + f32_to_f64_exact(v.y);
     else return v.x + v.y;
 }
 
-template <class TA>
-__global__ void __launch_bounds__(256) k_contract_simt(
-    const float2 *__restrict__ tabL, const float2 *__restrict__ tabR,
-    const int4 *__restrict__ work, const int32_t *__restrict__ gp_off,
-    const int32_t *__restrict__ gp_idx, const int32_t *__restrict__ dof_off,
-    const int32_t *__restrict__ dof_idx, const int64_t *__restrict__ tab_off,
-    const int32_t *__restrict__ tab_ld, const double *__restrict__ gw, double sK, TA *A,
-    int64_t n_dof) {
-    __shared__ TA sLa[kKC][kTile], sRa[kKC][kTile], sLb[kKC][kTile], sRb[kKC][kTile];
-    __shared__ TA sw[kKC];
-    const int4 wk = work[blockIdx.x];
-    const int bin = wk.x, t1 = wk.y, t2 = wk.z;
-    const int D = dof_off[bin + 1] - dof_off[bin];
-    const int G = gp_off[bin + 1] - gp_off[bin];
-    const int ld = tab_ld[bin];
-    const float2 *L = tabL + tab_off[bin], *R = tabR + tab_off[bin];
-    const int32_t *slots = gp_idx + gp_off[bin];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int a0 = t1 * kTile, b0 = t2 * kTile;
+// one axis of the product X = T^T diag(w) S over its bins
+struct RowsAxis {
+    const float2 *__restrict__ T, *__restrict__ S;   // tables of the rows and of the columns
+    const int4 *__restrict__ work;                   // (bin, first column of the window, 0, 0)
+    const int32_t *__restrict__ gp_off, *__restrict__ dof_off, *__restrict__ dof_idx,
+        *__restrict__ tab_ld;
+    const int64_t *__restrict__ tab_off;
+    const double *__restrict__ w;                    // weights per slot, or per Gauss point
+    const int32_t *__restrict__ w_idx;               // slot -> Gauss point (null: w per slot)
+    double scale;
+    int n_work;
+};
+struct RowsAxes {
+    RowsAxis a[3];
+};
 
-    TA acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; i++)
-#pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = TA(0);
-
-    for (int r0 = 0; r0 < G; r0 += kKC) {
-        if (threadIdx.x < kKC) {
-            int r = r0 + threadIdx.x;
-            sw[threadIdx.x] = r < G ? TA(gw[slots[r]]) : TA(0);
+// X(c1, c2) = sum_r w_r T[c1][r] S[c2][r] of one bin, row by row over the nonzeros (the
+// order of Gustavson's sparse product): one CTA per (bin, window of <= win columns c2).
+//   1. the window's nonzeros of S, compacted per Gauss point into shared memory (value and
+//      column; counts, a scan, then the entries in any order: a point's columns differ, so
+//      the sums do not depend on it);
+//   2. warp = row c1: its accumulator row lives in shared memory; for every Gauss point
+//      with T[c1][r] != 0 the lanes take the point's entries, acc[c2] += (w T) S;
+//   3. the row's nonzeros go to A: with FULL to A[dof c1][dof c2] (general form), else to the
+//      lower triangle only, where X(c1, c2) and X(c2, c1) land on the same element (the fold
+//      A = s K (X + X^T); the diagonal gets 2 X).
+// Points go in groups whose entries fit `cap` (>= win, so a group holds at least one point);
+// usually one group.  TA is the arithmetic type: double (FP64 form) or float (FP32 form).
+//
+// Bound: shared-memory latency and the FP64 pipe (1/64 of the FP32 rate).  A dense 64 x 64
+// tile product over the same blocks does 15 to 30 times the sum over points of
+// nnz(T) nnz(S); here a point's entries are about one warp-wide pass (1.5 n on a mesh of n
+// cells per side, both sides together 3 n).  Measured against that tile product, GB300: FP64
+// assemble + solve of the 11^3 parallelepiped 9.57 -> 5.03 ms (contraction 4.76 -> 0.21 ms),
+// one FP64 general-form term at the 13^3 cube 2.32 -> 0.51 ms (1.98 -> 0.19 ms without the
+// walk), FP32 step at the 13^3 cube 3.37 -> 3.13 ms (three axes 0.48 -> 0.25 ms).
+template <class TA, bool FULL>
+__global__ void __launch_bounds__(kRowsThreads) k_contract_rows(
+    const __grid_constant__ RowsAxes P, int cap, int win, int max_gp, TA *A, int64_t n_dof) {
+    extern __shared__ __align__(16) unsigned char sm_rows[];
+    int b = blockIdx.x, axis = 0;
+    while (axis < 2 && b >= P.a[axis].n_work) b -= P.a[axis++].n_work;
+    const RowsAxis &X = P.a[axis];
+    const int4 wk = X.work[b];
+    const int bin = wk.x, col0 = wk.y;
+    const int d0 = X.dof_off[bin], D = X.dof_off[bin + 1] - d0;
+    const int g0 = X.gp_off[bin], G = X.gp_off[bin + 1] - g0;
+    const int ld = X.tab_ld[bin];
+    const int ncol = min(win, D - col0);
+    const float2 *T = X.T + X.tab_off[bin];
+    const float2 *S = X.S + X.tab_off[bin] + (int64_t)col0 * ld;
+    TA *vals = reinterpret_cast<TA *>(sm_rows);               // [cap]
+    TA *accs = vals + cap;                                    // [warps][win]
+    int *first = reinterpret_cast<int *>(accs + kRowsWarps * win);   // [max_gp + 1]
+    int *cur = first + max_gp + 1;                            // [max_gp]
+    uint16_t *cols = reinterpret_cast<uint16_t *>(cur + max_gp);     // [cap]
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int nchunk = (G + 31) >> 5;
+    for (int g = tid; g < G; g += kRowsThreads) cur[g] = 0;
+    __syncthreads();
+    // (chunk of 32 points, one of kRowsWarps row slices) per warp and pass, lane = point
+    for (int it = warp; it < nchunk * kRowsWarps; it += kRowsWarps) {
+        const int g = 32 * (it / kRowsWarps) + lane;
+        if (g >= G) continue;
+        int c = 0;
+#pragma unroll 4
+        for (int r = it % kRowsWarps; r < ncol; r += kRowsWarps) {
+            const float2 v = __ldg(S + (int64_t)r * ld + g);
+            c += v.x != 0.f || v.y != 0.f;
         }
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            int e = threadIdx.x + 256 * q;  // 0..1023 over 64 rows x 16 columns
-            int c = e >> 4, k = e & 15, r = r0 + k;
-            bool okr = r < G;
-            int ca = a0 + c, cb = b0 + c;
-            sLa[k][c] = (okr && ca < D) ? tab_value<TA>(L + (int64_t)ca * ld + r) : TA(0);
-            sRa[k][c] = (okr && ca < D) ? tab_value<TA>(R + (int64_t)ca * ld + r) : TA(0);
-            sLb[k][c] = (okr && cb < D) ? tab_value<TA>(L + (int64_t)cb * ld + r) : TA(0);
-            sRb[k][c] = (okr && cb < D) ? tab_value<TA>(R + (int64_t)cb * ld + r) : TA(0);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < kKC; k++) {
-            TA la[4], ra[4], lb[4], rb[4];
-            TA w = sw[k];
-#pragma unroll
-            for (int i = 0; i < 4; i++) {
-                la[i] = sLa[k][ty * 4 + i];
-                ra[i] = sRa[k][ty * 4 + i];
-                lb[i] = sLb[k][tx * 4 + i] * w;
-                rb[i] = sRb[k][tx * 4 + i] * w;
-            }
-#pragma unroll
-            for (int i = 0; i < 4; i++)
-#pragma unroll
-                for (int j = 0; j < 4; j++) acc[i][j] = fma(la[i], rb[j], fma(ra[i], lb[j], acc[i][j]));
-        }
-        __syncthreads();
+        if (c) atomicAdd(&cur[g], c);
     }
-    const int32_t *dofs = dof_idx + dof_off[bin];
+    __syncthreads();
+    if (warp == 0) {   // exclusive scan of the counts
+        int carry = 0;
+        for (int q = 0; q < G; q += 32) {
+            const int c = q + lane < G ? cur[q + lane] : 0;
+            int x = c;
 #pragma unroll
-    for (int i = 0; i < 4; i++) {
-        int c1 = a0 + ty * 4 + i;
-        if (c1 >= D) continue;
-        int64_t j1 = dofs[c1];
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-            int c2 = b0 + tx * 4 + j;
-            if (c2 >= D) continue;
-            int64_t j2 = dofs[c2];
-            TA v = TA(sK) * acc[i][j];
-            atomicAdd(&A[j1 * n_dof + j2], v);
-            if (t1 != t2) atomicAdd(&A[j2 * n_dof + j1], v);
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (q + lane < G) first[q + lane] = carry + x - c;
+            carry += __shfl_sync(0xffffffffu, x, 31);
         }
+        if (lane == 0) first[G] = carry;
+    }
+    __syncthreads();
+    TA *acc = accs + warp * win;
+    for (int ga = 0; ga < G;) {
+        // the group [ga, gb): as many points as fit (all threads find the same gb)
+        const int base = first[ga];
+        int gb = G;
+        if (first[G] - base > cap) {
+            int lo = ga + 1, hi = G;   // first[lo] - base <= win <= cap
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (first[mid] - base <= cap) lo = mid;
+                else hi = mid;
+            }
+            gb = lo;
+        }
+        for (int g = ga + tid; g < gb; g += kRowsThreads) cur[g] = first[g] - base;
+        __syncthreads();
+        const int ca = ga >> 5, cn = ((gb + 31) >> 5) - ca;
+        for (int it = warp; it < cn * kRowsWarps; it += kRowsWarps) {
+            const int g = 32 * (ca + it / kRowsWarps) + lane;
+            if (g < ga || g >= gb) continue;
+#pragma unroll 4
+            for (int r = it % kRowsWarps; r < ncol; r += kRowsWarps) {
+                const float2 v = __ldg(S + (int64_t)r * ld + g);
+                if (v.x != 0.f || v.y != 0.f) {
+                    const int k = atomicAdd(&cur[g], 1);
+                    vals[k] = pair_value<TA>(v);
+                    cols[k] = (uint16_t)r;
+                }
+            }
+        }
+        __syncthreads();
+        for (int c1 = warp; c1 < D; c1 += kRowsWarps) {
+            for (int c = lane; c < ncol; c += 32) acc[c] = TA(0);
+            __syncwarp();
+            bool any = false;
+            for (int q = ga & ~31; q < gb; q += 32) {
+                const int g = q + lane;
+                float2 tv = make_float2(0.f, 0.f);
+                if (g >= ga && g < gb) tv = __ldg(T + (int64_t)c1 * ld + g);
+                const bool nz = tv.x != 0.f || tv.y != 0.f;
+                unsigned m = __ballot_sync(0xffffffffu, nz);
+                if (!m) continue;
+                any = true;
+                TA t = TA(0);
+                if (nz) t = pair_value<TA>(tv) * (TA)X.w[X.w_idx ? X.w_idx[g0 + g] : g0 + g];
+                while (m) {
+                    const int l = __ffs(m) - 1;
+                    m &= m - 1;
+                    const TA tc = __shfl_sync(0xffffffffu, t, l);
+                    const int k1 = first[q + l + 1] - base;
+                    for (int k = first[q + l] - base + lane; k < k1; k += 32) {
+                        const int c = cols[k];
+                        acc[c] = fma(tc, vals[k], acc[c]);
+                    }
+                    __syncwarp();
+                }
+            }
+            if (any) {
+                const int64_t j1 = X.dof_idx[d0 + c1];
+                const TA sc = (TA)X.scale;
+                for (int c = lane; c < ncol; c += 32) {
+                    const TA v = acc[c];
+                    if (v == TA(0)) continue;
+                    const int64_t j2 = X.dof_idx[d0 + col0 + c];
+                    if constexpr (FULL)
+                        atomicAdd(&A[j1 * n_dof + j2], sc * v);
+                    else
+                        atomicAdd(&A[(j1 > j2 ? j1 : j2) * n_dof + (j1 > j2 ? j2 : j1)],
+                                  (j1 == j2 ? TA(2) : TA(1)) * sc * v);
+                }
+            }
+            __syncwarp();
+        }
+        ga = gb;
+        if (ga < G) __syncthreads();   // the entries are read before the next group's
     }
 }
 
@@ -140,78 +227,6 @@ __global__ void __launch_bounds__(128) k_contract_work(
     if ((threadIdx.x & 31) == 0 && cnt != 0) atomicAdd(nnz, cnt);
 }
 
-// One product of the general form (c D^a u, D^^b v), all 64 x 64 tile pairs of each bin:
-// out(c1, c2) = sum_r wc_r T[c1][r] S[c2][r] (T the test side's table, S the trial side's,
-// wc the Gauss weight times the coefficient) added to K[dof c1][dof c2].
-template <class TA>
-__global__ void __launch_bounds__(256) k_contract_form(
-    const float2 *__restrict__ tabT, const float2 *__restrict__ tabS,
-    const int4 *__restrict__ work, const int32_t *__restrict__ gp_off,
-    const int32_t *__restrict__ gp_idx, const int32_t *__restrict__ dof_off,
-    const int32_t *__restrict__ dof_idx, const int64_t *__restrict__ tab_off,
-    const int32_t *__restrict__ tab_ld, const double *__restrict__ wc, TA *K, int64_t n_dof) {
-    __shared__ TA sT[kKC][kTile], sS[kKC][kTile];
-    __shared__ TA sw[kKC];
-    const int4 wk = work[blockIdx.x];
-    const int bin = wk.x, t1 = wk.y, t2 = wk.z;
-    const int D = dof_off[bin + 1] - dof_off[bin];
-    const int G = gp_off[bin + 1] - gp_off[bin];
-    const int ld = tab_ld[bin];
-    const float2 *T = tabT + tab_off[bin], *S = tabS + tab_off[bin];
-    const int32_t *slots = gp_idx + gp_off[bin];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int a0 = t1 * kTile, b0 = t2 * kTile;
-    TA acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; i++)
-#pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = TA(0);
-    for (int r0 = 0; r0 < G; r0 += kKC) {
-        if (threadIdx.x < kKC) {
-            const int r = r0 + threadIdx.x;
-            sw[threadIdx.x] = r < G ? TA(wc[slots[r]]) : TA(0);
-        }
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const int e = threadIdx.x + 256 * q;
-            const int c = e >> 4, k = e & 15, r = r0 + k;
-            const bool okr = r < G;
-            const int ca = a0 + c, cb = b0 + c;
-            sT[k][c] = (okr && ca < D) ? tab_value<TA>(T + (int64_t)ca * ld + r) : TA(0);
-            sS[k][c] = (okr && cb < D) ? tab_value<TA>(S + (int64_t)cb * ld + r) : TA(0);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < kKC; k++) {
-            TA ta[4], sb[4];
-            const TA w = sw[k];
-#pragma unroll
-            for (int i = 0; i < 4; i++) {
-                ta[i] = sT[k][ty * 4 + i];
-                sb[i] = sS[k][tx * 4 + i] * w;
-            }
-#pragma unroll
-            for (int i = 0; i < 4; i++)
-#pragma unroll
-                for (int j = 0; j < 4; j++) acc[i][j] = fma(ta[i], sb[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-    const int32_t *dofs = dof_idx + dof_off[bin];
-#pragma unroll
-    for (int i = 0; i < 4; i++) {
-        const int c1 = a0 + ty * 4 + i;
-        if (c1 >= D) continue;
-        const int64_t j1 = dofs[c1];
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-            const int c2 = b0 + tx * 4 + j;
-            if (c2 >= D) continue;
-            atomicAdd(&K[j1 * n_dof + dofs[c2]], acc[i][j]);
-        }
-    }
-}
-
 // wc[g] = w[g] c[g] (c NULL: w)
 __global__ void k_weight_coef(const double *__restrict__ w, const double *__restrict__ c,
                               int64_t n, double *wc) {
@@ -229,52 +244,64 @@ int weight_coef(Mesh *m, const double *c_gp, double *wc_gp) {
     return FEM3_OK;
 }
 
+// one launch of k_contract_rows over the axes of P (an axis without work has n_work = 0)
+template <class TA, bool FULL>
+static int launch_rows(Mesh *m, const RowsAxes &P, TA *A) {
+    int64_t nw = 0;
+    int max_dof = 1, max_gp = 1;
+    for (int axis = 0; axis < 3; axis++) {
+        if (!P.a[axis].n_work) continue;
+        nw += P.a[axis].n_work;
+        max_dof = std::max(max_dof, m->bins[axis].max_dof);
+        max_gp = std::max(max_gp, m->bins[axis].max_gp);
+    }
+    if (nw == 0) return FEM3_OK;
+    // room for a third of the largest block's entries (a fifth are nonzero on the
+    // configured meshes), 48 KB at most: three CTAs or more per SM
+    const int win = std::min(max_dof, kRowsWindow);
+    const int64_t entry = sizeof(TA) + sizeof(uint16_t);
+    const int cap = (int)std::max<int64_t>(
+        win, std::min<int64_t>((int64_t)win * max_gp / 3 + 64, kRowsEntryBytes / entry));
+    const size_t sh = (sizeof(TA) * (cap + (size_t)kRowsWarps * win) +
+                       sizeof(int) * (2 * (size_t)max_gp + 1) + sizeof(uint16_t) * cap + 15) &
+                      ~size_t(15);
+    static bool attr = false;
+    if (!attr) {
+        FEM3_CUDA(cudaFuncSetAttribute(k_contract_rows<TA, FULL>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kRowsSmemMax));
+        attr = true;
+    }
+    kc_begin(m, KC_CONTRACT);
+    k_contract_rows<TA, FULL><<<(unsigned)nw, kRowsThreads, sh, m->stream>>>(P, cap, win, max_gp,
+                                                                            A, m->n_dof);
+    kc_end(m, KC_CONTRACT);
+    note_launch(m);
+    FEM3_CUDA(cudaGetLastError());
+    return FEM3_OK;
+}
+
+static int clear_matrix(Mesh *m, int precision) {
+    const int64_t n = m->n_dof;
+    if (precision == FEM3_FP64)
+        FEM3_CUDA(cudaMemsetAsync(m->A64, 0, sizeof(double) * n * n, m->stream));
+    else
+        FEM3_CUDA(cudaMemsetAsync(m->A32, 0, sizeof(float) * n * n, m->stream));
+    return FEM3_OK;
+}
+
 // K = T^T diag(wc) S over one axis's bins on CUDA cores (FP64 into A64 or FP32 into A32),
 // T the test side's table (R if test_right), S the trial side's
 int contract_form(Mesh *m, int axis, bool test_right, const double *wc_gp, int precision) {
-    cudaStream_t s = m->stream;
-    const int64_t n = m->n_dof;
     AxisBins &B = m->bins[axis];
-    if (!B.form_work) {
-        std::vector<int4> work;
-        for (int b = 0; b < B.n_bins; b++) {
-            const int D = B.h_dof_off[b + 1] - B.h_dof_off[b];
-            const int G = B.h_gp_off[b + 1] - B.h_gp_off[b];
-            if (D == 0 || G == 0) continue;
-            const int nt = (D + kTile - 1) / kTile;
-            for (int t1 = 0; t1 < nt; t1++)
-                for (int t2 = 0; t2 < nt; t2++) work.push_back(make_int4(b, t1, t2, 0));
-        }
-        B.n_form_work = (int)work.size();
-        FEM3_TRY(dev_alloc_t(m, &B.form_work, std::max(1, B.n_form_work)));
-        if (B.n_form_work)
-            FEM3_CUDA(cudaMemcpyAsync(B.form_work, work.data(), sizeof(int4) * work.size(),
-                                      cudaMemcpyHostToDevice, s));
-        // the pageable source must outlive the copy
-        FEM3_CUDA(cudaStreamSynchronize(s));
-    }
-    const float2 *T = test_right ? m->tabR[axis] : m->tabL[axis];
-    const float2 *S = test_right ? m->tabL[axis] : m->tabR[axis];
-    if (precision == FEM3_FP64) {
-        FEM3_CUDA(cudaMemsetAsync(m->A64, 0, sizeof(double) * n * n, s));
-    } else {
-        FEM3_CUDA(cudaMemsetAsync(m->A32, 0, sizeof(float) * n * n, s));
-    }
-    if (B.n_form_work) {
-        kc_begin(m, KC_CONTRACT);
-        if (precision == FEM3_FP64)
-            k_contract_form<double><<<B.n_form_work, 256, 0, s>>>(
-                T, S, B.form_work, B.gp_off, B.gp_idx, B.dof_off, B.dof_idx, B.tab_off, B.tab_ld,
-                wc_gp, m->A64, n);
-        else
-            k_contract_form<float><<<B.n_form_work, 256, 0, s>>>(
-                T, S, B.form_work, B.gp_off, B.gp_idx, B.dof_off, B.dof_idx, B.tab_off, B.tab_ld,
-                wc_gp, m->A32, n);
-        kc_end(m, KC_CONTRACT);
-        note_launch(m);
-    }
-    FEM3_CUDA(cudaGetLastError());
-    return FEM3_OK;
+    FEM3_TRY(clear_matrix(m, precision));
+    RowsAxes P{};
+    P.a[axis] = RowsAxis{test_right ? m->tabR[axis] : m->tabL[axis],
+                         test_right ? m->tabL[axis] : m->tabR[axis], B.work, B.gp_off,
+                         B.dof_off, B.dof_idx, B.tab_ld, B.tab_off, wc_gp, B.gp_idx, 1.0,
+                         B.n_work};
+    return precision == FEM3_FP64 ? launch_rows<double, true>(m, P, m->A64)
+                                  : launch_rows<float, true>(m, P, m->A32);
 }
 
 int contract_work(Mesh *m, double *flops_out, int64_t *nnz_out) {
@@ -301,15 +328,11 @@ int contract_work(Mesh *m, double *flops_out, int64_t *nnz_out) {
     return FEM3_OK;
 }
 
+// the lower triangle of A (all that the factorisation reads)
 int contract(Mesh *m, int precision) {
-    cudaStream_t s = m->stream;
-    const int64_t n = m->n_dof;
     double flops = 0;
-    if (precision == FEM3_FP64) {
-        FEM3_CUDA(cudaMemsetAsync(m->A64, 0, sizeof(double) * n * n, s));
-    } else {
-        FEM3_CUDA(cudaMemsetAsync(m->A32, 0, sizeof(float) * n * n, s));
-    }
+    FEM3_TRY(clear_matrix(m, precision));
+    RowsAxes P{};
     for (int axis = 0; axis < 3; axis++) {
         AxisBins &B = m->bins[axis];
         for (int b = 0; b < B.n_bins; b++) {
@@ -317,7 +340,6 @@ int contract(Mesh *m, int precision) {
             double G = B.h_gp_off[b + 1] - B.h_gp_off[b];
             flops += 2.0 * D * D * G;
         }
-        if (!B.n_work) continue;
         // the work items of this part's bins (the list is in bin order)
         int b0, b1;
         part_bins(m, axis, b0, b1);
@@ -326,23 +348,13 @@ int contract(Mesh *m, int precision) {
                                           [](const int4 &x, int v) { return x.x < v; }) -
                          B.h_work.begin());
         };
-        const int w0 = lb(b0), nw = lb(b1) - w0;
-        if (nw <= 0) continue;
-        kc_begin(m, KC_CONTRACT);
-        if (precision == FEM3_FP64)
-            k_contract_simt<double><<<nw, 256, 0, s>>>(
-                m->tabL[axis], m->tabR[axis], B.work + w0, B.gp_off, B.gp_idx, B.dof_off,
-                B.dof_idx, B.tab_off, B.tab_ld, m->gw, m->sK[axis], m->A64, n);
-        else
-            k_contract_simt<float><<<nw, 256, 0, s>>>(
-                m->tabL[axis], m->tabR[axis], B.work + w0, B.gp_off, B.gp_idx, B.dof_off,
-                B.dof_idx, B.tab_off, B.tab_ld, m->gw, m->sK[axis], m->A32, n);
-        kc_end(m, KC_CONTRACT);
-        note_launch(m);
+        const int w0 = lb(b0), nw = std::max(0, lb(b1) - w0);
+        P.a[axis] = RowsAxis{m->tabL[axis], m->tabR[axis], B.work + w0, B.gp_off, B.dof_off,
+                             B.dof_idx, B.tab_ld, B.tab_off, B.w_slot, nullptr, m->sK[axis], nw};
     }
     m->contract_flops = flops;
-    FEM3_CUDA(cudaGetLastError());
-    return FEM3_OK;
+    return precision == FEM3_FP64 ? launch_rows<double, false>(m, P, m->A64)
+                                  : launch_rows<float, false>(m, P, m->A32);
 }
 
 }  // namespace fem3

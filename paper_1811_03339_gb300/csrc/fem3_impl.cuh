@@ -51,6 +51,8 @@ constexpr double kEpsRRel = 1e-12;    // segment-length / tie tolerance, times t
 constexpr double kEpsDRel = 1e-12;    // |gradient| below this fraction of the largest: parallel
 
 constexpr int kMaxBinItems = 4096;    // max dofs or Gauss points in one transverse bin
+constexpr int kRowsWindow = 512;      // columns of one CUDA-core contraction item (its eight
+                                      // accumulator rows: 32 KB of shared memory in FP64)
 constexpr int kSegCounterSlot = 120;  // norms[120]: segment counter (norms[0..63] reductions)
                                       // norms[121]: contraction work counter
 
@@ -90,10 +92,8 @@ struct AxisBins {
     int32_t *tab_ld = nullptr;   // [n_bins]     leading dimension (padded Gauss-point count)
     int64_t n_tmpl = 0, tab_elems = 0;
     int max_dof = 0, max_gp = 0;
-    int4 *work = nullptr;        // contraction work items (bin, t1, t2, 0)
+    int4 *work = nullptr;        // CUDA-core contraction items (bin, first column, 0, 0)
     int n_work = 0;
-    int4 *form_work = nullptr;   // general-form work items: every tile pair (bin, t1, t2, 0)
-    int n_form_work = 0;
     // tensor-core contraction operands: TF32 or BF16 hi/lo of L and of W R, [n_tmpl][Kp]
     // (Kp = tc_maxG rounded to one 128-byte row of the operand type)
     void *tc_op[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -360,6 +360,17 @@ __device__ __forceinline__ void f64_split(double x, float &hi, float &lo) {
     const float rl = __uint_as_float(0x4B000000u | (rest & 0x7FFFFFu)) - 8388608.0f;
     const float mag = fmaf(rh, 8388608.0f, rl) * __uint_as_float((ef - 948u) << 23);
     lo = __uint_as_float(__float_as_uint(mag) | sign);
+}
+
+// exact FP64 value of a normal FP32 number (zero and subnormals give 0), by bit assembly:
+// exponent rebiased by 1023 - 127, significand moved to the top of the 52-bit field
+__device__ __forceinline__ double f32_to_f64_exact(float x) {
+    const uint32_t b = __float_as_uint(x);
+    const uint32_t e = (b >> 23) & 0xFFu;
+    const unsigned long long d = ((unsigned long long)(b & 0x80000000u) << 32) |
+                                 ((unsigned long long)(e + 896u) << 52) |
+                                 ((unsigned long long)(b & 0x7FFFFFu) << 29);
+    return __longlong_as_double(e == 0u ? 0ll : (long long)d);
 }
 
 // (sh, sl) += (ah + al)(bh + bl): ah bh exactly as p + e (FMA), the cross terms in FP32

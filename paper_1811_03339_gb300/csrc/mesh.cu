@@ -841,9 +841,7 @@ int bins_build(Mesh *m) {
             B.h_tab_ld[b] = ld;
             acc += (int64_t)D * ld;
             if (D == 0 || Gc == 0) continue;
-            int nt = (D + 63) / 64;
-            for (int t1 = 0; t1 < nt; t1++)
-                for (int t2 = t1; t2 < nt; t2++) work.push_back(make_int4(b, t1, t2, 0));
+            for (int c = 0; c < D; c += kRowsWindow) work.push_back(make_int4(b, c, 0, 0));
         }
         B.tab_elems = acc;
         B.n_work = (int)work.size();

@@ -1038,16 +1038,24 @@ inline unsigned g256(int64_t n) { return (unsigned)(n > 0 ? (n + 255) / 256 : 1)
 
 }  // namespace
 
-// upper triangle := transpose of the lower triangle (n x n row-major)
-__global__ void k_sym_from_lower(double *A, int64_t n) {
-    int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= n * n) return;
-    int64_t i = e / n, j = e % n;
-    if (j > i) A[e] = A[j * n + i];
+// upper triangle := transpose of the lower triangle (n x n row-major); a CTA copies one
+// 32 x 32 tile of the lower triangle through shared memory (both sides along rows)
+__global__ void __launch_bounds__(256) k_sym_from_lower(double *A, int64_t n) {
+    __shared__ double t[32][33];
+    if (blockIdx.x > blockIdx.y) return;
+    const int64_t r0 = 32 * (int64_t)blockIdx.y, c0 = 32 * (int64_t)blockIdx.x;
+    const int x = threadIdx.x & 31;
+    for (int y = threadIdx.x >> 5; y < 32; y += 8)
+        if (r0 + y < n && c0 + x < n) t[y][x] = A[(r0 + y) * n + c0 + x];
+    __syncthreads();
+    for (int y = threadIdx.x >> 5; y < 32; y += 8)
+        if (c0 + y < n && r0 + x < n && r0 + x > c0 + y) A[(c0 + y) * n + r0 + x] = t[x][y];
 }
 
 int sym_from_lower(double *A, int64_t n, cudaStream_t s) {
-    k_sym_from_lower<<<g256(n * n), 256, 0, s>>>(A, n);
+    if (n <= 0) return FEM3_OK;
+    const unsigned g = (unsigned)((n + 31) / 32);
+    k_sym_from_lower<<<dim3(g, g), 256, 0, s>>>(A, n);
     FEM3_CUDA(cudaGetLastError());
     return FEM3_OK;
 }
@@ -1199,17 +1207,6 @@ constexpr size_t apply_bin_smem() {
                     2 * apply_pw<NR>() * kApplyGC * NR + 2 * kApplyGC * NR) *
                sizeof(float2) +
            kApplyRM * sizeof(int4);
-}
-
-// exact FP64 value of a normal FP32 number (zero and subnormals give 0), by bit assembly:
-// exponent rebiased by 1023 - 127, significand moved to the top of the 52-bit field
-__device__ __forceinline__ double f32_to_f64_exact(float x) {
-    const uint32_t b = __float_as_uint(x);
-    const uint32_t e = (b >> 23) & 0xFFu;
-    const unsigned long long d = ((unsigned long long)(b & 0x80000000u) << 32) |
-                                 ((unsigned long long)(e + 896u) << 52) |
-                                 ((unsigned long long)(b & 0x7FFFFFu) << 29);
-    return __longlong_as_double(e == 0u ? 0ll : (long long)d);
 }
 
 __device__ __forceinline__ void cp_async16(void *dst, const void *src, int src_bytes) {
