@@ -8,6 +8,7 @@
 #include <string>
 #include <vector>
 
+#include "chol_f64.cuh"
 #include "fem3_impl.cuh"
 
 namespace fem3 {
@@ -297,8 +298,8 @@ int fem3_mesh_upload(const double *verts, int64_t n_nodes, const int32_t *tets, 
     if ((st = dev_alloc(m, &m->dinv, sizeof(double) * 64 * 64 * ((n + 63) / 64))) != FEM3_OK)
         return fail(st);
     {
-        const int64_t nblk = (n + 63) / 64;
-        if ((st = dev_alloc_t(m, &m->chol_flags, nblk * (nblk + 1) + 2)) != FEM3_OK)
+        // the FP64 factorisation's 32 x 32 tiles have more flags than the FP32 one's 64 x 64
+        if ((st = dev_alloc_t(m, &m->chol_flags, chol_f64_flags(n))) != FEM3_OK)
             return fail(st);
     }
     if (cudaMemsetAsync(m->flags, 0, sizeof(int32_t) * (2 * ((n + 63) / 64) + 2), m->stream) != cudaSuccess)

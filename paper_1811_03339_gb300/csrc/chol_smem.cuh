@@ -4,7 +4,7 @@
 // diagonal-block factor-and-invert routine.  Included inside `namespace fem3 { namespace {`
 // by each translation unit (every unit gets its own internal copy).
 
-constexpr int NB = 64;   // block (tile) width of the factorisation
+constexpr int NB = 64;   // block width of the FP32 factorisations and of the triangular solves
 
 // ---------------------------------------------------------------------------------
 // Cholesky
@@ -30,6 +30,34 @@ template <> __device__ __forceinline__ float rsqrt_t<float>(float x) {
     return fmaf(0.5f * y, r, y);
 }
 template <> __device__ __forceinline__ double rsqrt_t<double>(double x) { return rsqrt(x); }
+
+// a positive pivot (false for NaN); FP64 by its bits, since a comparison takes the FP64 pipe
+__device__ __forceinline__ bool pivot_pos(float d) { return d > 0.f; }
+__device__ __forceinline__ bool pivot_pos(double d) {
+    const long long b = __double_as_longlong(d);
+    return b > 0 && b <= 0x7FF0000000000000LL;
+}
+
+// 1 / d of a positive pivot, the only function on the serial path of the diagonal factor.
+// FP64: the FP32 reciprocal estimate of the leading 24 bits of d (together below 2^-21 off)
+// as the start and one cubic Newton step y <- y (1 + e + e^2), e = 1 - d y (error e^3 <
+// 2^-63): three dependent FP64 operations where the division takes several more.
+template <class TF> __device__ __forceinline__ TF recip_t(TF d);
+template <> __device__ __forceinline__ float recip_t<float>(float d) { return __frcp_rn(d); }
+template <> __device__ __forceinline__ double recip_t<double>(double d) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(d);
+    const int e = (int)(b >> 52);   // d > 0: the sign bit is 0
+    if (e < 8 || e > 2038) return 1.0 / d;
+    const float m = __uint_as_float(0x3F800000u | (uint32_t)((b >> 29) & 0x7FFFFFu));
+    float ym;   // in [0.5, 1]
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ym) : "f"(m));
+    const uint32_t y32 = __float_as_uint(ym);
+    const double y = __longlong_as_double(
+        (long long)(((unsigned long long)((int)(y32 >> 23) + 896 + 1023 - e) << 52) |
+                    ((unsigned long long)(y32 & 0x7FFFFFu) << 29)));
+    const double r = fma(-d, y, 1.0);
+    return fma(y, fma(r, r, r), y);
+}
 
 template <class TF>
 __device__ __forceinline__ void lds4(const TF *p, TF v[4]) {   // 16-byte aligned (float) / 32 (double)
@@ -69,13 +97,14 @@ __device__ __forceinline__ void bar_arrive_n(int id, int count) {
 // warp 0: 16 x 16 Cholesky of block p of a_s and its inverse in one pass.  Lanes 0..15 hold
 // row r of the block (lower part), lanes 16..31 column r of the identity; step j broadcasts
 // the pivot column (a_kj, k >= j, from lanes k) and every lane applies the same update,
-// x_k -= (x_j / a_jj) a_kj (k > j), x_j /= sqrt(a_jj): on the rows this is the right-looking
-// factorisation, on the identity's columns forward substitution with the new column of
-// L_pp, so the inverse needs no pass of its own.  Entries above the diagonal of the row
-// lanes are never read.  Writes L_pp into a_s, L_pp^{-1} into x_s and
-// lt[k][c] = L_pp^{-1}[c][k].
-template <class TF>
-__device__ __forceinline__ void chol_inv16(TF (*a_s)[NB + 1], TF (*x_s)[NB + 1], TF (*lt)[PB + 4],
+// x_k -= (x_j / a_jj) a_kj (k > j): on the rows this is the right-looking factorisation, on
+// the identity's columns forward substitution with the new column of L_pp, so the inverse
+// needs no pass of its own.  The square roots stay off this serial path: column j (row j of
+// the inverse) is scaled by 1 / sqrt(a_jj) after the last step, all sixteen roots at once on
+// the lanes.  Entries above the diagonal of the row lanes are never read.  Writes L_pp into
+// a_s, L_pp^{-1} into x_s and lt[k][c] = L_pp^{-1}[c][k].
+template <class TF, int N>
+__device__ __forceinline__ void chol_inv16(TF (*a_s)[N + 1], TF (*x_s)[N + 1], TF (*lt)[PB + 4],
                                            int P, int nb, int64_t k0, int32_t *err) {
     const int lane = threadIdx.x & 31;
     const int r = lane & (PB - 1);
@@ -85,19 +114,23 @@ __device__ __forceinline__ void chol_inv16(TF (*a_s)[NB + 1], TF (*x_s)[NB + 1],
     for (int c = 0; c < PB; c++)
         x[c] = inv ? (c == r ? TF(1) : TF(0)) : (c <= r ? a_s[P + r][P + c] : TF(0));
     int bad = -1;
+    TF dr = TF(1);   // pivot r (of lane r)
 #pragma unroll
     for (int j = 0; j < PB; j++) {
         TF col[PB];
 #pragma unroll
         for (int k = j; k < PB; k++) col[k] = __shfl_sync(0xffffffffu, x[j], k);
         const TF d = col[j];
-        if (!(d > TF(0)) && bad < 0) bad = j;
-        const TF rs = d > TF(0) ? rsqrt_t<TF>(d) : TF(1);
-        const TF f = x[j] * rs * rs;
+        const bool pos = pivot_pos(d);
+        if (!pos && bad < 0) bad = j;
+        const TF f = x[j] * (pos ? recip_t<TF>(d) : TF(1));
+        if (r == j) dr = d;
 #pragma unroll
         for (int k = j + 1; k < PB; k++) x[k] -= f * col[k];
-        x[j] *= rs;
     }
+    const TF rs = pivot_pos(dr) ? rsqrt_t<TF>(dr) : TF(1);
+#pragma unroll
+    for (int j = 0; j < PB; j++) x[j] *= __shfl_sync(0xffffffffu, rs, j);
     if (bad >= 0 && lane == 0 && P + bad < nb)
         atomicCAS(&err[ERR_NOT_SPD], 0, (int32_t)(k0 + P + bad + 1));
     if (!inv) {
@@ -113,7 +146,7 @@ __device__ __forceinline__ void chol_inv16(TF (*a_s)[NB + 1], TF (*x_s)[NB + 1],
     }
 }
 
-// Diagonal block: factor A_kk = L_kk L_kk^T and form L_kk^{-1} (512 threads), blocked by
+// Diagonal block: factor A_kk = L_kk L_kk^T and form L_kk^{-1} (N x N, N = 64 or 32; 512 threads), blocked by
 // 16 with look-ahead.  Warp 0 factors and inverts the 16 x 16 diagonal block p; 12 other
 // warps then (a) solve the 16 rows of block p + 1 in panel p (L_{p+1,p} = A L_pp^{-T})
 // and update diagonal block p + 1, which releases warp 0 for block p + 1 at once, and
@@ -126,27 +159,27 @@ __device__ __forceinline__ void chol_inv16(TF (*a_s)[NB + 1], TF (*x_s)[NB + 1],
 // (zero above the diagonal); the caller stores them.  A non-positive pivot records 1 + its
 // global column (k0 + local).  Needs exactly 512 threads, all of the CTA; ends with a
 // barrier.
-template <class TF>
-__device__ void potrf_inv_smem(TF (*a_s)[NB + 1], TF (*x_s)[NB + 1], int nb, int64_t k0,
+template <class TF, int N>
+__device__ void potrf_inv_smem(TF (*a_s)[N + 1], TF (*x_s)[N + 1], int nb, int64_t k0,
                                int32_t *err) {
     // warps 4, 8 and 12 share warp 0's SM sub-partition and sit out: the 12 other warps
     // do the update work, so warp 0's serial factor competes with no issuing neighbour
-    constexpr int NT = 416, NU = 384, NP = NB / PB;
+    constexpr int NT = 416, NU = 384, NP = N / PB;
     __shared__ __align__(16) TF lt[2][PB][PB + 4];     // lt[p & 1][k][c] = L_pp^{-1}[c][k]
-    __shared__ __align__(16) TF pant[PB][NB + 4];      // pant[k][r] = L[r][P + k], r >= P + 16
-    __shared__ __align__(16) TF tq[PB][NB - PB + 4];   // T_pJ, columns c < P
+    __shared__ __align__(16) TF pant[PB][N + 4];      // pant[k][r] = L[r][P + k], r >= P + 16
+    __shared__ __align__(16) TF tq[PB][N - PB + 4];   // T_pJ, columns c < P
     const int tid = threadIdx.x;
     if (tid < 32) {
         for (int p = 0; p < NP; p++) {
             if (p > 0) bar_sync_n(kBarNextReady, NT);
-            chol_inv16<TF>(a_s, x_s, lt[p & 1], p * PB, nb, k0, err);
+            chol_inv16<TF, N>(a_s, x_s, lt[p & 1], p * PB, nb, k0, err);
             __syncwarp();
             bar_arrive_n(kBarPanelReady, NT);
         }
     } else if (((tid >> 5) & 3) != 0) {
         const int ut = ((tid >> 5) - 1 - (tid >> 7)) * 32 + (tid & 31);   // 0 .. NU - 1
-        for (int e = ut; e < NB * NB; e += NU) {
-            const int i = e >> 6, c = e & 63;
+        for (int e = ut; e < N * N; e += NU) {
+            const int i = e / N, c = e & (N - 1);
             if (c >= ((i >> 4) + 1) * PB) x_s[i][c] = TF(0);
         }
         for (int p = 0; p < NP; p++) {
@@ -178,7 +211,7 @@ __device__ void potrf_inv_smem(TF (*a_s)[NB + 1], TF (*x_s)[NB + 1], int nb, int
             }
             // (b1) rows below block p + 1 (four columns per thread); the inverse's block
             // row p from T_pJ (formed in the previous panel)
-            const int R1 = R0 + PB, m2 = NB - R1;
+            const int R1 = R0 + PB, m2 = N - R1;
             const bool panel = m2 > 0 && ut < 4 * m2;
             const int pr = R1 + (ut >> 2), pc = (ut & 3) * 4;
             TF pv[4] = {TF(0), TF(0), TF(0), TF(0)};
@@ -241,7 +274,7 @@ __device__ void potrf_inv_smem(TF (*a_s)[NB + 1], TF (*x_s)[NB + 1], int nb, int
             }
             // trailing update of blocks (i, k), i >= k >= p + 1, except block (p + 1, p + 1),
             // in 2 x 2 blocks (rows i0, i0 + 1 >= R1; columns j0, j0 + 1 >= R0)
-            const int mr = (NB - R1) / 2, mc = (NB - R0) / 2;
+            const int mr = (N - R1) / 2, mc = (N - R0) / 2;
             for (int e = ut; e < mr * mc; e += NU) {
                 const int i0 = R1 + 2 * (e / mc), j0 = R0 + 2 * (e % mc);
                 if (j0 > i0) continue;

@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(512, 1) k_cholp_diag(float *A, int64_t n, int6
         d22[i][c] = (i < nb2 && c < nb2) ? A[(j0 + NB + i) * n + j0 + NB + c] : (i == c ? 1.f : 0.f);
     }
     __syncthreads();
-    potrf_inv_smem<float>(a_s, x_s, nb1, j0, err);
+    potrf_inv_smem<float, NB>(a_s, x_s, nb1, j0, err);
     float *d1 = dinv + (j0 / NB) * (int64_t)NB * NB;
     for (int e = tid; e < NB * NB; e += 512) {
         const int i = e >> 6, c = e & 63;
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(512, 1) k_cholp_diag(float *A, int64_t n, int6
             a_s[i][c] = d22[i][c] - t_s[i][c];
         }
         __syncthreads();
-        potrf_inv_smem<float>(a_s, x_s, nb2, j0 + NB, err);    // x_s = X22
+        potrf_inv_smem<float, NB>(a_s, x_s, nb2, j0 + NB, err);    // x_s = X22
         float *d2 = d1 + (int64_t)NB * NB;
         for (int e = tid; e < NB * NB; e += 512) {
             d2[e] = x_s[e >> 6][e & 63];

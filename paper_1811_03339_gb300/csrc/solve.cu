@@ -2,10 +2,10 @@
 //
 //  - b = M f with the P1 mass matrix (|T|/20 (1 + delta_ab) per tet), the weak
 //    right-hand side (f, v) of Section 3.
-//  - Right-looking blocked Cholesky A = L L^T (block 64): diagonal block in shared
-//    memory, panel triangular solve, trailing symmetric update; row-major storage: the
-//    tiles below the diagonal in A's lower triangle, each diagonal tile as its inverse
-//    L_jj^{-1} (all the solves use).  TF is double (FP64 form) or float (mixed forms).
+//  - Cholesky A = L L^T: by tile tasks (FP32 here, FP64 in chol_f64.cu) or blocked on the
+//    tensor cores (chol_tc.cu); row-major storage: the tiles below the diagonal in A's
+//    lower triangle, each 64 x 64 diagonal block as its inverse L_jj^{-1} (all the solves
+//    use).
 //  - Blocked forward / backward substitution.
 //  - Refinement for the mixed forms: r = b - A u with A u applied in FP64 from the FP64
 //    derivative tables (A u = sum_i s_i K_i (L_i^T W (R_i u) + R_i^T W (L_i u))), the
@@ -15,6 +15,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "chol_f64.cuh"
 #include "fem3_impl.cuh"
 
 namespace fem3 {
@@ -60,7 +61,8 @@ __global__ void k_load_T(const int32_t *__restrict__ tets, const double *__restr
 #include "chol_smem.cuh"
 
 // ---------------------------------------------------------------------------------
-// Tile-task Cholesky in one launch.  CTA 0 runs the diagonal chain: for each block
+// Tile-task Cholesky of the FP32 factor in one launch, 64 x 64 tiles (the FP64 form has its
+// own, chol_f64.cu).  CTA 0 runs the diagonal chain: for each block
 // column j it applies the last update (k = j - 1) to the diagonal tile, factors it
 // (L_jj and L_jj^{-1}), solves the tile below it, L_{j+1,j} = A_{j+1,j} L_jj^{-T}, and
 // keeps that tile in shared memory for the next diagonal update, so the critical path
@@ -100,19 +102,17 @@ __device__ __forceinline__ bool wait_tile(const int *f, int *abort_w, int32_t *e
 // load instruction covers 32 consecutive entries of one row), element e = 2k + h of a
 // thread is (row 4w + k, column lane + 32h).  L2 loads: the tile was written by another CTA
 // of the same launch.
-template <class TF>
-__device__ __forceinline__ void tile_regs(const TF *src, int64_t ld, int64_t rows, TF v[8]) {
+__device__ __forceinline__ void tile_regs(const float *src, int64_t ld, int64_t rows, float v[8]) {
     const int lane = threadIdx.x & 31, r0 = (threadIdx.x >> 5) * 4;
 #pragma unroll
     for (int k = 0; k < 4; k++)
 #pragma unroll
         for (int h = 0; h < 2; h++)
             v[2 * k + h] = r0 + k < rows ? __ldcg(src + (int64_t)(r0 + k) * ld + lane + 32 * h)
-                                         : TF(0);
+                                         : 0.f;
 }
 // dst[c][r] = the loaded tile's entry (r, c)
-template <class TF>
-__device__ __forceinline__ void tile_store_T(const TF v[8], TF (*dst)[kTileLd]) {
+__device__ __forceinline__ void tile_store_T(const float v[8], float (*dst)[kTileLd]) {
     const int lane = threadIdx.x & 31, r0 = (threadIdx.x >> 5) * 4;
 #pragma unroll
     for (int k = 0; k < 4; k++)
@@ -120,31 +120,30 @@ __device__ __forceinline__ void tile_store_T(const TF v[8], TF (*dst)[kTileLd]) 
         for (int h = 0; h < 2; h++) dst[lane + 32 * h][r0 + k] = v[2 * k + h];
 }
 // dst[c][r] = src[r * ld + c] (r < rows, else 0), c < 64
-template <class TF>
-__device__ __forceinline__ void load_tile_T(const TF *src, int64_t ld, int64_t rows,
-                                            TF (*dst)[kTileLd]) {
-    TF v[8];
-    tile_regs<TF>(src, ld, rows, v);
-    tile_store_T<TF>(v, dst);
+__device__ __forceinline__ void load_tile_T(const float *src, int64_t ld, int64_t rows,
+                                            float (*dst)[kTileLd]) {
+    float v[8];
+    tile_regs(src, ld, rows, v);
+    tile_store_T(v, dst);
 }
 
 // acc[p][q] += sgn * sum_c bi[c][ty*2+p] bj[c][tx*4+q] (operands in transposed layout).
 // The 64-term product is summed from zero and added to acc once: summing into acc
 // directly would round every term at the magnitude of the (much larger) tile entry,
 // which made the FP32 factor several times less accurate.
-template <class TF, bool SUB>
-__device__ __forceinline__ void tile_gemm_T(TF acc[2][4], const TF (*bi)[kTileLd],
-                                            const TF (*bj)[kTileLd], int tx, int ty) {
-    TF t[2][4];
+template <bool SUB>
+__device__ __forceinline__ void tile_gemm_T(float acc[2][4], const float (*bi)[kTileLd],
+                                            const float (*bj)[kTileLd], int tx, int ty) {
+    float t[2][4];
 #pragma unroll
     for (int p = 0; p < 2; p++)
 #pragma unroll
-        for (int q = 0; q < 4; q++) t[p][q] = TF(0);
+        for (int q = 0; q < 4; q++) t[p][q] = 0.f;
 #pragma unroll 8
     for (int c = 0; c < NB; c++) {
-        TF u[2], v[4];
-        lds2<TF>(&bi[c][ty * 2], u);
-        lds4<TF>(&bj[c][tx * 4], v);
+        float u[2], v[4];
+        lds2<float>(&bi[c][ty * 2], u);
+        lds4<float>(&bj[c][tx * 4], v);
 #pragma unroll
         for (int p = 0; p < 2; p++)
 #pragma unroll
@@ -157,22 +156,20 @@ __device__ __forceinline__ void tile_gemm_T(TF acc[2][4], const TF (*bi)[kTileLd
 }
 
 // load tile (r0, c0) of A into acc (rows/columns beyond n: identity on the diagonal tile)
-template <class TF>
-__device__ __forceinline__ void load_acc(const TF *A, int64_t n, int64_t r0, int64_t c0,
-                                         bool diag, TF acc[2][4], int tx, int ty) {
+__device__ __forceinline__ void load_acc(const float *A, int64_t n, int64_t r0, int64_t c0,
+                                         bool diag, float acc[2][4], int tx, int ty) {
 #pragma unroll
     for (int p = 0; p < 2; p++)
 #pragma unroll
         for (int q = 0; q < 4; q++) {
             const int r = ty * 2 + p, c = tx * 4 + q;
             acc[p][q] = (r0 + r < n && c0 + c < n) ? __ldcg(&A[(r0 + r) * n + c0 + c])
-                                                   : ((diag && r == c) ? TF(1) : TF(0));
+                                                   : ((diag && r == c) ? 1.f : 0.f);
         }
 }
 
-template <class TF>
-__device__ __forceinline__ void store_acc(TF *A, int64_t n, int64_t r0, int64_t c0,
-                                          const TF acc[2][4], int tx, int ty) {
+__device__ __forceinline__ void store_acc(float *A, int64_t n, int64_t r0, int64_t c0,
+                                          const float acc[2][4], int tx, int ty) {
 #pragma unroll
     for (int p = 0; p < 2; p++) {
         const int r = ty * 2 + p;
@@ -190,32 +187,31 @@ __device__ __forceinline__ void publish(int *f) {
     if (threadIdx.x == 0) st_release_gpu(f, 1);
 }
 
-template <class TF>
-__device__ void chol_chain(TF *A, int64_t n, int nblk, TF *dinv, int *F, int *U, int *abort_w,
+__device__ void chol_chain(float *A, int64_t n, int nblk, float *dinv, int *F, int *U, int *abort_w,
                            int32_t *err, unsigned char *smem_raw) {
-    TF(*b0)[kTileLd] = reinterpret_cast<TF(*)[kTileLd]>(smem_raw);
-    TF(*b1)[kTileLd] = b0 + NB;
-    TF(*xt)[kTileLd] = b1 + NB;   // L_{j+1,j}^T (from the sub-solve, for the next update)
-    TF(*at)[kTileLd] = xt + NB;   // A_{j+1,j}^T as the sub-solve reads it
-    TF(*a_s)[NB + 1] = reinterpret_cast<TF(*)[NB + 1]>(&b0[0][0]);
-    TF(*x_s)[NB + 1] = reinterpret_cast<TF(*)[NB + 1]>(&b1[0][0]);
+    float (*b0)[kTileLd] = reinterpret_cast<float (*)[kTileLd]>(smem_raw);
+    float (*b1)[kTileLd] = b0 + NB;
+    float (*xt)[kTileLd] = b1 + NB;   // L_{j+1,j}^T (from the sub-solve, for the next update)
+    float (*at)[kTileLd] = xt + NB;   // A_{j+1,j}^T as the sub-solve reads it
+    float (*a_s)[NB + 1] = reinterpret_cast<float (*)[NB + 1]>(&b0[0][0]);
+    float (*x_s)[NB + 1] = reinterpret_cast<float (*)[NB + 1]>(&b1[0][0]);
     __shared__ int s_ok, s_pre;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    TF acc[2][4];   // the diagonal tile A~_jj of the coming step (loaded one step ahead)
+    float acc[2][4];   // the diagonal tile A~_jj of the coming step (loaded one step ahead)
     if (tid == 0) s_ok = wait_tile(&U[tile_id(0, 0)], abort_w, err);
     __syncthreads();
     if (!s_ok) return;
-    load_acc<TF>(A, n, 0, 0, true, acc, tx, ty);
+    load_acc(A, n, 0, 0, true, acc, tx, ty);
     for (int j = 0; j < nblk; j++) {
         const int64_t c0 = (int64_t)j * NB, r0 = c0 + NB;
         const bool next = j + 1 < nblk;
-        if (j > 0) tile_gemm_T<TF, true>(acc, xt, xt, tx, ty);   // the update k = j - 1
+        if (j > 0) tile_gemm_T<true>(acc, xt, xt, tx, ty);   // the update k = j - 1
 #pragma unroll
         for (int p = 0; p < 2; p++)
 #pragma unroll
             for (int q = 0; q < 4; q++) a_s[ty * 2 + p][tx * 4 + q] = acc[p][q];
         __syncthreads();
-        potrf_inv_smem<TF>(a_s, x_s, (int)min((int64_t)NB, n - c0), c0, err);
+        potrf_inv_smem<float, NB>(a_s, x_s, (int)min((int64_t)NB, n - c0), c0, err);
         if (next) {
             // L_{j+1,j} = A~_{j+1,j} L_jj^{-T}, computed transposed: xt = L_jj^{-1} A~_{j+1,j}^T
             // the next diagonal tile's flag is looked at now, beside this wait, and once more
@@ -224,18 +220,18 @@ __device__ void chol_chain(TF *A, int64_t n, int nblk, TF *dinv, int *F, int *U,
             if (tid == 32) s_pre = ld_acquire_gpu(&U[tile_id(j + 1, j + 1)]) != 0;
             __syncthreads();
             if (!s_ok) return;
-            load_tile_T<TF>(A + r0 * n + c0, n, n - r0, at);   // at[k][r] = A_{j+1,j}[r][k]
+            load_tile_T(A + r0 * n + c0, n, n - r0, at);   // at[k][r] = A_{j+1,j}[r][k]
             __syncthreads();
-            TF o[2][4];
+            float o[2][4];
 #pragma unroll
             for (int p = 0; p < 2; p++)
 #pragma unroll
-                for (int q = 0; q < 4; q++) o[p][q] = TF(0);
+                for (int q = 0; q < 4; q++) o[p][q] = 0.f;
 #pragma unroll 8
             for (int k = 0; k < NB; k++) {
-                TF v[4];
-                lds4<TF>(&at[k][tx * 4], v);
-                const TF u0 = x_s[ty * 2][k], u1 = x_s[ty * 2 + 1][k];
+                float v[4];
+                lds4<float>(&at[k][tx * 4], v);
+                const float u0 = x_s[ty * 2][k], u1 = x_s[ty * 2 + 1][k];
 #pragma unroll
                 for (int q = 0; q < 4; q++) {
                     o[0][q] = fma(u0, v[q], o[0][q]);
@@ -245,13 +241,8 @@ __device__ void chol_chain(TF *A, int64_t n, int nblk, TF *dinv, int *F, int *U,
             // o[p][q] = L_{j+1,j}[tx*4+q][ty*2+p]; xt was last read by this step's update
 #pragma unroll
             for (int p = 0; p < 2; p++) {
-                TF *dst = &xt[ty * 2 + p][tx * 4];
-                if constexpr (sizeof(TF) == 4) {
-                    *reinterpret_cast<float4 *>(dst) = make_float4(o[p][0], o[p][1], o[p][2], o[p][3]);
-                } else {
-                    *reinterpret_cast<double2 *>(dst) = make_double2(o[p][0], o[p][1]);
-                    *reinterpret_cast<double2 *>(dst + 2) = make_double2(o[p][2], o[p][3]);
-                }
+                float *dst = &xt[ty * 2 + p][tx * 4];
+                *reinterpret_cast<float4 *>(dst) = make_float4(o[p][0], o[p][1], o[p][2], o[p][3]);
             }
             // the next diagonal tile goes into registers now if it is ready.  It is not
             // waited for here: its task may be queued behind tasks of this column that
@@ -260,11 +251,11 @@ __device__ void chol_chain(TF *A, int64_t n, int nblk, TF *dinv, int *F, int *U,
         }
         __syncthreads();   // xt complete; the next diagonal tile's flag seen
         const bool pre = next && s_pre;
-        if (pre) load_acc<TF>(A, n, r0, r0, true, acc, tx, ty);
+        if (pre) load_acc(A, n, r0, r0, true, acc, tx, ty);
         // L_jj^{-1} into dinv, L_{j+1,j} into A: rows of 64, coalesced.  L_jj itself is not
         // stored: every solve with the factor applies L_jj^{-1}, so A's diagonal tiles keep
         // their last update.
-        TF *Lj = dinv + (int64_t)j * NB * NB;
+        float *Lj = dinv + (int64_t)j * NB * NB;
         for (int e = tid; e < NB * NB; e += blockDim.x) {
             const int i = e >> 6, c = e & 63;
             Lj[e] = x_s[i][c];
@@ -279,22 +270,21 @@ __device__ void chol_chain(TF *A, int64_t n, int nblk, TF *dinv, int *F, int *U,
             if (tid == 0) s_ok = wait_tile(&U[tile_id(j + 1, j + 1)], abort_w, err);
             __syncthreads();
             if (!s_ok) return;
-            load_acc<TF>(A, n, r0, r0, true, acc, tx, ty);
+            load_acc(A, n, r0, r0, true, acc, tx, ty);
         }
     }
 }
 
-template <class TF>
-__global__ void __launch_bounds__(512, 1) k_chol_tiles(TF *A, int64_t n, int nblk, TF *dinv,
+__global__ void __launch_bounds__(512, 1) k_chol_tiles(float *A, int64_t n, int nblk, float *dinv,
                                                        int *flags, int32_t *err) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    TF(*b0)[kTileLd] = reinterpret_cast<TF(*)[kTileLd]>(smem_raw);
-    TF(*b1)[kTileLd] = b0 + NB;
+    float (*b0)[kTileLd] = reinterpret_cast<float (*)[kTileLd]>(smem_raw);
+    float (*b1)[kTileLd] = b0 + NB;
     __shared__ int s_task, s_ok, s_fa, s_fb, s_pa[2], s_pb[2];
     const int ntask = nblk * (nblk + 1) / 2;
     int *F = flags, *U = flags + ntask, *ticket = flags + 2 * ntask, *abort_w = ticket + 1;
     if (blockIdx.x == 0) {
-        chol_chain<TF>(A, n, nblk, dinv, F, U, abort_w, err, smem_raw);
+        chol_chain(A, n, nblk, dinv, F, U, abort_w, err, smem_raw);
         return;
     }
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;   // rows ty*2+{0,1}, cols tx*4+{0..3}
@@ -309,27 +299,27 @@ __global__ void __launch_bounds__(512, 1) k_chol_tiles(TF *A, int64_t n, int nbl
         const int64_t r0 = (int64_t)i * NB, c0 = (int64_t)j * NB;
         const int64_t rows_i = n - r0;
         const int kmax = i == j ? max(j - 1, 0) : j;   // the chain applies k = j - 1 to (j, j)
-        TF acc[2][4];
-        load_acc<TF>(A, n, r0, c0, false, acc, tx, ty);
+        float acc[2][4];
+        load_acc(A, n, r0, c0, false, acc, tx, ty);
         // Updates k = 0 .. kmax-1, pipelined: the tiles L_ik, L_jk of update k + 1 are
         // loaded into registers while update k's product runs (when their flags are
         // already set; otherwise after it, with a blocking wait), and stored into the other
         // pair of shared tiles.  Threads 0 and 32 read the two flags at the same time.
-        TF va[8], vb[8];
+        float va[8], vb[8];
         bool have = false;   // va / vb hold the tiles of update k
         for (int k = 0; k < kmax; k++) {
-            TF(*ta)[kTileLd] = b0 + (k & 1) * 2 * NB;
-            TF(*tb)[kTileLd] = ta + NB;
+            float (*ta)[kTileLd] = b0 + (k & 1) * 2 * NB;
+            float (*tb)[kTileLd] = ta + NB;
             if (!have) {
                 if (tid == 0) s_fa = wait_tile(&F[tile_id(i, k)], abort_w, err);
                 if (tid == 32) s_fb = wait_tile(&F[tile_id(j, k)], abort_w, err);
                 __syncthreads();
                 if (!(s_fa && s_fb)) return;
-                tile_regs<TF>(A + r0 * n + (int64_t)k * NB, n, rows_i, va);
-                if (i != j) tile_regs<TF>(A + c0 * n + (int64_t)k * NB, n, n - c0, vb);
+                tile_regs(A + r0 * n + (int64_t)k * NB, n, rows_i, va);
+                if (i != j) tile_regs(A + c0 * n + (int64_t)k * NB, n, n - c0, vb);
             }
-            tile_store_T<TF>(va, ta);
-            if (i != j) tile_store_T<TF>(vb, tb);
+            tile_store_T(va, ta);
+            if (i != j) tile_store_T(vb, tb);
             const int q = (k + 1) & 1;
             if (k + 1 < kmax) {   // a look at update k + 1's flags, without waiting
                 if (tid == 0) s_pa[q] = ld_acquire_gpu(&F[tile_id(i, k + 1)]) != 0;
@@ -339,20 +329,20 @@ __global__ void __launch_bounds__(512, 1) k_chol_tiles(TF *A, int64_t n, int nbl
                                // is no longer read); update k + 1's flags seen
             have = k + 1 < kmax && s_pa[q] && s_pb[q];
             if (have) {
-                tile_regs<TF>(A + r0 * n + (int64_t)(k + 1) * NB, n, rows_i, va);
-                if (i != j) tile_regs<TF>(A + c0 * n + (int64_t)(k + 1) * NB, n, n - c0, vb);
+                tile_regs(A + r0 * n + (int64_t)(k + 1) * NB, n, rows_i, va);
+                if (i != j) tile_regs(A + c0 * n + (int64_t)(k + 1) * NB, n, n - c0, vb);
             }
-            tile_gemm_T<TF, true>(acc, ta, i == j ? ta : tb, tx, ty);
+            tile_gemm_T<true>(acc, ta, i == j ? ta : tb, tx, ty);
         }
         __syncthreads();   // the last product is done before the shared tiles are reused
         if (i <= j + 1) {
             // diagonal or sub-diagonal tile: the chain finishes it
-            store_acc<TF>(A, n, r0, c0, acc, tx, ty);
+            store_acc(A, n, r0, c0, acc, tx, ty);
             publish(&U[tile_id(i, j)]);
             continue;
         }
         // L_ij = A_ij L_jj^{-T}: o[p][q] = sum_c acc[ty*2+p][c] Linv[tx*4+q][c]
-        TF(*a)[NB + 1] = reinterpret_cast<TF(*)[NB + 1]>(smem_raw);   // overlays b0 only
+        float (*a)[NB + 1] = reinterpret_cast<float (*)[NB + 1]>(smem_raw);   // overlays b0 only
 #pragma unroll
         for (int p = 0; p < 2; p++)
 #pragma unroll
@@ -360,25 +350,25 @@ __global__ void __launch_bounds__(512, 1) k_chol_tiles(TF *A, int64_t n, int nbl
         if (tid == 0) s_ok = wait_tile(&F[tile_id(j, j)], abort_w, err);
         __syncthreads();
         if (!s_ok) return;
-        load_tile_T<TF>(dinv + (int64_t)j * NB * NB, NB, NB, b1);   // b1[c][q] = Linv[q][c]
+        load_tile_T(dinv + (int64_t)j * NB * NB, NB, NB, b1);   // b1[c][q] = Linv[q][c]
         __syncthreads();
-        TF o[2][4];
+        float o[2][4];
 #pragma unroll
         for (int p = 0; p < 2; p++)
 #pragma unroll
-            for (int q = 0; q < 4; q++) o[p][q] = TF(0);
+            for (int q = 0; q < 4; q++) o[p][q] = 0.f;
 #pragma unroll 8
         for (int c = 0; c < NB; c++) {
-            TF v[4];
-            lds4<TF>(&b1[c][tx * 4], v);
-            const TF u0 = a[ty * 2][c], u1 = a[ty * 2 + 1][c];
+            float v[4];
+            lds4<float>(&b1[c][tx * 4], v);
+            const float u0 = a[ty * 2][c], u1 = a[ty * 2 + 1][c];
 #pragma unroll
             for (int q = 0; q < 4; q++) {
                 o[0][q] = fma(u0, v[q], o[0][q]);
                 o[1][q] = fma(u1, v[q], o[1][q]);
             }
         }
-        store_acc<TF>(A, n, r0, c0, o, tx, ty);
+        store_acc(A, n, r0, c0, o, tx, ty);
         publish(&F[tile_id(i, j)]);
     }
 }
@@ -457,8 +447,7 @@ __global__ void __launch_bounds__(256) k_btrsm_update(const BatchTrsmDesc *__res
     }
 }
 
-template <class TF>
-int chol_tiles_t(TF *A, int64_t n, cudaStream_t s, Mesh *m) {
+int chol_tiles(float *A, int64_t n, cudaStream_t s, Mesh *m) {
     if (n <= 0) return FEM3_OK;
     const int nblk = (int)((n + NB - 1) / NB);
     const int ntask = nblk * (nblk + 1) / 2;
@@ -472,8 +461,8 @@ int chol_tiles_t(TF *A, int64_t n, cudaStream_t s, Mesh *m) {
     // one CTA per SM: the chain CTA gets an SM of its own
     const int grid = std::min(ntask + 1, std::max(sms, 2));
     kc_begin(m, KC_FACTOR);
-    k_chol_tiles<TF><<<grid, 512, kCholTilesSmem * sizeof(TF), s>>>(
-        A, n, nblk, reinterpret_cast<TF *>(m->dinv), m->chol_flags, m->err);
+    k_chol_tiles<<<grid, 512, kCholTilesSmem * sizeof(float), s>>>(
+        A, n, nblk, reinterpret_cast<float *>(m->dinv), m->chol_flags, m->err);
     kc_end(m, KC_FACTOR);
     note_launch(m);
     FEM3_CUDA(cudaGetLastError());
@@ -1130,31 +1119,20 @@ int load_vector_T(Mesh *m, const double *lam_d, double *out_d) {
     return FEM3_OK;
 }
 
-// The factorisation is a fixed sequence of ~3 n/64 launches for a given handle and
-// precision.  The first factorisation of a handle launches it directly; a second one
-// (a new assemble with other alpha or K on the same mesh) captures the sequence into a
-// CUDA graph on a private stream, and later ones replay the graph on the caller's stream.
-static int chol_attributes() {
-    static bool done = false;
-    if (done) return FEM3_OK;
-    FEM3_CUDA(cudaFuncSetAttribute(k_chol_tiles<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)(kCholTilesSmem * sizeof(double))));
-    FEM3_CUDA(cudaFuncSetAttribute(k_chol_tiles<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)(kCholTilesSmem * sizeof(float))));
-    done = true;
-    return FEM3_OK;
-}
-
 // FP32 factorisations of at least this order take the blocked factorisation with
 // tensor-core trailing updates (chol_tc.cu); smaller ones the one-launch tile-task
 // factorisation, whose diagonal chain is the shorter critical path there.
 constexpr int64_t kCholTcMinN = 4096;
 
 int factor(Mesh *m) {
-    FEM3_TRY(chol_attributes());
     m->chol_tc_used = false;
     if (m->precision == FEM3_FP64) {
-        FEM3_TRY(chol_tiles_t<double>(m->A64, m->n_dof, m->stream, m));
+        int launches = 0;
+        kc_begin(m, KC_FACTOR);
+        FEM3_TRY(chol_f64(m->A64, m->n_dof, reinterpret_cast<double *>(m->dinv), m->chol_flags,
+                          m->err, m->stream, &launches));
+        kc_end(m, KC_FACTOR);
+        m->launches += launches;
         return solve_prep_t<double>(m->A64, m->n_dof, m->stream, m);
     }
     const bool tc = m->chol_tc_opt > 0 || (m->chol_tc_opt == 0 && m->n_dof >= kCholTcMinN);
@@ -1162,7 +1140,13 @@ int factor(Mesh *m) {
         FEM3_TRY(chol_tc(m, m->A32, m->n_dof));
         m->chol_tc_used = true;
     } else {
-        FEM3_TRY(chol_tiles_t<float>(m->A32, m->n_dof, m->stream, m));
+        static bool attr = false;
+        if (!attr) {
+            FEM3_CUDA(cudaFuncSetAttribute(k_chol_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)(kCholTilesSmem * sizeof(float))));
+            attr = true;
+        }
+        FEM3_TRY(chol_tiles(m->A32, m->n_dof, m->stream, m));
     }
     return solve_prep_t<float>(m->A32, m->n_dof, m->stream, m);
 }

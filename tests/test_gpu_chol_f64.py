@@ -1,0 +1,37 @@
+"""The FP64 tile factorisation (csrc/chol_f64.cu) at the edges of its 32-column tiles and of
+the 64-column diagonal inverses that the solves use: integer-order problems of chosen order
+against the oracle's matrix, solved by numpy."""
+import numpy as np
+import pytest
+
+import oracle
+from test_gpu_contract_rows import _bar_mesh
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA device", allow_module_level=True)
+
+from paper_1811_03339_gb300 import fem3  # noqa: E402
+
+# interior dofs of a box of cells: (a - 1)(b - 1)(c - 1)
+SIZES = {1: (2, 2, 2), 8: (3, 3, 3), 9: (10, 2, 2), 31: (32, 2, 2), 32: (3, 5, 5), 33: (4, 12, 2),
+         63: (8, 10, 2), 64: (5, 5, 5), 65: (6, 14, 2), 96: (4, 5, 9), 98: (8, 15, 2),
+         130: (14, 11, 2)}
+
+
+@pytest.mark.parametrize("n", sorted(SIZES))
+def test_f64_factor_sizes(n):
+    mesh = _bar_mesh(SIZES[n])
+    o = oracle.Oracle.from_mesh(mesh)
+    assert o.n_dof == n
+    K = (1.0, 2.0, 0.5)
+    A = o.assemble((2.0, 2.0, 2.0), K)
+    f = np.random.default_rng(n).standard_normal((mesh.n_nodes, 3))
+    m = fem3.Mesh(mesh.verts, mesh.tets)
+    m.assemble_integer(K)
+    u = m.solve(f).cpu().numpy().reshape(n, 3)
+    ref = np.linalg.solve(A, o.load(f))
+    assert np.linalg.norm(u - ref) <= 1e-10 * np.linalg.norm(ref)
+    m.free()
