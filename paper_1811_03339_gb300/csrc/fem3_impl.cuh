@@ -156,6 +156,7 @@ struct Mesh {
     bool tc_tuned = false;     // the last contraction ran the tuner
     bool ap_ready = false;     // ap_R holds W R of the current tables
     bool integer_order = false;   // the matrix came from fem3_assemble_integer (no tables)
+    int32_t *p1_first = nullptr;  // integer order: first tile column of each block row of A64
     double *form_wc = nullptr;    // general form: w c per Gauss point, and per slot of one axis
     double *A_ns = nullptr;       // divergence-form (non-symmetric) matrix, FP64 [n_dof][n_dof]
     bool nonsym = false;          // the current operator is A_ns (GMRES solve)

@@ -6,17 +6,19 @@
 // (its one-sided order-1 derivatives are the slope on the Gauss point's tet, and
 // s_i = -1/2); this is its fast special case.  The matrix is FP64 and is solved by the
 // FP64 form.
+#include "chol_f64.cuh"
 #include "fem3_impl.cuh"
 
 namespace fem3 {
 
 namespace {
 
-// one thread per tet: the 4 x 4 element matrix added into the dof rows and columns
+// one thread per tet: the 4 x 4 element matrix added into the dof rows and columns, and the
+// matrix's profile by the factorisation's tiles (first[i] starts at its largest value)
 __global__ void k_p1_stiffness(const double *__restrict__ M, const double *__restrict__ vol,
                                const int32_t *__restrict__ tets, const int32_t *__restrict__ dof,
                                int64_t n_tets, double K0, double K1, double K2, double *A,
-                               int64_t n) {
+                               int64_t n, int32_t *first) {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= n_tets) return;
     const double *Mt = M + 16 * t;
@@ -27,8 +29,13 @@ __global__ void k_p1_stiffness(const double *__restrict__ M, const double *__res
         j[a] = dof[tets[4 * t + a]];
         for (int i = 0; i < 3; i++) g[a][i] = Mt[4 * a + 1 + i];
     }
+    int32_t lo = INT32_MAX;
+    for (int a = 0; a < 4; a++)
+        if (j[a] >= 0) lo = min(lo, j[a]);
     for (int a = 0; a < 4; a++) {
         if (j[a] < 0) continue;
+        int32_t *fr = first + j[a] / kChol64Tile;
+        if (lo / kChol64Tile < *fr) atomicMin(fr, lo / kChol64Tile);
         for (int b = 0; b < 4; b++) {
             if (j[b] < 0) continue;
             const double e = v * (K0 * g[a][0] * g[b][0] + K1 * g[a][1] * g[b][1] +
@@ -100,11 +107,15 @@ int assemble_integer(Mesh *m, const double K[3]) {
     cudaStream_t s = m->stream;
     const int64_t n = m->n_dof;
     if (!m->A64) FEM3_TRY(dev_alloc_t(m, &m->A64, n * n));
+    const int64_t nblk = std::max<int64_t>(1, (n + kChol64Tile - 1) / kChol64Tile);
+    if (!m->p1_first) FEM3_TRY(dev_alloc_t(m, &m->p1_first, nblk));
     FEM3_CUDA(cudaMemsetAsync(m->A64, 0, sizeof(double) * n * n, s));
+    FEM3_CUDA(cudaMemsetAsync(m->p1_first, 0x7f, sizeof(int32_t) * nblk, s));
     if (n > 0 && m->n_tets > 0) {
         kc_begin(m, KC_CONTRACT);
         k_p1_stiffness<<<grid_tets(m->n_tets), 256, 0, s>>>(m->M, m->vol, m->tets, m->dof,
-                                                             m->n_tets, K[0], K[1], K[2], m->A64, n);
+                                                             m->n_tets, K[0], K[1], K[2], m->A64, n,
+                                                             m->p1_first);
         kc_end(m, KC_CONTRACT);
         note_launch(m);
     }

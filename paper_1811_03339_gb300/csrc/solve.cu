@@ -1129,8 +1129,9 @@ int factor(Mesh *m) {
     if (m->precision == FEM3_FP64) {
         int launches = 0;
         kc_begin(m, KC_FACTOR);
-        FEM3_TRY(chol_f64(m->A64, m->n_dof, reinterpret_cast<double *>(m->dinv), m->chol_flags,
-                          m->err, m->stream, &launches));
+        FEM3_TRY(chol_f64(m->A64, m->n_dof, reinterpret_cast<double *>(m->dinv),
+                          m->integer_order ? m->p1_first : nullptr, m->chol_flags, m->err,
+                          m->stream, &launches));
         kc_end(m, KC_FACTOR);
         m->launches += launches;
         return solve_prep_t<double>(m->A64, m->n_dof, m->stream, m);
