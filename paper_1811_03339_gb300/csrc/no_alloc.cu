@@ -4,20 +4,22 @@
 // latency-critical loops that must never enter the allocator, and host applications or
 // plugin hosts that own every device allocation themselves and hand the library only the
 // buffers of the problem.  This entry point serves them: its working memory (the
-// Cholesky factor, the inverse of the current 64 x 64 diagonal block and an error word)
-// is one file-scope static device array, so the caller passes only the matrix, the
-// right-hand side and the output.  Each call ends by reading the error word back and
+// Cholesky factor, the inverses of its 64 x 64 diagonal blocks, flags and error words) is
+// one file-scope static device array, so the caller passes only the matrix, the
+// right-hand side and the output.  Each call ends by reading the error words back and
 // synchronising its stream.
 //
-// The factorisation is its own multi-launch blocked right-looking Cholesky (64-wide
-// blocks: diagonal factor and inverse, panel product, trailing update of the lower
-// triangle, one launch each per block column) followed by blocked forward and backward
-// substitution.  It shares no kernel with fem3_solve, whose FP64 form serves only as the
-// reference in the test of this entry point.
+// Three steps: copy A (the factorisation works in place), the FP64 tile factorisation of
+// chol_f64.cu, and one launch for both substitutions (k_na_solve).  What bounds it is the
+// factorisation's diagonal chain (12 steps of 28 us at n = 384) and, for the substitutions,
+// a hand-over between SMs per 64-row block.  Measured at n = 384 (GB300): 2.58 ms as one
+// launch per 64-column step and phase, with a column-by-column 64 x 64 factor and one-warp
+// substitutions; 0.42 ms now.
 #include <math.h>
 
 #include <mutex>
 
+#include "chol_f64.cuh"
 #include "fem3_impl.cuh"
 
 namespace fem3 {
@@ -27,161 +29,136 @@ namespace {
 constexpr int kNaMaxN = 512;   // largest system this entry point accepts
 constexpr int NBS = 64;
 
-// factor [kNaMaxN^2] | diagonal-block inverse [64*64] | error word (as 8 doubles)
+// factor [kNaMaxN^2] | diagonal-block inverses [8][64 * 64] | flags of the factorisation, then
+// of the substitutions (2 kNaBlocks, a ticket, an abort word) | ERR_COUNT error words
+constexpr int kNaBlocks = kNaMaxN / NBS;
 constexpr size_t kNaFactor = (size_t)kNaMaxN * kNaMaxN;
-constexpr size_t kNaElems = kNaFactor + NBS * NBS + 8;
+constexpr size_t kNaInv = (size_t)kNaBlocks * NBS * NBS;
+constexpr int kNaCholTiles = kNaMaxN / kChol64Tile;
+constexpr size_t kNaCholFlags = (size_t)kNaCholTiles * (kNaCholTiles + 1) + 2;
+constexpr size_t kNaSolveFlags = 2 * kNaBlocks + 2;
+constexpr size_t kNaElems =
+    kNaFactor + kNaInv + (kNaCholFlags + kNaSolveFlags + ERR_COUNT + 1) / 2;
 static __device__ __align__(256) double g_na_scratch[kNaElems];
+
+#include "chol_smem.cuh"
 
 std::mutex g_na_mutex;
 void *g_na_ptr[256];   // per device: device address of g_na_scratch (host-side table)
 
-// F = A (row-major n x n), x = b
-__global__ void k_na_copy(const double *__restrict__ A, const double *__restrict__ b, int n,
-                          double *F, double *x) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < (int64_t)n * n) F[i] = A[i];
-    if (i < n) x[i] = b[i];
+// F = the lower triangle of A (row-major n x n); flags and error words cleared
+__global__ void __launch_bounds__(256) k_na_copy(const double *__restrict__ A, int n, double *F,
+                                                 int *flags, int n_flags) {
+    const int i = blockIdx.x;
+    for (int c = threadIdx.x; c <= i; c += blockDim.x) F[(int64_t)i * n + c] = A[(int64_t)i * n + c];
+    if (i == 0)
+        for (int q = threadIdx.x; q < n_flags; q += blockDim.x) flags[q] = 0;
 }
 
-__global__ void __launch_bounds__(256) k_na_potrf_inv(double *F, int n, int k0, double *Linv,
-                                                      int *err) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double(*a)[NBS + 1] = reinterpret_cast<double(*)[NBS + 1]>(smem_raw);
-    double(*li)[NBS + 1] = a + NBS;
-    const int nb = min(NBS, n - k0);
-    for (int e = threadIdx.x; e < NBS * NBS; e += blockDim.x) {
-        int i = e / NBS, j = e % NBS;
-        a[i][j] = (i < nb && j < nb) ? F[(int64_t)(k0 + i) * n + k0 + j] : (i == j ? 1.0 : 0.0);
-    }
-    __syncthreads();
-    for (int j = 0; j < nb; j++) {
-        if (threadIdx.x == 0) {
-            double d = a[j][j];
-            if (!(d > 0.0)) {
-                atomicCAS(err, 0, k0 + j + 1);
-                d = 1.0;
-            }
-            a[j][j] = sqrt(d);
-        }
-        __syncthreads();
-        double djj = a[j][j];
-        for (int i = j + 1 + threadIdx.x; i < nb; i += blockDim.x) a[i][j] /= djj;
-        __syncthreads();
-        const int m = nb - j - 1;
-        for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-            int i = j + 1 + e / m, c = j + 1 + e % m;
-            if (c <= i) a[i][c] -= a[i][j] * a[c][j];
-        }
-        __syncthreads();
-    }
-    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-        int i = e / nb, j = e % nb;
-        F[(int64_t)(k0 + i) * n + k0 + j] = j <= i ? a[i][j] : 0.0;
-    }
-    if (threadIdx.x < NBS) {
-        const int c = threadIdx.x;
-        for (int r = 0; r < NBS; r++) li[r][c] = 0.0;
-        li[c][c] = 1.0 / a[c][c];
-        for (int r = c + 1; r < NBS; r++) {
-            double s = 0.0;
-            for (int k = c; k < r; k++) s += a[r][k] * li[k][c];
-            li[r][c] = -s / a[r][r];
-        }
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < NBS * NBS; e += blockDim.x) Linv[e] = li[e / NBS][e % NBS];
-}
-
-__global__ void __launch_bounds__(256) k_na_trsm(double *F, int n, int k0, const double *Linv) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double(*bt)[NBS + 1] = reinterpret_cast<double(*)[NBS + 1]>(smem_raw);
-    double(*li)[NBS + 1] = bt + NBS;
-    const int row0 = k0 + NBS + blockIdx.x * NBS;
-    for (int e = threadIdx.x; e < NBS * NBS; e += blockDim.x) {
-        int i = e / NBS, j = e % NBS;
-        bt[i][j] = (row0 + i < n) ? F[(int64_t)(row0 + i) * n + k0 + j] : 0.0;
-        li[i][j] = Linv[e];
-    }
-    __syncthreads();
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    double acc[4][4] = {};
-    for (int k = 0; k < NBS; k++)
-        for (int p = 0; p < 4; p++)
-            for (int q = 0; q < 4; q++) acc[p][q] = fma(bt[ty * 4 + p][k], li[tx * 4 + q][k], acc[p][q]);
-    for (int p = 0; p < 4; p++) {
-        int r = row0 + ty * 4 + p;
-        if (r >= n) continue;
-        for (int q = 0; q < 4; q++) F[(int64_t)r * n + k0 + tx * 4 + q] = acc[p][q];
-    }
-}
-
-__global__ void __launch_bounds__(256) k_na_syrk(double *F, int n, int k0) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double(*pi)[NBS + 1] = reinterpret_cast<double(*)[NBS + 1]>(smem_raw);
-    double(*pj)[NBS + 1] = pi + NBS;
-    int idx = blockIdx.x, ti = 0;
-    while (idx > ti) { idx -= ti + 1; ti++; }
-    const int tj = idx;
-    const int i0 = k0 + NBS + ti * NBS, j0 = k0 + NBS + tj * NBS;
-    for (int e = threadIdx.x; e < NBS * NBS; e += blockDim.x) {
-        int r = e / NBS, c = e % NBS;
-        pi[r][c] = (i0 + r < n) ? F[(int64_t)(i0 + r) * n + k0 + c] : 0.0;
-        pj[r][c] = (j0 + r < n) ? F[(int64_t)(j0 + r) * n + k0 + c] : 0.0;
-    }
-    __syncthreads();
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    double acc[4][4] = {};
-    for (int c = 0; c < NBS; c++)
-        for (int a = 0; a < 4; a++)
-            for (int b = 0; b < 4; b++) acc[a][b] = fma(pi[ty * 4 + a][c], pj[tx * 4 + b][c], acc[a][b]);
-    for (int a = 0; a < 4; a++) {
-        int r = i0 + ty * 4 + a;
-        if (r >= n) continue;
-        for (int b = 0; b < 4; b++) {
-            int c = j0 + tx * 4 + b;
-            if (c < n && c <= r) F[(int64_t)r * n + c] -= acc[a][b];
-        }
-    }
-}
-
-// substitution on one 64-row block by one warp (backward = 1 uses the transpose)
-__global__ void k_na_trsv_diag(const double *F, int n, int k0, double *y, int backward) {
-    const int nb = min(NBS, n - k0), lane = threadIdx.x;
-    double t0 = lane < nb ? y[k0 + lane] : 0.0, t1 = lane + 32 < nb ? y[k0 + lane + 32] : 0.0;
-    if (!backward) {
-        for (int c = 0; c < nb; c++) {
-            double tc = c < 32 ? __shfl_sync(0xffffffffu, t0, c) : __shfl_sync(0xffffffffu, t1, c - 32);
-            double v = tc / F[(int64_t)(k0 + c) * n + k0 + c];
-            if (lane == (c & 31)) { if (c < 32) t0 = v; else t1 = v; }
-            if (lane > c && lane < nb) t0 -= F[(int64_t)(k0 + lane) * n + k0 + c] * v;
-            if (lane + 32 > c && lane + 32 < nb) t1 -= F[(int64_t)(k0 + lane + 32) * n + k0 + c] * v;
-        }
-    } else {
-        for (int c = nb - 1; c >= 0; c--) {
-            double tc = c < 32 ? __shfl_sync(0xffffffffu, t0, c) : __shfl_sync(0xffffffffu, t1, c - 32);
-            double v = tc / F[(int64_t)(k0 + c) * n + k0 + c];
-            if (lane == (c & 31)) { if (c < 32) t0 = v; else t1 = v; }
-            if (lane < c) t0 -= F[(int64_t)(k0 + c) * n + k0 + lane] * v;
-            if (lane + 32 < c) t1 -= F[(int64_t)(k0 + c) * n + k0 + lane + 32] * v;
-        }
-    }
-    if (lane < nb) y[k0 + lane] = t0;
-    if (lane + 32 < nb) y[k0 + lane + 32] = t1;
-}
-
-// forward: rows below the block; backward: rows above the block
-__global__ void k_na_trsv_update(const double *F, int n, int k0, double *y, int backward) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nb = min(NBS, n - k0);
+// part[16 columns 16 q ..] of row r of a 64 x 64 block times v: thread (r, q)
+__device__ __forceinline__ double dot16(const double m[16], const double *v, int q) {
     double s = 0.0;
-    if (!backward) {
-        if (i < k0 + nb || i >= n) return;
-        for (int c = 0; c < nb; c++) s += F[(int64_t)i * n + k0 + c] * y[k0 + c];
-    } else {
-        if (i >= k0) return;
-        for (int c = 0; c < nb; c++) s += F[(int64_t)(k0 + c) * n + i] * y[k0 + c];
+#pragma unroll
+    for (int e = 0; e < 16; e++) s = fma(m[e], v[16 * q + e], s);
+    return s;
+}
+
+// Both substitutions in one launch: L y = b, then L^T x = y, in blocks of 64 rows.  A CTA takes
+// roles from a ticket: role s < nb is the forward step of block s, role nb + s the backward
+// step of block nb - 1 - s.  A step reads the tiles of its block row (column) into registers
+// one ahead, adds each solved block as its flag appears, multiplies by the diagonal inverse
+// and publishes the block.  A role waits only for earlier tickets, so the launch needs no
+// co-residency; the waits are bounded (ERR_SOLVE, abort word).
+// 256 threads, thread (row r = t & 63, quarter q = t >> 6 of the columns).
+__global__ void __launch_bounds__(256) k_na_solve(const double *__restrict__ F,
+                                                  const double *__restrict__ dinv, int n, int nb,
+                                                  const double *__restrict__ b, double *y,
+                                                  double *x, int *flags, int *err) {
+    __shared__ double v[NBS], red[4][NBS];
+    __shared__ int s_role, s_ok;
+    int *done = flags, *ticket = flags + 2 * nb, *abort_w = ticket + 1;
+    const int t = threadIdx.x, r = t & 63, q = t >> 6;
+    for (;;) {
+        if (t == 0) s_role = atomicAdd(ticket, 1);
+        __syncthreads();
+        const int role = s_role;
+        if (role >= 2 * nb) return;
+        const bool bw = role >= nb;
+        const int blk = bw ? 2 * nb - 1 - role : role;   // this step's block
+        const int nd = bw ? role - nb : role;            // blocks it depends on
+        const int row = blk * NBS + r;
+        // the tile between this block and dependency d as applied (transposed when backward)
+        auto tile = [&](int d, double m[16]) {
+            const int jd = bw ? nb - 1 - d : d;
+#pragma unroll
+            for (int e = 0; e < 16; e++) {
+                const int o = jd * NBS + 16 * q + e;     // row of the other block
+                m[e] = (row < n && o < n) ? (bw ? __ldcg(F + (int64_t)o * n + row)
+                                                : __ldcg(F + (int64_t)row * n + o))
+                                          : 0.0;
+            }
+        };
+        double mt[16], mn[16], acc = 0.0;
+        if (nd > 0) tile(0, mt);
+        for (int d = 0; d < nd; d++) {
+            const int jd = bw ? nb - 1 - d : d;
+            if (t == 0) {
+                s_ok = 1;
+                for (int spins = 0; ld_acquire_gpu(&done[bw ? nb + d : d]) == 0; spins++) {
+                    if (ld_acquire_gpu(abort_w) != 0 || spins > kSpinLimit) {
+                        if (spins > kSpinLimit) atomicAdd(&err[ERR_SOLVE], 1);
+                        atomicExch(abort_w, 1);
+                        s_ok = 0;
+                        break;
+                    }
+                }
+            }
+            __syncthreads();
+            if (!s_ok) return;
+            if (t < NBS) v[t] = jd * NBS + t < n ? __ldcg((bw ? x : y) + jd * NBS + t) : 0.0;
+            if (d + 1 < nd) tile(d + 1, mn);
+            __syncthreads();
+            acc += dot16(mt, v, q);
+#pragma unroll
+            for (int e = 0; e < 16; e++) mt[e] = mn[e];
+        }
+        // the diagonal inverse as applied: X or X^T (loaded before the reduction's barriers)
+#pragma unroll
+        for (int e = 0; e < 16; e++) {
+            const int c = 16 * q + e;
+            mt[e] = __ldcg(dinv + (int64_t)blk * NBS * NBS + (bw ? c * NBS + r : r * NBS + c));
+        }
+        red[q][r] = acc;
+        if (bw && nd == 0) {   // y of the last block comes from its forward role
+            if (t == 0) {
+                s_ok = 1;
+                for (int spins = 0; ld_acquire_gpu(&done[nb - 1]) == 0; spins++) {
+                    if (ld_acquire_gpu(abort_w) != 0 || spins > kSpinLimit) {
+                        if (spins > kSpinLimit) atomicAdd(&err[ERR_SOLVE], 1);
+                        atomicExch(abort_w, 1);
+                        s_ok = 0;
+                        break;
+                    }
+                }
+            }
+        } else if (t == 0) {
+            s_ok = 1;
+        }
+        __syncthreads();
+        if (!s_ok) return;
+        if (t < NBS) {
+            const double rhs = blk * NBS + t < n ? (bw ? __ldcg(y + blk * NBS + t) : b[blk * NBS + t])
+                                                 : 0.0;
+            v[t] = rhs - ((red[0][t] + red[1][t]) + (red[2][t] + red[3][t]));
+        }
+        __syncthreads();
+        red[q][r] = dot16(mt, v, q);
+        __syncthreads();
+        if (t < NBS && blk * NBS + t < n)
+            (bw ? x : y)[blk * NBS + t] = (red[0][t] + red[1][t]) + (red[2][t] + red[3][t]);
+        __syncthreads();   // the block's stores are issued before the (cumulative) release
+        if (t == 0) st_release_gpu(&done[role], 1);
     }
-    y[i] -= s;
 }
 
 // device address of the static scratch for the current device (set up once per device)
@@ -194,10 +171,6 @@ int na_scratch(double **out) {
         void *p = nullptr;
         cudaError_t e = cudaGetSymbolAddress(&p, g_na_scratch);
         if (e != cudaSuccess) return cuda_error(e, "cudaGetSymbolAddress(static scratch)");
-        const size_t sh = 2 * NBS * (NBS + 1) * sizeof(double);
-        FEM3_CUDA(cudaFuncSetAttribute(k_na_potrf_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
-        FEM3_CUDA(cudaFuncSetAttribute(k_na_trsm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
-        FEM3_CUDA(cudaFuncSetAttribute(k_na_syrk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
         g_na_ptr[dev] = p;
     }
     *out = static_cast<double *>(g_na_ptr[dev]);
@@ -240,37 +213,24 @@ extern "C" int fem3_spd_solve_static(const double *A, int64_t n, const double *b
     double *scratch = nullptr;
     FEM3_TRY(na_scratch(&scratch));
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    double *F = scratch;
-    double *Linv = scratch + kNaFactor;
-    int *err = reinterpret_cast<int *>(scratch + kNaFactor + NBS * NBS);
-    const int nn = (int)n;
-    const size_t sh = 2 * NBS * (NBS + 1) * sizeof(double);
-    // the error word must start at zero; the factor and inverse are fully rewritten
-    FEM3_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
-    k_na_copy<<<(unsigned)((n * n + 255) / 256), 256, 0, s>>>(A, b, nn, F, x);
-    for (int k0 = 0; k0 < nn; k0 += NBS) {
-        k_na_potrf_inv<<<1, 256, sh, s>>>(F, nn, k0, Linv, err);
-        const int rest = nn - k0 - NBS;
-        if (rest > 0) {
-            const int nblk = (rest + NBS - 1) / NBS;
-            k_na_trsm<<<nblk, 256, sh, s>>>(F, nn, k0, Linv);
-            k_na_syrk<<<nblk * (nblk + 1) / 2, 256, sh, s>>>(F, nn, k0);
-        }
-    }
-    for (int k0 = 0; k0 < nn; k0 += NBS) {
-        k_na_trsv_diag<<<1, 32, 0, s>>>(F, nn, k0, x, 0);
-        if (k0 + NBS < nn) k_na_trsv_update<<<(nn + 255) / 256, 256, 0, s>>>(F, nn, k0, x, 0);
-    }
-    for (int k0 = ((nn - 1) / NBS) * NBS; k0 >= 0; k0 -= NBS) {
-        k_na_trsv_diag<<<1, 32, 0, s>>>(F, nn, k0, x, 1);
-        if (k0 > 0) k_na_trsv_update<<<(k0 + 255) / 256, 256, 0, s>>>(F, nn, k0, x, 1);
-    }
+    const int nn = (int)n, nb = (nn + NBS - 1) / NBS;
+    double *F = scratch, *dinv = F + kNaFactor;
+    int *chol_flags = reinterpret_cast<int *>(dinv + kNaInv);
+    int *flags = chol_flags + kNaCholFlags;
+    int *err = flags + kNaSolveFlags;   // cleared with the substitutions' flags
+    int launches = 0;
+    k_na_copy<<<(unsigned)nn, 256, 0, s>>>(A, nn, F, flags, (int)(kNaSolveFlags + ERR_COUNT));
+    FEM3_TRY(chol_f64(F, n, dinv, nullptr, chol_flags, err, s, &launches));
+    // y shares x: a backward step reads its block of y before it writes that block of x
+    k_na_solve<<<(unsigned)nb, 256, 0, s>>>(F, dinv, nn, nb, b, x, x, flags, err);
     FEM3_CUDA(cudaGetLastError());
-    int h_err = 0;
-    FEM3_CUDA(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    int h_err[ERR_COUNT];
+    FEM3_CUDA(cudaMemcpyAsync(h_err, err, sizeof(h_err), cudaMemcpyDeviceToHost, s));
     FEM3_CUDA(cudaStreamSynchronize(s));
-    if (h_err)
-        return set_error(FEM3_E_NOT_SPD,
-                         "non-positive pivot in Cholesky at column " + std::to_string(h_err - 1));
+    if (h_err[ERR_NOT_SPD])
+        return set_error(FEM3_E_NOT_SPD, "non-positive pivot in Cholesky at column " +
+                                             std::to_string(h_err[ERR_NOT_SPD] - 1));
+    if (h_err[ERR_CHOL] || h_err[ERR_SOLVE])
+        return set_error(FEM3_E_CUDA, "a factorisation or solve wait gave up (bounded wait expired)");
     return FEM3_OK;
 }

@@ -1,6 +1,7 @@
 """The FP64 tile factorisation (csrc/chol_f64.cu) at the edges of its 32-column tiles and of
 the 64-column diagonal inverses that the solves use: integer-order problems of chosen order
-against the oracle's matrix, solved by numpy."""
+against the oracle's matrix, solved by numpy; and the allocation-free solve, which shares it, on dense
+systems of the same kind of sizes."""
 import numpy as np
 import pytest
 
@@ -35,3 +36,19 @@ def test_f64_factor_sizes(n):
     ref = np.linalg.solve(A, o.load(f))
     assert np.linalg.norm(u - ref) <= 1e-10 * np.linalg.norm(ref)
     m.free()
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 63, 64, 65, 127, 160, 384, 511, 512])
+def test_static_solve_sizes(n):
+    """B B^T + n I has a condition number below about 5 (Gaussian B), so numpy's and the
+    library's solutions agree to n u 5 < 3e-13"""
+    rng = np.random.default_rng(n)
+    B = rng.standard_normal((n, n))
+    A, b = B @ B.T + n * np.eye(n), rng.standard_normal(n)
+    x = torch.empty(n, dtype=torch.float64, device="cuda")
+    fem3.spd_solve_static(torch.from_numpy(A).cuda(), torch.from_numpy(b).cuda(), x)
+    ref = np.linalg.solve(A, b)
+    assert np.linalg.norm(x.cpu().numpy() - ref) <= 1e-12 * np.linalg.norm(ref)
+    y = torch.from_numpy(b).cuda()        # in place
+    fem3.spd_solve_static(torch.from_numpy(A).cuda(), y, y)
+    assert torch.equal(x, y)
