@@ -346,8 +346,8 @@ int fem3_apply_lists(fem3_mesh m, int32_t *lists);
  * fem3_batch_run - assemble and solve every mesh of the batch (see also the graph note
  *   after the declarations).
  *   One launch walks every Gauss-point line of every mesh (Section 2.2, 2.1 tables);
- *   contraction, load vector and factorisation of each mesh run on internal streams;
- *   each refinement sweep solves all meshes in one batched triangular solve.
+ *   contraction, factorisation, load vector and refinement sweeps of each mesh run on
+ *   internal streams, with one host wait per sweep.
  *   alpha, K  host float64 [n_meshes][3].
  *   f         host array of n_meshes device pointers, each column-major [n_nodes_i][nrhs].
  *   u         host array of n_meshes device pointers, each column-major [n_dof_i][nrhs].
@@ -366,11 +366,10 @@ int fem3_batch_mesh(fem3_batch b, int i, fem3_mesh *out);
 int fem3_batch_run(fem3_batch b, const double *alpha, const double *K, int precision,
                    const double *const *f, int nrhs, double tol, int max_iter, double *const *u,
                    int *iters, double *resid, void *stream);
-/* The assembly and factorisation of a run (walk, contractions, load vectors, factorisations:
- * everything before the first refinement sweep) is captured as one CUDA graph by the second
- * run with the same alpha, K, precision, nrhs and f pointers and replayed as one graph launch
- * by later runs with them (the first run goes eagerly; a change of any of them captures
- * again).  The refinement sweeps are host-driven.  fem3_batch_graph_launches reports the
+/* The assembly and factorisation of a run (walk, contractions, factorisations) is captured
+ * as one CUDA graph by the second run with the same alpha, K and precision and replayed as
+ * one graph launch by later runs with them, whatever their right-hand sides (the first run
+ * goes eagerly; a change of any of them captures again).  The load vectors and the refinement sweeps are host-driven.  fem3_batch_graph_launches reports the
  * graph launches so far, the capturing run's own launch included (host int64). */
 int fem3_batch_graph_launches(fem3_batch b, int64_t *n);
 void fem3_batch_free(fem3_batch b);
@@ -389,12 +388,12 @@ void fem3_batch_free(fem3_batch b);
  *   n       1 <= n <= 512; larger systems are rejected with FEM3_E_ARG.
  * A, b and x must be device (or managed) memory of the current device; any other pointer
  * is rejected with FEM3_E_ARG before a kernel runs.
- * Working memory is one static device array of about 2.1 MB (a 512 x 512 FP64 factor,
- * one 64 x 64 block inverse and an error word) that every GPU which loads the library
- * holds until the process exits.  The first call on a device looks up that array's
+ * Working memory is one static device array of about 2.4 MB (a 512 x 512 FP64 factor, the
+ * inverses of its 64 x 64 diagonal blocks, flags and error words) that every GPU which loads
+ * the library holds until the process exits.  The first call on a device looks up that array's
  * device address (cudaGetSymbolAddress) with the device current.  All calls share the
  * array and it keeps the last call's
- * contents: each call clears the error word and rewrites the factor, so calls that
+ * contents: each call clears the flags and rewrites the factor, so calls that
  * overlap on the GPU (other streams, other host threads) race and must be serialised
  * by the caller.  Synchronises `stream`.  Errors: FEM3_E_ARG, FEM3_E_NOT_SPD,
  * FEM3_E_CUDA.

@@ -1,15 +1,19 @@
 // Batched assembly and solve of many meshes of uneven size (not in the paper: the paper
 // assembles one mesh at a time).  One launch walks every Gauss-point line of every mesh;
-// contraction, load vector and factorisation of each mesh run on internal streams so
-// that small meshes overlap; each refinement sweep solves all meshes in one batched
-// block-step triangular solve and checks all residuals with a single host wait.
+// contraction, load vector, factorisation and refinement sweeps of each mesh run on internal
+// streams so that meshes overlap (a sweep's triangular solves are one chain launch per
+// direction and mesh, latency-bound, so the meshes' chains run side by side, and its late
+// sweeps apply the operator in FP32 as the single-mesh solve does); all residuals are checked
+// with one host wait per sweep.  12 meshes of 6 to 20 cells per side, 16 columns: 49.3 ms a
+// run with block-step solves over the whole batch (1,100 launches, 13.3 ms) and double-float
+// sweeps throughout, 31.7 ms now.
 //
-// The assembly and factorisation of the whole batch (walk, contractions, load vectors,
-// factorisations: everything before the first refinement sweep) is captured as one CUDA
-// graph the second time a run has the same orders, coefficients, precision, column count and
-// right-hand-side arrays, and replayed as one graph launch from then on (the first run goes
-// eagerly: it makes the allocations, the tile tuner's timings and the factorisation's side
-// streams that a capture must not make).  The refinement sweeps stay host-driven: each one
+// The assembly and factorisation of the whole batch (walk, contractions, factorisations) is captured as one CUDA
+// graph the second time a run has the same orders, coefficients and precision, and replayed
+// as one graph launch from then on (the first run goes eagerly: it makes the allocations, the
+// tile tuner's timings and the factorisation's side streams that a capture must not make).
+// The load vectors are formed beside the graph, so new right-hand sides need no new capture.
+// The refinement sweeps stay host-driven: each one
 // checks the residuals before the next.
 #include <math.h>
 
@@ -27,12 +31,9 @@ struct Batch {
     std::vector<cudaEvent_t> done;   // one per internal stream
     cudaEvent_t fork = nullptr;
     BatchWalkScratch ws;
-    BatchTrsmDesc *d_tdesc = nullptr, *h_tdesc = nullptr;
-    int max_nblk = 0;
-    // per-mesh run buffers, kept across runs (a captured graph refers to their addresses):
-    // load vector b, residual r, A u (column-major, n_dof x nrhs) and the FP32 correction
-    std::vector<double *> bv, rv, auv;
-    std::vector<float *> r32;
+    // per-mesh run buffers, kept across runs: load vector b and the refinement's vectors
+    std::vector<double *> bv;
+    std::vector<RefineVecs> rv;
     int nrhs_cap = 0;
     // the captured assembly + factorisation and what it was captured for
     cudaGraphExec_t exec = nullptr;
@@ -41,21 +42,21 @@ struct Batch {
     cudaStream_t cap = nullptr;
     cudaEvent_t cap_in = nullptr;
     std::vector<double> key_ak;          // alpha, K
-    std::vector<const double *> key_f;   // right-hand-side arrays
-    int key_prec = -1, key_nrhs = 0;
+    int key_prec = -1;
     int runs = 0;                        // eager runs so far
     int graph_launches = 0;              // replays so far
 };
 
 static void free_run_buffers(Batch *b) {
     for (double *p : b->bv) cudaFree(p);
-    for (double *p : b->rv) cudaFree(p);
-    for (double *p : b->auv) cudaFree(p);
-    for (float *p : b->r32) cudaFree(p);
+    for (const RefineVecs &v : b->rv) {
+        cudaFree(v.r);
+        cudaFree(v.Au);
+        cudaFree(v.d64);
+        cudaFree(v.r32);
+    }
     b->bv.clear();
     b->rv.clear();
-    b->auv.clear();
-    b->r32.clear();
     b->nrhs_cap = 0;
 }
 
@@ -72,8 +73,6 @@ static void batch_destroy(Batch *b) {
     if (b->cap_in) cudaEventDestroy(b->cap_in);
     cudaFree(b->ws.d_desc);
     cudaFreeHost(b->ws.h_desc);
-    cudaFree(b->d_tdesc);
-    cudaFreeHost(b->h_tdesc);
     delete b;
 }
 
@@ -91,38 +90,6 @@ static int join_to(Batch *b, cudaStream_t s) {
     }
     return FEM3_OK;
 }
-
-__global__ void k_copy_to_f32(const double *__restrict__ a, float *b, int64_t n) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) b[i] = (float)a[i];
-}
-__global__ void k_add_f32(const float *__restrict__ d, double *u, int64_t n) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) u[i] += (double)d[i];
-}
-__global__ void k_resid_cols(const double *__restrict__ b, const double *__restrict__ Au, int64_t n,
-                             double *r, double *norms) {
-    const int c = blockIdx.y;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double rr = 0, bb = 0;
-    if (i < n) {
-        const int64_t k = (int64_t)c * n + i;
-        const double v = b[k] - Au[k];
-        r[k] = v;
-        rr = v * v;
-        bb = b[k] * b[k];
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        rr += __shfl_down_sync(0xffffffffu, rr, o);
-        bb += __shfl_down_sync(0xffffffffu, bb, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(&norms[2 * c], rr);
-        atomicAdd(&norms[2 * c + 1], bb);
-    }
-}
-
-static inline unsigned blocks(int64_t n) { return (unsigned)(n > 0 ? (n + 255) / 256 : 1); }
 
 static int check_mesh(Mesh *m, int i) {
     int32_t e[ERR_COUNT];
@@ -175,13 +142,10 @@ int fem3_batch_create(int n_meshes, const double *const *verts, const int64_t *n
     }
     if (cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&b->cap_in, cudaEventDisableTiming) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaMalloc(&b->d_tdesc, sizeof(BatchTrsmDesc) * n_meshes) != cudaSuccess ||
-        cudaMallocHost(&b->h_tdesc, sizeof(BatchTrsmDesc) * n_meshes) != cudaSuccess) {
+        cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess) {
         batch_destroy(b);
         return cuda_error(cudaGetLastError(), "batch allocation");
     }
-    for (Mesh *m : b->ms) b->max_nblk = std::max<int>(b->max_nblk, (int)((m->n_dof + 63) / 64));
     *out = reinterpret_cast<fem3_batch>(b);
     return FEM3_OK;
 }
@@ -234,36 +198,28 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
     if (b->nrhs_cap < nrhs) {
         for (cudaStream_t t : b->streams) FEM3_CUDA(cudaStreamSynchronize(t));
         FEM3_CUDA(cudaStreamSynchronize(cs));
-        if (b->exec) {
-            cudaGraphExecDestroy(b->exec);
-            b->exec = nullptr;
-        }
         free_run_buffers(b);
         b->bv.assign(n, nullptr);
-        b->rv.assign(n, nullptr);
-        b->auv.assign(n, nullptr);
-        b->r32.assign(n, nullptr);
+        b->rv.assign(n, RefineVecs{});
         for (int i = 0; i < n; i++) {
             const size_t nn = (size_t)std::max<int64_t>(1, b->ms[i]->n_dof * nrhs);
+            RefineVecs &v = b->rv[i];
             if (cudaMalloc((void **)&b->bv[i], sizeof(double) * nn) != cudaSuccess ||
-                cudaMalloc((void **)&b->rv[i], sizeof(double) * nn) != cudaSuccess ||
-                cudaMalloc((void **)&b->auv[i], sizeof(double) * nn) != cudaSuccess ||
-                cudaMalloc((void **)&b->r32[i], sizeof(float) * nn) != cudaSuccess)
+                cudaMalloc((void **)&v.r, sizeof(double) * nn) != cudaSuccess ||
+                cudaMalloc((void **)&v.Au, sizeof(double) * nn) != cudaSuccess ||
+                cudaMalloc((void **)&v.d64, sizeof(double) * nn) != cudaSuccess ||
+                cudaMalloc((void **)&v.r32, sizeof(float) * nn) != cudaSuccess)
                 return cuda_error(cudaGetLastError(), "cudaMalloc (batch run buffers)");
         }
         b->nrhs_cap = nrhs;
     }
-    std::vector<double *> &bv = b->bv, &rv = b->rv, &auv = b->auv;
-    std::vector<float *> &r32 = b->r32;
 
     // 1 + 2: walk of every line of every mesh (one launch on the caller's stream), then per
-    // mesh on the internal streams contraction, load vector and factorisation; replayed
-    // from the captured graph when the run matches the one it was captured for
+    // mesh on the internal streams contraction and factorisation; replayed from
+    // the captured graph when the run matches the one it was captured for
     std::vector<double> ak(alpha, alpha + 3 * n);
     ak.insert(ak.end(), K, K + 3 * n);
-    std::vector<const double *> fk(f, f + n);
-    const bool same = b->exec && b->key_prec == precision && b->key_nrhs == nrhs &&
-                      b->key_ak == ak && b->key_f == fk;
+    const bool same = b->exec && b->key_prec == precision && b->key_ak == ak;
     auto enqueue_assembly = [&](cudaStream_t os) -> int {
         FEM3_TRY(walk_tables_batch(b->ms.data(), n, alpha, os, &b->ws));
         FEM3_TRY(fork_to(b, os));
@@ -275,7 +231,6 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
                 FEM3_TRY(contract_tc(m, precision == FEM3_BF16X3));
             else
                 FEM3_TRY(contract(m, precision));
-            FEM3_TRY(load_vector(m, f[i], nrhs, bv[i]));
             FEM3_TRY(factor(m));
         }
         FEM3_TRY(join_to(b, os));
@@ -306,9 +261,7 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
                 cudaGraphInstantiate(&b->exec, g, 0) == cudaSuccess) {
                 captured = true;
                 b->key_prec = precision;
-                b->key_nrhs = nrhs;
                 b->key_ak = ak;
-                b->key_f = fk;
             }
             if (g) cudaGraphDestroy(g);
         }
@@ -324,77 +277,42 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
         st = enqueue_assembly(cs);
         b->runs++;
     }
-    // the first correction starts from u = 0: the residual is b
+    // 3. per mesh on its stream: load vector, then refinement from u = 0 (FP64: a direct solve)
     if (st == FEM3_OK) st = fork_to(b, cs);
+    std::vector<int> it(n, 0);
+    std::vector<double> worst(n, 0.0);
+    std::vector<char> active(n, 0), late(n, 0);
+    int n_active = 0;
     for (int i = 0; i < n && st == FEM3_OK; i++) {
         Mesh *m = b->ms[i];
         m->stream = b->streams[i % b->streams.size()];
         if (m->n_dof == 0) continue;
         m->factored = true;
-        FEM3_CUDA(cudaMemcpyAsync(rv[i], bv[i], sizeof(double) * m->n_dof * nrhs,
-                                  cudaMemcpyDeviceToDevice, m->stream));
-        FEM3_CUDA(cudaMemsetAsync(u[i], 0, sizeof(double) * m->n_dof * nrhs, m->stream));
+        if ((st = load_vector(m, f[i], nrhs, b->bv[i])) != FEM3_OK) break;
+        if (fp64) {
+            st = solve_direct(m, b->bv[i], nrhs, u[i]);
+            continue;
+        }
+        b->rv[i].b = b->bv[i];
+        b->rv[i].u = u[i];
+        st = refine_start(b->rv[i], m->n_dof, nrhs, m->stream);
+        active[i] = 1;
+        n_active++;
     }
-
-    // 3. refinement (FP64: a single direct sweep)
-    std::vector<int> it(n, 0);
-    std::vector<double> worst(n, 0.0);
-    std::vector<char> active(n, 1);
-    for (int i = 0; i < n; i++) active[i] = b->ms[i]->n_dof > 0;
-    BatchTrsmDesc *hd = b->h_tdesc;
-    int sweep = 0;
-    while (st == FEM3_OK) {
-        // right-hand sides of the triangular solves
-        int n_active = 0;
-        for (int i = 0; i < n; i++) {
-            Mesh *m = b->ms[i];
-            hd[i] = BatchTrsmDesc{fp64 ? (const void *)m->A64 : (const void *)m->A32, m->dinv,
-                                  fp64 ? (void *)u[i] : (void *)r32[i], m->n_dof,
-                                  (int)((m->n_dof + 63) / 64), active[i] ? 1 : 0};
-            if (!active[i]) continue;
-            n_active++;
-            const int64_t nn = m->n_dof * nrhs;
-            if (fp64) {
-                FEM3_CUDA(cudaMemcpyAsync(u[i], bv[i], sizeof(double) * nn, cudaMemcpyDeviceToDevice,
-                                          m->stream));
-            } else {
-                k_copy_to_f32<<<blocks(nn), 256, 0, m->stream>>>(rv[i], r32[i], nn);
-                note_launch(m);
-            }
-        }
-        if (n_active == 0) break;
-        FEM3_TRY(join_to(b, cs));
-        FEM3_CUDA(cudaMemcpyAsync(b->d_tdesc, hd, sizeof(BatchTrsmDesc) * n, cudaMemcpyHostToDevice, cs));
-        FEM3_TRY(trsm_batch(b->d_tdesc, n, b->max_nblk, nrhs, fp64, cs));
-        FEM3_TRY(fork_to(b, cs));
-        sweep++;
-        if (fp64) break;
-        for (int i = 0; i < n; i++) {
-            if (!active[i]) continue;
-            Mesh *m = b->ms[i];
-            const int64_t nn = m->n_dof * nrhs;
-            k_add_f32<<<blocks(nn), 256, 0, m->stream>>>(r32[i], u[i], nn);
-            note_launch(m);
-            if ((st = apply_multi(m, u[i], nrhs, auv[i])) != FEM3_OK) break;
-            FEM3_CUDA(cudaMemsetAsync(m->norms, 0, sizeof(double) * 2 * nrhs, m->stream));
-            k_resid_cols<<<dim3(blocks(m->n_dof), nrhs), 256, 0, m->stream>>>(bv[i], auv[i], m->n_dof,
-                                                                           rv[i], m->norms);
-            note_launch(m);
-            FEM3_CUDA(cudaMemcpyAsync(m->h_norms, m->norms, sizeof(double) * 2 * nrhs,
-                                      cudaMemcpyDeviceToHost, m->stream));
-        }
+    for (int sweep = 1; n_active > 0 && st == FEM3_OK; sweep++) {
+        for (int i = 0; i < n && st == FEM3_OK; i++)
+            if (active[i]) st = refine_sweep(b->ms[i], b->rv[i], nrhs, late[i]);
         for (cudaStream_t t : b->streams) FEM3_CUDA(cudaStreamSynchronize(t));
-        for (int i = 0; i < n; i++) {
+        for (int i = 0; i < n && st == FEM3_OK; i++) {
             if (!active[i]) continue;
-            Mesh *m = b->ms[i];
-            double w = 0;
-            for (int c = 0; c < nrhs; c++) {
-                const double rel = m->h_norms[2 * c + 1] > 0 ? sqrt(m->h_norms[2 * c] / m->h_norms[2 * c + 1]) : 0.0;
-                w = rel == rel ? std::max(w, rel) : INFINITY;
-            }
-            worst[i] = w;
+            bool l = false;
+            worst[i] = refine_worst(b->ms[i], nrhs, tol, &l);
+            late[i] = l;
             it[i] = sweep;
-            if (w <= tol || sweep >= max_iter || !(w < INFINITY)) active[i] = 0;
+            if (worst[i] <= tol || sweep >= max_iter || !(worst[i] < INFINITY)) {
+                active[i] = 0;
+                n_active--;
+            }
         }
     }
 

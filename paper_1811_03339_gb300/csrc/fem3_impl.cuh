@@ -254,14 +254,12 @@ struct BatchWalkScratch {
     void *d_desc = nullptr, *h_desc = nullptr;
 };
 
-// one mesh of a batched triangular solve (device-resident descriptor)
-struct BatchTrsmDesc {
-    const void *L;      // factor, row-major n x n (float or double)
-    const void *dinv;   // inverses of the 64 x 64 diagonal blocks
-    void *y;            // right-hand sides / solutions, column-major [n][nrhs]
-    int64_t n;
-    int nblk;
-    int active;         // 0: skip this mesh
+// vectors of a refinement (column-major [n_dof][nrhs]): right-hand sides, solutions, A u or
+// A d, residuals, the correction widened for a late sweep's apply, and the FP32 correction
+struct RefineVecs {
+    const double *b;
+    double *u, *Au, *r, *d64;
+    float *r32;
 };
 
 // translation-unit entry points
@@ -300,8 +298,9 @@ int solve_refined(Mesh *m, const double *b_d, int nrhs, double tol, int max_iter
 int apply_A64(Mesh *m, const double *u_d, double *Au_d);
 int axis_forms(Mesh *m, const double *u_d, const double *lam_d, double out[3]);
 int read_errors(Mesh *m, int32_t *h_err);
-int trsm_batch(const BatchTrsmDesc *d_desc, int n_mesh, int max_nblk, int nrhs, bool fp64,
-               cudaStream_t s);
+int refine_start(const RefineVecs &v, int64_t n, int nrhs, cudaStream_t s);
+int refine_sweep(Mesh *m, const RefineVecs &v, int nrhs, bool late);
+double refine_worst(const Mesh *m, int nrhs, double tol, bool *late);
 int apply_multi(Mesh *m, const double *u_d, int nv, double *Au_d, bool df = true);
 int f32_to_f64(const float *a, double *b, int64_t n, cudaStream_t s);
 int sym_from_lower(double *A, int64_t n, cudaStream_t s);

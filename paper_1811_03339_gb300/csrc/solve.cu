@@ -376,77 +376,6 @@ __global__ void __launch_bounds__(512, 1) k_chol_tiles(float *A, int64_t n, int 
 // at most this many right-hand sides per triangular-solve launch
 constexpr int kMaxRhs = 24;
 
-// ---------------------------------------------------------------------------------
-// Batched block-step triangular solves across meshes (no waiting between CTAs, so the
-// meshes of a batch share launches).  Step s: mesh m solves its block k = s (forward)
-// or nblk_m - 1 - s (backward) with the diagonal inverse, then updates the blocks that
-// depend on it.  All right-hand sides of a mesh (<= 24, column-major, ld = n) together.
-// ---------------------------------------------------------------------------------
-template <class TF>
-__global__ void __launch_bounds__(256) k_btrsm_diag(const BatchTrsmDesc *__restrict__ d, int s,
-                                                    int nrhs, int backward) {
-    __shared__ TF dv[NB][NB + 1];
-    __shared__ TF tt[NB][kMaxRhs + 1];
-    const BatchTrsmDesc &D = d[blockIdx.x];
-    if (!D.active || s >= D.nblk) return;
-    const int k = backward ? D.nblk - 1 - s : s;
-    const int64_t n = D.n, r0 = (int64_t)k * NB;
-    const int nb = (int)min((int64_t)NB, n - r0);
-    const TF *Dinv = reinterpret_cast<const TF *>(D.dinv) + (int64_t)k * NB * NB;
-    TF *Y = reinterpret_cast<TF *>(D.y);
-    for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) dv[e >> 6][e & 63] = Dinv[e];
-    for (int e = threadIdx.x; e < NB * nrhs; e += blockDim.x) {
-        const int r = e & 63, c = e >> 6;
-        tt[r][c] = r < nb ? Y[(int64_t)c * n + r0 + r] : TF(0);
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < NB * nrhs; e += blockDim.x) {
-        const int r = e & 63, c = e >> 6;
-        TF acc = TF(0);
-        if (!backward)
-            for (int q = 0; q <= r; q++) acc += dv[r][q] * tt[q][c];
-        else
-            for (int q = r; q < NB; q++) acc += dv[q][r] * tt[q][c];
-        if (r < nb) Y[(int64_t)c * n + r0 + r] = acc;
-    }
-}
-
-template <class TF>
-__global__ void __launch_bounds__(256) k_btrsm_update(const BatchTrsmDesc *__restrict__ d, int s,
-                                                      int nrhs, int backward) {
-    __shared__ TF lt[NB][NB + 1];
-    __shared__ TF xs[NB][kMaxRhs + 1];
-    const BatchTrsmDesc &D = d[blockIdx.y];
-    if (!D.active || s >= D.nblk) return;
-    const int k = backward ? D.nblk - 1 - s : s;
-    const int i = backward ? k - 1 - (int)blockIdx.x : k + 1 + (int)blockIdx.x;
-    if (i < 0 || i >= D.nblk) return;
-    const int64_t n = D.n, r0 = (int64_t)i * NB, c0 = (int64_t)k * NB;
-    const int nb = (int)min((int64_t)NB, n - r0), nk = (int)min((int64_t)NB, n - c0);
-    const TF *L = reinterpret_cast<const TF *>(D.L);
-    TF *Y = reinterpret_cast<TF *>(D.y);
-    for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-        const int a = e >> 6, b = e & 63;
-        if (!backward) {   // lt[r][q] = L[r0 + r][c0 + q]
-            lt[a][b] = (a < nb && b < nk) ? L[(r0 + a) * n + c0 + b] : TF(0);
-        } else {           // lt[r][q] = L[c0 + q][r0 + r]
-            lt[b][a] = (a < nk && b < nb) ? L[(c0 + a) * n + r0 + b] : TF(0);
-        }
-    }
-    for (int e = threadIdx.x; e < NB * nrhs; e += blockDim.x) {
-        const int q = e & 63, c = e >> 6;
-        xs[q][c] = q < nk ? Y[(int64_t)c * n + c0 + q] : TF(0);
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < NB * nrhs; e += blockDim.x) {
-        const int r = e & 63, c = e >> 6;
-        TF acc = TF(0);
-#pragma unroll 8
-        for (int q = 0; q < NB; q++) acc += lt[r][q] * xs[q][c];
-        if (r < nb) Y[(int64_t)c * n + r0 + r] -= acc;
-    }
-}
-
 int chol_tiles(float *A, int64_t n, cudaStream_t s, Mesh *m) {
     if (n <= 0) return FEM3_OK;
     const int nblk = (int)((n + NB - 1) / NB);
@@ -1077,27 +1006,6 @@ int residual_norm(Mesh *m, const double *b, const double *Au, double *rel) {
 template <class TF>
 int trsm_t(const TF *L, int64_t n, TF *Y, int nrhs, cudaStream_t s, Mesh *m) {
     return solve_chain_t<TF>(L, n, Y, nrhs, s, m);
-}
-
-// Forward then backward block-step sweeps over all meshes of a batch (descriptors in
-// device memory, nrhs <= 16, max_nblk = largest block count).
-template <class TF>
-int trsm_batch_t(const BatchTrsmDesc *d_desc, int n_mesh, int max_nblk, int nrhs, cudaStream_t s) {
-    for (int backward = 0; backward < 2; backward++)
-        for (int st = 0; st < max_nblk; st++) {
-            k_btrsm_diag<TF><<<n_mesh, 256, 0, s>>>(d_desc, st, nrhs, backward);
-            if (st + 1 < max_nblk)
-                k_btrsm_update<TF><<<dim3(max_nblk - 1 - st, n_mesh), 256, 0, s>>>(d_desc, st, nrhs,
-                                                                                   backward);
-        }
-    FEM3_CUDA(cudaGetLastError());
-    return FEM3_OK;
-}
-
-int trsm_batch(const BatchTrsmDesc *d_desc, int n_mesh, int max_nblk, int nrhs, bool fp64,
-               cudaStream_t s) {
-    return fp64 ? trsm_batch_t<double>(d_desc, n_mesh, max_nblk, nrhs, s)
-                : trsm_batch_t<float>(d_desc, n_mesh, max_nblk, nrhs, s);
 }
 
 int load_vector(Mesh *m, const double *f_d, int nrhs, double *b_d) {
@@ -1899,59 +1807,77 @@ int solve_direct(Mesh *m, const double *b_d, int nrhs, double *u_d) {
 // while the double-float apply of A u costs six times the instructions.
 constexpr double kLateFactor = 1e4;
 
+int refine_start(const RefineVecs &v, int64_t n, int nrhs, cudaStream_t s) {
+    const int64_t nn = n * nrhs;
+    FEM3_CUDA(cudaMemsetAsync(v.u, 0, sizeof(double) * nn, s));
+    FEM3_CUDA(cudaMemcpyAsync(v.r, v.b, sizeof(double) * nn, cudaMemcpyDeviceToDevice, s));
+    return FEM3_OK;
+}
+
+// one sweep, enqueued on m->stream; the norms arrive in m->h_norms (2 nrhs values)
+int refine_sweep(Mesh *m, const RefineVecs &v, int nrhs, bool late) {
+    cudaStream_t s = m->stream;
+    const int64_t n = m->n_dof, nn = n * nrhs;
+    k_to_f32<<<g256(nn), 256, 0, s>>>(v.r, v.r32, nn);
+    note_launch(m);
+    for (int c0 = 0; c0 < nrhs; c0 += kMaxRhs)
+        FEM3_TRY(trsm_t<float>(m->A32, n, v.r32 + c0 * n, std::min(kMaxRhs, nrhs - c0), s, m));
+    k_axpy_f32<<<g256(nn), 256, 0, s>>>(v.r32, v.u, nn);
+    note_launch(m);
+    FEM3_CUDA(cudaMemsetAsync(m->norms, 0, sizeof(double) * 2 * nrhs, s));
+    if (late) {
+        k_f32_to_f64_n<<<g256(nn), 256, 0, s>>>(v.r32, v.d64, nn);
+        note_launch(m);
+        FEM3_TRY(apply_multi(m, v.d64, nrhs, v.Au, false));
+        k_residual_update_cols<<<dim3(g256(n), nrhs), 256, 0, s>>>(v.b, v.Au, n, v.r, m->norms);
+    } else {
+        FEM3_TRY(apply_multi(m, v.u, nrhs, v.Au, true));
+        k_residual_cols<<<dim3(g256(n), nrhs), 256, 0, s>>>(v.b, v.Au, n, v.r, m->norms);
+    }
+    note_launch(m);
+    FEM3_CUDA(cudaMemcpyAsync(m->h_norms, m->norms, sizeof(double) * 2 * nrhs,
+                              cudaMemcpyDeviceToHost, s));
+    return FEM3_OK;
+}
+
+// largest relative residual of the sweep whose norms have arrived (infinity for NaN), and
+// whether the next sweep is a late one
+double refine_worst(const Mesh *m, int nrhs, double tol, bool *late) {
+    double worst = 0;
+    for (int c = 0; c < nrhs; c++) {
+        const double rel = m->h_norms[2 * c + 1] > 0 ? sqrt(m->h_norms[2 * c] / m->h_norms[2 * c + 1]) : 0.0;
+        worst = (rel == rel) ? std::max(worst, rel) : INFINITY;
+    }
+    *late = worst <= kLateFactor * tol;
+    return worst;
+}
+
 int solve_refined(Mesh *m, const double *b_d, int nrhs, double tol, int max_iter, double *u_d,
                   int *iters, double *resid) {
     cudaStream_t s = m->stream;
     const int64_t n = m->n_dof;
     const int64_t nn = n * nrhs;
     if (nrhs > 32) return set_error(FEM3_E_ARG, "at most 32 right-hand sides per solve");
-    double *Au = nullptr, *r = nullptr, *d64 = nullptr;
-    float *r32 = nullptr;
-    FEM3_CUDA(cudaMallocAsync((void **)&Au, sizeof(double) * nn, s));
-    FEM3_CUDA(cudaMallocAsync((void **)&r, sizeof(double) * nn, s));
-    FEM3_CUDA(cudaMallocAsync((void **)&d64, sizeof(double) * nn, s));
-    FEM3_CUDA(cudaMallocAsync((void **)&r32, sizeof(float) * nn, s));
-    FEM3_CUDA(cudaMemsetAsync(u_d, 0, sizeof(double) * nn, s));
-    FEM3_CUDA(cudaMemcpyAsync(r, b_d, sizeof(double) * nn, cudaMemcpyDeviceToDevice, s));
+    RefineVecs v{b_d, u_d, nullptr, nullptr, nullptr, nullptr};
+    FEM3_CUDA(cudaMallocAsync((void **)&v.Au, sizeof(double) * nn, s));
+    FEM3_CUDA(cudaMallocAsync((void **)&v.r, sizeof(double) * nn, s));
+    FEM3_CUDA(cudaMallocAsync((void **)&v.d64, sizeof(double) * nn, s));
+    FEM3_CUDA(cudaMallocAsync((void **)&v.r32, sizeof(float) * nn, s));
     int it = 0;
     double worst = 1.0;
     bool late = false;
-    int st = FEM3_OK;
-    for (;;) {
-        k_to_f32<<<g256(nn), 256, 0, s>>>(r, r32, nn);
-        note_launch(m);
-        for (int c0 = 0; c0 < nrhs && st == FEM3_OK; c0 += kMaxRhs)
-            st = trsm_t<float>(m->A32, n, r32 + c0 * n, std::min(kMaxRhs, nrhs - c0), s, m);
-        if (st != FEM3_OK) break;
-        k_axpy_f32<<<g256(nn), 256, 0, s>>>(r32, u_d, nn);
-        note_launch(m);
-        FEM3_CUDA(cudaMemsetAsync(m->norms, 0, sizeof(double) * 2 * nrhs, s));
-        if (late) {
-            k_f32_to_f64_n<<<g256(nn), 256, 0, s>>>(r32, d64, nn);
-            note_launch(m);
-            if ((st = apply_multi(m, d64, nrhs, Au, false)) != FEM3_OK) break;
-            k_residual_update_cols<<<dim3(g256(n), nrhs), 256, 0, s>>>(b_d, Au, n, r, m->norms);
-        } else {
-            if ((st = apply_multi(m, u_d, nrhs, Au, true)) != FEM3_OK) break;
-            k_residual_cols<<<dim3(g256(n), nrhs), 256, 0, s>>>(b_d, Au, n, r, m->norms);
-        }
-        note_launch(m);
-        FEM3_CUDA(cudaMemcpyAsync(m->h_norms, m->norms, sizeof(double) * 2 * nrhs,
-                                  cudaMemcpyDeviceToHost, s));
+    int st = refine_start(v, n, nrhs, s);
+    while (st == FEM3_OK) {
+        if ((st = refine_sweep(m, v, nrhs, late)) != FEM3_OK) break;
         FEM3_CUDA(cudaStreamSynchronize(s));
-        worst = 0;
-        for (int c = 0; c < nrhs; c++) {
-            const double rel = m->h_norms[2 * c + 1] > 0 ? sqrt(m->h_norms[2 * c] / m->h_norms[2 * c + 1]) : 0.0;
-            worst = (rel == rel) ? std::max(worst, rel) : INFINITY;
-        }
+        worst = refine_worst(m, nrhs, tol, &late);
         it++;
         if (worst <= tol || it >= max_iter || !(worst < INFINITY)) break;
-        late = worst <= kLateFactor * tol;
     }
-    cudaFreeAsync(d64, s);
-    cudaFreeAsync(Au, s);
-    cudaFreeAsync(r, s);
-    cudaFreeAsync(r32, s);
+    cudaFreeAsync(v.d64, s);
+    cudaFreeAsync(v.Au, s);
+    cudaFreeAsync(v.r, s);
+    cudaFreeAsync(v.r32, s);
     if (iters) *iters = it;
     if (resid) *resid = worst;
     if (st != FEM3_OK) return st;
