@@ -219,11 +219,12 @@ int fem3_load(fem3_mesh m, const double *f, int nrhs, double *b, void *stream);
  * fem3_solve - u = A^{-1} M f for the last assembled A.
  *   FP64: FP64 Cholesky and triangular solves.
  *   TF32X3 / BF16X3 / FP32: FP32 Cholesky of the mixed-precision A, then iterative
- *   refinement: d = A32^{-1} r, u += d, r = M f - A u with A u applied from the tables
- *   in double-float FP32 arithmetic (FP64-accurate), until ||r||_2 <= tol ||M f||_2 for
- *   every column or max_iter corrections.  Once every column's residual is below
- *   1e4 tol, a sweep updates r -= A d instead, with A d in plain FP32 (about 1e-6
- *   relative; d is as small as r, so the update's error stays near tol / 100).
+ *   refinement: d = A32^{-1} r, u += d, r = M f - A u with A u in FP64 from an
+ *   FP64-accurate A (formed from the tables on the first solve after an assemble, its nonzero
+ *   32 x 32 blocks), until ||r||_2 <= tol ||M f||_2 for every column or max_iter
+ *   corrections.  Once every column's residual is below 1e-3, a sweep updates r -= A d
+ *   instead, d being as small as r: in double-float FP32 arithmetic (2^-46 relative), and
+ *   below 1e4 tol in plain FP32 (about 1e-6 relative: an error near tol / 100).
  *   f         host or device float64 column-major [n_nodes][nrhs].
  *   u         device float64 column-major [n_dof][nrhs].
  *   iters_out host int or NULL: refinement steps taken (0 for FP64).
@@ -328,11 +329,12 @@ int fem3_bin_stats(fem3_mesh m, int axis, int64_t *n_bins, int64_t *n_tmpl, int3
  * (0).  Any output pointer may be NULL. */
 int fem3_tc_tile(fem3_mesh m, int32_t *tile_n, int32_t *tuned);
 
-/* Which form the refinement's operator apply A u (Section 2.3 tables) takes for this mesh:
- * *lists = 1 from the nonzero lists of the tables (the bins' template rows and Gauss-point
- * sums of 17 vectors fit the list kernel's 112 KB of shared memory and its threads' items),
- * 0 from the dense table blocks of the bins.  Decided by the bins alone, so known once the
- * mesh is uploaded.  lists: host int32.  Errors: FEM3_E_ARG. */
+/* Whether the bins are narrow (Section 2.3 template): *lists = 1 if 17 vectors' hi + lo pairs over
+ * the largest bin's template rows and Gauss points take at most 112 KB and no bin has more
+ * than 256 template rows, else 0.  Decided by the bins alone, so known once the mesh is
+ * uploaded.  (It once chose how the refinement applies A u from the tables; the apply now
+ * runs from the operator's nonzero blocks whatever the bins.)  lists: host int32.
+ * Errors: FEM3_E_ARG. */
 int fem3_apply_lists(fem3_mesh m, int32_t *lists);
 
 /*

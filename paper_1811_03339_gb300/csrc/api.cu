@@ -352,7 +352,7 @@ int fem3_assemble(fem3_mesh h, const double alpha[3], const double K[3], int pre
     }
     m->precision = precision;
     m->factored = false;
-    m->ap_ready = false;
+    m->op_ready = false;
     m->integer_order = false;
     m->nonsym = false;
     kc_reset(m);
@@ -392,7 +392,7 @@ int fem3_assemble_part(fem3_mesh h, const double alpha[3], const double K[3], in
     // a part of the matrix (and of the tables) is no operator to solve with
     m->precision = -1;
     m->factored = false;
-    m->ap_ready = false;
+    m->op_ready = false;
     return st;
 }
 
@@ -411,7 +411,7 @@ int fem3_assemble_integer(fem3_mesh h, const double K[3], double *A_out, void *s
     }
     m->precision = FEM3_FP64;
     m->factored = false;
-    m->ap_ready = false;
+    m->op_ready = false;
     m->integer_order = true;
     m->nonsym = false;
     kc_reset(m);
@@ -439,7 +439,7 @@ int fem3_assemble_form(fem3_mesh h, int axis, double alpha, double beta, int tri
     // the tables of this axis are rewritten: no assembled operator remains for fem3_solve
     m->precision = -1;
     m->factored = false;
-    m->ap_ready = false;
+    m->op_ready = false;
     m->integer_order = false;
     m->nonsym = false;
     kc_reset(m);
@@ -490,7 +490,7 @@ int fem3_assemble_divergence(fem3_mesh h, const double beta[3], const double *p,
     const int64_t n = m->n_dof;
     m->precision = -1;
     m->factored = false;
-    m->ap_ready = false;
+    m->op_ready = false;
     m->integer_order = false;
     m->nonsym = false;
     kc_reset(m);
@@ -589,17 +589,7 @@ int fem3_solve(fem3_mesh h, const double *f, int nrhs, double tol, int max_iter,
     if (st == FEM3_OK) {
         if (m->precision == FEM3_FP64) {
             st = solve_direct(m, b, nrhs, u);
-            if (st == FEM3_OK && resid_out) {
-                double worst = 0;
-                for (int r = 0; r < nrhs && st == FEM3_OK; r++) {
-                    st = m->integer_order ? apply_integer(m, u + r * n, m->vec64[0])
-                                          : apply_A64(m, u + r * n, m->vec64[0]);
-                    double rel = 0;
-                    if (st == FEM3_OK) st = residual_norm(m, b + r * n, m->vec64[0], &rel);
-                    worst = std::max(worst, rel);
-                }
-                *resid_out = worst;
-            }
+            if (st == FEM3_OK && resid_out) st = residual_worst(m, b, u, nrhs, resid_out);
             if (iters_out) *iters_out = 0;
         } else {
             st = solve_refined(m, b, nrhs, tol, max_iter > 0 ? max_iter : 50, u, iters_out, resid_out);
@@ -714,7 +704,14 @@ int fem3_tc_tile(fem3_mesh h, int32_t *tile_n, int32_t *tuned) {
 int fem3_apply_lists(fem3_mesh h, int32_t *lists) {
     Mesh *m = reinterpret_cast<Mesh *>(h);
     if (!m || !lists) return set_error(FEM3_E_ARG, "bad argument");
-    *lists = apply_lists_fit(m) ? 1 : 0;
+    // 17 vectors' pairs over the largest bin's template rows and Gauss points in 112 KB, and at
+    // most 256 template rows
+    int md = 0, mg = 0;
+    for (int a = 0; a < 3; a++) {
+        md = std::max(md, m->bins[a].max_dof);
+        mg = std::max(mg, m->bins[a].max_gp);
+    }
+    *lists = 8 * 17 * ((int64_t)md + mg) <= 112 * 1024 && md <= 256 ? 1 : 0;
     return FEM3_OK;
 }
 

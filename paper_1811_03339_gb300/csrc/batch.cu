@@ -52,7 +52,6 @@ static void free_run_buffers(Batch *b) {
     for (const RefineVecs &v : b->rv) {
         cudaFree(v.r);
         cudaFree(v.Au);
-        cudaFree(v.d64);
         cudaFree(v.r32);
     }
     b->bv.clear();
@@ -192,7 +191,7 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
         }
         m->precision = precision;
         m->factored = false;
-        m->ap_ready = false;
+        m->op_ready = false;
     }
     // run buffers for nrhs columns (kept across runs)
     if (b->nrhs_cap < nrhs) {
@@ -207,7 +206,6 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
             if (cudaMalloc((void **)&b->bv[i], sizeof(double) * nn) != cudaSuccess ||
                 cudaMalloc((void **)&v.r, sizeof(double) * nn) != cudaSuccess ||
                 cudaMalloc((void **)&v.Au, sizeof(double) * nn) != cudaSuccess ||
-                cudaMalloc((void **)&v.d64, sizeof(double) * nn) != cudaSuccess ||
                 cudaMalloc((void **)&v.r32, sizeof(float) * nn) != cudaSuccess)
                 return cuda_error(cudaGetLastError(), "cudaMalloc (batch run buffers)");
         }
@@ -240,9 +238,8 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
     if (same) {
         FEM3_CUDA(cudaGraphLaunch(b->exec, cs));
         b->graph_launches++;
-        // the replayed contraction wrote the apply operands, as the captured one did
-        const bool tc = precision == FEM3_TF32X3 || precision == FEM3_BF16X3;
-        for (Mesh *m : b->ms) m->ap_ready = tc && m->n_dof > 0;
+        // a replayed FP64 run has copied its operator, as the captured one did
+        for (Mesh *m : b->ms) m->op_ready = fp64 && m->n_dof > 0;
     } else if (b->runs >= 1) {
         // capture the assembly + factorisation; on any failure discard it and run eagerly
         if (b->exec) {
@@ -281,7 +278,8 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
     if (st == FEM3_OK) st = fork_to(b, cs);
     std::vector<int> it(n, 0);
     std::vector<double> worst(n, 0.0);
-    std::vector<char> active(n, 0), late(n, 0);
+    std::vector<char> active(n, 0);
+    std::vector<RefineMode> mode(n, kRefineFull);
     int n_active = 0;
     for (int i = 0; i < n && st == FEM3_OK; i++) {
         Mesh *m = b->ms[i];
@@ -301,13 +299,11 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
     }
     for (int sweep = 1; n_active > 0 && st == FEM3_OK; sweep++) {
         for (int i = 0; i < n && st == FEM3_OK; i++)
-            if (active[i]) st = refine_sweep(b->ms[i], b->rv[i], nrhs, late[i]);
+            if (active[i]) st = refine_sweep(b->ms[i], b->rv[i], nrhs, mode[i]);
         for (cudaStream_t t : b->streams) FEM3_CUDA(cudaStreamSynchronize(t));
         for (int i = 0; i < n && st == FEM3_OK; i++) {
             if (!active[i]) continue;
-            bool l = false;
-            worst[i] = refine_worst(b->ms[i], nrhs, tol, &l);
-            late[i] = l;
+            worst[i] = refine_worst(b->ms[i], nrhs, tol, &mode[i]);
             it[i] = sweep;
             if (worst[i] <= tol || sweep >= max_iter || !(worst[i] < INFINITY)) {
                 active[i] = 0;

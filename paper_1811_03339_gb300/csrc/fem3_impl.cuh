@@ -51,8 +51,8 @@ constexpr double kEpsRRel = 1e-12;    // segment-length / tie tolerance, times t
 constexpr double kEpsDRel = 1e-12;    // |gradient| below this fraction of the largest: parallel
 
 constexpr int kMaxBinItems = 4096;    // max dofs or Gauss points in one transverse bin
-constexpr int kRowsWindow = 512;      // columns of one CUDA-core contraction item (its eight
-                                      // accumulator rows: 32 KB of shared memory in FP64)
+constexpr int kRowsWindow = 512;      // columns of one CUDA-core contraction item (its
+                                      // accumulator rows: 32 or 64 KB of shared memory)
 constexpr int kSegCounterSlot = 120;  // norms[120]: segment counter (norms[0..63] reductions)
                                       // norms[121]: contraction work counter
 
@@ -74,20 +74,6 @@ struct AxisBins {
     // 30 bits) << 32 | dof id, ascending within a bin; [n_dof] that quantised position
     unsigned long long *dof_key = nullptr;
     uint32_t *dof_q = nullptr;
-    // [n_tmpl] Gauss-point ranges [first, end) of the nonzeros of each row of L and of R
-    // (x, y: L; z, w: R), written with the apply operands
-    int4 *ap_rng = nullptr;
-    // the nonzeros of L and W R (t = 0: L, 1: W R) as lists, written with the apply operands:
-    // row-major, a template row's list in the place of its dense table row (Gauss-point index
-    // in the bin, value), and Gauss-point major in chunks of 32 points within the bin's block
-    // (row index in the bin, value; layout at k_gp_lists); list lengths per template row and
-    // per Gauss-point slot
-    uint16_t *rl_g[2] = {nullptr, nullptr};
-    float2 *rl_v[2] = {nullptr, nullptr};
-    int32_t *rl_n[2] = {nullptr, nullptr};
-    uint16_t *gl_r[2] = {nullptr, nullptr};
-    float2 *gl_v[2] = {nullptr, nullptr};
-    int32_t *gl_n[2] = {nullptr, nullptr};
     int64_t *tab_off = nullptr;  // [n_bins]     element offset of the bin's table block
     int32_t *tab_ld = nullptr;   // [n_bins]     leading dimension (padded Gauss-point count)
     int64_t n_tmpl = 0, tab_elems = 0;
@@ -100,13 +86,24 @@ struct AxisBins {
     int32_t *row_bin = nullptr;  // [n_tmpl] template row -> bin
     int tc_maxG = 0;             // largest Gauss-point count of a bin
     int4 *tc_work[2] = {nullptr, nullptr};   // (bin, m-tile, n-tile, 0) per tile width
-    // operator-apply operand W R as hi + lo FP32 pairs in the table layout (L is the table)
-    float2 *ap_R = nullptr;
     int tc_n_work[2] = {0, 0};
     std::vector<int32_t> h_gp_off, h_dof_off;
     std::vector<int4> h_work, h_tc_work[2];   // host copies of the work lists
     std::vector<int64_t> h_tab_off;
     std::vector<int32_t> h_tab_ld;
+};
+
+// The operator at FP64 accuracy in 32 x 32 blocks (operator.cu)
+constexpr int kOpBlock = 32;
+constexpr int kOpVecs = 18;   // vectors of one apply pass (17, padded to even)
+struct OpBlocks {
+    int nb = 0;                   // block rows
+    int64_t n_low = 0, n_full = 0;
+    int32_t *map = nullptr;       // [nb (nb + 1) / 2] block (i, j <= i) -> lower block or -1
+    int32_t *row_off = nullptr;   // [nb + 1] blocks of each block row, both triangles
+    int32_t *col = nullptr, *src = nullptr, *row_of = nullptr;   // [n_full]
+    double *low = nullptr;        // [n_low][32][32] lower blocks as the contraction adds them
+    double *full = nullptr;       // [n_full][32][32] column-major
 };
 
 struct Mesh {
@@ -154,7 +151,8 @@ struct Mesh {
     int tc_tile_opt = 0;       // tensor-core tile width asked for: 0 tuned, 128 or 256
     int tc_tile_used = 0;      // width of the last tensor-core contraction
     bool tc_tuned = false;     // the last contraction ran the tuner
-    bool ap_ready = false;     // ap_R holds W R of the current tables
+    OpBlocks op;
+    bool op_ready = false;     // op holds the operator of the current tables
     bool integer_order = false;   // the matrix came from fem3_assemble_integer (no tables)
     int32_t *p1_first = nullptr;  // integer order: first tile column of each block row of A64
     double *form_wc = nullptr;    // general form: w c per Gauss point, and per slot of one axis
@@ -228,7 +226,7 @@ void stage_collect(Mesh *m);
 // CUDA events on the launch stream around every launch of the class.
 enum KernelClass {
     KC_WALK = 0,      // k_walk_tables: walk + derivative tables, three axes in one launch
-    KC_SPLIT = 1,     // k_split_ops: operand split of the tables
+    KC_SPLIT = 1,     // operand splits: the tables' (k_split_ops), the operator's (k_op_mirror)
     KC_CONTRACT = 2,  // contraction GEMMs (tensor-core or CUDA-core)
     KC_FACTOR = 3,    // Cholesky factorisation
     KC_CHAIN = 4,     // triangular-solve chains
@@ -243,24 +241,20 @@ void kc_reset(Mesh *m);
 int scan_i32(const int32_t *in, int32_t *out, int64_t n, cudaStream_t s, Mesh *m);
 
 // scratch of the batched walk (descriptor arrays; freed by the batch)
-// row-major lists of a table pair (L, W R) as k_split_ops writes them (null: not written)
-struct RowLists {
-    uint16_t *g0, *g1;   // Gauss-point index in the bin
-    float2 *v0, *v1;     // L, W R values (hi + lo)
-    int32_t *n0, *n1;    // [n_tmpl] lengths
-};
-
 struct BatchWalkScratch {
     void *d_desc = nullptr, *h_desc = nullptr;
 };
 
 // vectors of a refinement (column-major [n_dof][nrhs]): right-hand sides, solutions, A u or
-// A d, residuals, the correction widened for a late sweep's apply, and the FP32 correction
+// A d, residuals, and the FP32 correction
 struct RefineVecs {
     const double *b;
-    double *u, *Au, *r, *d64;
+    double *u, *Au, *r;
     float *r32;
 };
+// how a sweep forms its residual: b - A u in FP64, or r - A d of its correction in double-float
+// or plain FP32 arithmetic
+enum RefineMode { kRefineFull = 0, kRefineUpdate = 1, kRefineLate = 2 };
 
 // translation-unit entry points
 int mesh_build(Mesh *m, const double *verts_d, const int32_t *tets_d);
@@ -299,36 +293,18 @@ int apply_A64(Mesh *m, const double *u_d, double *Au_d);
 int axis_forms(Mesh *m, const double *u_d, const double *lam_d, double out[3]);
 int read_errors(Mesh *m, int32_t *h_err);
 int refine_start(const RefineVecs &v, int64_t n, int nrhs, cudaStream_t s);
-int refine_sweep(Mesh *m, const RefineVecs &v, int nrhs, bool late);
-double refine_worst(const Mesh *m, int nrhs, double tol, bool *late);
-int apply_multi(Mesh *m, const double *u_d, int nv, double *Au_d, bool df = true);
+int refine_sweep(Mesh *m, const RefineVecs &v, int nrhs, RefineMode mode);
+double refine_worst(const Mesh *m, int nrhs, double tol, RefineMode *next);
+int residual_worst(Mesh *m, const double *b, const double *u, int nrhs, double *worst);
+// A u in FP64 and A d of FP32 corrections d in double-float or (late) plain FP32 arithmetic
+int apply_multi(Mesh *m, const double *u_d, int nv, double *Au_d);
+int apply_correction(Mesh *m, const float *d, int nv, double *Ad, bool late);
 int f32_to_f64(const float *a, double *b, int64_t n, cudaStream_t s);
 int sym_from_lower(double *A, int64_t n, cudaStream_t s);
 int sub_vec(const double *a, const double *b, double *c, int64_t n, cudaStream_t s);
-// rel = ||b - Au|| / ||b|| (synchronises)
-int residual_norm(Mesh *m, const double *b, const double *Au, double *rel);
-
-int ap_alloc(Mesh *m, int axis);   // operator-apply operand buffers of one axis
-int ap_prepare(Mesh *m);           // split the current tables into the apply operands
-// The operator apply runs from the lists of the tables' nonzeros when a bin's u rows and its
-// Gauss points' sums of 17 vectors fit the list kernel's shared memory and its rows its
-// threads' items (kListItems per thread, two vector groups); otherwise from the dense table
-// blocks (with the W R operand in the table layout)
-constexpr size_t kListSmemMax = 112 * 1024;   // two CTAs per SM at least
-constexpr int kListItems = 2;                  // phase-2 items (row, vector group) per thread
-inline size_t apply_lists_smem(int nr, int max_dof, int max_gp) {
-    return 8 * (size_t)nr * ((size_t)max_dof + (size_t)max_gp);
-}
-inline bool apply_lists_fit(const Mesh *m) {
-    int md = 0, mg = 0;
-    for (int a = 0; a < 3; a++) {
-        md = std::max(md, m->bins[a].max_dof);
-        mg = std::max(mg, m->bins[a].max_gp);
-    }
-    return apply_lists_smem(17, md, mg) <= kListSmemMax && 2 * md <= 256 * kListItems;
-}
-RowLists row_lists(AxisBins &B);   // the axis's row-major list arrays
-void launch_gp_lists(Mesh *m, int axis);   // Gauss-point-major lists of L and W R
+int op_build(Mesh *m);                          // the operator of the current tables
+int op_from_dense(Mesh *m, const double *A);    // ... of the FP64 form, from its matrix
+int contract_blocks(Mesh *m, const OpBlocks &O);   // the element sum into the lower blocks
 
 // ---------------------------------------------------------------------------------
 // FP64 values in FP32 arithmetic.  GB300 runs FP64 arithmetic and f64 <-> f32

@@ -7,9 +7,8 @@
 //    lower triangle, each 64 x 64 diagonal block as its inverse L_jj^{-1} (all the solves
 //    use).
 //  - Blocked forward / backward substitution.
-//  - Refinement for the mixed forms: r = b - A u with A u applied in FP64 from the FP64
-//    derivative tables (A u = sum_i s_i K_i (L_i^T W (R_i u) + R_i^T W (L_i u))), the
-//    correction solved with the FP32 factor.
+//  - Refinement for the mixed forms: r = b - A u with A u applied at FP64 accuracy
+//    (operator.cu), the correction solved with the FP32 factor.
 #include <math.h>
 
 #include <algorithm>
@@ -851,30 +850,9 @@ __global__ void __launch_bounds__(256) k_axis_form(
     }
 }
 
-// r = b - Au; norms[0] += |r|^2, norms[1] += |b|^2
-__global__ void k_residual(const double *__restrict__ b, const double *__restrict__ Au, int64_t n,
-                           double *r, double *norms) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double rr = 0, bb = 0;
-    if (i < n) {
-        double v = b[i] - Au[i];
-        r[i] = v;
-        rr = v * v;
-        bb = b[i] * b[i];
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        rr += __shfl_down_sync(0xffffffffu, rr, o);
-        bb += __shfl_down_sync(0xffffffffu, bb, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(&norms[0], rr);
-        atomicAdd(&norms[1], bb);
-    }
-}
-
-// r = b - Au for column blockIdx.y; norms[2c] += |r_c|^2, norms[2c+1] += |b_c|^2
-__global__ void k_residual_cols(const double *__restrict__ b, const double *__restrict__ Au,
-                                int64_t n, double *r, double *norms) {
+// (r may be Au)
+__global__ void k_residual_cols(const double *__restrict__ b, const double *Au, int64_t n,
+                                double *r, double *norms) {
     const int c = blockIdx.y;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     double rr = 0, bb = 0;
@@ -916,21 +894,6 @@ __global__ void k_residual_update_cols(const double *__restrict__ b, const doubl
         atomicAdd(&norms[2 * c], rr);
         atomicAdd(&norms[2 * c + 1], bb);
     }
-}
-
-__global__ void k_f32_to_f64_n(const float *__restrict__ a, double *b, int64_t n) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) b[i] = (double)a[i];
-}
-
-// ui[i][v] = u[v * n + i] for v < nv, zero for nv <= v < NR (NR = 4 or 8 vectors a pass)
-template <int NR>
-__global__ void k_interleave(const double *__restrict__ u, int64_t n, int nv, double *ui) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= NR * n) return;
-    const int64_t i = e / NR;
-    const int v = (int)(e - i * NR);
-    ui[e] = v < nv ? u[(int64_t)v * n + i] : 0.0;
 }
 
 __global__ void k_to_f32(const double *__restrict__ a, float *b, int64_t n) {
@@ -990,18 +953,6 @@ int sub_vec(const double *a, const double *b, double *c, int64_t n, cudaStream_t
     return FEM3_OK;
 }
 
-int residual_norm(Mesh *m, const double *b, const double *Au, double *rel) {
-    cudaStream_t s = m->stream;
-    const int64_t n = m->n_dof;
-    FEM3_CUDA(cudaMemsetAsync(m->norms, 0, sizeof(double) * 2, s));
-    k_residual<<<g256(n), 256, 0, s>>>(b, Au, n, m->vec64[1], m->norms);
-    note_launch(m);
-    FEM3_CUDA(cudaMemcpyAsync(m->h_norms, m->norms, sizeof(double) * 2, cudaMemcpyDeviceToHost, s));
-    FEM3_CUDA(cudaStreamSynchronize(s));
-    *rel = m->h_norms[1] > 0 ? sqrt(m->h_norms[0] / m->h_norms[1]) : 0.0;
-    return FEM3_OK;
-}
-
 // L Y = B then L^T X = Y for nrhs <= 24 columns (column-major, leading dimension n)
 template <class TF>
 int trsm_t(const TF *L, int64_t n, TF *Y, int nrhs, cudaStream_t s, Mesh *m) {
@@ -1035,6 +986,8 @@ constexpr int64_t kCholTcMinN = 4096;
 int factor(Mesh *m) {
     m->chol_tc_used = false;
     if (m->precision == FEM3_FP64) {
+        // the residual's operator, before the factor takes the matrix's place
+        if (!m->integer_order && !m->nonsym) FEM3_TRY(op_from_dense(m, m->A64));
         int launches = 0;
         kc_begin(m, KC_FACTOR);
         FEM3_TRY(chol_f64(m->A64, m->n_dof, reinterpret_cast<double *>(m->dinv),
@@ -1059,715 +1012,6 @@ int factor(Mesh *m) {
     }
     return solve_prep_t<float>(m->A32, m->n_dof, m->stream, m);
 }
-
-// Fused operator apply, one CTA per transverse bin, in double-float arithmetic on the FP32
-// pipes.  With R~ = W R (split once per assembly, see k_split_ops), A u restricted to
-// the bin is L^T (R~ u) + R~^T (L u) (L read from the table itself).  The bin's Gauss
-// points go in chunks of 32, and the chunks are independent: for a chunk, yR = R~ u_b and
-// yL = L u_b over its Gauss points (phase 1), then Au += s K (L^T yR + R~^T yL) over the
-// chunk's columns (phase 2).  The template rows go in pieces of kApplyRM: a piece's L and
-// R~ columns of the chunk are staged in shared memory (cp.async 16-byte copies, zero-filled
-// past the bin's Gauss points; rows of 34 pairs, 272 bytes) with u_b as hi + lo pairs and
-// the rows' nonzero ranges; phase 2 takes the piece staged last first and stages the others
-// again (from L2).
-// Rows and Gauss points of a bin are both ordered along the axis, so a row's nonzeros in L
-// (paths towards -x) start at a Gauss point that grows with the row and its nonzeros in R~
-// end at one: each row carries its exact ranges (k_split_ops) and both phases skip the
-// entries outside them, which are exact zeros.
-// Phase 1: warp w sums rows w, w + 8, ... (lane = Gauss point, all NR vectors); the eight
-// partial sums are added in shared memory.  Phase 2: thread = (row, group of NV vectors) for
-// NR = 4 and 8, each over the pairs of Gauss points that hold nonzeros of some row of its
-// warp (a warp-uniform range: the yL / yR reads are broadcasts); for NR = 1 thread = (row,
-// slice of the pairs), the slices added by shuffles.
-// Every product is exact up to 2^-48 relative and sums carry their rounding errors
-// (df_fma), so Au matches an FP64 evaluation to a few units in 2^-48.  The kernel has no
-// FP64 arithmetic: s K z is formed in double-float FP32 operations and its two parts go to
-// Au as exact FP64 values (bit assembly) through FP64 atomics.  NR = 1: u plain; NR = 4, 8:
-// u interleaved [dof][NR].
-constexpr int kApplyThreads = 256;
-constexpr int kApplyGC = 32;                  // Gauss points per chunk
-constexpr int kApplyStride = kApplyGC + 2;    // staged row, float2 units: 272 B, 16-B aligned
-constexpr int kApplyRM = 64;                  // rows per staged piece
-
-// phase-1 partial-sum buffers: one per warp, or four for NR > 8 (warps 4-7 first add into
-// those of warps 0-3)
-template <int NR> __host__ __device__ constexpr int apply_pw() { return NR > 8 ? 4 : 8; }
-// 76,800 bytes at NR = 8: three CTAs per SM (233,472 bytes less 1,024 reserved per CTA);
-// 88,064 bytes at NR = 17: two
-template <int NR>
-constexpr size_t apply_bin_smem() {
-    return (size_t)(2 * kApplyRM * kApplyStride + kApplyRM * NR +
-                    2 * apply_pw<NR>() * kApplyGC * NR + 2 * kApplyGC * NR) *
-               sizeof(float2) +
-           kApplyRM * sizeof(int4);
-}
-
-__device__ __forceinline__ void cp_async16(void *dst, const void *src, int src_bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
-                     (uint32_t)__cvta_generic_to_shared(dst)),
-                 "l"(src), "r"(src_bytes)
-                 : "memory");
-}
-
-// stage rows [r0, r0 + rn) of the chunk's L and R~ columns [gc0, gc0 + 32): one 16-byte
-// copy per (row, pair of Gauss points), the part past the bin's G Gauss points zero-filled
-// (and not read: entries past G in a table row are padding); and the rows' nonzero ranges.
-// The caller waits (cp.async.wait_all) and synchronises.
-__device__ __forceinline__ void apply_stage_ops(const float2 *__restrict__ TL,
-                                                const float2 *__restrict__ TR,
-                                                const int4 *__restrict__ rng, int ld, int G,
-                                                int gc0, int r0, int rn, float2 *Ls,
-                                                float2 *Rs, int4 *Qs) {
-    for (int e = threadIdx.x; e < rn * 16; e += kApplyThreads) {
-        const int r = e >> 4, q = e & 15, g = gc0 + 2 * q;
-        const int nb = g + 1 < G ? 16 : (g < G ? 8 : 0);
-        const int64_t o = (int64_t)(r0 + r) * ld + (nb ? g : 0);   // in the row when nb = 0
-        cp_async16(Ls + r * kApplyStride + 2 * q, TL + o, nb);
-        cp_async16(Rs + r * kApplyStride + 2 * q, TR + o, nb);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    for (int r = threadIdx.x; r < rn; r += kApplyThreads) Qs[r] = __ldg(rng + r0 + r);
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-    asm volatile("cp.async.wait_all;" ::: "memory");
-}
-
-// pairs [p0, p1) of the chunk's Gauss points that hold a row's nonzeros in [first, end)
-__device__ __forceinline__ void pair_range(int first, int end, int gc0, int gn, int &p0,
-                                           int &p1) {
-    p0 = max(first - gc0, 0) >> 1;
-    p1 = (min(end - gc0, gn) + 1) >> 1;
-}
-
-// phase 2 of one staged piece: thread = (row, group of NV vectors, slice of S of the 16
-// pairs of Gauss points); adds s K (L^T yR + R~^T yL) of the chunk to Au
-template <int NR, int NV, int S, bool DF>
-__device__ __forceinline__ void apply_phase2(const float2 *Ls, const float2 *Rs, const int4 *Qs,
-                                             const float2 *yL, const float2 *yR, int rn,
-                                             int gc0, int gn, const int32_t *__restrict__ dofs,
-                                             float sKh, float sKl, int nv, double *Au,
-                                             int64_t ldA) {
-    constexpr int VS = NR / NV;   // vector groups per row
-    const int t = threadIdx.x;
-    const int r = t / (VS * S), vg = (t / S) % VS, s = t % S;   // compile-time divisors
-    const bool act = r < rn;
-    const int rr = act ? r : 0;
-    const int4 q = Qs[rr];
-    int l0, l1, q0, q1;
-    pair_range(q.x, q.y, gc0, gn, l0, l1);
-    pair_range(q.z, q.w, gc0, gn, q0, q1);
-    if (!act) { l0 = q0 = kApplyGC; l1 = q1 = 0; }
-    if constexpr (S == 1) {
-        // the union over the warp's rows (entries outside a row's own range are zeros)
-        l0 = __reduce_min_sync(0xffffffffu, l0);
-        l1 = __reduce_max_sync(0xffffffffu, l1);
-        q0 = __reduce_min_sync(0xffffffffu, q0);
-        q1 = __reduce_max_sync(0xffffffffu, q1);
-    } else {
-        constexpr int PS = (kApplyGC / 2) / S;   // pairs per slice
-        l0 = max(l0, s * PS);
-        l1 = min(l1, (s + 1) * PS);
-        q0 = max(q0, s * PS);
-        q1 = min(q1, (s + 1) * PS);
-    }
-    const float4 *Lr = reinterpret_cast<const float4 *>(Ls + rr * kApplyStride);
-    const float4 *Rr = reinterpret_cast<const float4 *>(Rs + rr * kApplyStride);
-    const float2 *yRv = yR + vg * NV, *yLv = yL + vg * NV;
-    float zh[NV], zl[NV];
-#pragma unroll
-    for (int k = 0; k < NV; k++) { zh[k] = 0.f; zl[k] = 0.f; }
-    for (int g2 = l0; g2 < l1; g2++) {   // two Gauss points per 16-byte read
-        const float4 lv = Lr[g2];
-#pragma unroll
-        for (int k = 0; k < NV; k++) {
-            const float2 a0 = yRv[2 * g2 * NR + k], a1 = yRv[(2 * g2 + 1) * NR + k];
-            if constexpr (DF) {
-                df_fma(lv.x, lv.y, a0.x, a0.y, zh[k], zl[k]);
-                df_fma(lv.z, lv.w, a1.x, a1.y, zh[k], zl[k]);
-            } else {
-                zh[k] = fmaf(lv.x, a0.x, zh[k]);
-                zh[k] = fmaf(lv.z, a1.x, zh[k]);
-            }
-        }
-    }
-    for (int g2 = q0; g2 < q1; g2++) {
-        const float4 rv = Rr[g2];
-#pragma unroll
-        for (int k = 0; k < NV; k++) {
-            const float2 a0 = yLv[2 * g2 * NR + k], a1 = yLv[(2 * g2 + 1) * NR + k];
-            if constexpr (DF) {
-                df_fma(rv.x, rv.y, a0.x, a0.y, zh[k], zl[k]);
-                df_fma(rv.z, rv.w, a1.x, a1.y, zh[k], zl[k]);
-            } else {
-                zh[k] = fmaf(rv.x, a0.x, zh[k]);
-                zh[k] = fmaf(rv.z, a1.x, zh[k]);
-            }
-        }
-    }
-    if constexpr (S > 1) {   // the row's S slices sit in neighbouring lanes
-#pragma unroll
-        for (int o = 1; o < S; o <<= 1)
-#pragma unroll
-            for (int k = 0; k < NV; k++) {
-                const float xh = __shfl_xor_sync(0xffffffffu, zh[k], o);
-                const float xl = __shfl_xor_sync(0xffffffffu, zl[k], o);
-                if constexpr (DF) df_add(xh, xl, zh[k], zl[k]);
-                else zh[k] += xh;
-            }
-    }
-    // after the butterfly every slice lane holds the row's sums: lane s writes the vectors
-    // k = s (mod S)
-    if (!act) return;
-    const int64_t dof = dofs[r];
-#pragma unroll
-    for (int k = 0; k < NV; k++) {
-        const int v = vg * NV + k;
-        if (v >= nv) break;
-        if (k % S != s) continue;
-        if constexpr (DF) {
-            float ph, pl;
-            df_mul(zh[k], zl[k], sKh, sKl, ph, pl);
-            atomicAdd(&Au[(int64_t)v * ldA + dof], f32_to_f64_exact(ph));
-            atomicAdd(&Au[(int64_t)v * ldA + dof], f32_to_f64_exact(pl));
-        } else {
-            atomicAdd(&Au[(int64_t)v * ldA + dof], (double)(zh[k] * sKh));
-        }
-    }
-}
-
-// one axis of the apply: its bins' operands and s K as an FP32 pair
-struct ApplyAxis {
-    const float2 *apL, *apR;
-    const int4 *rng;   // per template row: Gauss-point ranges of the nonzeros of L and W R
-    const int32_t *gp_off, *dof_off, *dof_idx, *tab_ld;
-    const int64_t *tab_off;
-    float sKh, sKl;
-    int n_bins;
-};
-struct ApplyAxes {
-    ApplyAxis a[3];
-};
-
-// grid: the bins of the three axes (block x -> axis, bin)
-// DF = false: the same operator in plain FP32 arithmetic (hi parts of the table pairs and of
-// u, FMA accumulation), about 1e-6 relative: the refinement's late sweeps, whose residual
-// update r -= A d has a tiny correction d (see solve_refined)
-template <int NR, bool DF = true>
-__global__ void __launch_bounds__(kApplyThreads, NR > 8 ? 2 : 3)
-    k_apply_bin(const __grid_constant__ ApplyAxes P, const double *__restrict__ u, int nv,
-                double *Au, int64_t ldA) {
-    static_assert(NR == 1 || NR == 4 || NR == 8 || NR == 17, "vectors per pass");
-    constexpr int RM = kApplyRM, PW = apply_pw<NR>();
-    int b = blockIdx.x, axis = 0;
-    while (axis < 2 && b >= P.a[axis].n_bins) b -= P.a[axis++].n_bins;
-    const ApplyAxis &X = P.a[axis];
-    const float2 *__restrict__ apL = X.apL, *__restrict__ apR = X.apR;
-    const int32_t *__restrict__ gp_off = X.gp_off, *__restrict__ dof_off = X.dof_off,
-                  *__restrict__ dof_idx = X.dof_idx, *__restrict__ tab_ld = X.tab_ld;
-    const int64_t *__restrict__ tab_off = X.tab_off;
-    const float sKh = X.sKh, sKl = X.sKl;
-    extern __shared__ __align__(16) float2 sm_apply[];
-    float2 *Ls = sm_apply;                       // [RM][34]
-    float2 *Rs = Ls + RM * kApplyStride;         // [RM][34]
-    float2 *us = Rs + RM * kApplyStride;         // [RM][NR]
-    float2 *pL = us + RM * NR;                   // [PW][32][NR] phase-1 partial sums, L u
-    float2 *pR = pL + PW * kApplyGC * NR;        // [PW][32][NR] R~ u
-    float2 *yL = pR + PW * kApplyGC * NR;        // [32][NR]
-    float2 *yR = yL + kApplyGC * NR;             // [32][NR]
-    int4 *Qs = reinterpret_cast<int4 *>(yR + kApplyGC * NR);   // [RM] row ranges
-    const int d0 = dof_off[b], D = dof_off[b + 1] - d0;
-    const int G = gp_off[b + 1] - gp_off[b], ld = tab_ld[b];
-    if (D == 0 || G == 0) return;
-    const float2 *TL = apL + tab_off[b], *TR = apR + tab_off[b];
-    const int4 *rng = X.rng + d0;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int np = (D + RM - 1) / RM;
-    for (int gc0 = 0; gc0 < G; gc0 += kApplyGC) {
-        const int gn = min(kApplyGC, G - gc0);
-        // ---- phase 1: lane = Gauss point gc0 + lane, warp = row slice ----
-        float lh[NR], ll[NR], rh[NR], rl[NR];
-#pragma unroll
-        for (int v = 0; v < NR; v++) { lh[v] = 0.f; ll[v] = 0.f; rh[v] = 0.f; rl[v] = 0.f; }
-        for (int p = 0; p < np; p++) {
-            const int rc0 = p * RM, rn = min(RM, D - rc0);
-            __syncthreads();   // earlier readers of the staged rows are done
-            apply_stage_ops(TL, TR, rng, ld, G, gc0, rc0, rn, Ls, Rs, Qs);
-            for (int e = tid; e < rn * NR; e += kApplyThreads) {
-                const int r = e / NR, v = e - r * NR;
-                const int64_t dof = dof_idx[d0 + rc0 + r];
-                float a, a2;
-                f64_split(NR == 1 ? u[dof] : u[dof * NR + v], a, a2);
-                us[e] = make_float2(a, a2);
-            }
-            cp_async_wait_all();
-            __syncthreads();
-            for (int r = warp; r < rn; r += kApplyThreads / 32) {
-                // does the row's nonzero range meet this chunk in L, in R~?  (usually one)
-                const int4 q = Qs[r];
-                if (q.x < gc0 + kApplyGC && q.y > gc0) {
-                    const float2 lv = Ls[r * kApplyStride + lane];
-#pragma unroll
-                    for (int v = 0; v < NR; v++) {
-                        const float2 uv = us[r * NR + v];
-                        if constexpr (DF) df_fma(lv.x, lv.y, uv.x, uv.y, lh[v], ll[v]);
-                        else lh[v] = fmaf(lv.x, uv.x, lh[v]);
-                    }
-                }
-                if (q.z < gc0 + kApplyGC && q.w > gc0) {
-                    const float2 rv = Rs[r * kApplyStride + lane];
-#pragma unroll
-                    for (int v = 0; v < NR; v++) {
-                        const float2 uv = us[r * NR + v];
-                        if constexpr (DF) df_fma(rv.x, rv.y, uv.x, uv.y, rh[v], rl[v]);
-                        else rh[v] = fmaf(rv.x, uv.x, rh[v]);
-                    }
-                }
-            }
-        }
-        if constexpr (PW == 8) {
-#pragma unroll
-            for (int v = 0; v < NR; v++) {
-                pL[(warp * kApplyGC + lane) * NR + v] = make_float2(lh[v], ll[v]);
-                pR[(warp * kApplyGC + lane) * NR + v] = make_float2(rh[v], rl[v]);
-            }
-        } else {
-            // warps 4-7 store, warps 0-3 add their own sums to them
-            const int w4 = warp & 3;
-            if (warp >= 4) {
-#pragma unroll
-                for (int v = 0; v < NR; v++) {
-                    pL[(w4 * kApplyGC + lane) * NR + v] = make_float2(lh[v], ll[v]);
-                    pR[(w4 * kApplyGC + lane) * NR + v] = make_float2(rh[v], rl[v]);
-                }
-            }
-            __syncthreads();
-            if (warp < 4) {
-#pragma unroll
-                for (int v = 0; v < NR; v++) {
-                    const int e = (w4 * kApplyGC + lane) * NR + v;
-                    const float2 x = pL[e], z = pR[e];
-                    if constexpr (DF) {
-                        df_add(x.x, x.y, lh[v], ll[v]);
-                        df_add(z.x, z.y, rh[v], rl[v]);
-                    } else {
-                        lh[v] += x.x;
-                        rh[v] += z.x;
-                    }
-                    pL[e] = make_float2(lh[v], ll[v]);
-                    pR[e] = make_float2(rh[v], rl[v]);
-                }
-            }
-        }
-        __syncthreads();
-        for (int e = tid; e < kApplyGC * NR; e += kApplyThreads) {
-            float2 a = pL[e], c = pR[e];
-            float ah = a.x, al = a.y, ch = c.x, cl = c.y;
-#pragma unroll
-            for (int w = 1; w < PW; w++) {
-                const float2 x = pL[w * kApplyGC * NR + e], z = pR[w * kApplyGC * NR + e];
-                if constexpr (DF) {
-                    df_add(x.x, x.y, ah, al);
-                    df_add(z.x, z.y, ch, cl);
-                } else {
-                    ah += x.x;
-                    ch += z.x;
-                }
-            }
-            yL[e] = make_float2(ah, al);
-            yR[e] = make_float2(ch, cl);
-        }
-        __syncthreads();
-        // ---- phase 2: the piece staged last first ----
-        for (int pass = 0; pass < np; pass++) {
-            const int p = pass == 0 ? np - 1 : pass - 1;
-            const int rc0 = p * RM, rn = min(RM, D - rc0);
-            if (pass > 0) {
-                __syncthreads();
-                apply_stage_ops(TL, TR, rng, ld, G, gc0, rc0, rn, Ls, Rs, Qs);
-                cp_async_wait_all();
-                __syncthreads();
-            }
-            const int32_t *dofs = dof_idx + d0 + rc0;
-            if constexpr (NR == 8) {
-                if (rn <= 32)
-                    apply_phase2<8, 1, 1, DF>(Ls, Rs, Qs, yL, yR, rn, gc0, gn, dofs, sKh, sKl, nv,
-                                              Au, ldA);
-                else
-                    apply_phase2<8, 2, 1, DF>(Ls, Rs, Qs, yL, yR, rn, gc0, gn, dofs, sKh, sKl, nv,
-                                              Au, ldA);
-            } else if constexpr (NR == 4) {
-                if (rn <= 32)
-                    apply_phase2<4, 1, 2, DF>(Ls, Rs, Qs, yL, yR, rn, gc0, gn, dofs, sKh, sKl, nv,
-                                              Au, ldA);
-                else
-                    apply_phase2<4, 1, 1, DF>(Ls, Rs, Qs, yL, yR, rn, gc0, gn, dofs, sKh, sKl, nv,
-                                              Au, ldA);
-            } else if constexpr (NR == 17) {
-                if (rn <= 32)
-                    apply_phase2<17, 17, 8, DF>(Ls, Rs, Qs, yL, yR, rn, gc0, gn, dofs, sKh, sKl,
-                                                nv, Au, ldA);
-                else
-                    apply_phase2<17, 17, 4, DF>(Ls, Rs, Qs, yL, yR, rn, gc0, gn, dofs, sKh, sKl,
-                                                nv, Au, ldA);
-            } else {
-                if (rn <= 32)
-                    apply_phase2<1, 1, 8, DF>(Ls, Rs, Qs, yL, yR, rn, gc0, gn, dofs, sKh, sKl, nv,
-                                              Au, ldA);
-                else
-                    apply_phase2<1, 1, 4, DF>(Ls, Rs, Qs, yL, yR, rn, gc0, gn, dofs, sKh, sKl, nv,
-                                              Au, ldA);
-            }
-        }
-    }
-}
-
-// The same operator from the lists of the tables' nonzeros (the Gauss-point-major and
-// row-major lists that k_gp_lists and k_split_ops write with the apply operands): the work is
-// the nonzeros, about a fifth of the dense bin blocks (a Gauss point's line crosses the
-// element patches of a few of its bin's template dofs).  One CTA per bin, one y buffer:
-//   phase 0: u of the bin's template rows into shared memory (hi + lo pairs, [D][NR]);
-//   then two rounds, (point table, row table) = (W R, L) and then (L, W R):
-//   phase 1, warp = (chunk of 32 Gauss points, half of the vectors), lane = point: y[g] =
-//     sum over g's list in the point table of T[r][g] u[r], into shared memory ([G][NR]; the
-//     chunk layout puts the lanes' entries k side by side);
-//   phase 2, thread = up to two items (template row r, group of NV vectors): z += sum over
-//     r's list in the row table of T'[r][g] y[g], z kept in registers across the rounds;
-//   at the end Au[dof(r)] += s K z (FP64 atomics of the double-float parts, as in
-//   k_apply_bin).
-// With rows and Gauss points ordered along the axis, a point's L list grows along the bin as
-// its W R list shrinks (and likewise for a row), so the lanes of a warp do similar work.
-// u comes split into hi + lo FP32 pairs, [dof][NR] (k_split_vec).  The bin's rows, Gauss
-// points and their NR sums must fit the launch's shared memory (apply_multi checks).
-template <int NR>
-__global__ void k_split_vec(const double *__restrict__ u, int64_t n, int nv, float2 *uf) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= NR * n) return;
-    const int64_t i = e / NR;
-    const int v = (int)(e - i * NR);
-    float h = 0.f, l = 0.f;
-    if (v < nv) f64_split(u[(int64_t)v * n + i], h, l);
-    uf[e] = make_float2(h, l);
-}
-
-// loads that do not happen when `pred` is false (a predicated PTX load: no access is made, the
-// address need not be valid, and the result keeps its zero)
-__device__ __forceinline__ float2 ldg_if(const float2 *p, bool pred) {
-    float x = 0.f, y = 0.f;
-    asm volatile(
-        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
-        "@q ld.global.nc.v2.f32 {%0, %1}, [%3];\n\t}"
-        : "+f"(x), "+f"(y)
-        : "r"((int)pred), "l"(p));
-    return make_float2(x, y);
-}
-__device__ __forceinline__ int ldg_if(const uint16_t *p, bool pred) {
-    uint32_t v = 0;
-    asm volatile(
-        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
-        "@q ld.global.nc.u16 %0, [%2];\n\t}"
-        : "+r"(v)
-        : "r"((int)pred), "l"(p));
-    return (int)v;
-}
-
-struct ListAxis {
-    const uint16_t *rg[2];          // row-major lists: Gauss-point index, value (t = 0 L, 1 W R)
-    const float2 *rv[2];
-    const int32_t *rn[2];
-    const uint16_t *gr[2];          // Gauss-point-major lists (chunk layout): row index, value
-    const float2 *gv[2];
-    const int32_t *gn[2];
-    const int32_t *gp_off, *dof_off, *dof_idx, *tab_ld;
-    const int64_t *tab_off;
-    float sKh, sKl;
-    int n_bins;
-};
-struct ListAxes {
-    ListAxis a[3];
-};
-
-constexpr int kListThreads = 256;
-constexpr int kListBatch = 3;   // list entries whose loads are in flight together (timed: 3 of 2, 3, 4)
-
-template <int NR, int VS, bool DF>
-__global__ void __launch_bounds__(kListThreads, 3) k_apply_lists(const __grid_constant__ ListAxes P,
-                                                              const float2 *__restrict__ uf,
-                                                              int nv, double *Au, int64_t ldA,
-                                                              int max_dof) {
-    constexpr int NV = (NR + VS - 1) / VS;   // phase-2 vectors per item (the last group short)
-    constexpr int NH = (NR + 1) / 2;         // phase-1 vectors per warp item (two halves)
-    int b = blockIdx.x, axis = 0;
-    while (axis < 2 && b >= P.a[axis].n_bins) b -= P.a[axis++].n_bins;
-    const ListAxis &X = P.a[axis];
-    const int d0 = X.dof_off[b], D = X.dof_off[b + 1] - d0;
-    const int g0 = X.gp_off[b], G = X.gp_off[b + 1] - g0;
-    if (D == 0 || G == 0) return;
-    const int ld = X.tab_ld[b];
-    const int64_t t0 = X.tab_off[b];
-    extern __shared__ __align__(16) float2 sm_lists[];
-    float2 *us = sm_lists;                         // [max_dof][NR]
-    float2 *y = us + (int64_t)max_dof * NR;        // [G][NR]: R~ u, then L u
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // phase-2 items (row, vector group) of this thread, fixed for both rounds
-    float zh[kListItems][NV], zl[kListItems][NV];
-#pragma unroll
-    for (int i = 0; i < kListItems; i++)
-#pragma unroll
-        for (int k = 0; k < NV; k++) { zh[i][k] = 0.f; zl[i][k] = 0.f; }
-    // ---- phase 0 ----
-    for (int e = tid; e < D * NR; e += kListThreads) {
-        const int c = e / NR, v = e - c * NR;
-        us[e] = __ldg(uf + (int64_t)__ldg(X.dof_idx + d0 + c) * NR + v);
-    }
-    // Round 0: y = R~ u from the points' W R lists, then the rows' L lists against it;
-    // round 1: y = L u from the points' L lists, then the rows' W R lists.
-#pragma unroll
-    for (int round = 0; round < 2; round++) {
-        const int tg = 1 - round, tr = round;   // point-list table, row-list table
-        __syncthreads();   // u staged / the rows are done with the previous round's y
-        // ---- phase 1: warp = (chunk of 32 Gauss points, half of the vectors), lane = point
-        const int nchunk = (G + 31) >> 5;
-        for (int wi = warp; wi < 2 * nchunk; wi += kListThreads / 32) {
-            const int gc = 32 * (wi >> 1), v0 = NH * (wi & 1);
-            const int g = gc + lane, wc = min(32, G - gc);
-            const bool in = g < G;
-            const int64_t base = t0 + (int64_t)gc * D + lane;
-            float h[NH], l[NH];
-#pragma unroll
-            for (int k = 0; k < NH; k++) { h[k] = 0.f; l[k] = 0.f; }
-            const int cnt = in ? X.gn[tg][g0 + g] : 0;
-            const int cmax = __reduce_max_sync(0xffffffffu, cnt);
-            const uint16_t *__restrict__ rl = X.gr[tg] + base;
-            const float2 *__restrict__ vl = X.gv[tg] + base;
-            for (int q0 = 0; q0 < cmax; q0 += kListBatch) {
-                float2 a[kListBatch];
-                int r[kListBatch];
-#pragma unroll
-                for (int j = 0; j < kListBatch; j++) {
-                    // only the lane's own entries are read (cnt = 0 past the bin's points)
-                    const bool ok = q0 + j < cnt;
-                    const int64_t o = (int64_t)(q0 + j) * wc;
-                    a[j] = ldg_if(vl + o, ok);
-                    r[j] = ldg_if(rl + o, ok);
-                }
-#pragma unroll
-                for (int j = 0; j < kListBatch; j++) {
-                    const float2 *ur = us + r[j] * NR + v0;
-#pragma unroll
-                    for (int k = 0; k < NH; k++) {
-                        if (v0 + k >= NR) break;
-                        const float2 uu = ur[k];
-                        if constexpr (DF) df_fma(a[j].x, a[j].y, uu.x, uu.y, h[k], l[k]);
-                        else h[k] = fmaf(a[j].x, uu.x, h[k]);
-                    }
-                }
-            }
-            if (in) {
-                float2 *yg = y + (int64_t)g * NR + v0;
-#pragma unroll
-                for (int k = 0; k < NH; k++)
-                    if (v0 + k < NR) yg[k] = make_float2(h[k], l[k]);
-            }
-        }
-        __syncthreads();
-        // ---- phase 2: the thread's rows, their table-tr lists against y ----
-#pragma unroll
-        for (int i = 0; i < kListItems; i++) {
-            const int it = tid + i * kListThreads;
-            if (it >= D * VS) break;
-            const int c = it / VS, v0 = (it - c * VS) * NV;
-            const int64_t base = t0 + (int64_t)c * ld;
-            const int cnt = X.rn[tr][d0 + c];
-            const uint16_t *__restrict__ gl = X.rg[tr] + base;
-            const float2 *__restrict__ vl = X.rv[tr] + base;
-            for (int q0 = 0; q0 < cnt; q0 += kListBatch) {
-                float2 a[kListBatch];
-                int gi[kListBatch];
-#pragma unroll
-                for (int j = 0; j < kListBatch; j++) {
-                    // the row's own entries only
-                    const bool ok = q0 + j < cnt;
-                    a[j] = ldg_if(vl + q0 + j, ok);
-                    gi[j] = ldg_if(gl + q0 + j, ok);
-                }
-#pragma unroll
-                for (int j = 0; j < kListBatch; j++) {
-                    const float2 *yr = y + gi[j] * NR + v0;
-#pragma unroll
-                    for (int k = 0; k < NV; k++) {
-                        if (v0 + k >= NR) break;
-                        const float2 yy = yr[k];
-                        if constexpr (DF) df_fma(a[j].x, a[j].y, yy.x, yy.y, zh[i][k], zl[i][k]);
-                        else zh[i][k] = fmaf(a[j].x, yy.x, zh[i][k]);
-                    }
-                }
-            }
-        }
-    }
-    // ---- the thread's rows into Au ----
-#pragma unroll
-    for (int i = 0; i < kListItems; i++) {
-        const int it = tid + i * kListThreads;
-        if (it >= D * VS) break;
-        const int c = it / VS, v0 = (it - c * VS) * NV;
-        const int64_t dof = X.dof_idx[d0 + c];
-#pragma unroll
-        for (int k = 0; k < NV; k++) {
-            const int v = v0 + k;
-            if (v >= NR || v >= nv) break;
-            if constexpr (DF) {
-                float ph, pl;
-                df_mul(zh[i][k], zl[i][k], X.sKh, X.sKl, ph, pl);
-                atomicAdd(&Au[(int64_t)v * ldA + dof], f32_to_f64_exact(ph));
-                atomicAdd(&Au[(int64_t)v * ldA + dof], f32_to_f64_exact(pl));
-            } else {
-                atomicAdd(&Au[(int64_t)v * ldA + dof], (double)(zh[i][k] * X.sKh));
-            }
-        }
-    }
-}
-
-// Au = A u for nv vectors (column-major, leading dimension n_dof), applied from
-// the tables; vectors go through the tables in groups: up to 17 per pass while at least 13
-// are left, then up to eight, and a last group of one or up to four vectors takes the
-// narrower form of the kernel (a pass costs a fixed part, staging and the phases' overhead,
-// plus about its vectors' arithmetic: an eight-wide pass for one leftover vector cost as much
-// as a full group).
-int apply_multi(Mesh *m, const double *u_d, int nv, double *Au_d, bool df) {
-    cudaStream_t s = m->stream;
-    const int64_t n = m->n_dof;
-    FEM3_CUDA(cudaMemsetAsync(Au_d, 0, sizeof(double) * n * nv, s));
-    static bool attr = false;
-    if (!attr) {
-        FEM3_CUDA(cudaFuncSetAttribute(k_apply_bin<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)apply_bin_smem<1>()));
-        FEM3_CUDA(cudaFuncSetAttribute(k_apply_bin<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)apply_bin_smem<4>()));
-        FEM3_CUDA(cudaFuncSetAttribute(k_apply_bin<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)apply_bin_smem<8>()));
-        FEM3_CUDA(cudaFuncSetAttribute(k_apply_bin<1, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)apply_bin_smem<1>()));
-        FEM3_CUDA(cudaFuncSetAttribute(k_apply_bin<4, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)apply_bin_smem<4>()));
-        FEM3_CUDA(cudaFuncSetAttribute(k_apply_bin<8, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)apply_bin_smem<8>()));
-        FEM3_CUDA(cudaFuncSetAttribute(k_apply_bin<17>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)apply_bin_smem<17>()));
-        FEM3_CUDA(cudaFuncSetAttribute(k_apply_bin<17, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)apply_bin_smem<17>()));
-        attr = true;
-    }
-    FEM3_TRY(ap_prepare(m));
-    ApplyAxes P;
-    ListAxes PL;
-    int64_t nblk = 0;
-    int max_gp = 0, max_dof = 0;
-    for (int axis = 0; axis < 3; axis++) {
-        AxisBins &B = m->bins[axis];
-        const bool on = B.n_tmpl > 0 && B.n_bins > 0;
-        const float skh = (float)m->sK[axis], skl = (float)(m->sK[axis] - (double)skh);
-        P.a[axis] = ApplyAxis{m->tabL[axis], B.ap_R, B.ap_rng, B.gp_off, B.dof_off, B.dof_idx,
-                              B.tab_ld, B.tab_off, skh, skl, on ? B.n_bins : 0};
-        PL.a[axis] = ListAxis{{B.rl_g[0], B.rl_g[1]}, {B.rl_v[0], B.rl_v[1]},
-                              {B.rl_n[0], B.rl_n[1]}, {B.gl_r[0], B.gl_r[1]},
-                              {B.gl_v[0], B.gl_v[1]}, {B.gl_n[0], B.gl_n[1]},
-                              B.gp_off, B.dof_off, B.dof_idx, B.tab_ld, B.tab_off, skh, skl,
-                              on ? B.n_bins : 0};
-        nblk += on ? B.n_bins : 0;
-        if (on) {
-            max_gp = std::max(max_gp, B.max_gp);
-            max_dof = std::max(max_dof, B.max_dof);
-        }
-    }
-    // the lists' kernel when the largest bin's Gauss points and their 17 sums fit
-    const bool lists = apply_lists_fit(m);
-    if (lists) {
-        static bool lattr = false;
-        if (!lattr) {
-#define FEM3_LATTR(NR_, VS_)                                                                     \
-    FEM3_CUDA(cudaFuncSetAttribute(k_apply_lists<NR_, VS_, true>,                                \
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kListSmemMax)); \
-    FEM3_CUDA(cudaFuncSetAttribute(k_apply_lists<NR_, VS_, false>,                               \
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kListSmemMax))
-            FEM3_LATTR(17, 2);
-            FEM3_LATTR(8, 2);
-            FEM3_LATTR(4, 2);
-            FEM3_LATTR(1, 1);
-#undef FEM3_LATTR
-            lattr = true;
-        }
-    }
-    double *ui = nullptr;
-    if (nv > 1 || lists)
-        FEM3_CUDA(cudaMallocAsync((void **)&ui, sizeof(double) * 17 * std::max<int64_t>(1, n), s));
-    float2 *uf = reinterpret_cast<float2 *>(ui);
-    for (int v0 = 0, cnt = 0; v0 < nv && nblk > 0; v0 += cnt) {
-        const int left = nv - v0;
-        const int nri = left >= 13 ? 17 : (left >= 5 ? 8 : (left >= 2 ? 4 : 1));
-        cnt = std::min(nri, left);
-        double *out = Au_d + (int64_t)v0 * n;
-        if (lists) {
-            const double *us = u_d + (int64_t)v0 * n;
-            const size_t sh = apply_lists_smem(nri, max_dof, max_gp);
-#define FEM3_LISTS(NR_, VS_)                                                                     \
-    do {                                                                                         \
-        k_split_vec<NR_><<<g256((int64_t)NR_ * n), 256, 0, s>>>(us, n, cnt, uf);                 \
-        note_launch(m);                                                                          \
-        kc_begin(m, KC_APPLY);                                                                   \
-        if (df)                                                                                  \
-            k_apply_lists<NR_, VS_, true><<<(unsigned)nblk, kListThreads, sh, s>>>(PL, uf, cnt,  \
-                                                                                 out, n, max_dof); \
-        else                                                                                     \
-            k_apply_lists<NR_, VS_, false><<<(unsigned)nblk, kListThreads, sh, s>>>(PL, uf, cnt, \
-                                                                                  out, n, max_dof); \
-        kc_end(m, KC_APPLY);                                                                     \
-        note_launch(m);                                                                          \
-    } while (0)
-            if (nri == 17) FEM3_LISTS(17, 2);
-            else if (nri == 8) FEM3_LISTS(8, 2);
-            else if (nri == 4) FEM3_LISTS(4, 2);
-            else FEM3_LISTS(1, 1);
-#undef FEM3_LISTS
-            continue;
-        }
-        if (nri == 4)
-            k_interleave<4><<<g256(4 * n), 256, 0, s>>>(u_d + (int64_t)v0 * n, n, cnt, ui);
-        else if (nri == 8)
-            k_interleave<8><<<g256(8 * n), 256, 0, s>>>(u_d + (int64_t)v0 * n, n, cnt, ui);
-        else if (nri == 17)
-            k_interleave<17><<<g256(17 * n), 256, 0, s>>>(u_d + (int64_t)v0 * n, n, cnt, ui);
-        if (nri > 1) note_launch(m);
-        kc_begin(m, KC_APPLY);
-#define FEM3_APPLY(NR_, DF_, U_, CNT_)                                                          \
-    k_apply_bin<NR_, DF_><<<(unsigned)nblk, kApplyThreads, apply_bin_smem<NR_>(), s>>>(P, U_, CNT_, \
-                                                                                   out, n)
-        if (nri == 1) {
-            if (df) FEM3_APPLY(1, true, u_d + (int64_t)v0 * n, 1);
-            else FEM3_APPLY(1, false, u_d + (int64_t)v0 * n, 1);
-        } else if (nri == 4) {
-            if (df) FEM3_APPLY(4, true, ui, cnt);
-            else FEM3_APPLY(4, false, ui, cnt);
-        } else if (nri == 8) {
-            if (df) FEM3_APPLY(8, true, ui, cnt);
-            else FEM3_APPLY(8, false, ui, cnt);
-        } else {
-            if (df) FEM3_APPLY(17, true, ui, cnt);
-            else FEM3_APPLY(17, false, ui, cnt);
-        }
-#undef FEM3_APPLY
-        kc_end(m, KC_APPLY);
-        note_launch(m);
-    }
-    if (ui) FEM3_CUDA(cudaFreeAsync(ui, s));
-    FEM3_CUDA(cudaGetLastError());
-    return FEM3_OK;
-}
-
-int apply_A64(Mesh *m, const double *u_d, double *Au_d) { return apply_multi(m, u_d, 1, Au_d, true); }
 
 int axis_forms(Mesh *m, const double *u_d, const double *lam_d, double out[3]) {
     cudaStream_t s = m->stream;
@@ -1799,12 +1043,13 @@ int solve_direct(Mesh *m, const double *b_d, int nrhs, double *u_d) {
 
 // Refinement for all right-hand sides together: u = 0, r = b; repeat
 //   d = A32^{-1} r (FP32 factor, all columns in one wavefront sweep pair), u += d,
-//   r = b - A u (FP64 operator from the tables, double-float arithmetic),
-// until every column has ||r|| <= tol ||b|| or max_iter sweeps.  Once the residual is below
-// kLateFactor * tol, a sweep's residual is updated from its correction alone,
-// r = r - A d, with A d applied in plain FP32 (about 1e-6 relative): d is as small as r, so
-// the update's error is about 1e-6 ||r|| <= 1e-6 kLateFactor tol ||b|| = tol ||b|| / 100,
-// while the double-float apply of A u costs six times the instructions.
+//   r = b - A u in FP64, or r -= A d,
+// until every column has ||r|| <= tol ||b|| or max_iter sweeps.  The first sweep's residual is
+// formed from u in FP64.  Once the residual is below kUpdateBelow the correction is as small
+// against u, and r -= A d in double-float arithmetic (2^-46 relative to A d) keeps the FP64
+// residual's accuracy; below kLateFactor * tol plain FP32 (about 1e-6 relative) does: its
+// error is about 1e-6 ||r|| <= 1e-6 kLateFactor tol ||b|| = tol ||b|| / 100.
+constexpr double kUpdateBelow = 1e-3;
 constexpr double kLateFactor = 1e4;
 
 int refine_start(const RefineVecs &v, int64_t n, int nrhs, cudaStream_t s) {
@@ -1815,7 +1060,7 @@ int refine_start(const RefineVecs &v, int64_t n, int nrhs, cudaStream_t s) {
 }
 
 // one sweep, enqueued on m->stream; the norms arrive in m->h_norms (2 nrhs values)
-int refine_sweep(Mesh *m, const RefineVecs &v, int nrhs, bool late) {
+int refine_sweep(Mesh *m, const RefineVecs &v, int nrhs, RefineMode mode) {
     cudaStream_t s = m->stream;
     const int64_t n = m->n_dof, nn = n * nrhs;
     k_to_f32<<<g256(nn), 256, 0, s>>>(v.r, v.r32, nn);
@@ -1825,14 +1070,12 @@ int refine_sweep(Mesh *m, const RefineVecs &v, int nrhs, bool late) {
     k_axpy_f32<<<g256(nn), 256, 0, s>>>(v.r32, v.u, nn);
     note_launch(m);
     FEM3_CUDA(cudaMemsetAsync(m->norms, 0, sizeof(double) * 2 * nrhs, s));
-    if (late) {
-        k_f32_to_f64_n<<<g256(nn), 256, 0, s>>>(v.r32, v.d64, nn);
-        note_launch(m);
-        FEM3_TRY(apply_multi(m, v.d64, nrhs, v.Au, false));
-        k_residual_update_cols<<<dim3(g256(n), nrhs), 256, 0, s>>>(v.b, v.Au, n, v.r, m->norms);
-    } else {
-        FEM3_TRY(apply_multi(m, v.u, nrhs, v.Au, true));
+    if (mode == kRefineFull) {
+        FEM3_TRY(apply_multi(m, v.u, nrhs, v.Au));
         k_residual_cols<<<dim3(g256(n), nrhs), 256, 0, s>>>(v.b, v.Au, n, v.r, m->norms);
+    } else {
+        FEM3_TRY(apply_correction(m, v.r32, nrhs, v.Au, mode == kRefineLate));
+        k_residual_update_cols<<<dim3(g256(n), nrhs), 256, 0, s>>>(v.b, v.Au, n, v.r, m->norms);
     }
     note_launch(m);
     FEM3_CUDA(cudaMemcpyAsync(m->h_norms, m->norms, sizeof(double) * 2 * nrhs,
@@ -1840,16 +1083,53 @@ int refine_sweep(Mesh *m, const RefineVecs &v, int nrhs, bool late) {
     return FEM3_OK;
 }
 
-// largest relative residual of the sweep whose norms have arrived (infinity for NaN), and
-// whether the next sweep is a late one
-double refine_worst(const Mesh *m, int nrhs, double tol, bool *late) {
+static double worst_norm(const Mesh *m, int nrhs) {
     double worst = 0;
     for (int c = 0; c < nrhs; c++) {
         const double rel = m->h_norms[2 * c + 1] > 0 ? sqrt(m->h_norms[2 * c] / m->h_norms[2 * c + 1]) : 0.0;
         worst = (rel == rel) ? std::max(worst, rel) : INFINITY;
     }
-    *late = worst <= kLateFactor * tol;
     return worst;
+}
+
+// largest relative residual of the sweep whose norms have arrived (infinity for NaN), and
+// how the next sweep forms its residual
+double refine_worst(const Mesh *m, int nrhs, double tol, RefineMode *next) {
+    const double worst = worst_norm(m, nrhs);
+    *next = worst <= kLateFactor * tol ? kRefineLate
+                                       : (worst <= kUpdateBelow ? kRefineUpdate : kRefineFull);
+    return worst;
+}
+
+// largest ||b - A u|| / ||b|| over the columns (synchronises)
+int residual_worst(Mesh *m, const double *b, const double *u, int nrhs, double *worst) {
+    cudaStream_t s = m->stream;
+    const int64_t n = m->n_dof;
+    const int group = std::min(nrhs, kMaxRhs);
+    double *Au = nullptr;   // A u, then the residual
+    FEM3_CUDA(cudaMallocAsync((void **)&Au, sizeof(double) * n * group, s));
+    int st = FEM3_OK;
+    *worst = 0.0;
+    for (int c0 = 0; c0 < nrhs && st == FEM3_OK; c0 += group) {
+        const int cnt = std::min(group, nrhs - c0);
+        if (m->integer_order) {
+            for (int c = 0; c < cnt && st == FEM3_OK; c++)
+                st = apply_integer(m, u + (int64_t)(c0 + c) * n, Au + (int64_t)c * n);
+        } else {
+            st = apply_multi(m, u + (int64_t)c0 * n, cnt, Au);
+        }
+        if (st != FEM3_OK) break;
+        cudaMemsetAsync(m->norms, 0, sizeof(double) * 2 * cnt, s);
+        k_residual_cols<<<dim3(g256(n), cnt), 256, 0, s>>>(b + (int64_t)c0 * n, Au, n, Au, m->norms);
+        note_launch(m);
+        cudaError_t e = cudaMemcpyAsync(m->h_norms, m->norms, sizeof(double) * 2 * cnt,
+                                        cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) st = cuda_error(e, "residual norms");
+        else *worst = std::max(*worst, worst_norm(m, cnt));
+    }
+    cudaFreeAsync(Au, s);
+    return st;
 }
 
 int solve_refined(Mesh *m, const double *b_d, int nrhs, double tol, int max_iter, double *u_d,
@@ -1858,23 +1138,21 @@ int solve_refined(Mesh *m, const double *b_d, int nrhs, double tol, int max_iter
     const int64_t n = m->n_dof;
     const int64_t nn = n * nrhs;
     if (nrhs > 32) return set_error(FEM3_E_ARG, "at most 32 right-hand sides per solve");
-    RefineVecs v{b_d, u_d, nullptr, nullptr, nullptr, nullptr};
+    RefineVecs v{b_d, u_d, nullptr, nullptr, nullptr};
     FEM3_CUDA(cudaMallocAsync((void **)&v.Au, sizeof(double) * nn, s));
     FEM3_CUDA(cudaMallocAsync((void **)&v.r, sizeof(double) * nn, s));
-    FEM3_CUDA(cudaMallocAsync((void **)&v.d64, sizeof(double) * nn, s));
     FEM3_CUDA(cudaMallocAsync((void **)&v.r32, sizeof(float) * nn, s));
     int it = 0;
     double worst = 1.0;
-    bool late = false;
+    RefineMode mode = kRefineFull;
     int st = refine_start(v, n, nrhs, s);
     while (st == FEM3_OK) {
-        if ((st = refine_sweep(m, v, nrhs, late)) != FEM3_OK) break;
+        if ((st = refine_sweep(m, v, nrhs, mode)) != FEM3_OK) break;
         FEM3_CUDA(cudaStreamSynchronize(s));
-        worst = refine_worst(m, nrhs, tol, &late);
+        worst = refine_worst(m, nrhs, tol, &mode);
         it++;
         if (worst <= tol || it >= max_iter || !(worst < INFINITY)) break;
     }
-    cudaFreeAsync(v.d64, s);
     cudaFreeAsync(v.Au, s);
     cudaFreeAsync(v.r, s);
     cudaFreeAsync(v.r32, s);

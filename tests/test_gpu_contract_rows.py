@@ -42,7 +42,7 @@ def _bar_mesh(cells, h=(1.0, 1.0, 1.0)):
 
 
 # cells, bin_scale, least columns of the widest bin: one dof; a bin of a few dofs; one over 512
-# columns (two windows, more than 4,915 entries: several groups)
+# columns (three windows of 256, more entries than shared memory holds: several groups)
 SHAPES = [((2, 2, 2), 0.5, 1), ((5, 3, 4), 0.5, 4), ((45, 4, 5), 1.5, 513)]
 
 
@@ -66,4 +66,28 @@ def test_rows_contraction_matches_oracle(cells, scale, least, precision):
         m.sync()
         F_ref = o.assemble_form(0, 0.7, 0.4, left, coef)
         assert np.abs(F - F_ref).max() <= BAR[precision] * np.abs(F_ref).max()
+    m.free()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "tf32x3", "bf16x3"])
+@pytest.mark.parametrize("cells,scale", [(SHAPES[0][0], SHAPES[0][1]), (SHAPES[1][0], SHAPES[1][1]),
+                                         (SHAPES[2][0], SHAPES[2][1])])
+def test_operator_of_the_refinement(cells, scale, precision):
+    """The refinement's operator from the same meshes (its contraction is the double-float one):
+    1, 3 and 21 columns (one-, four- and 17-wide passes) refined to 1e-13 equal the oracle's
+    solutions to 1e-10, and the mixed form's residual is that of the oracle's matrix."""
+    mesh = _bar_mesh(cells)
+    o = oracle.Oracle.from_mesh(mesh)
+    alpha, K = (1.3, 1.6, 1.8), (1.0, 2.0, 0.5)
+    A = o.assemble(alpha, K)
+    m = fem3.Mesh(mesh.verts, mesh.tets, bin_scale=scale)
+    m.assemble(alpha, K, precision)
+    for nrhs in (1, 3, 21):
+        f = np.random.default_rng(nrhs).standard_normal((mesh.n_nodes, nrhs))
+        b = o.load(f)
+        u = m.solve(f, tol=1e-13).cpu().numpy().reshape(o.n_dof, nrhs)
+        ref = np.linalg.solve(A, b)
+        assert np.linalg.norm(u - ref) <= 1e-10 * np.linalg.norm(ref)
+        res = np.linalg.norm(b - A @ u, axis=0) / np.linalg.norm(b, axis=0)
+        assert res.max() <= 1e-12, res
     m.free()
