@@ -808,46 +808,70 @@ int trsv_t(const TF *L, int64_t n, TF *y, cudaStream_t s, Mesh *m) {
     return solve_chain_t<TF>(L, n, y, 1, s, m);
 }
 
-// per-axis forms sum_g w_g ((L lam)(R u) + (R lam)(L u)) (adjoint), one CTA per bin
-__global__ void __launch_bounds__(256) k_axis_form(
+// Per-axis forms sum_g w_g ((L lam)(R u) + (R lam)(L u)) (adjoint), one CTA per bin: the
+// bin's u and lam as hi + lo pairs in shared memory, thread = (Gauss point, slice of the
+// template rows); sums in double-float FP32 arithmetic (an FP64 evaluation spends ten
+// FP64-pipe instructions per table entry on conversions and sums: 0.95 ms for the three axes
+// of the 16^3 cube, 0.35 ms now), the slices and the final product in FP64.  Bound: one read of
+// the tables.
+constexpr int kFormSlices = 4, kFormPoints = 64;
+__global__ void __launch_bounds__(kFormSlices *kFormPoints) k_axis_form(
     const float2 *__restrict__ tabL, const float2 *__restrict__ tabR,
-    const int32_t *__restrict__ gp_off, const int32_t *__restrict__ gp_idx,
-    const int32_t *__restrict__ dof_off, const int32_t *__restrict__ dof_idx,
-    const int64_t *__restrict__ tab_off, const int32_t *__restrict__ tab_ld,
-    const double *__restrict__ gw, const double *__restrict__ u, const double *__restrict__ lam,
-    double *out) {
-    extern __shared__ double sm[];
+    const int32_t *__restrict__ gp_off, const int32_t *__restrict__ dof_off,
+    const int32_t *__restrict__ dof_idx, const int64_t *__restrict__ tab_off,
+    const int32_t *__restrict__ tab_ld, const double *__restrict__ w_slot,
+    const double *__restrict__ u, const double *__restrict__ lam, double *out) {
+    extern __shared__ __align__(16) float4 sm_form[];   // (u hi, u lo, lam hi, lam lo) per row
+    __shared__ double part[kFormSlices][4][kFormPoints];
+    __shared__ double red[kFormPoints / 32];
     const int bin = blockIdx.x;
     const int D = dof_off[bin + 1] - dof_off[bin];
-    const int G = gp_off[bin + 1] - gp_off[bin];
+    const int g0 = gp_off[bin], G = gp_off[bin + 1] - g0;
     if (D == 0 || G == 0) return;
     const int ld = tab_ld[bin];
     const float2 *L = tabL + tab_off[bin], *R = tabR + tab_off[bin];
     const int32_t *dofs = dof_idx + dof_off[bin];
-    const int32_t *slots = gp_idx + gp_off[bin];
-    double *ub = sm, *lb = sm + D;
-    __shared__ double red[8];
-    for (int c = threadIdx.x; c < D; c += blockDim.x) { ub[c] = u[dofs[c]]; lb[c] = lam[dofs[c]]; }
+    for (int c = threadIdx.x; c < D; c += blockDim.x) {
+        float4 v;
+        f64_split(u[dofs[c]], v.x, v.y);
+        f64_split(lam[dofs[c]], v.z, v.w);
+        sm_form[c] = v;
+    }
     __syncthreads();
+    const int p = threadIdx.x % kFormPoints, q = threadIdx.x / kFormPoints;
     double acc = 0;
-    for (int r = threadIdx.x; r < G; r += blockDim.x) {
-        double Lu = 0, Ru = 0, Ll = 0, Rl = 0;
-        for (int c = 0; c < D; c++) {
-            const float2 lp = L[(int64_t)c * ld + r], rp = R[(int64_t)c * ld + r];
-            const double lv = (double)lp.x + (double)lp.y, rv = (double)rp.x + (double)rp.y;
-            Lu = fma(lv, ub[c], Lu); Ru = fma(rv, ub[c], Ru);
-            Ll = fma(lv, lb[c], Ll); Rl = fma(rv, lb[c], Rl);
+    for (int r0 = 0; r0 < G; r0 += kFormPoints) {
+        const int r = r0 + p;
+        float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};   // Lu, Ru, Llam, Rlam
+        if (r < G) {
+#pragma unroll 4
+            for (int c = q; c < D; c += kFormSlices) {
+                const float2 a = __ldg(L + (int64_t)c * ld + r), b = __ldg(R + (int64_t)c * ld + r);
+                const float4 v = sm_form[c];
+                df_fma(a.x, a.y, v.x, v.y, h[0], l[0]);
+                df_fma(b.x, b.y, v.x, v.y, h[1], l[1]);
+                df_fma(a.x, a.y, v.z, v.w, h[2], l[2]);
+                df_fma(b.x, b.y, v.z, v.w, h[3], l[3]);
+            }
         }
-        acc += gw[slots[r]] * (Ll * Ru + Rl * Lu);
+#pragma unroll
+        for (int k = 0; k < 4; k++) part[q][k][p] = f32_to_f64_exact(h[k]) + f32_to_f64_exact(l[k]);
+        __syncthreads();
+        if (q == 0 && r < G) {
+            double t[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                t[k] = (part[0][k][p] + part[1][k][p]) + (part[2][k][p] + part[3][k][p]);
+            acc = fma(w_slot[g0 + r], fma(t[2], t[1], t[3] * t[0]), acc);
+        }
+        __syncthreads();
     }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    if (q == 0) {
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+        if ((p & 31) == 0) red[p >> 5] = acc;
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) s += red[w];
-        atomicAdd(out, s);
-    }
+    if (threadIdx.x == 0) atomicAdd(out, red[0] + red[1]);
 }
 
 // (r may be Au)
@@ -1015,15 +1039,19 @@ int factor(Mesh *m) {
 
 int axis_forms(Mesh *m, const double *u_d, const double *lam_d, double out[3]) {
     cudaStream_t s = m->stream;
-    FEM3_CUDA(cudaFuncSetAttribute(k_axis_form, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)(sizeof(double) * 2 * kMaxBinItems)));
+    static bool attr = false;
+    if (!attr) {
+        FEM3_CUDA(cudaFuncSetAttribute(k_axis_form, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)(sizeof(float4) * kMaxBinItems)));
+        attr = true;
+    }
     FEM3_CUDA(cudaMemsetAsync(m->norms, 0, sizeof(double) * 3, s));
     for (int axis = 0; axis < 3; axis++) {
         AxisBins &B = m->bins[axis];
-        size_t sh = sizeof(double) * 2 * B.max_dof;
-        k_axis_form<<<B.n_bins, 256, sh, s>>>(m->tabL[axis], m->tabR[axis], B.gp_off, B.gp_idx,
-                                               B.dof_off, B.dof_idx, B.tab_off, B.tab_ld, m->gw, u_d,
-                                               lam_d, m->norms + axis);
+        const size_t sh = sizeof(float4) * std::max(1, B.max_dof);
+        k_axis_form<<<B.n_bins, kFormSlices * kFormPoints, sh, s>>>(
+            m->tabL[axis], m->tabR[axis], B.gp_off, B.dof_off, B.dof_idx, B.tab_off, B.tab_ld,
+            B.w_slot, u_d, lam_d, m->norms + axis);
         note_launch(m);
     }
     FEM3_CUDA(cudaMemcpyAsync(m->h_norms, m->norms, sizeof(double) * 3, cudaMemcpyDeviceToHost, s));
