@@ -290,11 +290,6 @@ int fem3_mesh_upload(const double *verts, int64_t n_nodes, const int32_t *tets, 
     if ((st = bins_build(m)) != FEM3_OK) return fail(st);
     stage_end(m, 1);
     const int64_t n = std::max<int64_t>(1, m->n_dof);
-    if ((st = dev_alloc_t(m, &m->flags, 2 * ((n + 63) / 64) + 2)) != FEM3_OK) return fail(st);
-    if ((st = dev_alloc(m, &m->solve_ws, sizeof(double) * 64 * 24 * ((n + 63) / 64))) != FEM3_OK)
-        return fail(st);
-    if ((st = dev_alloc(m, &m->solve_G, sizeof(double) * 2 * 3 * 64 * 64 * ((n + 63) / 64))) != FEM3_OK)
-        return fail(st);
     if ((st = dev_alloc(m, &m->dinv, sizeof(double) * 64 * 64 * ((n + 63) / 64))) != FEM3_OK)
         return fail(st);
     {
@@ -302,14 +297,10 @@ int fem3_mesh_upload(const double *verts, int64_t n_nodes, const int32_t *tets, 
         if ((st = dev_alloc_t(m, &m->chol_flags, chol_f64_flags(n))) != FEM3_OK)
             return fail(st);
     }
-    if (cudaMemsetAsync(m->flags, 0, sizeof(int32_t) * (2 * ((n + 63) / 64) + 2), m->stream) != cudaSuccess)
-        return fail(cuda_error(cudaGetLastError(), "cudaMemsetAsync"));
     for (int k = 0; k < 6; k++)
         if ((st = dev_alloc_t(m, &m->vec64[k], std::max<int64_t>(std::max<int64_t>(n, m->n_nodes),
                                                                  64 * 64))) != FEM3_OK)
             return fail(st);
-    for (int k = 0; k < 2; k++)
-        if ((st = dev_alloc_t(m, &m->vec32[k], n)) != FEM3_OK) return fail(st);
     if ((st = check_errors(m)) != FEM3_OK) return fail(st);
     *out = reinterpret_cast<fem3_mesh>(m);
     return FEM3_OK;

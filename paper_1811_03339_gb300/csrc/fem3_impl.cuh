@@ -162,17 +162,14 @@ struct Mesh {
 
     // workspaces
     double *vec64[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-    float *vec32[2] = {nullptr, nullptr};
-    int32_t *flags = nullptr;  // triangular-solve flags: [2 nblk + 2]
-    void *solve_ws = nullptr;  // triangular-solve z blocks: nblk x 64 x 24 doubles
-    void *solve_G = nullptr;   // triangular-solve chain operators: nblk x 2 x 3 x 64 x 64 doubles
+    void *solve_ws = nullptr;  // triangular solves: [kTriRhs][n_dof], FP64 or FP32
+    void *tri_inv = nullptr;   // inverses of the factor's wide diagonal blocks (trisolve.cu)
     int32_t *chol_flags = nullptr;  // tile-factorisation flags, then ticket and abort words
     void *dinv = nullptr;      // inverses of the 64 x 64 diagonal blocks of the factor
     float *chol_w = nullptr;   // tensor-core factorisation: TF32 hi / lo operand rows, panel inverse
     int64_t chol_w_rows = 0;
     int chol_tc_opt = 0;       // 0: by size, 1: always, -1: never (tensor-core factorisation)
     bool chol_tc_used = false; // the last factorisation ran on the tensor cores
-    int flag_epoch = 0;        // value that marks "ready" in the current solve
     double *norms = nullptr;   // device scratch for reductions
     double *h_norms = nullptr; // pinned host mirror
 
@@ -229,7 +226,7 @@ enum KernelClass {
     KC_SPLIT = 1,     // operand splits: the tables' (k_split_ops), the operator's (k_op_mirror)
     KC_CONTRACT = 2,  // contraction GEMMs (tensor-core or CUDA-core)
     KC_FACTOR = 3,    // Cholesky factorisation
-    KC_CHAIN = 4,     // triangular-solve chains
+    KC_CHAIN = 4,     // triangular solves (both directions of a group of columns)
     KC_APPLY = 5,     // operator apply of the refinement residual
     KC_COUNT = 6
 };
@@ -278,6 +275,12 @@ int load_vector(Mesh *m, const double *f_d, int nrhs, double *b_d);
 int load_vector_T(Mesh *m, const double *lam_d, double *out_d);
 int factor(Mesh *m);
 int chol_tc(Mesh *m, float *A, int64_t n);
+// triangular solves with a factor (A's tiles below the 64 x 64 diagonal blocks, their inverses in
+// dinv): the wide diagonal inverses, once per factorisation, then L L^T x = y in place for
+// column-major [n][nrhs]
+constexpr int kTriRhs = 24;
+template <class TF> int tri_prepare(Mesh *m, const TF *L, int64_t n);
+template <class TF> int tri_solve(Mesh *m, const TF *L, int64_t n, TF *Y, int nrhs);
 int assemble_integer(Mesh *m, const double K[3]);       // P1 stiffness, alpha_i = 2
 int axis_forms_integer(Mesh *m, const double *u, const double *lam, double out[3]);
 int apply_integer(Mesh *m, const double *x, double *y); // y = A x, element by element

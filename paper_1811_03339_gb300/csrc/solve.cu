@@ -6,7 +6,7 @@
 //    tensor cores (chol_tc.cu); row-major storage: the tiles below the diagonal in A's
 //    lower triangle, each 64 x 64 diagonal block as its inverse L_jj^{-1} (all the solves
 //    use).
-//  - Blocked forward / backward substitution.
+//  - Triangular solves: trisolve.cu.
 //  - Refinement for the mixed forms: r = b - A u with A u applied at FP64 accuracy
 //    (operator.cu), the correction solved with the FP32 factor.
 #include <math.h>
@@ -372,9 +372,6 @@ __global__ void __launch_bounds__(512, 1) k_chol_tiles(float *A, int64_t n, int 
     }
 }
 
-// at most this many right-hand sides per triangular-solve launch
-constexpr int kMaxRhs = 24;
-
 int chol_tiles(float *A, int64_t n, cudaStream_t s, Mesh *m) {
     if (n <= 0) return FEM3_OK;
     const int nblk = (int)((n + NB - 1) / NB);
@@ -395,417 +392,6 @@ int chol_tiles(float *A, int64_t n, cudaStream_t s, Mesh *m) {
     note_launch(m);
     FEM3_CUDA(cudaGetLastError());
     return FEM3_OK;
-}
-
-// ---------------------------------------------------------------------------------
-// Chain triangular solves (one launch per direction, 1..24 right-hand sides).
-// Forward: y_j = Dinv_j (b_j - sum_{k<j} L_jk y_k); backward: x_j = Dinv_j^T (y_j -
-// sum_{k>j} L_kj^T x_k).  Step s solves block j(s) (j = s forward, nblk-1-s backward);
-// M(s, s') is the coefficient tile between the blocks of steps s and s' < s.
-// CTA 0 runs the chain: at step s it waits for the workers' partial sum S_s (all
-// dependencies s' < s - D), applies the D nearest tiles M(s, s-1 .. s-D) itself from
-// registers loaded one step ahead, multiplies by the diagonal inverse and publishes the
-// block (flag Yf).  Worker CTAs take steps s > D from an atomic ticket in increasing order,
-// accumulate S_s as the blocks s' <= s - D - 1 appear and publish it (flag Pf).  The
-// chain only waits for tickets that precede the ones any worker can be blocked on, so the
-// launch needs no co-residency; waits are bounded (ERR_SOLVE, abort word).
-// Y is column-major (n x nrhs, leading dimension n), solved in place.  flags: Yf [nblk],
-// Pf [nblk], ticket, abort word, all zero at launch; Z: nblk x 64 x 24 workspace.
-// ---------------------------------------------------------------------------------
-constexpr int kSolveThreads = 512;            // thread (r, g): row r = t & 63, column chunk g = t >> 6
-
-template <class TF> struct SolveCfg {
-    // dependency tiles the chain applies itself: one more lengthens every chain step, one
-    // fewer puts the workers' hand-over on the critical path (2 timed fastest, both types)
-    static constexpr int D = 2;
-};
-
-// shared memory: ring of D + 1 solved blocks [64][NR] (chain) or one dependency block and
-// one right-hand-side block (worker), and 8 partial buffers [64][NR + 1]
-template <class TF, int NR>
-constexpr size_t solve_chain_smem() {
-    return ((size_t)(SolveCfg<TF>::D + 1) * NB * NR + (size_t)8 * NB * (NR + 1)) * sizeof(TF);
-}
-
-// Precomputed chain operators.  Step s of a direction solves block j; its dependency d
-// (d < D) is the block solved at step s - 1 - d.  G(s, d) = Dm_j M(s, s-1-d), with Dm_j
-// the diagonal inverse as applied (transposed when backward) and M the coefficient tile,
-// so that the chain step is y_s = z_s - sum_d G(s, d) y_{s-1-d}, z_s = Dm_j (b_s - S_s).
-// Layout per (direction, s, d): element (r, c = 8g + e) at (g * 64 + r) * 8 + e, i.e. the
-// eight values thread (r, g) needs are 32 contiguous bytes.
-__device__ __forceinline__ int64_t gop_index(int dir, int s, int d, int nblk, int D) {
-    return (((int64_t)dir * nblk + s) * D + d) * (NB * NB);
-}
-
-__device__ __forceinline__ int solve_blk(int s, int nblk, bool backward) {
-    return backward ? nblk - 1 - s : s;
-}
-
-// NR consecutive values of a shared row (16-byte aligned when NR > 1)
-template <class TF, int NR>
-__device__ __forceinline__ void ld_row(const TF *p, TF out[NR]) {
-    if constexpr (NR == 1) {
-        out[0] = p[0];
-    } else if constexpr (sizeof(TF) == 4) {
-#pragma unroll
-        for (int k = 0; k < NR / 4; k++) {
-            const float4 q = reinterpret_cast<const float4 *>(p)[k];
-            out[4 * k] = q.x; out[4 * k + 1] = q.y; out[4 * k + 2] = q.z; out[4 * k + 3] = q.w;
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < NR / 2; k++) {
-            const double2 q = reinterpret_cast<const double2 *>(p)[k];
-            out[2 * k] = q.x; out[2 * k + 1] = q.y;
-        }
-    }
-}
-
-// this thread's eight entries M[r][8g .. 8g+7] of the tile between blocks j (solved) and jd
-template <class TF>
-__device__ __forceinline__ void load_coef(const TF *__restrict__ L, int64_t n, int j, int jd,
-                                          bool backward, int r, int g, TF out[8]) {
-#pragma unroll
-    for (int e = 0; e < 8; e++) {
-        const int c = g * 8 + e;
-        const int64_t row = backward ? (int64_t)jd * NB + c : (int64_t)j * NB + r;
-        const int64_t col = backward ? (int64_t)j * NB + r : (int64_t)jd * NB + c;
-        out[e] = row < n ? __ldg(&L[row * n + col]) : TF(0);
-    }
-}
-
-// diagonal inverse of block j as applied at this step (transposed when backward)
-template <class TF>
-__device__ __forceinline__ void load_dinv(const TF *__restrict__ Dinv, int j, bool backward, int r,
-                                          int g, TF out[8]) {
-    const TF *Dj = Dinv + (int64_t)j * NB * NB;
-#pragma unroll
-    for (int e = 0; e < 8; e++) {
-        const int c = g * 8 + e;
-        out[e] = __ldg(&Dj[backward ? c * NB + r : r * NB + c]);
-    }
-}
-
-__device__ __forceinline__ bool wait_flag(const int *f, int *abort_w, int32_t *err) {
-    int spins = 0;
-    while (ld_acquire_gpu(f) == 0) {
-        if (ld_acquire_gpu(abort_w) != 0) return false;
-        if (++spins > kSpinLimit) {
-            atomicAdd(&err[ERR_SOLVE], 1);
-            atomicExch(abort_w, 1);
-            return false;
-        }
-        if (spins > 64) __nanosleep(32);
-    }
-    return true;
-}
-
-// part[v] += sum_e m[e] rows[8g + e][v], v < NR
-template <class TF, int NR>
-__device__ __forceinline__ void chunk_gemv(const TF m[8], const TF *rows, int g, TF part[NR]) {
-#pragma unroll
-    for (int e = 0; e < 8; e++) {
-        TF yv[NR];
-        ld_row<TF, NR>(rows + (g * 8 + e) * NR, yv);
-#pragma unroll
-        for (int v = 0; v < NR; v++) part[v] = fma(m[e], yv[v], part[v]);
-    }
-}
-
-// red[g][r][v] = part[v]; after a barrier, the owner of (r, v) adds the eight partials
-template <class TF, int NR>
-__device__ __forceinline__ void store_partial(TF *red, int r, int g, const TF part[NR]) {
-#pragma unroll
-    for (int v = 0; v < NR; v++) red[(g * NB + r) * (NR + 1) + v] = part[v];
-}
-template <class TF, int NR>
-__device__ __forceinline__ TF sum_partials(const TF *red, int r, int v) {
-    TF t = TF(0);
-#pragma unroll
-    for (int q = 0; q < 8; q++) t += red[(q * NB + r) * (NR + 1) + v];
-    return t;
-}
-
-// G(s, d) for one direction, step and dependency (grid: nblk x D x 2 directions)
-template <class TF>
-__global__ void __launch_bounds__(256) k_solve_prep(const TF *__restrict__ L,
-                                                    const TF *__restrict__ Dinv, int64_t n,
-                                                    int nblk, TF *Gop) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int D = SolveCfg<TF>::D;
-    TF(*dm)[NB + 1] = reinterpret_cast<TF(*)[NB + 1]>(smem_raw);   // Dm[r][k]
-    TF(*mm)[NB + 1] = dm + NB;                                     // M[k][c]
-    const int s = blockIdx.x, d = blockIdx.y, dir = blockIdx.z;
-    if (s - 1 - d < 0) return;
-    const bool bw = dir != 0;
-    const int j = solve_blk(s, nblk, bw), jd = solve_blk(s - 1 - d, nblk, bw);
-    const TF *Dj = Dinv + (int64_t)j * NB * NB;
-    for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-        const int hi = e >> 6, lo = e & 63;
-        // Dm[r][k] = Dinv_j[r][k] (forward) or Dinv_j[k][r] (backward); read row-major
-        if (!bw) dm[hi][lo] = Dj[e];
-        else dm[lo][hi] = Dj[e];
-        // M[k][c] = L[j*64 + k][jd*64 + c] (forward) or L[jd*64 + c][j*64 + k] (backward)
-        const int64_t grow = (bw ? (int64_t)jd : (int64_t)j) * NB + hi;
-        const int64_t gcol = (bw ? (int64_t)j : (int64_t)jd) * NB + lo;
-        const TF v = grow < n ? L[grow * n + gcol] : TF(0);
-        if (!bw) mm[hi][lo] = v;
-        else mm[lo][hi] = v;
-    }
-    __syncthreads();
-    TF *G = Gop + gop_index(dir, s, d, nblk, D);
-    for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-        const int r = e & 63, c = e >> 6;
-        TF acc = TF(0);
-#pragma unroll 8
-        for (int k = 0; k < NB; k++) acc = fma(dm[r][k], mm[k][c], acc);
-        G[((c >> 3) * NB + r) * 8 + (c & 7)] = acc;
-    }
-}
-
-template <class TF>
-__device__ __forceinline__ void load_g(const TF *G, int r, int g, TF out[8]) {
-    const TF *p = G + (g * NB + r) * 8;
-    if constexpr (sizeof(TF) == 4) {
-        const float4 a = __ldg(reinterpret_cast<const float4 *>(p));
-        const float4 b = __ldg(reinterpret_cast<const float4 *>(p) + 1);
-        out[0] = a.x; out[1] = a.y; out[2] = a.z; out[3] = a.w;
-        out[4] = b.x; out[5] = b.y; out[6] = b.z; out[7] = b.w;
-    } else {
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            const double2 a = __ldg(reinterpret_cast<const double2 *>(p) + k);
-            out[2 * k] = a.x; out[2 * k + 1] = a.y;
-        }
-    }
-}
-
-template <class TF, int NR>
-__device__ void solve_chain(int64_t n, int nblk, TF *Y, int nrhs, bool backward, const TF *Gop,
-                            const TF *Z, int *Yf, const int *Pf, int *abort_w, int32_t *err,
-                            unsigned char *smem_raw) {
-    constexpr int D = SolveCfg<TF>::D;
-    TF *yr = reinterpret_cast<TF *>(smem_raw);        // [D + 1][64][NR] ring of solved blocks
-    TF *red = yr + (D + 1) * NB * NR;                 // [8][64][NR + 1]
-    __shared__ int s_ok;
-    const int tid = threadIdx.x, r = tid & 63, g = tid >> 6;
-    const int dir = backward ? 1 : 0;
-    TF gc[D][8], gn[D][8];
-#pragma unroll
-    for (int d = 0; d < D; d++)
-#pragma unroll
-        for (int e = 0; e < 8; e++) { gc[d][e] = TF(0); gn[d][e] = TF(0); }
-    for (int s = 0; s < nblk; s++) {
-        const int j = solve_blk(s, nblk, backward);
-        const int64_t row = (int64_t)j * NB + r;
-        // warp 1 waits for z_s while thread 0 may still be publishing the last block
-        if (tid == 32) s_ok = wait_flag(&Pf[s], abort_w, err);
-        if (s + 1 < nblk) {
-#pragma unroll
-            for (int d = 0; d < D; d++)
-                if (s - d >= 0) load_g<TF>(Gop + gop_index(dir, s + 1, d, nblk, D), r, g, gn[d]);
-        }
-        TF part[NR];
-#pragma unroll
-        for (int v = 0; v < NR; v++) part[v] = TF(0);
-#pragma unroll
-        for (int d = 0; d < D; d++)
-            if (s - 1 - d >= 0)
-                chunk_gemv<TF, NR>(gc[d], yr + ((s - 1 - d) % (D + 1)) * NB * NR, g, part);
-        store_partial<TF, NR>(red, r, g, part);
-        __syncthreads();
-        if (!s_ok) return;
-        TF *ys = yr + (s % (D + 1)) * NB * NR;
-#pragma unroll
-        for (int h = 0; h < (NR + 7) / 8; h++) {
-            const int v = g + 8 * h;
-            if (v < NR) {
-                const TF y = __ldcg(&Z[((int64_t)s * NB + r) * kMaxRhs + v]) -
-                             sum_partials<TF, NR>(red, r, v);
-                ys[r * NR + v] = y;
-                if (row < n && v < nrhs) Y[row + (int64_t)v * n] = y;
-            }
-        }
-        __syncthreads();
-        // the barrier orders every thread's stores of the block before thread 0's release,
-        // which carries them to the consumers that acquire the flag (release is cumulative)
-        if (tid == 0) st_release_gpu(&Yf[s], 1);
-#pragma unroll
-        for (int d = 0; d < D; d++)
-#pragma unroll
-            for (int e = 0; e < 8; e++) gc[d][e] = gn[d][e];
-    }
-}
-
-template <class TF, int NR>
-__global__ void __launch_bounds__(kSolveThreads, 1) k_solve_chain(
-    const TF *__restrict__ L, const TF *__restrict__ Dinv, int64_t n, int nblk, TF *Y, int nrhs,
-    int backward, const TF *__restrict__ Gop, TF *Z, int *flags, int32_t *err) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int D = SolveCfg<TF>::D;
-    int *Yf = flags, *Pf = flags + nblk, *ticket = flags + 2 * nblk, *abort_w = ticket + 1;
-    if (blockIdx.x == 0) {
-        solve_chain<TF, NR>(n, nblk, Y, nrhs, backward != 0, Gop, Z, Yf, Pf, abort_w, err, smem_raw);
-        return;
-    }
-    TF *yb = reinterpret_cast<TF *>(smem_raw);   // [2][64][NR] dependency blocks, then b - S
-    TF *red = yb + 2 * NB * NR;                  // [8][64][NR + 1]
-    __shared__ int s_task, s_ok, s_pre[2];
-    const int tid = threadIdx.x, r = tid & 63, g = tid >> 6;
-    const bool bw = backward != 0;
-    for (;;) {
-        if (tid == 0) s_task = atomicAdd(ticket, 1);
-        __syncthreads();
-        const int s = s_task;
-        if (s >= nblk) return;
-        const int j = solve_blk(s, nblk, bw);
-        TF part[NR];
-#pragma unroll
-        for (int v = 0; v < NR; v++) part[v] = TF(0);
-        // Dependencies sd = 0 .. last, pipelined: the solved block y_{sd+1} is loaded into
-        // registers while the product with y_sd runs (when its flag is already set;
-        // otherwise after it, with a blocking wait) and stored into the other shared buffer.
-        constexpr int PY = (NB * NR + kSolveThreads - 1) / kSolveThreads;   // y values / thread
-        const int last = s - D - 1;
-        auto load_y = [&](int sd, TF yv[PY]) {
-            const int jd = solve_blk(sd, nblk, bw);
-#pragma unroll
-            for (int k = 0; k < PY; k++) {
-                const int e = tid + k * kSolveThreads;
-                const int c = e / NR, v = e % NR;
-                const int64_t rr = (int64_t)jd * NB + c;
-                yv[k] = (e < NB * NR && rr < n && v < nrhs) ? __ldcg(&Y[rr + (int64_t)v * n]) : TF(0);
-            }
-        };
-        TF tc[8], yv[PY];
-        bool have = false;   // yv holds y_sd
-        if (last >= 0) load_coef<TF>(L, n, j, solve_blk(0, nblk, bw), bw, r, g, tc);
-        for (int sd = 0; sd <= last; sd++) {
-            TF *ybs = yb + (sd & 1) * NB * NR;
-            if (!have) {
-                if (tid == 0) s_ok = wait_flag(&Yf[sd], abort_w, err);
-                __syncthreads();
-                if (!s_ok) return;
-                load_y(sd, yv);
-            }
-#pragma unroll
-            for (int k = 0; k < PY; k++)
-                if (tid + k * kSolveThreads < NB * NR) ybs[tid + k * kSolveThreads] = yv[k];
-            const int q = (sd + 1) & 1;
-            if (tid == 0 && sd + 1 <= last) s_pre[q] = ld_acquire_gpu(&Yf[sd + 1]) != 0;
-            __syncthreads();   // y_sd stored (the buffer written two dependencies ago is no
-                               // longer read); y_{sd+1}'s flag seen
-            have = sd + 1 <= last && s_pre[q];
-            if (have) load_y(sd + 1, yv);
-            TF tn[8];
-            if (sd + 1 <= last) load_coef<TF>(L, n, j, solve_blk(sd + 1, nblk, bw), bw, r, g, tn);
-            chunk_gemv<TF, NR>(tc, ybs, g, part);
-#pragma unroll
-            for (int e = 0; e < 8; e++) tc[e] = tn[e];
-        }
-        __syncthreads();   // the last product is done before yb is reused
-        // t = b_s - S_s into yb, then z_s = Dm_j t
-        store_partial<TF, NR>(red, r, g, part);
-        __syncthreads();
-#pragma unroll
-        for (int h = 0; h < (NR + 7) / 8; h++) {
-            const int v = g + 8 * h;
-            if (v < NR) {
-                const int64_t row = (int64_t)j * NB + r;
-                const TF b = (row < n && v < nrhs) ? __ldcg(&Y[row + (int64_t)v * n]) : TF(0);
-                yb[r * NR + v] = b - sum_partials<TF, NR>(red, r, v);
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int v = 0; v < NR; v++) part[v] = TF(0);
-        {
-            TF dm[8];
-            load_dinv<TF>(Dinv, j, bw, r, g, dm);
-            chunk_gemv<TF, NR>(dm, yb, g, part);
-        }
-        store_partial<TF, NR>(red, r, g, part);
-        __syncthreads();
-#pragma unroll
-        for (int h = 0; h < (NR + 7) / 8; h++) {
-            const int v = g + 8 * h;
-            if (v < NR) Z[((int64_t)s * NB + r) * kMaxRhs + v] = sum_partials<TF, NR>(red, r, v);
-        }
-        __syncthreads();
-        if (tid == 0) st_release_gpu(&Pf[s], 1);
-    }
-}
-
-template <class TF, int NR>
-static int launch_solve_chain(const TF *L, const TF *Dinv, int64_t n, int nblk, TF *Y, int nrhs,
-                              const TF *Gop, TF *Z, int workers, cudaStream_t s, Mesh *m) {
-    static bool attr = false;
-    if (!attr) {
-        FEM3_CUDA(cudaFuncSetAttribute(k_solve_chain<TF, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)solve_chain_smem<TF, NR>()));
-        attr = true;
-    }
-    for (int backward = 0; backward < 2; backward++) {
-        FEM3_CUDA(cudaMemsetAsync(m->flags, 0, sizeof(int32_t) * (2 * nblk + 2), s));
-        kc_begin(m, KC_CHAIN);
-        k_solve_chain<TF, NR><<<1 + workers, kSolveThreads, solve_chain_smem<TF, NR>(), s>>>(
-            L, Dinv, n, nblk, Y, nrhs, backward, Gop, Z, m->flags, m->err);
-        kc_end(m, KC_CHAIN);
-        note_launch(m);
-    }
-    return FEM3_OK;
-}
-
-// Chain operators of the current factor (run once per factorisation).
-template <class TF>
-int solve_prep_t(const TF *L, int64_t n, cudaStream_t s, Mesh *m) {
-    if (n <= 0) return FEM3_OK;
-    const int nblk = (int)((n + NB - 1) / NB);
-    const size_t sh = 2 * NB * (NB + 1) * sizeof(TF);
-    static bool attr = false;
-    if (!attr) {
-        FEM3_CUDA(cudaFuncSetAttribute(k_solve_prep<TF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
-        attr = true;
-    }
-    k_solve_prep<TF><<<dim3(nblk, SolveCfg<TF>::D, 2), 256, sh, s>>>(
-        L, reinterpret_cast<const TF *>(m->dinv), n, nblk, reinterpret_cast<TF *>(m->solve_G));
-    note_launch(m);
-    FEM3_CUDA(cudaGetLastError());
-    return FEM3_OK;
-}
-
-// L y = b (forward) then L^T x = y (backward), in place in Y (n x nrhs, nrhs <= 24);
-// uses the operators of solve_prep_t for the same factor.
-template <class TF>
-int solve_chain_t(const TF *L, int64_t n, TF *Y, int nrhs, cudaStream_t s, Mesh *m) {
-    if (n <= 0) return FEM3_OK;
-    if (nrhs < 1 || nrhs > kMaxRhs) return set_error(FEM3_E_ARG, "1..24 right-hand sides per block solve");
-    const int nblk = (int)((n + NB - 1) / NB);
-    static int sms = 0;
-    if (sms == 0) {
-        int dev = 0;
-        FEM3_CUDA(cudaGetDevice(&dev));
-        FEM3_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    }
-    const int workers = std::max(1, std::min(nblk, sms - 1));
-    const TF *Dinv = reinterpret_cast<const TF *>(m->dinv);
-    const TF *Gop = reinterpret_cast<const TF *>(m->solve_G);
-    TF *Z = reinterpret_cast<TF *>(m->solve_ws);
-    if (nrhs == 1) FEM3_TRY((launch_solve_chain<TF, 1>(L, Dinv, n, nblk, Y, nrhs, Gop, Z, workers, s, m)));
-    else if (nrhs <= 4) FEM3_TRY((launch_solve_chain<TF, 4>(L, Dinv, n, nblk, Y, nrhs, Gop, Z, workers, s, m)));
-    else if (nrhs <= 8) FEM3_TRY((launch_solve_chain<TF, 8>(L, Dinv, n, nblk, Y, nrhs, Gop, Z, workers, s, m)));
-    else if (nrhs <= 16) FEM3_TRY((launch_solve_chain<TF, 16>(L, Dinv, n, nblk, Y, nrhs, Gop, Z, workers, s, m)));
-    else if (nrhs <= 20) FEM3_TRY((launch_solve_chain<TF, 20>(L, Dinv, n, nblk, Y, nrhs, Gop, Z, workers, s, m)));
-    else FEM3_TRY((launch_solve_chain<TF, 24>(L, Dinv, n, nblk, Y, nrhs, Gop, Z, workers, s, m)));
-    FEM3_CUDA(cudaGetLastError());
-    return FEM3_OK;
-}
-
-// L y = b then L^T x = y, in place; cooperative wavefront kernel when all block CTAs
-// fit on the device at once, otherwise blocked substitution with one launch per block.
-template <class TF>
-int trsv_t(const TF *L, int64_t n, TF *y, cudaStream_t s, Mesh *m) {
-    return solve_chain_t<TF>(L, n, y, 1, s, m);
 }
 
 // Per-axis forms sum_g w_g ((L lam)(R u) + (R lam)(L u)) (adjoint), one CTA per bin: the
@@ -977,12 +563,6 @@ int sub_vec(const double *a, const double *b, double *c, int64_t n, cudaStream_t
     return FEM3_OK;
 }
 
-// L Y = B then L^T X = Y for nrhs <= 24 columns (column-major, leading dimension n)
-template <class TF>
-int trsm_t(const TF *L, int64_t n, TF *Y, int nrhs, cudaStream_t s, Mesh *m) {
-    return solve_chain_t<TF>(L, n, Y, nrhs, s, m);
-}
-
 int load_vector(Mesh *m, const double *f_d, int nrhs, double *b_d) {
     cudaStream_t s = m->stream;
     FEM3_CUDA(cudaMemsetAsync(b_d, 0, sizeof(double) * m->n_dof * nrhs, s));
@@ -1019,7 +599,7 @@ int factor(Mesh *m) {
                           m->stream, &launches));
         kc_end(m, KC_FACTOR);
         m->launches += launches;
-        return solve_prep_t<double>(m->A64, m->n_dof, m->stream, m);
+        return tri_prepare<double>(m, m->A64, m->n_dof);
     }
     const bool tc = m->chol_tc_opt > 0 || (m->chol_tc_opt == 0 && m->n_dof >= kCholTcMinN);
     if (tc) {
@@ -1034,7 +614,7 @@ int factor(Mesh *m) {
         }
         FEM3_TRY(chol_tiles(m->A32, m->n_dof, m->stream, m));
     }
-    return solve_prep_t<float>(m->A32, m->n_dof, m->stream, m);
+    return tri_prepare<float>(m, m->A32, m->n_dof);
 }
 
 int axis_forms(Mesh *m, const double *u_d, const double *lam_d, double out[3]) {
@@ -1064,9 +644,7 @@ int solve_direct(Mesh *m, const double *b_d, int nrhs, double *u_d) {
     cudaStream_t s = m->stream;
     const int64_t n = m->n_dof;
     FEM3_CUDA(cudaMemcpyAsync(u_d, b_d, sizeof(double) * n * nrhs, cudaMemcpyDeviceToDevice, s));
-    for (int c0 = 0; c0 < nrhs; c0 += kMaxRhs)
-        FEM3_TRY(trsm_t<double>(m->A64, n, u_d + (int64_t)c0 * n, std::min(kMaxRhs, nrhs - c0), s, m));
-    return FEM3_OK;
+    return tri_solve<double>(m, m->A64, n, u_d, nrhs);
 }
 
 // Refinement for all right-hand sides together: u = 0, r = b; repeat
@@ -1093,8 +671,7 @@ int refine_sweep(Mesh *m, const RefineVecs &v, int nrhs, RefineMode mode) {
     const int64_t n = m->n_dof, nn = n * nrhs;
     k_to_f32<<<g256(nn), 256, 0, s>>>(v.r, v.r32, nn);
     note_launch(m);
-    for (int c0 = 0; c0 < nrhs; c0 += kMaxRhs)
-        FEM3_TRY(trsm_t<float>(m->A32, n, v.r32 + c0 * n, std::min(kMaxRhs, nrhs - c0), s, m));
+    FEM3_TRY(tri_solve<float>(m, m->A32, n, v.r32, nrhs));
     k_axpy_f32<<<g256(nn), 256, 0, s>>>(v.r32, v.u, nn);
     note_launch(m);
     FEM3_CUDA(cudaMemsetAsync(m->norms, 0, sizeof(double) * 2 * nrhs, s));
@@ -1133,7 +710,7 @@ double refine_worst(const Mesh *m, int nrhs, double tol, RefineMode *next) {
 int residual_worst(Mesh *m, const double *b, const double *u, int nrhs, double *worst) {
     cudaStream_t s = m->stream;
     const int64_t n = m->n_dof;
-    const int group = std::min(nrhs, kMaxRhs);
+    const int group = std::min(nrhs, 24);   // norms: 2 values a column
     double *Au = nullptr;   // A u, then the residual
     FEM3_CUDA(cudaMallocAsync((void **)&Au, sizeof(double) * n * group, s));
     int st = FEM3_OK;
