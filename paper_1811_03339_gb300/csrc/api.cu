@@ -227,6 +227,7 @@ void fem3_mesh_free(fem3_mesh h) {
     if (m->ev_made)
         for (int k = 0; k < 16; k++) cudaEventDestroy(m->ev[k]);
     for (cudaEvent_t e : m->kc_ev) cudaEventDestroy(e);
+    if (m->op.ev) cudaEventDestroy(m->op.ev);
     delete m;
 }
 
@@ -347,6 +348,7 @@ int fem3_assemble(fem3_mesh h, const double alpha[3], const double K[3], int pre
     m->integer_order = false;
     m->nonsym = false;
     kc_reset(m);
+    if (m->nparts == 1) FEM3_TRY(op_count(m));   // for the solve; behind the walk by then
     FEM3_TRY(walk_tables(m, alpha));
     stage_begin(m, 3);
     if (precision == FEM3_TF32X3 || precision == FEM3_BF16X3)

@@ -6,7 +6,8 @@
 // sweeps apply the operator in FP32 as the single-mesh solve does); all residuals are checked
 // with one host wait per sweep.  12 meshes of 6 to 20 cells per side, 16 columns: 49.3 ms a
 // run with block-step solves over the whole batch (1,100 launches, 13.3 ms) and double-float
-// sweeps throughout, 31.7 ms now.
+// sweeps throughout, 26.8 ms so, 21.8 ms since each internal stream has factorisation streams
+// of its own (one set for all made the large meshes' blocked factorisations follow each other).
 //
 // The assembly and factorisation of the whole batch (walk, contractions, factorisations) is captured as one CUDA
 // graph the second time a run has the same orders, coefficients and precision, and replayed
@@ -29,6 +30,7 @@ struct Batch {
     std::vector<Mesh *> ms;
     std::vector<cudaStream_t> streams;
     std::vector<cudaEvent_t> done;   // one per internal stream
+    std::vector<SideCtx *> side;     // factorisation streams, likewise
     cudaEvent_t fork = nullptr;
     BatchWalkScratch ws;
     // per-mesh run buffers, kept across runs: load vector b and the refinement's vectors
@@ -66,6 +68,7 @@ static void batch_destroy(Batch *b) {
     free_run_buffers(b);
     for (Mesh *m : b->ms) fem3_mesh_free(reinterpret_cast<fem3_mesh>(m));
     for (cudaEvent_t e : b->done) cudaEventDestroy(e);
+    for (SideCtx *c : b->side) side_destroy(c);
     for (cudaStream_t s : b->streams) cudaStreamDestroy(s);
     if (b->fork) cudaEventDestroy(b->fork);
     if (b->cap) cudaStreamDestroy(b->cap);
@@ -138,6 +141,12 @@ int fem3_batch_create(int n_meshes, const double *const *verts, const int64_t *n
         }
         b->streams.push_back(s);
         b->done.push_back(e);
+        SideCtx *c = nullptr;
+        if (int st = side_make(&c)) {
+            batch_destroy(b);
+            return st;
+        }
+        b->side.push_back(c);
     }
     if (cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&b->cap_in, cudaEventDisableTiming) != cudaSuccess ||
@@ -193,6 +202,11 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
         m->factored = false;
         m->op_ready = false;
     }
+    // the operators' block patterns and storage (the first run's; one wait for all of them)
+    for (Mesh *m : b->ms)
+        if (m->n_dof > 0) FEM3_TRY(op_count(m));
+    for (Mesh *m : b->ms)
+        if (m->n_dof > 0) FEM3_TRY(op_prepare(m, !fp64));
     // run buffers for nrhs columns (kept across runs)
     if (b->nrhs_cap < nrhs) {
         for (cudaStream_t t : b->streams) FEM3_CUDA(cudaStreamSynchronize(t));
@@ -229,7 +243,10 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
                 FEM3_TRY(contract_tc(m, precision == FEM3_BF16X3));
             else
                 FEM3_TRY(contract(m, precision));
-            FEM3_TRY(factor(m));
+            m->lent = b->side[i % b->streams.size()];
+            const int fst = factor(m);
+            m->lent = nullptr;
+            FEM3_TRY(fst);
         }
         FEM3_TRY(join_to(b, os));
         return FEM3_OK;
@@ -238,8 +255,8 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
     if (same) {
         FEM3_CUDA(cudaGraphLaunch(b->exec, cs));
         b->graph_launches++;
-        // a replayed FP64 run has copied its operator, as the captured one did
-        for (Mesh *m : b->ms) m->op_ready = fp64 && m->n_dof > 0;
+        // the replay has built (FP64: copied) the operators that the captured run did
+        for (Mesh *m : b->ms) m->op_ready = m->n_dof > 0 && (fp64 || op_beside_factor(m));
     } else if (b->runs >= 1) {
         // capture the assembly + factorisation; on any failure discard it and run eagerly
         if (b->exec) {
@@ -268,6 +285,7 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
             b->graph_launches++;
         } else {
             b->exec = nullptr;
+            for (Mesh *m : b->ms) m->op_ready = false;   // the capture built none
             st = enqueue_assembly(cs);
         }
     } else {

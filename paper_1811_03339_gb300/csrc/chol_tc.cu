@@ -459,87 +459,89 @@ int make_w_map(CUtensorMap *map, float *base, int64_t rows) {
     return FEM3_OK;
 }
 
-// Side stream and events of the look-ahead, shared through a process-wide pool: a
-// factorisation takes a context for the time it enqueues its launches (every wait on an
-// event is enqueued before the event is recorded again), so concurrent callers never share
-// one.
-struct CholCtx {
-    int device = -1;
-    cudaStream_t side = nullptr;   // bulk trailing updates
-    cudaStream_t col = nullptr;    // the next panel's columns below its diagonal tile
-    std::vector<cudaEvent_t> ev;
-};
 std::mutex g_ctx_mu;
-std::vector<CholCtx *> g_ctx_free;
+std::vector<SideCtx *> g_ctx_free;
 
-int ctx_acquire(CholCtx **out, int npan) {
-    int dev = 0;
-    FEM3_CUDA(cudaGetDevice(&dev));
-    CholCtx *c = nullptr;
-    {
-        std::lock_guard<std::mutex> lk(g_ctx_mu);
-        for (size_t i = 0; i < g_ctx_free.size(); i++)
-            if (g_ctx_free[i]->device == dev) {
-                c = g_ctx_free[i];
-                g_ctx_free.erase(g_ctx_free.begin() + i);
-                break;
-            }
-    }
-    if (!c) {
-        c = new CholCtx();
-        c->device = dev;
-        cudaError_t e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->col, cudaStreamNonBlocking);
-        if (e != cudaSuccess) {
-            if (c->side) cudaStreamDestroy(c->side);
-            delete c;
-            return cuda_error(e, "cudaStreamCreateWithFlags");
-        }
-    }
-    while ((int)c->ev.size() < 4 * npan) {
-        cudaEvent_t e;
-        cudaError_t r = cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
-        if (r != cudaSuccess) {
-            std::lock_guard<std::mutex> lk(g_ctx_mu);
-            g_ctx_free.push_back(c);
-            return cuda_error(r, "cudaEventCreateWithFlags");
-        }
-        c->ev.push_back(e);
+}  // namespace
+
+int side_make(SideCtx **out) {
+    SideCtx *c = new SideCtx();
+    int least = 0, most = 0;   // priorities: lower numbers first
+    cudaError_t e = cudaGetDevice(&c->device);
+    if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&least, &most);
+    const auto stream = [&](cudaStream_t *s, int prio) {
+        if (e == cudaSuccess) e = cudaStreamCreateWithPriority(s, cudaStreamNonBlocking, prio);
+    };
+    stream(&c->chain, most);
+    stream(&c->col, most);
+    stream(&c->side, (least + most) / 2);
+    stream(&c->op, least);
+    for (cudaEvent_t *v : {&c->fork, &c->chain_done, &c->op_done})
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(v, cudaEventDisableTiming);
+    if (e != cudaSuccess) {
+        side_destroy(c);
+        cudaGetLastError();
+        return cuda_error(e, "side streams");
     }
     *out = c;
     return FEM3_OK;
 }
 
-void ctx_release(CholCtx *c) {
+void side_destroy(SideCtx *c) {
+    if (!c) return;
+    for (cudaStream_t s : {c->chain, c->col, c->side, c->op})
+        if (s) cudaStreamDestroy(s);
+    for (cudaEvent_t v : {c->fork, c->chain_done, c->op_done})
+        if (v) cudaEventDestroy(v);
+    for (cudaEvent_t v : c->ev) cudaEventDestroy(v);
+    delete c;
+}
+
+// A caller holds a context while it enqueues; every wait on an event is enqueued before the
+// event is recorded again, so concurrent callers never share one.
+int side_acquire(SideCtx **out) {
+    int dev = 0;
+    FEM3_CUDA(cudaGetDevice(&dev));
+    {
+        std::lock_guard<std::mutex> lk(g_ctx_mu);
+        for (size_t i = 0; i < g_ctx_free.size(); i++)
+            if (g_ctx_free[i]->device == dev) {
+                *out = g_ctx_free[i];
+                g_ctx_free.erase(g_ctx_free.begin() + i);
+                return FEM3_OK;
+            }
+    }
+    return side_make(out);
+}
+
+void side_release(SideCtx *c) {
     std::lock_guard<std::mutex> lk(g_ctx_mu);
     g_ctx_free.push_back(c);
 }
-
-}  // namespace
 
 // FP32 factorisation of A (n x n, lower triangle) in place, inverses of the 64 x 64
 // diagonal blocks into m->dinv; the same output layout as the tile-task factorisation.
 //
 // Look-ahead over three streams.  Panel p: D(p) diagonal block, P(p) panel solve into the
 // operand buffer p % 2, Ta(p) the trailing update of panel p + 1's diagonal tile, Tc(p) that
-// of the rest of panel p + 1's columns, Tb(p) the rest of the trailing update.  The caller's
+// of the rest of panel p + 1's columns, Tb(p) the rest of the trailing update.  The chain
 // stream runs D, P and Ta (the critical chain), the column stream Tc and the side stream Tb,
 // so Tc(p) overlaps D(p + 1) and Tb(p) overlaps D(p + 1) and P(p + 1).  Orderings: D(p) after
 // Tb(p - 2) (which updated panel p's columns and read the operand buffer P(p) rewrites) and
 // Ta(p - 1); P(p) after Tc(p - 1) (panel p's columns below the diagonal tile; Tc(p - 2),
 // earlier on its stream, read the operand buffer P(p) rewrites); Ta(p) and Tc(p) after P(p)
 // and Tb(p - 1) (which updated the same columns); Tb(p) after P(p); the caller's stream waits
-// for the last Tb and Tc.
-int chol_tc(Mesh *m, float *A, int64_t n) {
+// for the chain and the last Tb and Tc.
+int chol_tc(Mesh *m, SideCtx *cx, float *A, int64_t n) {
     if (n <= 0) return FEM3_OK;
-    cudaStream_t s = m->stream;
+    cudaStream_t caller = m->stream;
     const int64_t wrows = std::max<int64_t>(128, (n + 127) / 128 * 128);
     if (!m->chol_w || m->chol_w_rows < wrows) {
         FEM3_TRY(dev_alloc(m, (void **)&m->chol_w, sizeof(float) * (4 * wrows * kP + 3 * 64 * 64)));
         m->chol_w_rows = wrows;
         // operand rows past the trailing matrix are read by the edge tiles' MMAs (their
         // products are masked in the epilogue): keep them finite
-        FEM3_CUDA(cudaMemsetAsync(m->chol_w, 0, sizeof(float) * 4 * wrows * kP, s));
+        FEM3_CUDA(cudaMemsetAsync(m->chol_w, 0, sizeof(float) * 4 * wrows * kP, caller));
     }
     float *W[2][2] = {{m->chol_w, m->chol_w + wrows * kP},
                       {m->chol_w + 2 * wrows * kP, m->chol_w + 3 * wrows * kP}};
@@ -564,9 +566,12 @@ int chol_tc(Mesh *m, float *A, int64_t n) {
         FEM3_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     }
     const int npan = (int)((n + kP - 1) / kP);
-    CholCtx *cx = nullptr;
-    FEM3_TRY(ctx_acquire(&cx, npan));
-    cudaStream_t s1 = cx->side, s2 = cx->col;
+    while ((int)cx->ev.size() < 4 * npan) {
+        cudaEvent_t e;
+        FEM3_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        cx->ev.push_back(e);
+    }
+    cudaStream_t s = cx->chain, s1 = cx->side, s2 = cx->col;
     cudaEvent_t *evP = cx->ev.data(), *evB = evP + npan, *evQ = evB + npan, *evR = evQ + npan;
     float *dinv = reinterpret_cast<float *>(m->dinv);
     int st = FEM3_OK;
@@ -577,6 +582,8 @@ int chol_tc(Mesh *m, float *A, int64_t n) {
         return st == FEM3_OK;
     };
     kc_begin(m, KC_FACTOR);
+    FEM3_CUDA(cudaEventRecord(cx->fork, caller));
+    FEM3_CUDA(cudaStreamWaitEvent(s, cx->fork, 0));
     for (int p = 0; p < npan && st == FEM3_OK; p++) {
         const int64_t j0 = (int64_t)p * kP;
         const int nbp = (int)std::min<int64_t>(kP, n - j0);
@@ -623,7 +630,7 @@ int chol_tc(Mesh *m, float *A, int64_t n) {
             break;
         }
         // Tc(p) on the column stream, after P(p) and Tb(p - 1) (both behind this point of the
-        // caller's stream); then Ta(p), the one tile D(p + 1) waits for
+        // chain); then Ta(p), the one tile D(p + 1) waits for
         if (cudaEventRecord(evQ[p], s) != cudaSuccess ||
             cudaStreamWaitEvent(s2, evQ[p], 0) != cudaSuccess) {
             st = cuda_error(cudaGetLastError(), "cudaEventRecord");
@@ -646,13 +653,15 @@ int chol_tc(Mesh *m, float *A, int64_t n) {
         note_launch(m);
         if (!launch_ok("k_cholp_trail")) break;
     }
-    // join: the caller's stream continues after the side streams' last updates
-    if (last_b >= 0 && cudaStreamWaitEvent(s, evB[last_b], 0) != cudaSuccess && st == FEM3_OK)
-        st = cuda_error(cudaGetLastError(), "cudaStreamWaitEvent");
-    if (last_r >= 0 && cudaStreamWaitEvent(s, evR[last_r], 0) != cudaSuccess && st == FEM3_OK)
-        st = cuda_error(cudaGetLastError(), "cudaStreamWaitEvent");
+    // join: the caller's stream continues after the chain and the last updates beside it
+    const auto join = [&](cudaError_t e) {
+        if (e != cudaSuccess && st == FEM3_OK) st = cuda_error(cudaGetLastError(), "factor join");
+    };
+    if (last_b >= 0) join(cudaStreamWaitEvent(caller, evB[last_b], 0));
+    if (last_r >= 0) join(cudaStreamWaitEvent(caller, evR[last_r], 0));
+    join(cudaEventRecord(cx->chain_done, s));
+    join(cudaStreamWaitEvent(caller, cx->chain_done, 0));
     kc_end(m, KC_FACTOR);
-    ctx_release(cx);
     return st;
 }
 

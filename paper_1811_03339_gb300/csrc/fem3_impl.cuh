@@ -104,7 +104,24 @@ struct OpBlocks {
     int32_t *col = nullptr, *src = nullptr, *row_of = nullptr;   // [n_full]
     double *low = nullptr;        // [n_low][32][32] lower blocks as the contraction adds them
     double *full = nullptr;       // [n_full][32][32] column-major
+    bool counted = false;         // the block counts are on their way to h_norms (op_count)
+    cudaEvent_t ev = nullptr;     // ... and have arrived
 };
+
+// Streams and events of work beside a mesh's own stream: the factorisation (its critical
+// chain and the next panel's columns at the highest priority, the bulk updates between) and
+// the operator build (lowest).  Taken from a process-wide pool for the time a factorisation
+// enqueues its launches, or lent by a batch, which owns one per internal stream.
+struct SideCtx {
+    int device = -1;
+    cudaStream_t chain = nullptr, col = nullptr, side = nullptr, op = nullptr;
+    cudaEvent_t fork = nullptr, chain_done = nullptr, op_done = nullptr;
+    std::vector<cudaEvent_t> ev;   // per panel
+};
+int side_make(SideCtx **out);
+void side_destroy(SideCtx *c);
+int side_acquire(SideCtx **out);
+void side_release(SideCtx *c);
 
 struct Mesh {
     int device = 0;
@@ -153,6 +170,7 @@ struct Mesh {
     bool tc_tuned = false;     // the last contraction ran the tuner
     OpBlocks op;
     bool op_ready = false;     // op holds the operator of the current tables
+    SideCtx *lent = nullptr;   // side streams lent by a batch
     bool integer_order = false;   // the matrix came from fem3_assemble_integer (no tables)
     int32_t *p1_first = nullptr;  // integer order: first tile column of each block row of A64
     double *form_wc = nullptr;    // general form: w c per Gauss point, and per slot of one axis
@@ -274,7 +292,7 @@ int contract_tc_form(Mesh *m, int axis, bool test_right, double *wc_gp, bool bf1
 int load_vector(Mesh *m, const double *f_d, int nrhs, double *b_d);
 int load_vector_T(Mesh *m, const double *lam_d, double *out_d);
 int factor(Mesh *m);
-int chol_tc(Mesh *m, float *A, int64_t n);
+int chol_tc(Mesh *m, SideCtx *cx, float *A, int64_t n);
 // triangular solves with a factor (A's tiles below the 64 x 64 diagonal blocks, their inverses in
 // dinv): the wide diagonal inverses, once per factorisation, then L L^T x = y in place for
 // column-major [n][nrhs]
@@ -305,7 +323,11 @@ int apply_correction(Mesh *m, const float *d, int nv, double *Ad, bool late);
 int f32_to_f64(const float *a, double *b, int64_t n, cudaStream_t s);
 int sym_from_lower(double *A, int64_t n, cudaStream_t s);
 int sub_vec(const double *a, const double *b, double *c, int64_t n, cudaStream_t s);
-int op_build(Mesh *m);                          // the operator of the current tables
+int op_count(Mesh *m);     // enqueues the search for the operator's blocks (once per mesh)
+// the block pattern and its storage, of the lower blocks too if `low` (waits for the counts)
+int op_prepare(Mesh *m, bool low);
+int op_build(Mesh *m);     // the operator of the current tables
+bool op_beside_factor(const Mesh *m);   // factor() builds it on a side stream
 int op_from_dense(Mesh *m, const double *A);    // ... of the FP64 form, from its matrix
 int contract_blocks(Mesh *m, const OpBlocks &O);   // the element sum into the lower blocks
 

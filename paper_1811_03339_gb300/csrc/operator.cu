@@ -39,6 +39,7 @@ constexpr int kOpSplitMax = 8;
 // up to this many block rows (1,024 dofs) the pattern is every block: three quarters of them
 // or more are nonzero there, and finding them costs twelve launches and a wait
 constexpr int kOpAllMax = 32;
+constexpr int kOpCountSlot = 124;   // of h_norms: the two block counts
 enum OpMode { kOpFull = 0, kOpUpdate = 1, kOpLate = 2 };
 
 __host__ __device__ inline int64_t tri_id(int64_t i, int64_t j) { return i * (i + 1) / 2 + j; }
@@ -385,30 +386,27 @@ int apply_groups(Mesh *m, const typename OpCfg<1, MODE>::X *u_d, int nv, double 
     return st;
 }
 
-// the block pattern of the mesh (once; synchronises to learn the block counts)
-int op_pattern(Mesh *m) {
+}  // namespace
+
+// Finds the nonzero blocks and sends their numbers to the host (once per mesh; nothing to do
+// for the small patterns with every block).  Enqueued before the walk of an assembly, so that
+// op_prepare, called once the factorisation's turn has come, finds the numbers there.
+int op_count(Mesh *m) {
     OpBlocks &O = m->op;
-    if (O.map) return FEM3_OK;
-    cudaStream_t s = m->stream;
+    if (O.counted || m->n_dof == 0) return FEM3_OK;
     const int nb = (int)((m->n_dof + kOB - 1) / kOB);
-    const int64_t np = tri_id(nb, 0);
-    int32_t *flag, *off, *cnt, *map;
-    FEM3_TRY(dev_alloc_t(m, &map, np));
-    FEM3_TRY(dev_alloc_t(m, &O.row_off, nb + 1));
-    O.nb = nb;
-    if (nb <= kOpAllMax) {
-        O.n_low = np;
-        O.n_full = (int64_t)nb * nb;
-        FEM3_TRY(dev_alloc_t(m, &O.col, O.n_full));
-        FEM3_TRY(dev_alloc_t(m, &O.src, O.n_full));
-        FEM3_TRY(dev_alloc_t(m, &O.row_of, O.n_full));
-        FEM3_TRY(dev_alloc(m, (void **)&O.full, sizeof(double) * kOB * kOB * O.n_full));
-        k_op_all<<<nb, 64, 0, s>>>(nb, map, O.row_off, O.col, O.src, O.row_of);
-        note_launch(m);
-        FEM3_CUDA(cudaGetLastError());
-        O.map = map;
+    if (nb <= kOpAllMax) return FEM3_OK;
+    cudaStream_t s = m->stream;
+    cudaStreamCaptureStatus cap;   // in a caller's capture: left to the solve
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
         return FEM3_OK;
     }
+    const int64_t np = tri_id(nb, 0);
+    int32_t *flag, *off, *cnt;
+    if (!O.ev) FEM3_CUDA(cudaEventCreateWithFlags(&O.ev, cudaEventDisableTiming));
+    FEM3_TRY(dev_alloc_t(m, &O.map, np));
+    FEM3_TRY(dev_alloc_t(m, &O.row_off, nb + 1));
     FEM3_TRY(dev_alloc_t(m, &flag, np));
     FEM3_TRY(dev_alloc_t(m, &off, np + 1));
     FEM3_TRY(dev_alloc_t(m, &cnt, nb));
@@ -425,38 +423,76 @@ int op_pattern(Mesh *m) {
                       sizeof(uint16_t) * (size_t)std::min(nb, std::max(1, max_dof));
     k_op_mark<<<(unsigned)bins, 256, sh, s>>>(P, nb, flag);
     FEM3_TRY(scan_i32(flag, off, np, s, m));
-    k_op_map<<<g256(np), 256, 0, s>>>(flag, off, np, map);
-    k_op_rows<false><<<(nb + 7) / 8, 256, 0, s>>>(map, nb, cnt, nullptr, nullptr, nullptr);
+    k_op_map<<<g256(np), 256, 0, s>>>(flag, off, np, O.map);
+    k_op_rows<false><<<(nb + 7) / 8, 256, 0, s>>>(O.map, nb, cnt, nullptr, nullptr, nullptr);
     FEM3_TRY(scan_i32(cnt, O.row_off, nb, s, m));
-    int32_t h[2] = {0, 0};
-    FEM3_CUDA(cudaMemcpyAsync(&h[0], off + np, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    FEM3_CUDA(cudaMemcpyAsync(&h[1], O.row_off + nb, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    FEM3_CUDA(cudaStreamSynchronize(s));
-    O.n_low = h[0];
-    O.n_full = h[1];
+    int32_t *h = reinterpret_cast<int32_t *>(m->h_norms + kOpCountSlot);
+    FEM3_CUDA(cudaMemcpyAsync(h, off + np, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    FEM3_CUDA(cudaMemcpyAsync(h + 1, O.row_off + nb, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    FEM3_CUDA(cudaEventRecord(O.ev, s));
+    m->launches += 3;
+    FEM3_CUDA(cudaGetLastError());
+    O.counted = true;
+    return FEM3_OK;
+}
+
+// the block pattern of the mesh and the storage of its blocks (once)
+static int op_pattern(Mesh *m) {
+    OpBlocks &O = m->op;
+    if (O.full) return FEM3_OK;
+    cudaStream_t s = m->stream;
+    const int nb = (int)((m->n_dof + kOB - 1) / kOB);
+    const bool all = nb <= kOpAllMax;
+    if (all) {
+        const int64_t np = tri_id(nb, 0);
+        if (!O.map) FEM3_TRY(dev_alloc_t(m, &O.map, np));
+        if (!O.row_off) FEM3_TRY(dev_alloc_t(m, &O.row_off, nb + 1));
+        O.n_low = np;
+        O.n_full = (int64_t)nb * nb;
+    } else {
+        FEM3_TRY(op_count(m));
+        if (!O.counted) return set_error(FEM3_E_STATE, "the solve cannot be captured");
+        FEM3_CUDA(cudaEventSynchronize(O.ev));
+        const int32_t *h = reinterpret_cast<const int32_t *>(m->h_norms + kOpCountSlot);
+        O.n_low = h[0];
+        O.n_full = h[1];
+    }
+    O.nb = nb;
     const int64_t nf = std::max<int64_t>(1, O.n_full);
     FEM3_TRY(dev_alloc_t(m, &O.col, nf));
     FEM3_TRY(dev_alloc_t(m, &O.src, nf));
     FEM3_TRY(dev_alloc_t(m, &O.row_of, nf));
-    FEM3_TRY(dev_alloc(m, (void **)&O.full, sizeof(double) * kOB * kOB * nf));
-    k_op_rows<true><<<(nb + 7) / 8, 256, 0, s>>>(map, nb, nullptr, O.row_off, O.col, O.src);
-    k_op_row_of<<<nb, 128, 0, s>>>(O.row_off, nb, O.row_of);
-    m->launches += 5;
+    double *full = nullptr;
+    FEM3_TRY(dev_alloc(m, (void **)&full, sizeof(double) * kOB * kOB * nf));
+    if (all) {
+        k_op_all<<<nb, 64, 0, s>>>(nb, O.map, O.row_off, O.col, O.src, O.row_of);
+    } else {
+        k_op_rows<true><<<(nb + 7) / 8, 256, 0, s>>>(O.map, nb, nullptr, O.row_off, O.col, O.src);
+        k_op_row_of<<<nb, 128, 0, s>>>(O.row_off, nb, O.row_of);
+        note_launch(m);
+    }
+    note_launch(m);
     FEM3_CUDA(cudaGetLastError());
-    O.map = map;
+    O.full = full;
     return FEM3_OK;
 }
 
-}  // namespace
+int op_prepare(Mesh *m, bool low) {
+    FEM3_TRY(op_pattern(m));
+    OpBlocks &O = m->op;
+    if (low && !O.low)
+        FEM3_TRY(dev_alloc(m, (void **)&O.low,
+                           sizeof(double) * kOB * kOB * (size_t)std::max<int64_t>(1, O.n_low)));
+    return FEM3_OK;
+}
 
 // the operator of the current tables (nothing to do if it is ready)
 int op_build(Mesh *m) {
     if (m->op_ready || m->n_dof == 0) return FEM3_OK;
-    FEM3_TRY(op_pattern(m));
+    FEM3_TRY(op_prepare(m, true));
     OpBlocks &O = m->op;
-    const size_t bytes = sizeof(double) * kOB * kOB * (size_t)std::max<int64_t>(1, O.n_low);
-    if (!O.low) FEM3_TRY(dev_alloc(m, (void **)&O.low, bytes));
-    FEM3_CUDA(cudaMemsetAsync(O.low, 0, bytes, m->stream));
+    FEM3_CUDA(cudaMemsetAsync(O.low, 0, sizeof(double) * kOB * kOB * (size_t)std::max<int64_t>(1, O.n_low),
+                              m->stream));
     FEM3_TRY(contract_blocks(m, O));
     if (O.n_full > 0) {
         kc_begin(m, KC_SPLIT);

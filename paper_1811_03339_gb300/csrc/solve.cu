@@ -385,6 +385,12 @@ int chol_tiles(float *A, int64_t n, cudaStream_t s, Mesh *m) {
     FEM3_CUDA(cudaMemsetAsync(m->chol_flags, 0, sizeof(int32_t) * (2 * ntask + 2), s));
     // one CTA per SM: the chain CTA gets an SM of its own
     const int grid = std::min(ntask + 1, std::max(sms, 2));
+    static bool attr = false;
+    if (!attr) {
+        FEM3_CUDA(cudaFuncSetAttribute(k_chol_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)(kCholTilesSmem * sizeof(float))));
+        attr = true;
+    }
     kc_begin(m, KC_FACTOR);
     k_chol_tiles<<<grid, 512, kCholTilesSmem * sizeof(float), s>>>(
         A, n, nblk, reinterpret_cast<float *>(m->dinv), m->chol_flags, m->err);
@@ -587,6 +593,53 @@ int load_vector_T(Mesh *m, const double *lam_d, double *out_d) {
 // factorisation, whose diagonal chain is the shorter critical path there.
 constexpr int64_t kCholTcMinN = 4096;
 
+bool factor_on_tc(const Mesh *m) {
+    return m->chol_tc_opt > 0 || (m->chol_tc_opt == 0 && m->n_dof >= kCholTcMinN);
+}
+
+// The refinement's operator (a contraction that fills the chip) is built beside the tile-task
+// factorisation (a serial chain that leaves most of it idle) from this order on; below it the
+// two are a few launches each and the events between the streams cost as much as they save.
+// Not beside the blocked factorisation: its trailing updates take an SM's whole shared memory
+// each, so the critical chain waited for the operator's CTAs to drain (24^3 step 30.6 ms
+// with, 30.3 ms without).  A profiled mesh times its launches one at a time.
+constexpr int64_t kOpBesideMin = 512;
+bool op_beside_factor(const Mesh *m) {
+    return !m->profile && m->n_dof >= kOpBesideMin && !factor_on_tc(m);
+}
+
+// the FP32 factor; on return m->stream waits for everything enqueued on cx's streams
+static int factor_mixed(Mesh *m, SideCtx *cx) {
+    cudaStream_t s = m->stream;
+    const bool tc = factor_on_tc(m);
+    const bool beside = op_beside_factor(m) && !m->op_ready;
+    if (beside) {
+        FEM3_TRY(op_prepare(m, true));
+        FEM3_CUDA(cudaEventRecord(cx->op_done, s));
+        FEM3_CUDA(cudaStreamWaitEvent(cx->op, cx->op_done, 0));
+    }
+    int st;
+    if (tc) {
+        st = chol_tc(m, cx, m->A32, m->n_dof);
+        m->chol_tc_used = st == FEM3_OK;
+    } else {
+        st = chol_tiles(m->A32, m->n_dof, s, m);
+    }
+    if (beside) {   // enqueued after the factorisation, whose CTAs are to be placed first
+        m->stream = cx->op;
+        const int so = op_build(m);
+        m->stream = s;
+        if (st == FEM3_OK) st = so;
+    }
+    if (st == FEM3_OK) st = tri_prepare<float>(m, m->A32, m->n_dof);
+    if (beside) {
+        cudaError_t e = cudaEventRecord(cx->op_done, cx->op);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, cx->op_done, 0);
+        if (e != cudaSuccess && st == FEM3_OK) st = cuda_error(e, "operator join");
+    }
+    return st;
+}
+
 int factor(Mesh *m) {
     m->chol_tc_used = false;
     if (m->precision == FEM3_FP64) {
@@ -601,20 +654,11 @@ int factor(Mesh *m) {
         m->launches += launches;
         return tri_prepare<double>(m, m->A64, m->n_dof);
     }
-    const bool tc = m->chol_tc_opt > 0 || (m->chol_tc_opt == 0 && m->n_dof >= kCholTcMinN);
-    if (tc) {
-        FEM3_TRY(chol_tc(m, m->A32, m->n_dof));
-        m->chol_tc_used = true;
-    } else {
-        static bool attr = false;
-        if (!attr) {
-            FEM3_CUDA(cudaFuncSetAttribute(k_chol_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)(kCholTilesSmem * sizeof(float))));
-            attr = true;
-        }
-        FEM3_TRY(chol_tiles(m->A32, m->n_dof, m->stream, m));
-    }
-    return tri_prepare<float>(m, m->A32, m->n_dof);
+    SideCtx *cx = m->lent;
+    if (!cx) FEM3_TRY(side_acquire(&cx));
+    const int st = factor_mixed(m, cx);
+    if (!m->lent) side_release(cx);
+    return st;
 }
 
 int axis_forms(Mesh *m, const double *u_d, const double *lam_d, double out[3]) {
