@@ -10,7 +10,7 @@
 //      and invert D11 (X11 = L11^{-1}), L21 = A21 X11^T, factor and invert D22 - L21 L21^T;
 //      X11 and X22 go to dinv and L21 to A, the layout the triangular-solve chains read (the
 //      strictly lower 64 x 64 tiles of A hold L; a diagonal tile is only used through its
-//      inverse), and [X11 | X22 | L21] to the panel solve;
+//      inverse), and their transposes to the panel solve;
 //   2. k_cholp_panel: for every row below the panel, L[:, 0:64] = A[:, 0:64] X11^T and
 //      L[:, 64:128] = (A[:, 64:128] - L[:, 0:64] L21^T) X22^T, into A and, split into TF32
 //      hi + lo pairs, into the K-major operand rows W_hi, W_lo;
@@ -40,8 +40,6 @@ constexpr int kWaitLimit = 1 << 22;
 
 constexpr int kP = 128;                        // panel width
 constexpr int kLd = NB + 1;                    // shared 64 x 64 block row stride
-constexpr int kDiagSmemFloats = 6 * NB * kLd;  // a_s, x_s, b_s (A21 -> L21), x11, t, A22
-constexpr int kPanelRows = 64;                 // rows of a panel-solve CTA
 constexpr uint32_t kTile = 128 * 128;          // bytes of one 128-row x 128-byte TMA box
 constexpr uint32_t kStage = 4 * kTile;         // A hi, A lo, B hi, B lo: 64 KB
 constexpr int kStages = 2;
@@ -53,47 +51,49 @@ constexpr int kEpiThreads = 512;
 constexpr int kReservedSms = 20;                // left to the critical chain by the bulk update
 
 // ------------------------------- diagonal block ----------------------------------
-// c[i][j] (+)= sgn * sum_k a[i][k] b(k, j) over a 64 x 64 x 64 product in shared memory,
-// 512 threads, 8 outputs each; BT selects b(k, j) = b[j][k] (transposed) or b[k][j].
-template <bool BT>
-__device__ __forceinline__ void smem_gemm64(float (*c)[kLd], const float (*a)[kLd],
-                                            const float (*b)[kLd], float sgn, bool accumulate) {
-    const int tid = threadIdx.x, r = tid >> 3, c0 = (tid & 7) * 8;
-    float acc[8];
-#pragma unroll
-    for (int q = 0; q < 8; q++) acc[q] = 0.f;
-    for (int k = 0; k < NB; k++) {
-        const float av = a[r][k];
-#pragma unroll
-        for (int q = 0; q < 8; q++) acc[q] = fmaf(av, BT ? b[c0 + q][k] : b[k][c0 + q], acc[q]);
-    }
-    __syncthreads();   // c may alias an operand's storage in the caller's sequence
-#pragma unroll
-    for (int q = 0; q < 8; q++) c[r][c0 + q] = (accumulate ? c[r][c0 + q] : 0.f) + sgn * acc[q];
-    __syncthreads();
-}
-
 // one CTA of 512 threads: the diagonal block [j0, j0 + nbp) of A (nbp <= 128).  Every global
 // load of the block is issued first; then D11 = L11 L11^T with X11 = L11^{-1}, L21 = A21 X11^T,
 // D22 - L21 L21^T = L22 L22^T with X22 = L22^{-1}.  Out: X11, X22 into dinv (the
-// triangular-solve chains' diagonal inverses), L21 into A, and [X11 | X22 | L21] (three
-// 64 x 64 blocks, row-major) into Pinv for the panel solve.
+// triangular solves' diagonal inverses), L21 into A, and [X11^T | X22^T | L21^T] (three
+// 64 x 64 blocks, row-major) into Pinv, as the panel solve reads them.
+//
+// On the critical chain of the factorisation, one SM.  Bound: the two serial 64 x 64 factors
+// (about 10 us each); the products take 2 x 4 outputs per thread from operands laid out so that
+// an output's row and columns come in one 16-byte and two broadcast reads a step.  One output
+// row of eight per thread, nine scalar reads a step, took 11 us a product: 46.7 -> 31.6 us a
+// launch.
+constexpr int kQ = 68;   // shared row stride (floats) of the 64-wide operand blocks: 16-byte rows
+constexpr int kDiagSmemFloats = NB * (2 * kLd + 2 * kQ);   // a_s, x_s; A21^T, L21^T
 __global__ void __launch_bounds__(512, 1) k_cholp_diag(float *A, int64_t n, int64_t j0, int nbp,
                                                        float *dinv, float *Pinv, int32_t *err) {
     extern __shared__ __align__(16) float sm_diag[];
     float(*a_s)[kLd] = reinterpret_cast<float(*)[kLd]>(sm_diag);
     float(*x_s)[kLd] = a_s + NB;
-    float(*b_s)[kLd] = x_s + NB;   // A21, then L21
-    float(*x11)[kLd] = b_s + NB;
-    float(*t_s)[kLd] = x11 + NB;   // L21 L21^T
-    float(*d22)[kLd] = t_s + NB;   // A22 as loaded
-    const int tid = threadIdx.x;
+    float(*at)[kQ] = reinterpret_cast<float(*)[kQ]>(sm_diag + 2 * NB * kLd);   // A21^T
+    float(*lt)[kQ] = at + NB;                                                  // L21^T
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int nb1 = min(NB, nbp), nb2 = nbp - nb1;
-    for (int e = tid; e < NB * NB; e += 512) {
-        const int i = e >> 6, c = e & 63;
-        a_s[i][c] = (i < nb1 && c < nb1) ? A[(j0 + i) * n + j0 + c] : (i == c ? 1.f : 0.f);
-        b_s[i][c] = (i < nb2) ? A[(j0 + NB + i) * n + j0 + c] : 0.f;
-        d22[i][c] = (i < nb2 && c < nb2) ? A[(j0 + NB + i) * n + j0 + NB + c] : (i == c ? 1.f : 0.f);
+    constexpr int E = NB * NB / 512;
+    float v11[E], v21[E], d22[2][4];   // d22: rows 2 ty + p, columns 4 tx + q
+#pragma unroll
+    for (int q = 0; q < E; q++) {
+        const int i = (tid >> 6) + 8 * q, c = tid & 63;
+        v11[q] = (i < nb1 && c < nb1) ? A[(j0 + i) * n + j0 + c] : (i == c ? 1.f : 0.f);
+        v21[q] = (i < nb2) ? A[(j0 + NB + i) * n + j0 + c] : 0.f;
+    }
+#pragma unroll
+    for (int p = 0; p < 2; p++)
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const int i = 2 * ty + p, c = 4 * tx + q;
+            d22[p][q] = (i < nb2 && c < nb2) ? A[(j0 + NB + i) * n + j0 + NB + c]
+                                             : (i == c ? 1.f : 0.f);
+        }
+#pragma unroll
+    for (int q = 0; q < E; q++) {
+        const int i = (tid >> 6) + 8 * q, c = tid & 63;
+        a_s[i][c] = v11[q];
+        at[c][i] = v21[q];
     }
     __syncthreads();
     potrf_inv_smem<float, NB>(a_s, x_s, nb1, j0, err);
@@ -101,118 +101,166 @@ __global__ void __launch_bounds__(512, 1) k_cholp_diag(float *A, int64_t n, int6
     for (int e = tid; e < NB * NB; e += 512) {
         const int i = e >> 6, c = e & 63;
         d1[e] = x_s[i][c];
-        x11[i][c] = x_s[i][c];
-        Pinv[e] = x_s[i][c];
+        Pinv[e] = x_s[c][i];
     }
-    if (nb2 > 0) {
-        __syncthreads();
-        smem_gemm64<true>(b_s, b_s, x11, 1.f, false);          // b_s = L21 = A21 X11^T
-        smem_gemm64<true>(t_s, b_s, b_s, 1.f, false);          // t = L21 L21^T
-        for (int e = tid; e < NB * NB; e += 512) {
-            const int i = e >> 6, c = e & 63;
-            if (i < nb2) A[(j0 + NB + i) * n + j0 + c] = b_s[i][c];
-            Pinv[2 * NB * NB + e] = b_s[i][c];
-            // the identity padding stays: L21's padded rows are zero
-            a_s[i][c] = d22[i][c] - t_s[i][c];
+    if (nb2 <= 0) return;
+    // L21^T = X11 A21^T: o[p][q] = L21[4 tx + q][2 ty + p]
+    float o[2][4], t[2][4];
+#pragma unroll
+    for (int p = 0; p < 2; p++)
+#pragma unroll
+        for (int q = 0; q < 4; q++) o[p][q] = t[p][q] = 0.f;
+#pragma unroll 8
+    for (int k = 0; k < NB; k++) {
+        float v[4];
+        lds4<float>(&at[k][4 * tx], v);
+        const float u0 = x_s[2 * ty][k], u1 = x_s[2 * ty + 1][k];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            o[0][q] = fmaf(u0, v[q], o[0][q]);
+            o[1][q] = fmaf(u1, v[q], o[1][q]);
         }
-        __syncthreads();
-        potrf_inv_smem<float, NB>(a_s, x_s, nb2, j0 + NB, err);    // x_s = X22
-        float *d2 = d1 + (int64_t)NB * NB;
-        for (int e = tid; e < NB * NB; e += 512) {
-            d2[e] = x_s[e >> 6][e & 63];
-            Pinv[NB * NB + e] = x_s[e >> 6][e & 63];
-        }
+    }
+#pragma unroll
+    for (int p = 0; p < 2; p++)
+        *reinterpret_cast<float4 *>(&lt[2 * ty + p][4 * tx]) =
+            make_float4(o[p][0], o[p][1], o[p][2], o[p][3]);
+    __syncthreads();
+    // t = L21 L21^T
+#pragma unroll 8
+    for (int k = 0; k < NB; k++) {
+        float u[2], v[4];
+        lds2<float>(&lt[k][2 * ty], u);
+        lds4<float>(&lt[k][4 * tx], v);
+#pragma unroll
+        for (int p = 0; p < 2; p++)
+#pragma unroll
+            for (int q = 0; q < 4; q++) t[p][q] = fmaf(u[p], v[q], t[p][q]);
+    }
+    // (the identity padding stays: L21's padded rows are zero)
+#pragma unroll
+    for (int p = 0; p < 2; p++)
+#pragma unroll
+        for (int q = 0; q < 4; q++) a_s[2 * ty + p][4 * tx + q] = d22[p][q] - t[p][q];
+    for (int e = tid; e < NB * NB; e += 512) {
+        const int i = e >> 6, c = e & 63;
+        if (i < nb2) A[(j0 + NB + i) * n + j0 + c] = lt[c][i];
+        Pinv[2 * NB * NB + e] = lt[i][c];
+    }
+    __syncthreads();
+    potrf_inv_smem<float, NB>(a_s, x_s, nb2, j0 + NB, err);    // x_s = X22
+    float *d2 = d1 + (int64_t)NB * NB;
+    for (int e = tid; e < NB * NB; e += 512) {
+        const int i = e >> 6, c = e & 63;
+        d2[e] = x_s[i][c];
+        Pinv[NB * NB + e] = x_s[c][i];
     }
 }
 
-// ------------------------------- panel solve --------------------------------------
-// rows [r0, r0 + 64) below the panel (r0 >= t0 = j0 + P), in two 64-column steps:
+// ------------------------------- panel solve ----------------------------------
+// ROWS rows of the panel per CTA, with [X11^T | X22^T | L21^T] in shared memory:
 //   L[:, 0:64]   = A[:, 0:64] X11^T
 //   L[:, 64:128] = (A[:, 64:128] - L[:, 0:64] L21^T) X22^T
 // written to A and, as TF32 hi + lo, to the operand rows W[i - t0] of the trailing update.
-// 256 threads, each 4 rows x 4 columns of every 64 x 64 product.
-constexpr int kQ = 68;   // shared row stride (floats) of the 64-wide blocks: 16-byte rows
-__device__ __forceinline__ void panel_gemm64(const float (*a)[kQ], const float (*bt)[kQ],
-                                             float acc[4][4], int ty, int tx) {
-    // acc[p][q] += sum_k a[4 ty + p][k] bt[k][4 tx + q]
+// 256 threads, each ROWS / 16 rows x 4 columns of every product; every global load is issued
+// before the first store to shared memory (one latency instead of sixteen).
+// On the critical chain, so latency counts: 64 rows when 32 would need more CTAs than SMs.
+// Measured at n = 12,167: 14.7 us a launch above 4,864 rows and 9.6 us below (24.4 us with the
+// loads and stores of each sixteenth in turn and scalar reads of the rows).
+template <int ROWS>
+__device__ __forceinline__ void panel_gemm(const float (*a)[kQ], const float (*bt)[kQ],
+                                           float acc[ROWS / 16][4], int ty, int tx) {
+    // acc[p][q] = sum_k a[ROWS / 16 * ty + p][k] bt[k][4 tx + q]
+    constexpr int R = ROWS / 16;
+#pragma unroll
+    for (int p = 0; p < R; p++)
+#pragma unroll
+        for (int q = 0; q < 4; q++) acc[p][q] = 0.f;
 #pragma unroll 4
-    for (int k = 0; k < 64; k++) {
-        const float4 b4 = *reinterpret_cast<const float4 *>(&bt[k][4 * tx]);
-        const float bv[4] = {b4.x, b4.y, b4.z, b4.w};
+    for (int k = 0; k < 64; k += 4) {
+        float av[R][4];
 #pragma unroll
-        for (int p = 0; p < 4; p++) {
-            const float av = a[4 * ty + p][k];
+        for (int p = 0; p < R; p++) lds4<float>(&a[R * ty + p][k], av[p]);
 #pragma unroll
-            for (int q = 0; q < 4; q++) acc[p][q] = fmaf(av, bv[q], acc[p][q]);
+        for (int kk = 0; kk < 4; kk++) {
+            float bv[4];
+            lds4<float>(&bt[k + kk][4 * tx], bv);
+#pragma unroll
+            for (int p = 0; p < R; p++)
+#pragma unroll
+                for (int q = 0; q < 4; q++) acc[p][q] = fmaf(av[p][kk], bv[q], acc[p][q]);
         }
     }
 }
 
+template <int ROWS> constexpr size_t panel_smem() { return sizeof(float) * (3 * 64 + 2 * ROWS) * kQ; }
+
+template <int ROWS>
 __global__ void __launch_bounds__(256) k_cholp_panel(float *A, int64_t n, int64_t j0,
                                                      const float *__restrict__ Pinv, float *Whi,
                                                      float *Wlo) {
+    constexpr int R = ROWS / 16, EA = ROWS * kP / 256;
     extern __shared__ __align__(16) float sm_panel[];
     float(*x11t)[kQ] = reinterpret_cast<float(*)[kQ]>(sm_panel);   // x11t[k][c] = X11[c][k]
     float(*x22t)[kQ] = x11t + 64;                                    // x22t[k][c] = X22[c][k]
     float(*l21t)[kQ] = x22t + 64;                                    // l21t[k][c] = L21[c][k]
-    float(*a1)[kQ] = l21t + 64;   // A[:, 0:64], then L[:, 0:64]
-    float(*a2)[kQ] = a1 + 64;     // A[:, 64:128], then T, then L[:, 64:128]
+    float(*a1)[kQ] = l21t + 64;     // A[:, 0:64], then L[:, 0:64]
+    float(*a2)[kQ] = a1 + ROWS;     // A[:, 64:128], then T, then L[:, 64:128]
     const int tid = threadIdx.x;
     const int64_t t0 = j0 + kP;
-    const int64_t r0 = t0 + (int64_t)blockIdx.x * kPanelRows;
-    for (int e = tid; e < 64 * 64; e += 256) {
-        const int c = e >> 6, k = e & 63;
-        x11t[k][c] = Pinv[e];
-        x22t[k][c] = Pinv[64 * 64 + e];
-        l21t[k][c] = Pinv[2 * 64 * 64 + e];
-    }
-    for (int e = tid; e < kPanelRows * kP; e += 256) {
-        const int r = e >> 7, k = e & 127;
-        const float v = r0 + r < n ? A[(r0 + r) * n + j0 + k] : 0.f;
-        if (k < 64) a1[r][k] = v; else a2[r][k - 64] = v;
+    const int64_t r0 = t0 + (int64_t)blockIdx.x * ROWS;
+    {
+        float va[EA];
+        float4 vp[12];
+#pragma unroll
+        for (int q = 0; q < EA; q++) {
+            const int r = (tid >> 7) + 2 * q, k = tid & 127;
+            va[q] = r0 + r < n ? A[(r0 + r) * n + j0 + k] : 0.f;
+        }
+#pragma unroll
+        for (int q = 0; q < 12; q++) vp[q] = reinterpret_cast<const float4 *>(Pinv)[tid + 256 * q];
+#pragma unroll
+        for (int q = 0; q < EA; q++) {
+            const int r = (tid >> 7) + 2 * q, k = tid & 127;
+            if (k < 64) a1[r][k] = va[q]; else a2[r][k - 64] = va[q];
+        }
+#pragma unroll
+        for (int q = 0; q < 12; q++) {
+            const int e = tid + 256 * q;   // sixteen float4 per row, 64 rows per block
+            *reinterpret_cast<float4 *>(&x11t[e >> 4][4 * (e & 15)]) = vp[q];
+        }
     }
     __syncthreads();
     const int ty = tid >> 4, tx = tid & 15;
-    float acc[4][4];
-    // L1 = A1 X11^T
+    float acc[R][4];
+    const auto put = [&](float(*d)[kQ]) {
 #pragma unroll
-    for (int p = 0; p < 4; p++)
-#pragma unroll
-        for (int q = 0; q < 4; q++) acc[p][q] = 0.f;
-    panel_gemm64(a1, x11t, acc, ty, tx);
+        for (int p = 0; p < R; p++)
+            *reinterpret_cast<float4 *>(&d[R * ty + p][4 * tx]) =
+                make_float4(acc[p][0], acc[p][1], acc[p][2], acc[p][3]);
+    };
+    panel_gemm<ROWS>(a1, x11t, acc, ty, tx);   // L1 = A1 X11^T
     __syncthreads();
-#pragma unroll
-    for (int p = 0; p < 4; p++)
-#pragma unroll
-        for (int q = 0; q < 4; q++) a1[4 * ty + p][4 * tx + q] = acc[p][q];
+    put(a1);
     __syncthreads();
-    // T = A2 - L1 L21^T
+    panel_gemm<ROWS>(a1, l21t, acc, ty, tx);   // T = A2 - L1 L21^T
 #pragma unroll
-    for (int p = 0; p < 4; p++)
+    for (int p = 0; p < R; p++) {
+        float v[4];
+        lds4<float>(&a2[R * ty + p][4 * tx], v);
 #pragma unroll
-        for (int q = 0; q < 4; q++) acc[p][q] = 0.f;
-    panel_gemm64(a1, l21t, acc, ty, tx);
+        for (int q = 0; q < 4; q++) acc[p][q] = v[q] - acc[p][q];
+    }
+    put(a2);   // (each thread its own entries)
     __syncthreads();
-#pragma unroll
-    for (int p = 0; p < 4; p++)
-#pragma unroll
-        for (int q = 0; q < 4; q++) a2[4 * ty + p][4 * tx + q] -= acc[p][q];
+    panel_gemm<ROWS>(a2, x22t, acc, ty, tx);   // L2 = T X22^T
     __syncthreads();
-    // L2 = T X22^T
-#pragma unroll
-    for (int p = 0; p < 4; p++)
-#pragma unroll
-        for (int q = 0; q < 4; q++) acc[p][q] = 0.f;
-    panel_gemm64(a2, x22t, acc, ty, tx);
-    __syncthreads();
-#pragma unroll
-    for (int p = 0; p < 4; p++)
-#pragma unroll
-        for (int q = 0; q < 4; q++) a2[4 * ty + p][4 * tx + q] = acc[p][q];
+    put(a2);
     __syncthreads();
     // stores: A rows (lanes along the row) and the TF32 hi / lo operand rows
-    for (int e = tid; e < kPanelRows * kP; e += 256) {
-        const int r = e >> 7, k = e & 127;
+#pragma unroll 8
+    for (int q = 0; q < EA; q++) {
+        const int r = (tid >> 7) + 2 * q, k = tid & 127;
         const int64_t i = r0 + r;
         if (i >= n) continue;
         const float v = k < 64 ? a1[r][k] : a2[r][k - 64];
@@ -545,7 +593,7 @@ int chol_tc(Mesh *m, SideCtx *cx, float *A, int64_t n) {
     }
     float *W[2][2] = {{m->chol_w, m->chol_w + wrows * kP},
                       {m->chol_w + 2 * wrows * kP, m->chol_w + 3 * wrows * kP}};
-    float *Linv = m->chol_w + 4 * wrows * kP;   // [X11 | X22 | L21] of the current panel
+    float *Linv = m->chol_w + 4 * wrows * kP;   // [X11^T | X22^T | L21^T] of the current panel
     CUtensorMap maps[2][2];
     for (int b = 0; b < 2; b++)
         for (int h = 0; h < 2; h++) FEM3_TRY(make_w_map(&maps[b][h], W[b][h], wrows));
@@ -553,8 +601,10 @@ int chol_tc(Mesh *m, SideCtx *cx, float *A, int64_t n) {
     if (!attr) {
         FEM3_CUDA(cudaFuncSetAttribute(k_cholp_diag, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)(sizeof(float) * kDiagSmemFloats)));
-        FEM3_CUDA(cudaFuncSetAttribute(k_cholp_panel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(sizeof(float) * 5 * 64 * kQ)));
+        FEM3_CUDA(cudaFuncSetAttribute(k_cholp_panel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)panel_smem<32>()));
+        FEM3_CUDA(cudaFuncSetAttribute(k_cholp_panel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)panel_smem<64>()));
         FEM3_CUDA(cudaFuncSetAttribute(k_cholp_trail, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kTrailSmem));
         attr = true;
@@ -602,8 +652,12 @@ int chol_tc(Mesh *m, SideCtx *cx, float *A, int64_t n) {
             st = cuda_error(cudaGetLastError(), "cudaStreamWaitEvent");
             break;
         }
-        k_cholp_panel<<<(unsigned)((mt + kPanelRows - 1) / kPanelRows), 256,
-                        sizeof(float) * 5 * 64 * kQ, s>>>(A, n, j0, Linv, W[b][0], W[b][1]);
+        if (mt <= 32 * (int64_t)sms)
+            k_cholp_panel<32><<<(unsigned)((mt + 31) / 32), 256, panel_smem<32>(), s>>>(
+                A, n, j0, Linv, W[b][0], W[b][1]);
+        else
+            k_cholp_panel<64><<<(unsigned)((mt + 63) / 64), 256, panel_smem<64>(), s>>>(
+                A, n, j0, Linv, W[b][0], W[b][1]);
         note_launch(m);
         if (!launch_ok("k_cholp_panel")) break;
         const int64_t T = (mt + 127) / 128;
