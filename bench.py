@@ -72,11 +72,6 @@ TRAFFIC = {
     "k_walk_tables": {"source": "walk.cu",
                       "sha256": "f5c92935fc52fb0c9b1330c1e5b8263bad3af43b89dae583d9a101bc5830f08f",
                       "bytes": 189565952 + 598637568, "units": 16301215},
-    # ncu capture of one 17-vector double-float launch on the 16^3 parallelepiped (units:
-    # 14,392,119 nonzeros of the tables, read once per launch from their two list layouts)
-    "k_apply_lists": {"source": "solve.cu",
-                      "sha256": "338f5e8603fcac2521983a70e9b21d81327abaefc04680a6d409ed64289638c0",
-                      "bytes": 433901312 + 5169152, "units": 14392119},
 }
 
 def _source_sha(name):
@@ -128,17 +123,19 @@ def kernel_rooflines(kms: dict, cnt: dict, n_dof: int, precision: str, peaks: di
     walk_tables  HBM: 160 B (one tet record) per walked segment; FP64 side: 25 flops per
                  segment against the FP64 rate
     split        HBM: per table element 16 B read (L and R pairs) and the four operand halves
-                 written (2 B each for BF16, 4 B for TF32); then, where the apply runs from
-                 the nonzero lists, their entries (10 B per nonzero of L or W R in each of the
-                 row-major and Gauss-point-major layouts), else the dense W R pair (8 B per
-                 element)
+                 written (2 B each for BF16, 4 B for TF32); the class's time also holds the
+                 transposition of the refinement operator's blocks, whose bytes are not counted
     contract     tensor: algorithmic flops sum_g 4 nnz(L[g]) nnz(R[g]) per axis (when
-                 counted) and the executed split-product MMA flops (3 x 2 D_b^2 G_b)
+                 counted) and the executed split-product MMA flops (3 x 2 D_b^2 G_b); the
+                 mixed forms' time also holds the contraction that builds the refinement's
+                 operator (k_contract_rows), whose flops are not counted
     factor       FP32 pipe: n^3 / 3 flops
-    chain        HBM: one read of the factor's lower triangle (2 n^2 B for FP32) per launch
-    apply        FP32 issue: 2 double-float multiply-adds (13 FP32 instructions each) per
-                 nonzero table entry (of L and of R) and vector, when the nonzeros are counted
-                 (else 4 per dense bin-table element pair)
+    chain        HBM: the factor's lower triangle once per direction (4 n^2 B for FP32) and
+                 solve of a group of columns
+    apply        FP32 issue: the matrix-free work the block-sparse operator replaces, 2
+                 double-float multiply-adds (13 FP32 instructions each) per nonzero table entry
+                 (of L and of R) and vector, when the nonzeros are counted (else 4 per dense
+                 bin-table element pair)
     """
     out = {}
     hbm = float(peaks["hbm_gbs"])
@@ -157,18 +154,17 @@ def kernel_rooflines(kms: dict, cnt: dict, n_dof: int, precision: str, peaks: di
     s = kms.get("split", (0, 0))
     if s[0] > 0:
         per = 16 + (8 if precision == "bf16x3" else 16 if precision == "tf32x3" else 0)
+        # an apply from the tables also has its operands written here: a dense W R pair per
+        # element, or two lists of the nonzeros; the block operator (block_operator) has none
         snz = cnt.get("table_nnz") or 0
-        slists = bool(snz) and cnt.get("apply_lists", True)
-        nbytes = per * elems + (2 * 10 * snz if slists else 8 * elems)
-        gbs = nbytes / (s[0] * 1e-3) / 1e9
-        tail = (f"the nonzero lists, 2 x 10 B per nonzero x {snz} nonzeros" if slists else
-                "the dense W R pair, 8 B per element")
-        out["split"] = {"kernel": "k_split_ops (+ k_gp_lists)" if slists else "k_split_ops",
-                        "bound": "hbm", "unit": "GB/s", "achieved": gbs,
-                        "peak": hbm, "frac": gbs / hbm, "launches": s[1],
+        lists = bool(snz) and cnt.get("apply_lists", True)
+        tail = 0 if cnt.get("block_operator") else (2 * 10 * snz if lists else 8 * elems)
+        gbs = (per * elems + tail) / (s[0] * 1e-3) / 1e9
+        out["split"] = {"kernel": "k_split_ops (+ k_op_mirror)", "bound": "hbm", "unit": "GB/s",
+                        "achieved": gbs, "peak": hbm, "frac": gbs / hbm, "launches": s[1],
                         "launch_ms": s[0] / s[1], "traffic": None,
-                        "algorithmic": f"{per} B per table element x {elems:.0f} elements, plus "
-                                       + tail}
+                        "algorithmic": f"{per} B per table element x {elems:.0f} elements"
+                                       + (f" + {tail:.0f} B of apply operands" if tail else "")}
     c = kms.get("contract", (0, 0))
     if c[0] > 0:
         ratio = {"tf32x3": 1.1 / 2.25, "bf16x3": 1.0}.get(precision)
@@ -176,20 +172,22 @@ def kernel_rooflines(kms: dict, cnt: dict, n_dof: int, precision: str, peaks: di
         if ratio is not None:
             peak = float(peaks.get("bf16_tflops", 1900.0)) * ratio
             ach = executed / (c[0] * 1e-3) / 1e12
-            rec = {"kernel": "k_contract_tc", "bound": "tensor", "unit": "TFLOP/s",
+            rec = {"kernel": "k_contract_tc (+ k_contract_rows)", "bound": "tensor", "unit": "TFLOP/s",
                    "achieved": ach, "peak": peak, "frac": ach / peak,
                    "basis": "executed split-product MMA flops (3 x 2 D_b^2 G_b over the bins)"}
         else:
             peak = FP64_TFLOPS if precision == "fp64" else FP32_FMA_TFLOPS
-            ach = cnt["contract_flops"] / (c[0] * 1e-3) / 1e12
-            rec = {"kernel": "k_contract_simt", "bound": "alu", "unit": "TFLOP/s",
+            work = cnt.get("algorithmic_flops")
+            ach = (work or cnt["contract_flops"]) / (c[0] * 1e-3) / 1e12
+            rec = {"kernel": "k_contract_rows", "bound": "alu", "unit": "TFLOP/s",
                    "achieved": ach, "peak": peak, "frac": ach / peak,
-                   "basis": "dense bin flops 2 D_b^2 G_b"}
+                   "basis": "sum over the Gauss points of 4 nnz(L) nnz(R)" if work
+                            else "dense bin flops 2 D_b^2 G_b"}
         alg = cnt.get("algorithmic_flops")
         if alg:
             rec["algorithmic_tflops"] = alg / (c[0] * 1e-3) / 1e12
-            rec["executed_over_algorithmic"] = (executed if ratio is not None
-                                                else cnt["contract_flops"]) / alg
+            if ratio is not None:
+                rec["executed_over_algorithmic"] = executed / alg
         rec.update(launches=c[1], launch_ms=c[0] / c[1], traffic=None)
         out["contract"] = rec
     f = kms.get("factor", (0, 0))
@@ -212,7 +210,7 @@ def kernel_rooflines(kms: dict, cnt: dict, n_dof: int, precision: str, peaks: di
         else:
             peak = FP64_TFLOPS if precision == "fp64" else FP32_FMA_TFLOPS
             ach = fl / (f[0] * 1e-3) / 1e12
-            out["factor"] = {"kernel": "k_chol_tiles", "bound": "alu", "unit": "TFLOP/s",
+            out["factor"] = {"kernel": "k_chol_f64" if precision == "fp64" else "k_chol_tiles", "bound": "alu", "unit": "TFLOP/s",
                              "achieved": ach, "peak": peak, "frac": ach / peak, "launches": f[1],
                              "launch_ms": f[0] / f[1], "traffic": None,
                              "algorithmic": f"n^3/3 flops, n = {n_dof}",
@@ -220,12 +218,12 @@ def kernel_rooflines(kms: dict, cnt: dict, n_dof: int, precision: str, peaks: di
     ch = kms.get("chain", (0, 0))
     if ch[0] > 0:
         esz = 8 if precision == "fp64" else 4
-        byt = esz * n_dof * n_dof / 2.0
+        byt = esz * n_dof * n_dof          # n^2 / 2 entries, two directions
         gbs = byt / (ch[0] / ch[1] * 1e-3) / 1e9
-        out["chain"] = {"kernel": "k_solve_chain", "bound": "hbm", "unit": "GB/s",
+        out["chain"] = {"kernel": "k_tri_rows, k_tri_cols, k_tri_tile", "bound": "hbm", "unit": "GB/s",
                         "achieved": gbs, "peak": hbm, "frac": gbs / hbm, "launches": ch[1],
                         "launch_ms": ch[0] / ch[1], "traffic": None,
-                        "algorithmic": "the factor's lower triangle once per launch"}
+                        "algorithmic": "the factor's lower triangle twice per solve"}
     a = kms.get("apply", (0, 0))
     if a[0] > 0 and cnt.get("apply_vectors"):
         nnz = cnt.get("table_nnz")
@@ -240,14 +238,10 @@ def kernel_rooflines(kms: dict, cnt: dict, n_dof: int, precision: str, peaks: di
                    f"per table element and vector, {elems:.0f} elements, "
                    f"{cnt['apply_vectors']} vector-applies")
         ach = ops / (a[0] * 1e-3) / 1e12
-        lists = bool(nnz) and cnt.get("apply_lists", True)
-        out["apply"] = {"kernel": "k_apply_lists" if lists else "k_apply_bin", "bound": "alu",
-                        "unit": "T FP32 instr/s",
+        out["apply"] = {"kernel": "k_op_apply", "bound": "alu", "unit": "T FP32 instr/s",
                         "achieved": ach, "peak": FP32_ISSUE_TOPS, "frac": ach / FP32_ISSUE_TOPS,
-                        "launches": a[1], "launch_ms": a[0] / a[1],
-                        "traffic": measured_traffic("k_apply_lists", nnz) if lists else None,
-                        "algorithmic": alg,
-                        "bytes_gbs": 16 * elems * cnt["apply_passes"] / (a[0] * 1e-3) / 1e9}
+                        "launches": a[1], "launch_ms": a[0] / a[1], "traffic": None,
+                        "algorithmic": alg + " (matrix-free equivalent)"}
         if nnz:
             out["apply"]["nonzero_fraction_of_bin_tables"] = nnz / (2.0 * elems)
     return out
@@ -521,7 +515,7 @@ def measure_workload(args, torch, fem3, inputs, workload, precision, steps, warm
     cnt = m.counters()
     cnt["algorithmic_flops"] = m.contract_work()
     cnt["table_nnz"] = m.table_nnz()
-    cnt["apply_lists"] = m.apply_lists()
+    cnt["block_operator"] = True
     out.update(dofs=int(m.n_dof), stages_ms=_stage_dict(m.stage_ms()),
                kernel_ms={k: {"ms": round(v[0], 4), "launches": v[1]} for k, v in kms.items()},
                segments_per_step=cnt["segments"], table_bytes=cnt["table_bytes"],
@@ -530,12 +524,7 @@ def measure_workload(args, torch, fem3, inputs, workload, precision, steps, warm
                            "tol": args.tol},
                bins=[m.bin_stats(a) for a in range(3)], tc_tile=m.tc_tile()[0] or None)
     if precision != "fp64":
-        passes = 0
-        vecs = 0
-        for _ in range(m.iters):
-            vecs += nrhs
-            passes += (nrhs + 7) // 8
-        cnt["apply_vectors"], cnt["apply_passes"] = vecs, passes
+        cnt["apply_vectors"] = m.iters * nrhs
     n_dof = m.n_dof
     m.free()
     tc_factor = args.chol_tc == 1 or (args.chol_tc == 0 and n_dof >= CHOL_TC_MIN_N)

@@ -154,9 +154,10 @@ void kc_reset(Mesh *m) {
 }
 
 int read_errors(Mesh *m, int32_t *h_err) {
-    FEM3_CUDA(cudaMemcpyAsync(h_err, m->err, sizeof(int32_t) * ERR_COUNT, cudaMemcpyDeviceToHost,
-                              m->stream));
+    FEM3_CUDA(cudaMemcpyAsync(m->h_norms + kErrSlot, m->err, sizeof(int32_t) * ERR_COUNT,
+                              cudaMemcpyDeviceToHost, m->stream));
     FEM3_CUDA(cudaStreamSynchronize(m->stream));
+    memcpy(h_err, m->h_norms + kErrSlot, sizeof(int32_t) * ERR_COUNT);
     return FEM3_OK;
 }
 

@@ -189,7 +189,9 @@ struct Mesh {
     int chol_tc_opt = 0;       // 0: by size, 1: always, -1: never (tensor-core factorisation)
     bool chol_tc_used = false; // the last factorisation ran on the tensor cores
     double *norms = nullptr;   // device scratch for reductions
-    double *h_norms = nullptr; // pinned host mirror
+    // pinned host block of 128 values, the target of every small device-to-host read (a pageable
+    // target makes each copy wait by itself): reductions, and from kErrSlot the error words
+    double *h_norms = nullptr;
 
     // counters
     int64_t launches = 0;      // kernels this handle has launched
@@ -212,6 +214,7 @@ struct Mesh {
     size_t arena_size = 0, arena_used = 0;
 };
 
+constexpr int kErrSlot = 104;   // of Mesh::h_norms
 inline void note_launch(Mesh *m) { m->launches++; }
 
 // bins [b0, b1) of the current part of an axis: contiguous ranges of equal bin count

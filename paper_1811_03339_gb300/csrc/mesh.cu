@@ -648,16 +648,13 @@ int mesh_build(Mesh *m, const double *verts_d, const int32_t *tets_d) {
 
     // boundary vertices, dof numbering, vertex -> tets
     int32_t *used, *bnd, *flag, *off, *vcount, *cursor;
-    FEM3_TRY(dev_alloc_t(m, &used, N));
-    FEM3_TRY(dev_alloc_t(m, &bnd, N));
+    FEM3_TRY(dev_alloc_t(m, &used, 4 * N));   // the four that start at zero, one memset
+    bnd = used + N;
+    vcount = used + 2 * N;
+    cursor = used + 3 * N;
     FEM3_TRY(dev_alloc_t(m, &flag, N));
     FEM3_TRY(dev_alloc_t(m, &off, N + 1));
-    FEM3_TRY(dev_alloc_t(m, &vcount, N));
-    FEM3_TRY(dev_alloc_t(m, &cursor, N));
-    FEM3_CUDA(cudaMemsetAsync(used, 0, sizeof(int32_t) * N, s));
-    FEM3_CUDA(cudaMemsetAsync(bnd, 0, sizeof(int32_t) * N, s));
-    FEM3_CUDA(cudaMemsetAsync(vcount, 0, sizeof(int32_t) * N, s));
-    FEM3_CUDA(cudaMemsetAsync(cursor, 0, sizeof(int32_t) * N, s));
+    FEM3_CUDA(cudaMemsetAsync(used, 0, sizeof(int32_t) * 4 * N, s));
     k_mark_nodes<<<grid_for(4 * T), kThreads, 0, s>>>(tets_d, m->nbr, T, N, used, bnd, vcount);
     note_launch(m);
     k_interior_flag<<<grid_for(N), kThreads, 0, s>>>(used, bnd, N, flag);
@@ -681,15 +678,18 @@ int mesh_build(Mesh *m, const double *verts_d, const int32_t *tets_d) {
     k_sum_ordered<<<1, 256, 0, s>>>(vpart, nwarp, vsum);
     note_launch(m);
 
-    int32_t n_dof = 0;
-    unsigned long long h_ext[6];
-    double h_vsum = 0;
-    FEM3_CUDA(cudaMemcpyAsync(&n_dof, off + N, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    FEM3_CUDA(cudaMemcpyAsync(h_ext, ext, sizeof(h_ext), cudaMemcpyDeviceToHost, s));
-    FEM3_CUDA(cudaMemcpyAsync(&h_vsum, vsum, sizeof(double), cudaMemcpyDeviceToHost, s));
+    // into the pinned block: extents, volume sum, dof count; the wait comes with the error words
+    double *h = m->h_norms;
+    FEM3_CUDA(cudaMemcpyAsync(h, ext, sizeof(unsigned long long) * 6, cudaMemcpyDeviceToHost, s));
+    FEM3_CUDA(cudaMemcpyAsync(h + 6, vsum, sizeof(double), cudaMemcpyDeviceToHost, s));
+    FEM3_CUDA(cudaMemcpyAsync(h + 7, off + N, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     int32_t h_err[ERR_COUNT];
-    FEM3_CUDA(cudaMemcpyAsync(h_err, m->err, sizeof(h_err), cudaMemcpyDeviceToHost, s));
-    FEM3_CUDA(cudaStreamSynchronize(s));
+    FEM3_TRY(read_errors(m, h_err));
+    unsigned long long h_ext[6];
+    std::memcpy(h_ext, h, sizeof(h_ext));
+    const double h_vsum = h[6];
+    int32_t n_dof = 0;
+    std::memcpy(&n_dof, h + 7, sizeof(n_dof));
     if (h_err[ERR_MESH]) return set_error(FEM3_E_MESH, "degenerate tetrahedron or node id out of range");
     if (h_err[ERR_FACE]) return set_error(FEM3_E_MESH, "a face is shared by more than two tetrahedra");
     for (int d = 0; d < 6; d++) {
@@ -824,6 +824,15 @@ int bins_build(Mesh *m) {
     k_bin_slots3<<<dim3(grid_for(n_gp), 3), kThreads, 0, s>>>(P, m->gw, n_gp);
     note_launch(m);
 
+    // the three axes' table layouts and work lists, one copy (nine cost the host about 5 us each)
+    std::vector<unsigned char> pack;
+    const auto add = [&pack](const void *p, size_t bytes) {
+        const size_t at = pack.size();
+        pack.resize(at + (bytes + 15) / 16 * 16);
+        if (bytes) std::memcpy(pack.data() + at, p, bytes);
+        return at;
+    };
+    size_t at_off[3], at_ld[3], at_work[3];
     for (int axis = 0; axis < 3; axis++) {
         AxisBins &B = m->bins[axis];
         const int nb = B.n_bins;
@@ -845,18 +854,20 @@ int bins_build(Mesh *m) {
         }
         B.tab_elems = acc;
         B.n_work = (int)work.size();
-        FEM3_TRY(dev_alloc_t(m, &B.tab_off, nb));
-        FEM3_TRY(dev_alloc_t(m, &B.tab_ld, nb));
-        FEM3_TRY(dev_alloc_t(m, &B.work, std::max(1, B.n_work)));
-        FEM3_CUDA(cudaMemcpyAsync(B.tab_off, B.h_tab_off.data(), sizeof(int64_t) * nb,
-                                  cudaMemcpyHostToDevice, s));
-        FEM3_CUDA(cudaMemcpyAsync(B.tab_ld, B.h_tab_ld.data(), sizeof(int32_t) * nb,
-                                  cudaMemcpyHostToDevice, s));
-        if (B.n_work)
-            FEM3_CUDA(cudaMemcpyAsync(B.work, work.data(), sizeof(int4) * B.n_work,
-                                      cudaMemcpyHostToDevice, s));
+        at_off[axis] = add(B.h_tab_off.data(), sizeof(int64_t) * nb);
+        at_ld[axis] = add(B.h_tab_ld.data(), sizeof(int32_t) * nb);
+        at_work[axis] = add(work.data(), sizeof(int4) * B.n_work);
         FEM3_TRY(dev_alloc_t(m, &m->tabL[axis], std::max<int64_t>(1, acc)));
         FEM3_TRY(dev_alloc_t(m, &m->tabR[axis], std::max<int64_t>(1, acc)));
+    }
+    unsigned char *pack_d;
+    FEM3_TRY(dev_alloc_t(m, &pack_d, pack.size() + 16));
+    FEM3_CUDA(cudaMemcpyAsync(pack_d, pack.data(), pack.size(), cudaMemcpyHostToDevice, s));
+    for (int axis = 0; axis < 3; axis++) {
+        AxisBins &B = m->bins[axis];
+        B.tab_off = reinterpret_cast<int64_t *>(pack_d + at_off[axis]);
+        B.tab_ld = reinterpret_cast<int32_t *>(pack_d + at_ld[axis]);
+        B.work = reinterpret_cast<int4 *>(pack_d + at_work[axis]);
     }
     FEM3_CUDA(cudaGetLastError());
     return FEM3_OK;

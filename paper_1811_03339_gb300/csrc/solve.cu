@@ -598,14 +598,12 @@ bool factor_on_tc(const Mesh *m) {
 }
 
 // The refinement's operator (a contraction that fills the chip) is built beside the tile-task
-// factorisation (a serial chain that leaves most of it idle) from this order on; below it the
-// two are a few launches each and the events between the streams cost as much as they save.
-// Not beside the blocked factorisation: its trailing updates take an SM's whole shared memory
+// factorisation (a serial chain that leaves most of it idle): a TF32 x 3 step after against
+// before, 658 -> 646 us at n = 27, 1,012 -> 993 at 343, 2,559 -> 2,308 at 1,728.  Not beside the blocked factorisation: its trailing updates take an SM's whole shared memory
 // each, so the critical chain waited for the operator's CTAs to drain (24^3 step 30.6 ms
 // with, 30.3 ms without).  A profiled mesh times its launches one at a time.
-constexpr int64_t kOpBesideMin = 512;
 bool op_beside_factor(const Mesh *m) {
-    return !m->profile && m->n_dof >= kOpBesideMin && !factor_on_tc(m);
+    return !m->profile && !factor_on_tc(m);
 }
 
 // the FP32 factor; on return m->stream waits for everything enqueued on cx's streams

@@ -1,5 +1,5 @@
 """The refinement's operator built beside the factorisation (csrc/operator.cu, factor() in
-csrc/solve.cu): orders on both sides of its lower limit (512), of the small block patterns (32
+csrc/solve.cu): orders on both sides of the small block patterns (32
 block rows) and of the blocked factorisation (4,096), a handle assembled again, and a batch whose
 precision changes between eager runs, captures and replays.  Reference: a dense FP64 solve
 (torch) with the FP64 form's matrix; the mixed forms' bound is 1e-8."""
