@@ -6,7 +6,7 @@
 // per block J and direction, two launches over the whole chip: y_J = L_JJ^{-1} t_J, and
 // t_I -= L_IJ y_J for every later block I (k_tri_rows forward, k_tri_cols, the transposes, on
 // the way back).  What bounds a launch is the read of its matrix block (HBM for the updates of
-// large factors) and the launch itself, about 2.5 us.
+// large factors) and the launch itself, about 2.5 us, of which the chaining hides a part.
 //
 // B: doubling to B costs n B^2 / 3 multiply-adds, a step less saves two launches per
 // direction and solve.  FP32: 1024 above n = 4,096 (n = 12,167: 0.29 ms once, 12 steps per
@@ -16,6 +16,9 @@
 // Measured (GB300), both directions, against one CTA walking 64-row blocks with worker CTAs
 // feeding it partial sums through flags: 17 columns at n = 12,167 1.40 -> 0.99 ms, eight at n = 6,859
 // 0.49 -> 0.32 ms, FP64 four columns at n = 1,000 0.31 -> 0.16 ms, one at n = 343 47 -> 14 us.
+// Chaining the launches (launch_chained) then took the eight-column refined solve at n = 6,859 from
+// 1.77 to 1.62 ms and the 16^3 TF32 x 3 step from 4.31 to 4.16 ms (24^3: 28.1 ms either way, the
+// updates are bound by HBM there).
 #include <algorithm>
 
 #include "fem3_impl.cuh"
@@ -26,6 +29,37 @@ namespace {
 
 constexpr int kTriThreads = 256, kTriWarps = kTriThreads / 32;   // k_tri_rows
 constexpr int kColThreads = 512, kColWarps = kColThreads / 32;   // k_tri_cols
+
+// The launches of a solve are chained (programmatic dependent launch): a kernel starts while
+// the one before it finishes, fetches its share of the matrix (which no launch of the solve
+// writes) into L2, and only then waits for the vectors.  Every wait is for the whole launch
+// before, which itself waited for its own, so the order of reads and writes is the stream's.
+__device__ __forceinline__ void chain_next() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void fetch_l2(const void *p) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
+template <class... KP, class... Args>
+int launch_chained(bool first, void (*kernel)(KP...), int64_t grid, int threads, size_t sh,
+                   cudaStream_t s, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = sh;
+    cfg.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = first ? 0 : 1;   // the first waits for whatever wrote the matrix
+    FEM3_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<KP>(args)...));
+    return FEM3_OK;
+}
 
 // diagonal 64 x 64 inverses into the B x B blocks
 template <class TF>
@@ -119,7 +153,7 @@ __global__ void __launch_bounds__(256) k_tri_double(const TF *__restrict__ L, in
 template <class TF, int NR, int R, bool TRI>
 __global__ void __launch_bounds__(kTriThreads) k_tri_rows(const TF *__restrict__ M, int64_t ldm,
                                                           int64_t rows, int K,
-                                                          const TF *__restrict__ x, int64_t n,
+                                                          const TF *x, int64_t n,
                                                           int nrhs, TF *out) {
     const int lane = threadIdx.x & 31;
     const int64_t r0 = ((int64_t)blockIdx.x * kTriWarps + (threadIdx.x >> 5)) * R;
@@ -131,6 +165,13 @@ __global__ void __launch_bounds__(kTriThreads) k_tri_rows(const TF *__restrict__
         for (int v = 0; v < NR; v++) acc[q][v] = TF(0);
     const TF *Mr = M + r0 * ldm;
     const int kend = TRI ? (int)min((int64_t)K, r0 + R) : K;
+    chain_next();
+#pragma unroll
+    for (int q = 0; q < R; q++)
+        if (r0 + q < rows)
+            for (int k = lane * (128 / (int)sizeof(TF)); k < kend; k += 32 * (128 / (int)sizeof(TF)))
+                fetch_l2(Mr + q * ldm + k);
+    chain_wait();
 #pragma unroll(R == 1 ? 4 : 2)
     for (int k = lane; k < kend; k += 32) {
         TF a[R];
@@ -139,7 +180,7 @@ __global__ void __launch_bounds__(kTriThreads) k_tri_rows(const TF *__restrict__
             a[q] = (r0 + q < rows && (!TRI || k <= r0 + q)) ? __ldg(Mr + q * ldm + k) : TF(0);
 #pragma unroll
         for (int v = 0; v < NR; v++) {
-            const TF xv = NR == 1 || v < nrhs ? __ldg(x + (int64_t)v * n + k) : TF(0);
+            const TF xv = NR == 1 || v < nrhs ? x[(int64_t)v * n + k] : TF(0);
 #pragma unroll
             for (int q = 0; q < R; q++) acc[q][v] = fma(a[q], xv, acc[q][v]);
         }
@@ -169,7 +210,7 @@ template <class TF, int NR> struct ColCfg {
 template <class TF, int NR, bool TRI>
 __global__ void __launch_bounds__(kColThreads) k_tri_cols(const TF *__restrict__ M, int64_t ldm,
                                                           int rows, int64_t cols,
-                                                          const TF *__restrict__ x, int64_t n,
+                                                          const TF *x, int64_t n,
                                                           int nrhs, TF *out) {
     constexpr int PAD = ColCfg<TF, NR>::PAD, U = 16;   // rows in flight
     extern __shared__ __align__(16) unsigned char sm_cols[];   // x of the warps' rows, then sums
@@ -183,6 +224,10 @@ __global__ void __launch_bounds__(kColThreads) k_tri_cols(const TF *__restrict__
     for (int v = 0; v < NR; v++) acc[v] = TF(0);
     // rows from the CTA's first column on when triangular
     const int first = TRI ? blockIdx.x : 0, pieces = (rows + 31) / 32;
+    chain_next();
+    for (int i = 32 * first + threadIdx.x; i < rows; i += kColThreads)
+        fetch_l2(M + (int64_t)i * ldm + (int64_t)blockIdx.x * 32);
+    chain_wait();
     for (int pc = first + warp; pc < pieces; pc += kColWarps) {
         const int i0 = 32 * pc;
         const TF *Mc = M + (int64_t)i0 * ldm + c;
@@ -197,7 +242,7 @@ __global__ void __launch_bounds__(kColThreads) k_tri_cols(const TF *__restrict__
         load(0, a);
 #pragma unroll
         for (int v = 0; v < NR; v++)
-            xs[lane][v] = i0 + lane < rows && v < nrhs ? __ldg(x + (int64_t)v * n + i0 + lane) : TF(0);
+            xs[lane][v] = i0 + lane < rows && v < nrhs ? x[(int64_t)v * n + i0 + lane] : TF(0);
         __syncwarp();
 #pragma unroll
         for (int i = 0; i < 32; i += U) {
@@ -237,7 +282,7 @@ constexpr int kTileOut = 32, kTileK = 128;
 constexpr size_t kTileRed = 24 * 1024;   // room of the final sums (24 columns)
 template <int NR, bool TRANS>
 __global__ void __launch_bounds__(256) k_tri_tile(const float *__restrict__ M, int64_t ldm,
-                                                  int64_t outs, int K, const float *__restrict__ x,
+                                                  int64_t outs, int K, const float *x,
                                                   int64_t n, int nrhs, float *out) {
     static_assert(NR % 4 == 0, "four column groups");
     constexpr int NV = NR / 4, LM = TRANS ? kTileOut + 4 : kTileK + 4, LX = kTileK + 4;
@@ -253,7 +298,7 @@ __global__ void __launch_bounds__(256) k_tri_tile(const float *__restrict__ M, i
     for (int q = 0; q < 4; q++)
 #pragma unroll
         for (int v = 0; v < NV; v++) acc[q][v] = 0.f;
-    auto load = [&](int kc) {
+    auto load_m = [&](int kc) {
 #pragma unroll
         for (int q = 0; q < EM; q++) {
             const int e = tid + 256 * q, r = e / W, c = e % W;
@@ -261,13 +306,24 @@ __global__ void __launch_bounds__(256) k_tri_tile(const float *__restrict__ M, i
             const int k = kc + (TRANS ? r : c);
             pm[q] = o < outs && k < K ? __ldg(M + (TRANS ? k * ldm + o : o * ldm + k)) : 0.f;
         }
+    };
+    auto load_x = [&](int kc) {
 #pragma unroll
         for (int q = 0; q < EX; q++) {
             const int e = tid + 256 * q, v = e / kTileK, k = kc + e % kTileK;
-            px[q] = v < nrhs && k < K ? __ldg(x + (int64_t)v * n + k) : 0.f;
+            px[q] = v < nrhs && k < K ? x[(int64_t)v * n + k] : 0.f;
         }
     };
-    load(0);
+    chain_next();
+    load_m(0);
+    // the rest of the CTA's part of M, a line of 32 entries per fetch
+    for (int e = tid + (TRANS ? kTileK : kTileOut * (kTileK / 32)); e < K * kTileOut / 32; e += 256) {
+        const int64_t o = o0 + (TRANS ? 0 : e % kTileOut);
+        const int k = TRANS ? e : e / kTileOut * 32;
+        if (o < outs && k < K) fetch_l2(M + (TRANS ? k * ldm + o : o * ldm + k));
+    }
+    chain_wait();
+    load_x(0);
     for (int kc = 0; kc < K; kc += kTileK) {
         __syncthreads();   // the previous chunk has been read
 #pragma unroll
@@ -281,7 +337,10 @@ __global__ void __launch_bounds__(256) k_tri_tile(const float *__restrict__ M, i
             if (e < NR * kTileK) xs[e / kTileK * LX + e % kTileK] = px[q];
         }
         __syncthreads();
-        if (kc + kTileK < K) load(kc + kTileK);
+        if (kc + kTileK < K) {
+            load_m(kc + kTileK);
+            load_x(kc + kTileK);
+        }
 #pragma unroll
         for (int kk = 0; kk < 16; kk += 4) {
             const int k = kg * 16 + kk;
@@ -336,15 +395,14 @@ template <class TF> int tri_width(int64_t n) {
 // rows of a launch: one per warp until that fills the chip (about eight warps per SM), then four
 // (NR sums each), which share the reads of x
 template <class TF, int NR, bool TRI>
-void launch_rows(const TF *M, int64_t ldm, int64_t rows, int K, const TF *x, int64_t n, int nrhs,
-                 TF *out, cudaStream_t s) {
+int launch_rows(const TF *M, int64_t ldm, int64_t rows, int K, const TF *x, int64_t n, int nrhs,
+                TF *out, cudaStream_t s, bool first = false) {
     if (rows <= 4 * 1216)
-        k_tri_rows<TF, NR, 1, TRI><<<(unsigned)((rows + kTriWarps - 1) / kTriWarps), kTriThreads, 0, s>>>(
-            M, ldm, rows, K, x, n, nrhs, out);
-    else
-        k_tri_rows<TF, NR, 4, TRI>
-            <<<(unsigned)((rows + 4 * kTriWarps - 1) / (4 * kTriWarps)), kTriThreads, 0, s>>>(
-                M, ldm, rows, K, x, n, nrhs, out);
+        return launch_chained(first, k_tri_rows<TF, NR, 1, TRI>, (rows + kTriWarps - 1) / kTriWarps,
+                              kTriThreads, 0, s, M, ldm, rows, K, x, n, nrhs, out);
+    return launch_chained(first, k_tri_rows<TF, NR, 4, TRI>,
+                          (rows + 4 * kTriWarps - 1) / (4 * kTriWarps), kTriThreads, 0, s, M, ldm,
+                          rows, K, x, n, nrhs, out);
 }
 
 template <class TF, int NR, bool TRI>
@@ -357,9 +415,8 @@ int launch_cols(const TF *M, int64_t ldm, int rows, int64_t cols, const TF *x, i
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
         attr = true;
     }
-    k_tri_cols<TF, NR, TRI><<<(unsigned)((cols + 31) / 32), kColThreads, sh, s>>>(M, ldm, rows, cols, x,
-                                                                                 n, nrhs, out);
-    return FEM3_OK;
+    return launch_chained(false, k_tri_cols<TF, NR, TRI>, (cols + 31) / 32, kColThreads, sh, s, M, ldm,
+                          rows, cols, x, n, nrhs, out);
 }
 
 // t -= M x or M^T x
@@ -368,14 +425,13 @@ int launch_update(const TF *M, int64_t ldm, int64_t outs, int K, const TF *x, in
                   TF *out, cudaStream_t s) {
     if constexpr (sizeof(TF) == 4 && NR > 1) {
         constexpr int NP = (NR + 3) / 4 * 4;
-        k_tri_tile<NP, TRANS><<<(unsigned)((outs + kTileOut - 1) / kTileOut), 256, 0, s>>>(
-            M, ldm, outs, K, x, n, nrhs, out);
+        return launch_chained(false, k_tri_tile<NP, TRANS>, (outs + kTileOut - 1) / kTileOut, 256, 0, s,
+                              M, ldm, outs, K, x, n, nrhs, out);
     } else if constexpr (TRANS) {
         return launch_cols<TF, NR, false>(M, ldm, K, outs, x, n, nrhs, out, s);
     } else {
-        launch_rows<TF, NR, false>(M, ldm, outs, K, x, n, nrhs, out, s);
+        return launch_rows<TF, NR, false>(M, ldm, outs, K, x, n, nrhs, out, s);
     }
-    return FEM3_OK;
 }
 
 template <class TF, int NR>
@@ -388,7 +444,8 @@ int solve_blocks(Mesh *m, const TF *L, int64_t n, TF *Y, int nrhs) {
     kc_begin(m, KC_CHAIN);
     for (int j = 0; j < nb; j++) {   // Y -> W
         const int64_t c0 = (int64_t)j * B, w = std::min<int64_t>(B, n - c0), rest = n - c0 - w;
-        launch_rows<TF, NR, true>(inv + (int64_t)j * B * B, B, w, (int)w, Y + c0, n, nrhs, W + c0, s);
+        FEM3_TRY((launch_rows<TF, NR, true>(inv + (int64_t)j * B * B, B, w, (int)w, Y + c0, n, nrhs,
+                                            W + c0, s, j == 0)));
         if (rest > 0)
             FEM3_TRY((launch_update<TF, NR, false>(L + (c0 + w) * n + c0, n, rest, (int)w, W + c0, n,
                                                    nrhs, Y + c0 + w, s)));
