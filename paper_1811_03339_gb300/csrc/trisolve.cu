@@ -18,7 +18,7 @@
 // 0.49 -> 0.32 ms, FP64 four columns at n = 1,000 0.31 -> 0.16 ms, one at n = 343 47 -> 14 us.
 // Chaining the launches (launch_chained) then took the eight-column refined solve at n = 6,859 from
 // 1.77 to 1.62 ms and the 16^3 TF32 x 3 step from 4.31 to 4.16 ms (24^3: 28.1 ms either way, the
-// updates are bound by HBM there).
+// updates are bound by HBM there); without the fetches into L2 the former is 1.70 ms.
 #include <algorithm>
 
 #include "fem3_impl.cuh"
