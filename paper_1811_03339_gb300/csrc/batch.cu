@@ -1,8 +1,8 @@
 // Batched assembly and solve of many meshes of uneven size (not in the paper: the paper
 // assembles one mesh at a time).  One launch walks every Gauss-point line of every mesh;
 // contraction, load vector, factorisation and refinement sweeps of each mesh run on internal
-// streams so that meshes overlap (a sweep's triangular solves are one chain launch per
-// direction and mesh, latency-bound, so the meshes' chains run side by side, and its late
+// streams so that meshes overlap (a sweep's triangular solves are a chain of launches per
+// mesh, latency-bound, so the meshes' chains run side by side, and its late
 // sweeps apply the operator in FP32 as the single-mesh solve does); all residuals are checked
 // with one host wait per sweep.  12 meshes of 6 to 20 cells per side, 16 columns: 49.3 ms a
 // run with block-step solves over the whole batch (1,100 launches, 13.3 ms) and double-float

@@ -18,8 +18,8 @@
 //      the trailing matrix - TMA loads (128-byte swizzle) into a two-stage ring, three MMAs
 //      per 32-column K step (hi hi, hi lo, lo hi) into one of two TMEM accumulators, and an
 //      epilogue (sixteen warps) that overlaps the next tile's MMAs.
-// Look-ahead: the next panel's block column is updated on the caller's stream and the rest of
-// the trailing matrix on a side stream, so the next diagonal block and panel overlap it.
+// Look-ahead: the next panel's diagonal tile is updated on a high-priority chain stream and the
+// rest of the trailing matrix on side streams, so the next diagonal block and panel overlap it.
 // No kernel waits for another CTA; the mbarrier waits are bounded (ERR_CHOL on expiry).
 #include <math.h>
 

@@ -690,7 +690,7 @@ int solve_direct(Mesh *m, const double *b_d, int nrhs, double *u_d) {
 }
 
 // Refinement for all right-hand sides together: u = 0, r = b; repeat
-//   d = A32^{-1} r (FP32 factor, all columns in one wavefront sweep pair), u += d,
+//   d = A32^{-1} r (FP32 factor, trisolve.cu), u += d,
 //   r = b - A u in FP64, or r -= A d,
 // until every column has ||r|| <= tol ||b|| or max_iter sweeps.  The first sweep's residual is
 // formed from u in FP64.  Once the residual is below kUpdateBelow the correction is as small
