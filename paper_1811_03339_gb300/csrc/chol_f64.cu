@@ -386,21 +386,31 @@ __global__ void __launch_bounds__(kThreads, 1) k_chol_f64(double *A, int64_t n, 
     const int rb = warp >> 2, cb = warp & 3;
     const int r = rb * 8 + (lane >> 2), c = cb * 8 + (lane & 3) * 2;
     int j = 0, first = 0;   // column of the last ticket and the first ticket of that column
+    const auto row_of = [&](int t) {   // (t in column j from here on)
+        while (t - first >= nblk - j) first += nblk - j++;
+        return j + (t - first);
+    };
     for (;;) {
-        if (tid == 0) s_task = atomicAdd(ticket, 1);
+        // Thread 0 draws until it holds a task inside the profile (the others are zero and never
+        // read) and stores that one: every task then passes a barrier between the reads of
+        // s_task and the next store to it.
+        if (tid == 0) {
+            int t = atomicAdd(ticket, 1);
+            while (first_col && t < ntask) {
+                const int i = row_of(t);
+                if (i <= j + 1 || j >= first_col[i]) break;
+                t = atomicAdd(ticket, 1);
+            }
+            s_task = t;
+        }
         __syncthreads();
         const int t = s_task;
         if (t >= ntask) return;
-        while (t - first >= nblk - j) first += nblk - j++;
-        const int i = j + (t - first);
+        const int i = row_of(t);
         const int64_t r0 = (int64_t)i * kT, c0 = (int64_t)j * kT;
         const int kmax = i == j ? max(j - 1, 0) : j;   // the chain applies k = j - 1 to (j, j)
         int kmin = 0;
-        if (first_col) {
-            const int fi = first_col[i];
-            if (j < fi && i > j + 1) continue;   // outside the profile: zero, and never read
-            kmin = max(fi, first_col[j]);
-        }
+        if (first_col) kmin = max(first_col[i], first_col[j]);
         double2 acc = load_acc(A, n, r0, c0, false, r, c);
         // Updates k = 0 .. kmax-1, pipelined: the tiles L_ik, L_jk of update k + 1 are
         // loaded into registers while update k's product runs (when their flags are

@@ -52,3 +52,25 @@ def test_static_solve_sizes(n):
     y = torch.from_numpy(b).cuda()        # in place
     fem3.spd_solve_static(torch.from_numpy(A).cuda(), y, y)
     assert torch.equal(x, y)
+
+
+# cells of a long box: 1,416 dofs, band 29 (every ticket below the chain's tiles is skipped);
+# 1,536, band 73; 2,760, band 93: two and three tiles of a column are left
+@pytest.mark.parametrize("cells", [(5, 7, 60), (9, 9, 25), (9, 11, 35)])
+def test_f64_factor_band(cells):
+    """The integer order's profile: most tickets are skipped, several by one CTA in a row.  Repeats
+    differ by the element sum's order only (a few rounding errors of a matrix of condition below
+    1e3), and every one is the dense solution."""
+    mesh = _bar_mesh(cells)
+    m = fem3.Mesh(mesh.verts, mesh.tets)
+    f = np.random.default_rng(3).standard_normal(mesh.n_nodes)
+    A = m.assemble_integer((1.0, 2.0, 0.5), return_matrix=True)
+    b = m.load(torch.from_numpy(f).cuda())
+    first = m.solve(f)
+    ref = torch.linalg.solve(A, b)
+    assert float((first - ref).norm() / ref.norm()) <= 1e-10
+    for _ in range(20):
+        m.assemble_integer((1.0, 2.0, 0.5))
+        u = m.solve(f)
+        assert float((u - first).norm() / first.norm()) <= 1e-11
+    m.free()
