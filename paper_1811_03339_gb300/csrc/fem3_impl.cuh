@@ -366,11 +366,13 @@ __device__ __forceinline__ void f64_split(double x, float &hi, float &lo) {
     lo = __uint_as_float(__float_as_uint(mag) | sign);
 }
 
-// exact FP64 value of a normal FP32 number (zero and subnormals give 0), by bit assembly:
-// exponent rebiased by 1023 - 127, significand moved to the top of the 52-bit field
+// exact FP64 value of an FP32 number by bit assembly: exponent rebiased by 1023 - 127,
+// significand moved to the top of the 52-bit field (zero gives +0; the conversion instruction is
+// left for subnormals, infinities and NaN)
 __device__ __forceinline__ double f32_to_f64_exact(float x) {
     const uint32_t b = __float_as_uint(x);
     const uint32_t e = (b >> 23) & 0xFFu;
+    if (e - 1u >= 254u && (b << 1) != 0u) return (double)x;
     const unsigned long long d = ((unsigned long long)(b & 0x80000000u) << 32) |
                                  ((unsigned long long)(e + 896u) << 52) |
                                  ((unsigned long long)(b & 0x7FFFFFu) << 29);

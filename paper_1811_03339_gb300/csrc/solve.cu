@@ -400,20 +400,24 @@ int chol_tiles(float *A, int64_t n, cudaStream_t s, Mesh *m) {
     return FEM3_OK;
 }
 
-// Per-axis forms sum_g w_g ((L lam)(R u) + (R lam)(L u)) (adjoint), one CTA per bin: the
-// bin's u and lam as hi + lo pairs in shared memory, thread = (Gauss point, slice of the
-// template rows); sums in double-float FP32 arithmetic (an FP64 evaluation spends ten
-// FP64-pipe instructions per table entry on conversions and sums: 0.95 ms for the three axes
-// of the 16^3 cube, 0.35 ms now), the slices and the final product in FP64.  Bound: one read of
-// the tables.
-constexpr int kFormSlices = 4, kFormPoints = 64;
+// Per-axis forms sum_g w_g ((L lam)(R u) + (R lam)(L u)) (adjoint), one CTA per bin: the bin's u
+// and lam in shared memory, thread = (Gauss point, slice of the template rows), all sums and
+// products in FP64 whatever the form, so that dK scales with u and lam over the FP64 range.
+// Bound: the FP64 pipe, which holds a warp's instruction for 16 clocks of the SM.  A nonzero
+// table entry takes three (the pair's sum, two multiply-adds): the pair is converted by its bits,
+// as f32 -> f64 conversions run at the FP64 rate, and entries that are zero for a warp's 32
+// points (sorted along the axis) are skipped.  Sums in double-float FP32 arithmetic took AXIS_DF
+// for the three axes of the 16^3 cube, but their 2^-48 per term and their range (nothing
+// below 2^-126 or from 2^128 on, 24 bits below 2^-74) are less than the FP64 form promises; the same
+// FP64 sums with conversion instructions and no skipping took 0.95 ms, AXIS_F64 now.
+constexpr int kFormSlices = 4, kFormPoints = 64, kFormRows = 4;   // rows of a slice in flight
 __global__ void __launch_bounds__(kFormSlices *kFormPoints) k_axis_form(
     const float2 *__restrict__ tabL, const float2 *__restrict__ tabR,
     const int32_t *__restrict__ gp_off, const int32_t *__restrict__ dof_off,
     const int32_t *__restrict__ dof_idx, const int64_t *__restrict__ tab_off,
     const int32_t *__restrict__ tab_ld, const double *__restrict__ w_slot,
     const double *__restrict__ u, const double *__restrict__ lam, double *out) {
-    extern __shared__ __align__(16) float4 sm_form[];   // (u hi, u lo, lam hi, lam lo) per row
+    extern __shared__ __align__(16) double2 sm_form[];   // (u, lam) per row
     __shared__ double part[kFormSlices][4][kFormPoints];
     __shared__ double red[kFormPoints / 32];
     const int bin = blockIdx.x;
@@ -423,34 +427,48 @@ __global__ void __launch_bounds__(kFormSlices *kFormPoints) k_axis_form(
     const int ld = tab_ld[bin];
     const float2 *L = tabL + tab_off[bin], *R = tabR + tab_off[bin];
     const int32_t *dofs = dof_idx + dof_off[bin];
-    for (int c = threadIdx.x; c < D; c += blockDim.x) {
-        float4 v;
-        f64_split(u[dofs[c]], v.x, v.y);
-        f64_split(lam[dofs[c]], v.z, v.w);
-        sm_form[c] = v;
-    }
+    for (int c = threadIdx.x; c < D; c += blockDim.x)
+        sm_form[c] = make_double2(u[dofs[c]], lam[dofs[c]]);
     __syncthreads();
     const int p = threadIdx.x % kFormPoints, q = threadIdx.x / kFormPoints;
     double acc = 0;
     for (int r0 = 0; r0 < G; r0 += kFormPoints) {
         const int r = r0 + p;
-        float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};   // Lu, Ru, Llam, Rlam
+        double t[4] = {0.0, 0.0, 0.0, 0.0};   // Lu, Ru, Llam, Rlam
         if (r < G) {
-#pragma unroll 4
-            for (int c = q; c < D; c += kFormSlices) {
-                const float2 a = __ldg(L + (int64_t)c * ld + r), b = __ldg(R + (int64_t)c * ld + r);
-                const float4 v = sm_form[c];
-                df_fma(a.x, a.y, v.x, v.y, h[0], l[0]);
-                df_fma(b.x, b.y, v.x, v.y, h[1], l[1]);
-                df_fma(a.x, a.y, v.z, v.w, h[2], l[2]);
-                df_fma(b.x, b.y, v.z, v.w, h[3], l[3]);
+            for (int c0 = q; c0 < D; c0 += kFormSlices * kFormRows) {
+                float2 a[kFormRows], b[kFormRows];
+#pragma unroll
+                for (int k = 0; k < kFormRows; k++) {
+                    const int c = c0 + kFormSlices * k;
+                    a[k] = b[k] = make_float2(0.f, 0.f);
+                    if (c < D) {
+                        a[k] = __ldg(L + (int64_t)c * ld + r);
+                        b[k] = __ldg(R + (int64_t)c * ld + r);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < kFormRows; k++) {
+                    const int c = c0 + kFormSlices * k;
+                    if (a[k].x != 0.f || a[k].y != 0.f) {
+                        const double2 v = sm_form[c];
+                        const double e = f32_to_f64_exact(a[k].x) + f32_to_f64_exact(a[k].y);
+                        t[0] = fma(e, v.x, t[0]);
+                        t[2] = fma(e, v.y, t[2]);
+                    }
+                    if (b[k].x != 0.f || b[k].y != 0.f) {
+                        const double2 v = sm_form[c];
+                        const double e = f32_to_f64_exact(b[k].x) + f32_to_f64_exact(b[k].y);
+                        t[1] = fma(e, v.x, t[1]);
+                        t[3] = fma(e, v.y, t[3]);
+                    }
+                }
             }
         }
 #pragma unroll
-        for (int k = 0; k < 4; k++) part[q][k][p] = f32_to_f64_exact(h[k]) + f32_to_f64_exact(l[k]);
+        for (int k = 0; k < 4; k++) part[q][k][p] = t[k];
         __syncthreads();
         if (q == 0 && r < G) {
-            double t[4];
 #pragma unroll
             for (int k = 0; k < 4; k++)
                 t[k] = (part[0][k][p] + part[1][k][p]) + (part[2][k][p] + part[3][k][p]);
@@ -664,13 +682,13 @@ int axis_forms(Mesh *m, const double *u_d, const double *lam_d, double out[3]) {
     static bool attr = false;
     if (!attr) {
         FEM3_CUDA(cudaFuncSetAttribute(k_axis_form, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(sizeof(float4) * kMaxBinItems)));
+                                       (int)(sizeof(double2) * kMaxBinItems)));
         attr = true;
     }
     FEM3_CUDA(cudaMemsetAsync(m->norms, 0, sizeof(double) * 3, s));
     for (int axis = 0; axis < 3; axis++) {
         AxisBins &B = m->bins[axis];
-        const size_t sh = sizeof(float4) * std::max(1, B.max_dof);
+        const size_t sh = sizeof(double2) * std::max(1, B.max_dof);
         k_axis_form<<<B.n_bins, kFormSlices * kFormPoints, sh, s>>>(
             m->tabL[axis], m->tabR[axis], B.gp_off, B.dof_off, B.dof_idx, B.tab_off, B.tab_ld,
             B.w_slot, u_d, lam_d, m->norms + axis);
