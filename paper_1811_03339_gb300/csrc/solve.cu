@@ -406,10 +406,10 @@ int chol_tiles(float *A, int64_t n, cudaStream_t s, Mesh *m) {
 // Bound: the FP64 pipe, which holds a warp's instruction for 16 clocks of the SM.  A nonzero
 // table entry takes three (the pair's sum, two multiply-adds): the pair is converted by its bits,
 // as f32 -> f64 conversions run at the FP64 rate, and entries that are zero for a warp's 32
-// points (sorted along the axis) are skipped.  Sums in double-float FP32 arithmetic took AXIS_DF
-// for the three axes of the 16^3 cube, but their 2^-48 per term and their range (nothing
-// below 2^-126 or from 2^128 on, 24 bits below 2^-74) are less than the FP64 form promises; the same
-// FP64 sums with conversion instructions and no skipping took 0.95 ms, AXIS_F64 now.
+// points (sorted along the axis) are skipped.  Measured, GB300: the three axes of the 16^3 cube
+// 0.95 ms with conversion instructions and nothing skipped; the 16^3 gradient 4.82 ms so, 4.85 ms with
+// double-float FP32 sums, which keep 2^-48 a term and not the range (nothing below 2^-126 or from
+// 2^128 on, 24 bits below 2^-74).
 constexpr int kFormSlices = 4, kFormPoints = 64, kFormRows = 4;   // rows of a slice in flight
 __global__ void __launch_bounds__(kFormSlices *kFormPoints) k_axis_form(
     const float2 *__restrict__ tabL, const float2 *__restrict__ tabR,
