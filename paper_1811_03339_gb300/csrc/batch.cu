@@ -2,12 +2,13 @@
 // assembles one mesh at a time).  One launch walks every Gauss-point line of every mesh;
 // contraction, load vector, factorisation and refinement sweeps of each mesh run on internal
 // streams so that meshes overlap (a sweep's triangular solves are a chain of launches per
-// mesh, latency-bound, so the meshes' chains run side by side, and its late
-// sweeps apply the operator in FP32 as the single-mesh solve does); all residuals are checked
-// with one host wait per sweep.  12 meshes of 6 to 20 cells per side, 16 columns: 49.3 ms a
-// run with block-step solves over the whole batch (1,100 launches, 13.3 ms) and double-float
-// sweeps throughout, 26.8 ms so, 21.8 ms since each internal stream has factorisation streams
-// of its own (one set for all made the large meshes' blocked factorisations follow each other).
+// mesh, latency-bound, so the meshes' chains run side by side); all residuals are checked
+// with one host wait per sweep, and none is formed in less than double-float arithmetic.  12 meshes of
+// 6 to 20 cells per side, 16 columns: 49.3 ms a run with block-step solves over the whole batch (1,100
+// launches, 13.3 ms), 21.3 ms now that each internal stream has factorisation streams of its own (one
+// set for all made the large meshes' blocked factorisations follow each other: 26.8 ms).  Last sweeps
+// in plain FP32, as the single-mesh solve has them, would take 20.8 ms, but a run's residuals have always
+// been FP64-accurate (those sweeps leave them off by up to 3e-14 of b).
 //
 // The assembly and factorisation of the whole batch (walk, contractions, factorisations) is captured as one CUDA
 // graph the second time a run has the same orders, coefficients and precision, and replayed
@@ -321,7 +322,7 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
         for (cudaStream_t t : b->streams) FEM3_CUDA(cudaStreamSynchronize(t));
         for (int i = 0; i < n && st == FEM3_OK; i++) {
             if (!active[i]) continue;
-            worst[i] = refine_worst(b->ms[i], nrhs, tol, &mode[i]);
+            worst[i] = refine_worst(b->ms[i], nrhs, tol, false, &mode[i]);
             it[i] = sweep;
             if (worst[i] <= tol || sweep >= max_iter || !(worst[i] < INFINITY)) {
                 active[i] = 0;

@@ -318,7 +318,7 @@ int axis_forms(Mesh *m, const double *u_d, const double *lam_d, double out[3]);
 int read_errors(Mesh *m, int32_t *h_err);
 int refine_start(const RefineVecs &v, int64_t n, int nrhs, cudaStream_t s);
 int refine_sweep(Mesh *m, const RefineVecs &v, int nrhs, RefineMode mode);
-double refine_worst(const Mesh *m, int nrhs, double tol, RefineMode *next);
+double refine_worst(const Mesh *m, int nrhs, double tol, bool late, RefineMode *next);
 int residual_worst(Mesh *m, const double *b, const double *u, int nrhs, double *worst);
 // A u in FP64 and A d of FP32 corrections d in double-float or (late) plain FP32 arithmetic
 int apply_multi(Mesh *m, const double *u_d, int nv, double *Au_d);

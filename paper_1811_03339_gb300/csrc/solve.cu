@@ -758,10 +758,10 @@ static double worst_norm(const Mesh *m, int nrhs) {
 }
 
 // largest relative residual of the sweep whose norms have arrived (infinity for NaN), and
-// how the next sweep forms its residual
-double refine_worst(const Mesh *m, int nrhs, double tol, RefineMode *next) {
+// how the next sweep forms its residual (late: in plain FP32 if it may)
+double refine_worst(const Mesh *m, int nrhs, double tol, bool late, RefineMode *next) {
     const double worst = worst_norm(m, nrhs);
-    *next = worst <= kLateFactor * tol ? kRefineLate
+    *next = late && worst <= kLateFactor * tol ? kRefineLate
                                        : (worst <= kUpdateBelow ? kRefineUpdate : kRefineFull);
     return worst;
 }
@@ -814,7 +814,7 @@ int solve_refined(Mesh *m, const double *b_d, int nrhs, double tol, int max_iter
     while (st == FEM3_OK) {
         if ((st = refine_sweep(m, v, nrhs, mode)) != FEM3_OK) break;
         FEM3_CUDA(cudaStreamSynchronize(s));
-        worst = refine_worst(m, nrhs, tol, &mode);
+        worst = refine_worst(m, nrhs, tol, true, &mode);
         it++;
         if (worst <= tol || it >= max_iter || !(worst < INFINITY)) break;
     }

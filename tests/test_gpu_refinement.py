@@ -1,0 +1,56 @@
+"""What the refinement (csrc/solve.cu, csrc/batch.cu) reports and accepts: residuals against
+b - A u formed from the FP64 form's matrix, tolerances that FP64 solutions cannot reach, and
+coefficients of any scale."""
+import numpy as np
+import pytest
+
+from test_gpu_contract_rows import _bar_mesh
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA device", allow_module_level=True)
+
+from paper_1811_03339_gb300 import fem3  # noqa: E402
+
+ALPHA, K = (1.3, 1.6, 1.8), (1.0, 2.0, 0.5)
+MIXED = ("tf32x3", "bf16x3", "fp32")
+
+
+def _dense(mesh, f, alpha=ALPHA, k=K):
+    """the FP64 form's matrix and load vectors [n_dof, nrhs]"""
+    m = fem3.Mesh(mesh.verts, mesh.tets)
+    A = m.assemble(alpha, k, "fp64", return_matrix=True)
+    b = m.load(f).reshape(m.n_dof, -1)
+    m.free()
+    return A, b
+
+
+def _residual(A, b, u):
+    r = b - A @ u.reshape(b.shape)
+    return float((r.norm(dim=0) / b.norm(dim=0)).max())
+
+
+def _source(mesh, nrhs, seed=1):
+    return torch.from_numpy(np.random.default_rng(seed).standard_normal((mesh.n_nodes, nrhs))).cuda()
+
+
+@pytest.mark.parametrize("precision", MIXED)
+def test_batch_residual_is_double_float(precision):
+    """The residual that a run reports is b - A u to what double-float products and the evaluation
+    here (FP64, a matrix that differs by 2^-48 of its terms) leave open: with |A| |u| near 10 |b|, as
+    on these meshes, below 1e-14 of b.  Updates in plain FP32 are off by 2^-24 of |A| |d| with d of
+    1e-6 of u, a few 1e-14."""
+    meshes = [_bar_mesh(c) for c in ((9, 8, 10), (14, 11, 9), (13, 13, 13))]
+    fs = [_source(m, 3, i) for i, m in enumerate(meshes)]
+    dense = [_dense(m, f) for m, f in zip(meshes, fs)]
+    b = fem3.Batch([(m.verts, m.tets) for m in meshes])
+    n = len(meshes)
+    for tol in (1e-6, 1e-7, 1e-8, 1e-9, 1e-10, 1e-12):
+        us = b.run(np.tile(ALPHA, (n, 1)), np.tile(K, (n, 1)), fs, precision, tol=tol)
+        for (A, rhs), u, res in zip(dense, us, b.resid):
+            true = _residual(A, rhs, u)
+            assert res <= tol
+            assert abs(res - true) <= 1e-14, (tol, res, true)
+    b.free()
