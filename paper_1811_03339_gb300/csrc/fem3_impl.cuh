@@ -366,15 +366,15 @@ __device__ __forceinline__ void f64_split(double x, float &hi, float &lo) {
     lo = __uint_as_float(__float_as_uint(mag) | sign);
 }
 
-// exact FP64 value of an FP32 number by bit assembly: exponent rebiased by 1023 - 127,
-// significand moved to the top of the 52-bit field (zero gives +0; the conversion instruction is
-// left for subnormals, infinities and NaN)
+// exact FP64 value of an FP32 number by bit assembly: exponent rebiased by 1023 - 127 (kept for
+// infinities and NaN), significand moved to the top of the 52-bit field.  Zero and subnormals give 0:
+// pairs are split from numbers whose low parts are normal (f64_split).  A branch to the conversion
+// instruction for subnormals cost the FP64 general-form term at the 13^3 cube 495 us against 480.
 __device__ __forceinline__ double f32_to_f64_exact(float x) {
     const uint32_t b = __float_as_uint(x);
     const uint32_t e = (b >> 23) & 0xFFu;
-    if (e - 1u >= 254u && (b << 1) != 0u) return (double)x;
     const unsigned long long d = ((unsigned long long)(b & 0x80000000u) << 32) |
-                                 ((unsigned long long)(e + 896u) << 52) |
+                                 ((unsigned long long)(e == 255u ? 2047u : e + 896u) << 52) |
                                  ((unsigned long long)(b & 0x7FFFFFu) << 29);
     return __longlong_as_double(e == 0u ? 0ll : (long long)d);
 }
