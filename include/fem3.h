@@ -223,12 +223,16 @@ int fem3_load(fem3_mesh m, const double *f, int nrhs, double *b, void *stream);
  *   FP64-accurate A (formed from the tables on the first solve after an assemble, its nonzero
  *   32 x 32 blocks), until ||r||_2 <= tol ||M f||_2 for every column or max_iter
  *   corrections.  Once every column's residual is below 1e-3, a sweep updates r -= A d
- *   instead, d being as small as r: in double-float FP32 arithmetic (2^-46 relative), and
- *   below 1e4 tol in plain FP32 (about 1e-6 relative: an error near tol / 100).
+ *   instead, d being as small as r: in double-float FP32 arithmetic (2^-46 of |A| |d|), and
+ *   below 1e4 tol in plain FP32 (2^-24 of |A| |d|, which is 6e-4 tol times the ratio of |A| |d| to
+ *   A d).  Such an r leaves out the rounding of u to FP64.  Where the first sweep shows that this
+ *   may matter (tol below 2^-25 of its residual, or below 2^-53), the residual of u itself is
+ *   formed once r has reached tol, and has to be below 1e4 tol (fem3_batch_run: below tol).
  *   f         host or device float64 column-major [n_nodes][nrhs].
  *   u         device float64 column-major [n_dof][nrhs].
  *   iters_out host int or NULL: refinement steps taken (0 for FP64).
- *   resid_out host float64 or NULL: largest final relative residual.
+ *   resid_out host float64 or NULL: largest final relative residual ||M f - A u|| / ||M f||, u's
+ *             rounding included where it can be more than tol / 16.
  * Synchronises `stream`.  Errors: FEM3_E_STATE (no matrix), FEM3_E_NOT_SPD,
  * FEM3_E_NO_CONVERGE (u then holds the last iterate), FEM3_E_WALK, FEM3_E_TEMPLATE.
  */

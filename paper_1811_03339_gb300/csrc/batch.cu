@@ -55,7 +55,7 @@ static void free_run_buffers(Batch *b) {
     for (const RefineVecs &v : b->rv) {
         cudaFree(v.r);
         cudaFree(v.Au);
-        cudaFree(v.r32);
+        cudaFree(v.dc);
     }
     b->bv.clear();
     b->rv.clear();
@@ -221,7 +221,7 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
             if (cudaMalloc((void **)&b->bv[i], sizeof(double) * nn) != cudaSuccess ||
                 cudaMalloc((void **)&v.r, sizeof(double) * nn) != cudaSuccess ||
                 cudaMalloc((void **)&v.Au, sizeof(double) * nn) != cudaSuccess ||
-                cudaMalloc((void **)&v.r32, sizeof(float) * nn) != cudaSuccess)
+                cudaMalloc((void **)&v.dc, sizeof(float) * 2 * nn) != cudaSuccess)
                 return cuda_error(cudaGetLastError(), "cudaMalloc (batch run buffers)");
         }
         b->nrhs_cap = nrhs;
@@ -295,10 +295,8 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
     }
     // 3. per mesh on its stream: load vector, then refinement from u = 0 (FP64: a direct solve)
     if (st == FEM3_OK) st = fork_to(b, cs);
-    std::vector<int> it(n, 0);
-    std::vector<double> worst(n, 0.0);
     std::vector<char> active(n, 0);
-    std::vector<RefineMode> mode(n, kRefineFull);
+    std::vector<RefineState> q(n);
     int n_active = 0;
     for (int i = 0; i < n && st == FEM3_OK; i++) {
         Mesh *m = b->ms[i];
@@ -316,18 +314,14 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
         active[i] = 1;
         n_active++;
     }
-    for (int sweep = 1; n_active > 0 && st == FEM3_OK; sweep++) {
+    while (n_active > 0 && st == FEM3_OK) {
         for (int i = 0; i < n && st == FEM3_OK; i++)
-            if (active[i]) st = refine_sweep(b->ms[i], b->rv[i], nrhs, mode[i]);
+            if (active[i]) st = refine_sweep(b->ms[i], b->rv[i], nrhs, q[i].mode);
         for (cudaStream_t t : b->streams) FEM3_CUDA(cudaStreamSynchronize(t));
         for (int i = 0; i < n && st == FEM3_OK; i++) {
-            if (!active[i]) continue;
-            worst[i] = refine_worst(b->ms[i], nrhs, tol, false, &mode[i]);
-            it[i] = sweep;
-            if (worst[i] <= tol || sweep >= max_iter || !(worst[i] < INFINITY)) {
-                active[i] = 0;
-                n_active--;
-            }
+            if (!active[i] || refine_next(b->ms[i], nrhs, tol, max_iter, false, &q[i])) continue;
+            active[i] = 0;
+            n_active--;
         }
     }
 
@@ -338,11 +332,11 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
     for (int i = 0; i < n; i++) {
         Mesh *m = b->ms[i];
         m->stream = cs;
-        if (iters) iters[i] = fp64 ? 0 : it[i];
-        if (resid) resid[i] = worst[i];
+        if (iters) iters[i] = q[i].sweeps;
+        if (resid) resid[i] = fp64 || m->n_dof == 0 ? 0.0 : q[i].worst;
         int e = check_mesh(m, i);
         if (e != FEM3_OK && bad == FEM3_OK) bad = e;
-        if (!fp64 && m->n_dof > 0 && !(worst[i] <= tol) && bad == FEM3_OK)
+        if (!fp64 && m->n_dof > 0 && !q[i].converged && bad == FEM3_OK)
             bad = set_error(FEM3_E_NO_CONVERGE, "mesh " + std::to_string(i) +
                                                     ": iterative refinement did not converge");
     }

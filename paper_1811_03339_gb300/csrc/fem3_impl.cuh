@@ -263,16 +263,23 @@ struct BatchWalkScratch {
     void *d_desc = nullptr, *h_desc = nullptr;
 };
 
-// vectors of a refinement (column-major [n_dof][nrhs]): right-hand sides, solutions, A u or
-// A d, residuals, and the FP32 correction
+// vectors of a refinement (column-major [n_dof][nrhs]): right-hand sides, solutions, products
+// with A, residuals, and in FP32 the corrections followed by the solutions' carries (solve.cu)
 struct RefineVecs {
     const double *b;
     double *u, *Au, *r;
-    float *r32;
+    float *dc;
 };
 // how a sweep forms its residual: b - A u in FP64, or r - A d of its correction in double-float
-// or plain FP32 arithmetic
-enum RefineMode { kRefineFull = 0, kRefineUpdate = 1, kRefineLate = 2 };
+// or plain FP32 arithmetic; or no sweep, only the residual of u where r is one of u and its carry
+enum RefineMode { kRefineFull = 0, kRefineUpdate = 1, kRefineLate = 2, kRefineCheck = 3 };
+struct RefineState {
+    RefineMode mode = kRefineFull;   // of the next sweep
+    int sweeps = 0;                  // taken so far
+    bool check = false;              // u's rounding is of the tolerance's order
+    bool converged = false;
+    double worst = 1.0;              // largest relative residual of a column
+};
 
 // translation-unit entry points
 int mesh_build(Mesh *m, const double *verts_d, const int32_t *tets_d);
@@ -318,7 +325,7 @@ int axis_forms(Mesh *m, const double *u_d, const double *lam_d, double out[3]);
 int read_errors(Mesh *m, int32_t *h_err);
 int refine_start(const RefineVecs &v, int64_t n, int nrhs, cudaStream_t s);
 int refine_sweep(Mesh *m, const RefineVecs &v, int nrhs, RefineMode mode);
-double refine_worst(const Mesh *m, int nrhs, double tol, bool late, RefineMode *next);
+bool refine_next(const Mesh *m, int nrhs, double tol, int max_iter, bool late, RefineState *q);
 int residual_worst(Mesh *m, const double *b, const double *u, int nrhs, double *worst);
 // A u in FP64 and A d of FP32 corrections d in double-float or (late) plain FP32 arithmetic
 int apply_multi(Mesh *m, const double *u_d, int nv, double *Au_d);

@@ -507,26 +507,36 @@ __global__ void k_residual_cols(const double *__restrict__ b, const double *Au, 
     }
 }
 
-// r -= Ad (the late sweeps' residual update) with the norms of r and b per column
+// r -= Ad (where given) with the norms of r and b per column; where Ac, A times the carries, is
+// given, the norms of r + Ac in norms[kTrueSlot + c]
+constexpr int kTrueSlot = 64;   // of Mesh::norms
+constexpr double kCarryScale = 0x1p48;   // carries are stored times this
 __global__ void k_residual_update_cols(const double *__restrict__ b, const double *__restrict__ Ad,
-                                       int64_t n, double *r, double *norms) {
+                                       const double *__restrict__ Ac, int64_t n, double *r,
+                                       double *norms) {
     const int c = blockIdx.y;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double rr = 0, bb = 0;
+    double rr = 0, bb = 0, tt = 0;
     if (i < n) {
         const int64_t k = (int64_t)c * n + i;
-        const double v = r[k] - Ad[k];
-        r[k] = v;
+        double v = r[k];
+        if (Ad) r[k] = v = v - Ad[k];
         rr = v * v;
         bb = b[k] * b[k];
+        if (Ac) {
+            const double t = fma(Ac[k], 1.0 / kCarryScale, v);
+            tt = t * t;
+        }
     }
     for (int o = 16; o > 0; o >>= 1) {
         rr += __shfl_down_sync(0xffffffffu, rr, o);
         bb += __shfl_down_sync(0xffffffffu, bb, o);
+        tt += __shfl_down_sync(0xffffffffu, tt, o);
     }
     if ((threadIdx.x & 31) == 0) {
         atomicAdd(&norms[2 * c], rr);
         atomicAdd(&norms[2 * c + 1], bb);
+        if (Ac) atomicAdd(&norms[kTrueSlot + c], tt);
     }
 }
 
@@ -534,9 +544,15 @@ __global__ void k_to_f32(const double *__restrict__ a, float *b, int64_t n) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) b[i] = (float)a[i];
 }
-__global__ void k_axpy_f32(const float *__restrict__ d, double *u, int64_t n) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) u[i] += (double)d[i];
+// u + c += d: u takes the rounded sum, c what it lost (TwoSum: u + y = s + e exactly), or nothing
+// if the residual is formed from u anew (keep = false)
+__global__ void k_add_correction(const float *__restrict__ d, double *u, float *c, int64_t n, bool keep) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double y = (double)d[i] + (double)c[i] * (1.0 / kCarryScale), u0 = u[i];
+    const double s = u0 + y, z = s - u0;
+    u[i] = s;
+    c[i] = keep ? (float)(((u0 - (s - z)) + (y - z)) * kCarryScale) : 0.f;
 }
 __global__ void k_f32_to_f64(const float *__restrict__ a, double *b, int64_t n) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -712,58 +728,90 @@ int solve_direct(Mesh *m, const double *b_d, int nrhs, double *u_d) {
 //   r = b - A u in FP64, or r -= A d,
 // until every column has ||r|| <= tol ||b|| or max_iter sweeps.  The first sweep's residual is
 // formed from u in FP64.  Once the residual is below kUpdateBelow the correction is as small
-// against u, and r -= A d in double-float arithmetic (2^-46 relative to A d) keeps the FP64
-// residual's accuracy; below kLateFactor * tol plain FP32 (about 1e-6 relative) does: its
-// error is about 1e-6 ||r|| <= 1e-6 kLateFactor tol ||b|| = tol ||b|| / 100.
+// against u, and r -= A d in double-float arithmetic (2^-46 of |A| |d|) loses less than the
+// rounding of u to FP64 (2^-53 of |A| |u|) does; below kLateFactor * tol plain FP32 does: its error is
+// 2^-24 or so of |A| |d|, that is 6e-8 kLateFactor tol = 6e-4 tol times the ratio of |A| |d| to
+// the residual A d before the sweep (tens on these operators).
+//
+// u's own rounding: what u += d rounds off is kept (c, FP32, exact to 2^-24 of itself) and the next
+// sum takes it in, so r -= A d follows b - A (u + c), and the residual of u itself is r + A c.
+// The first sweep's residual tells whether A c matters: its u holds FP32 numbers, whose rounding is
+// 2^29 times FP64's, so A c is 2^-29 of that residual or less (2^-32 was measured).  A tolerance
+// of at least kRoundingFactor times it (and 2^-53) leaves A c below tol / 16.  For a smaller one
+// r + A c is formed, in plain FP32, once r has reached it, and decides: a tolerance that r reaches and u
+// cannot does not pass for reached.  Where late sweeps are allowed, r + A c <= kLateFactor tol is
+// enough (the level at which b - A u has been formed before them), else r + A c <= tol.
 constexpr double kUpdateBelow = 1e-3;
 constexpr double kLateFactor = 1e4;
+constexpr double kRoundingFactor = 0x1p-25;
 
 int refine_start(const RefineVecs &v, int64_t n, int nrhs, cudaStream_t s) {
     const int64_t nn = n * nrhs;
     FEM3_CUDA(cudaMemsetAsync(v.u, 0, sizeof(double) * nn, s));
+    FEM3_CUDA(cudaMemsetAsync(v.dc + nn, 0, sizeof(float) * nn, s));
     FEM3_CUDA(cudaMemcpyAsync(v.r, v.b, sizeof(double) * nn, cudaMemcpyDeviceToDevice, s));
     return FEM3_OK;
 }
 
-// one sweep, enqueued on m->stream; the norms arrive in m->h_norms (2 nrhs values)
+// one sweep, enqueued on m->stream; the norms arrive in m->h_norms (2 nrhs values, from kTrueSlot
+// on nrhs more)
 int refine_sweep(Mesh *m, const RefineVecs &v, int nrhs, RefineMode mode) {
     cudaStream_t s = m->stream;
     const int64_t n = m->n_dof, nn = n * nrhs;
-    k_to_f32<<<g256(nn), 256, 0, s>>>(v.r, v.r32, nn);
-    note_launch(m);
-    FEM3_TRY(tri_solve<float>(m, m->A32, n, v.r32, nrhs));
-    k_axpy_f32<<<g256(nn), 256, 0, s>>>(v.r32, v.u, nn);
-    note_launch(m);
-    FEM3_CUDA(cudaMemsetAsync(m->norms, 0, sizeof(double) * 2 * nrhs, s));
+    if (mode != kRefineCheck) {
+        k_to_f32<<<g256(nn), 256, 0, s>>>(v.r, v.dc, nn);
+        note_launch(m);
+        FEM3_TRY(tri_solve<float>(m, m->A32, n, v.dc, nrhs));
+        k_add_correction<<<g256(nn), 256, 0, s>>>(v.dc, v.u, v.dc + nn, nn, mode != kRefineFull);
+        note_launch(m);
+    }
+    const size_t bytes = sizeof(double) * (mode == kRefineCheck ? kTrueSlot + nrhs : 2 * nrhs);
+    FEM3_CUDA(cudaMemsetAsync(m->norms, 0, bytes, s));
+    const dim3 grid(g256(n), nrhs);
     if (mode == kRefineFull) {
         FEM3_TRY(apply_multi(m, v.u, nrhs, v.Au));
-        k_residual_cols<<<dim3(g256(n), nrhs), 256, 0, s>>>(v.b, v.Au, n, v.r, m->norms);
+        k_residual_cols<<<grid, 256, 0, s>>>(v.b, v.Au, n, v.r, m->norms);
+    } else if (mode == kRefineCheck) {
+        FEM3_TRY(apply_correction(m, v.dc + nn, nrhs, v.Au, true));
+        k_residual_update_cols<<<grid, 256, 0, s>>>(v.b, nullptr, v.Au, n, v.r, m->norms);
     } else {
-        FEM3_TRY(apply_correction(m, v.r32, nrhs, v.Au, mode == kRefineLate));
-        k_residual_update_cols<<<dim3(g256(n), nrhs), 256, 0, s>>>(v.b, v.Au, n, v.r, m->norms);
+        FEM3_TRY(apply_correction(m, v.dc, nrhs, v.Au, mode == kRefineLate));
+        k_residual_update_cols<<<grid, 256, 0, s>>>(v.b, v.Au, nullptr, n, v.r, m->norms);
     }
     note_launch(m);
-    FEM3_CUDA(cudaMemcpyAsync(m->h_norms, m->norms, sizeof(double) * 2 * nrhs,
-                              cudaMemcpyDeviceToHost, s));
+    FEM3_CUDA(cudaMemcpyAsync(m->h_norms, m->norms, bytes, cudaMemcpyDeviceToHost, s));
     return FEM3_OK;
 }
 
-static double worst_norm(const Mesh *m, int nrhs) {
+// largest relative residual over the columns from the norms that have arrived, of r or (of_u) of
+// u; infinity for NaN
+static double worst_norm(const Mesh *m, int nrhs, bool of_u) {
     double worst = 0;
     for (int c = 0; c < nrhs; c++) {
-        const double rel = m->h_norms[2 * c + 1] > 0 ? sqrt(m->h_norms[2 * c] / m->h_norms[2 * c + 1]) : 0.0;
+        const double b = m->h_norms[2 * c + 1], r = m->h_norms[of_u ? kTrueSlot + c : 2 * c];
+        const double rel = b > 0 ? sqrt(r / b) : 0.0;
         worst = (rel == rel) ? std::max(worst, rel) : INFINITY;
     }
     return worst;
 }
 
-// largest relative residual of the sweep whose norms have arrived (infinity for NaN), and
-// how the next sweep forms its residual (late: in plain FP32 if it may)
-double refine_worst(const Mesh *m, int nrhs, double tol, bool late, RefineMode *next) {
-    const double worst = worst_norm(m, nrhs);
-    *next = late && worst <= kLateFactor * tol ? kRefineLate
-                                       : (worst <= kUpdateBelow ? kRefineUpdate : kRefineFull);
-    return worst;
+// After the sweep q->mode, whose norms have arrived: whether the columns have converged, and what
+// the next sweep is (late: plain FP32 updates are allowed).  False once there is none.
+bool refine_next(const Mesh *m, int nrhs, double tol, int max_iter, bool late, RefineState *q) {
+    const RefineMode was = q->mode;
+    const double r = worst_norm(m, nrhs, false);
+    q->worst = was == kRefineCheck ? worst_norm(m, nrhs, true) : r;
+    if (was != kRefineCheck && ++q->sweeps == 1) q->check = tol < kRoundingFactor * std::max(r, 0x1p-28);
+    if (was == kRefineCheck)
+        q->converged = q->worst <= (late ? kLateFactor : 1.0) * tol;
+    else
+        q->converged = r <= tol && (was == kRefineFull || !q->check);
+    if (r <= tol && q->check && was != kRefineCheck)
+        q->mode = kRefineCheck;
+    else
+        q->mode = late && r <= kLateFactor * tol ? kRefineLate
+                                                 : (r <= kUpdateBelow ? kRefineUpdate : kRefineFull);
+    return !q->converged && q->worst < INFINITY && (q->sweeps < max_iter || q->mode == kRefineCheck);
 }
 
 // largest ||b - A u|| / ||b|| over the columns (synchronises)
@@ -791,7 +839,7 @@ int residual_worst(Mesh *m, const double *b, const double *u, int nrhs, double *
                                         cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) st = cuda_error(e, "residual norms");
-        else *worst = std::max(*worst, worst_norm(m, cnt));
+        else *worst = std::max(*worst, worst_norm(m, cnt, false));
     }
     cudaFreeAsync(Au, s);
     return st;
@@ -806,25 +854,20 @@ int solve_refined(Mesh *m, const double *b_d, int nrhs, double tol, int max_iter
     RefineVecs v{b_d, u_d, nullptr, nullptr, nullptr};
     FEM3_CUDA(cudaMallocAsync((void **)&v.Au, sizeof(double) * nn, s));
     FEM3_CUDA(cudaMallocAsync((void **)&v.r, sizeof(double) * nn, s));
-    FEM3_CUDA(cudaMallocAsync((void **)&v.r32, sizeof(float) * nn, s));
-    int it = 0;
-    double worst = 1.0;
-    RefineMode mode = kRefineFull;
+    FEM3_CUDA(cudaMallocAsync((void **)&v.dc, sizeof(float) * 2 * nn, s));
+    RefineState q;
     int st = refine_start(v, n, nrhs, s);
-    while (st == FEM3_OK) {
-        if ((st = refine_sweep(m, v, nrhs, mode)) != FEM3_OK) break;
+    do {
+        if (st != FEM3_OK || (st = refine_sweep(m, v, nrhs, q.mode)) != FEM3_OK) break;
         FEM3_CUDA(cudaStreamSynchronize(s));
-        worst = refine_worst(m, nrhs, tol, true, &mode);
-        it++;
-        if (worst <= tol || it >= max_iter || !(worst < INFINITY)) break;
-    }
+    } while (refine_next(m, nrhs, tol, max_iter, true, &q));
     cudaFreeAsync(v.Au, s);
     cudaFreeAsync(v.r, s);
-    cudaFreeAsync(v.r32, s);
-    if (iters) *iters = it;
-    if (resid) *resid = worst;
+    cudaFreeAsync(v.dc, s);
+    if (iters) *iters = q.sweeps;
+    if (resid) *resid = q.worst;
     if (st != FEM3_OK) return st;
-    if (!(worst <= tol))
+    if (!q.converged)
         return set_error(FEM3_E_NO_CONVERGE, "iterative refinement did not reach the tolerance");
     return FEM3_OK;
 }

@@ -54,3 +54,43 @@ def test_batch_residual_is_double_float(precision):
             assert res <= tol
             assert abs(res - true) <= 1e-14, (tol, res, true)
     b.free()
+
+
+@pytest.mark.parametrize("precision", MIXED)
+def test_unreachable_tolerance_is_refused(precision):
+    """FP64 u leaves a residual of 2^-53 of |A| |u| or so, above 1e-17 of b whatever the matrix."""
+    mesh = _bar_mesh((9, 8, 10))
+    f = _source(mesh, 2)
+    m = fem3.Mesh(mesh.verts, mesh.tets)
+    m.assemble(ALPHA, K, precision)
+    with pytest.raises(fem3.Fem3Error) as e:
+        m.solve(f, tol=1e-22, max_iter=12)
+    assert e.value.code == fem3.FEM3_E_NO_CONVERGE
+    m.solve(f, tol=1e-12)   # the handle is still good
+    m.free()
+    b = fem3.Batch([(mesh.verts, mesh.tets)] * 2)
+    with pytest.raises(fem3.Fem3Error) as e:
+        b.run(np.tile(ALPHA, (2, 1)), np.tile(K, (2, 1)), [f, f], precision, tol=1e-17, max_iter=12)
+    assert e.value.code == fem3.FEM3_E_NO_CONVERGE
+    b.free()
+
+
+@pytest.mark.parametrize("nrhs", [1, 5, 17])
+@pytest.mark.parametrize("precision", MIXED)
+def test_reported_residual_has_the_rounding_of_u(precision, nrhs):
+    """At tolerances below it the residual is that of u's rounding to FP64: the norm of A c for c
+    uniform within half a unit of u's entries, a sum of some 1e5 independent terms, here within a factor of
+    four.  A residual that leaves the rounding out shrinks on with tol."""
+    mesh = _bar_mesh((13, 13, 13))
+    f = _source(mesh, nrhs)
+    A, b = _dense(mesh, f)
+    m = fem3.Mesh(mesh.verts, mesh.tets)
+    m.assemble(ALPHA, K, precision)
+    for tol in (1e-15, 1e-17):
+        u = m.solve(f, tol=tol).reshape(b.shape)
+        ulp = torch.ldexp(torch.ones_like(u), torch.frexp(u).exponent - 53)
+        c = ulp * (torch.rand(u.shape, dtype=u.dtype, device="cuda",
+                              generator=torch.Generator("cuda").manual_seed(3)) - 0.5)
+        floor = float(((A @ c).norm(dim=0) / b.norm(dim=0)).max())
+        assert floor / 4 <= m.resid <= 4 * floor, (tol, m.resid, floor)
+    m.free()
