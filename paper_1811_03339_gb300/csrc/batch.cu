@@ -21,6 +21,7 @@
 
 #include <algorithm>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "fem3_impl.cuh"
@@ -45,6 +46,8 @@ struct Batch {
     cudaStream_t cap = nullptr;
     cudaEvent_t cap_in = nullptr;
     std::vector<double> key_ak;          // alpha, K
+    // per mesh, what the captured work leaves: whether it builds the operator, and its scale
+    std::vector<std::pair<bool, double>> key_op;
     int key_prec = -1;
     int runs = 0;                        // eager runs so far
     int graph_launches = 0;              // replays so far
@@ -257,7 +260,10 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
         FEM3_CUDA(cudaGraphLaunch(b->exec, cs));
         b->graph_launches++;
         // the replay has built (FP64: copied) the operators that the captured run did
-        for (Mesh *m : b->ms) m->op_ready = m->n_dof > 0 && (fp64 || op_beside_factor(m));
+        for (int i = 0; i < n; i++) {
+            b->ms[i]->op_ready = b->key_op[i].first;
+            b->ms[i]->op.scale = b->key_op[i].second;
+        }
     } else if (b->runs >= 1) {
         // capture the assembly + factorisation; on any failure discard it and run eagerly
         if (b->exec) {
@@ -277,6 +283,8 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
                 captured = true;
                 b->key_prec = precision;
                 b->key_ak = ak;
+                b->key_op.clear();
+                for (const Mesh *m : b->ms) b->key_op.emplace_back(m->op_ready, m->op.scale);
             }
             if (g) cudaGraphDestroy(g);
         }

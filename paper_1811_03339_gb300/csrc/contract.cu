@@ -2,6 +2,8 @@
 // (Section 2.1 element sum, Section 2.3 template: only dofs of a bin's template set can
 // meet the bin's Gauss points, so each bin contributes to a D_b x D_b block), from the
 // nonzeros of the bin's table blocks (about a fifth of their entries: k_contract_rows).
+#include <math.h>
+
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -453,8 +455,18 @@ int contract_work(Mesh *m, double *flops_out, int64_t *nnz_out) {
     return FEM3_OK;
 }
 
-// the work items of this part's bins of every axis (the lists are in bin order)
-static RowsAxes riesz_axes(Mesh *m) {
+// Power of two next to the largest |s_i K_i|.  s K w is formed before the products, so as a pair (24 bits
+// below 2^-74, nothing below 2^-126) it has to be of the weights' order for the coefficients'
+// scale not to cost digits; the factor stays with the blocks, whose entries are split likewise.
+static int coef_exponent(const Mesh *m) {
+    int e;
+    frexp(std::max({fabs(m->sK[0]), fabs(m->sK[1]), fabs(m->sK[2])}), &e);
+    return std::min(std::max(e, -126), 126);
+}
+
+// the work items of this part's bins of every axis (the lists are in bin order), the
+// coefficients times 2^-e
+static RowsAxes riesz_axes(Mesh *m, int e) {
     RowsAxes P{};
     for (int axis = 0; axis < 3; axis++) {
         AxisBins &B = m->bins[axis];
@@ -467,7 +479,7 @@ static RowsAxes riesz_axes(Mesh *m) {
         };
         const int w0 = lb(b0), nw = std::max(0, lb(b1) - w0);
         P.a[axis] = RowsAxis{m->tabL[axis], m->tabR[axis], B.work + w0, B.gp_off, B.dof_off,
-                             B.dof_idx, B.tab_ld, B.tab_off, B.w_slot, nullptr, m->sK[axis], nw};
+                             B.dof_idx, B.tab_ld, B.tab_off, B.w_slot, nullptr, ldexp(m->sK[axis], -e), nw};
     }
     return P;
 }
@@ -484,15 +496,17 @@ int contract(Mesh *m, int precision) {
             flops += 2.0 * D * D * G;
         }
     }
-    const RowsAxes P = riesz_axes(m);
+    const RowsAxes P = riesz_axes(m, 0);
     m->contract_flops = flops;
     return precision == FEM3_FP64 ? launch_rows<double, kLower>(m, P, m->A64)
                                   : launch_rows<float, kLower>(m, P, m->A32);
 }
 
-// the lower blocks of the operator, added in FP64 from double-float row sums
-int contract_blocks(Mesh *m, const OpBlocks &O) {
-    return launch_rows<float2, kBlocks>(m, riesz_axes(m), O.low, O.map);
+// the lower blocks of the operator over O.scale, added in FP64 from double-float row sums
+int contract_blocks(Mesh *m, OpBlocks &O) {
+    const int e = coef_exponent(m);
+    O.scale = ldexp(1.0, e);
+    return launch_rows<float2, kBlocks>(m, riesz_axes(m, e), O.low, O.map);
 }
 
 }  // namespace fem3

@@ -104,6 +104,7 @@ struct OpBlocks {
     int32_t *col = nullptr, *src = nullptr, *row_of = nullptr;   // [n_full]
     double *low = nullptr;        // [n_low][32][32] lower blocks as the contraction adds them
     double *full = nullptr;       // [n_full][32][32] column-major
+    double scale = 1.0;           // A = scale * blocks, a power of two
     bool counted = false;         // the block counts are on their way to h_norms (op_count)
     cudaEvent_t ev = nullptr;     // ... and have arrived
 };
@@ -337,9 +338,8 @@ int op_count(Mesh *m);     // enqueues the search for the operator's blocks (onc
 // the block pattern and its storage, of the lower blocks too if `low` (waits for the counts)
 int op_prepare(Mesh *m, bool low);
 int op_build(Mesh *m);     // the operator of the current tables
-bool op_beside_factor(const Mesh *m);   // factor() builds it on a side stream
 int op_from_dense(Mesh *m, const double *A);    // ... of the FP64 form, from its matrix
-int contract_blocks(Mesh *m, const OpBlocks &O);   // the element sum into the lower blocks
+int contract_blocks(Mesh *m, OpBlocks &O);   // the element sum into the lower blocks
 
 // ---------------------------------------------------------------------------------
 // FP64 values in FP32 arithmetic.  GB300 runs FP64 arithmetic and f64 <-> f32

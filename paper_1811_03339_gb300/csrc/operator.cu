@@ -316,16 +316,16 @@ __global__ void __launch_bounds__(kOpThreads, NR > 8 ? 2 : 3)
     }
 }
 
-// Au[v][row] = the parts' sum, added in order (grid: block rows; thread: vector, row)
+// Au[v][row] = scale times the parts' sum, added in order (grid: block rows; thread: vector, row)
 __global__ void __launch_bounds__(256) k_op_sum(const double *__restrict__ part, int nb, int S,
-                                                int nr, int64_t n, int nv, double *Au) {
+                                                int nr, int64_t n, int nv, double scale, double *Au) {
     const int64_t i = blockIdx.x;
     for (int e = threadIdx.x; e < nv * kOB; e += 256) {
         const int64_t row = i * kOB + (e & 31);
         if (row >= n) continue;
         double y = part[i * (nr * kOB) + e];
         for (int s = 1; s < S; s++) y += part[((int64_t)s * nb + i) * (nr * kOB) + e];
-        Au[(int64_t)(e >> 5) * n + row] = y;
+        Au[(int64_t)(e >> 5) * n + row] = y * scale;
     }
 }
 
@@ -352,7 +352,7 @@ int apply_group(Mesh *m, const typename OpCfg<NR, MODE>::X *u, int nv, double *A
     k_op_apply<NR, MODE><<<dim3(O.nb, S), kOpThreads, sh, s>>>(O.row_off, O.col, O.full, x, part, O.nb);
     kc_end(m, KC_APPLY);
     note_launch(m);
-    k_op_sum<<<O.nb, 256, 0, s>>>(part, O.nb, S, NR, m->n_dof, nv, Au);
+    k_op_sum<<<O.nb, 256, 0, s>>>(part, O.nb, S, NR, m->n_dof, nv, O.scale, Au);
     note_launch(m);
     FEM3_CUDA(cudaGetLastError());
     return FEM3_OK;
@@ -516,6 +516,7 @@ int op_from_dense(Mesh *m, const double *A) {
         note_launch(m);
     }
     FEM3_CUDA(cudaGetLastError());
+    O.scale = 1.0;
     m->op_ready = true;
     return FEM3_OK;
 }

@@ -636,7 +636,7 @@ bool factor_on_tc(const Mesh *m) {
 // before, 658 -> 646 us at n = 27, 1,012 -> 993 at 343, 2,559 -> 2,308 at 1,728.  Not beside the blocked factorisation: its trailing updates take an SM's whole shared memory
 // each, so the critical chain waited for the operator's CTAs to drain (24^3 step 30.6 ms
 // with, 30.3 ms without).  A profiled mesh times its launches one at a time.
-bool op_beside_factor(const Mesh *m) {
+static bool op_beside_factor(const Mesh *m) {
     return !m->profile && !factor_on_tc(m);
 }
 

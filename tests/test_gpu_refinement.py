@@ -94,3 +94,42 @@ def test_reported_residual_has_the_rounding_of_u(precision, nrhs):
         floor = float(((A @ c).norm(dim=0) / b.norm(dim=0)).max())
         assert floor / 4 <= m.resid <= 4 * floor, (tol, m.resid, floor)
     m.free()
+
+
+@pytest.mark.parametrize("precision", MIXED)
+def test_coefficients_of_any_scale(precision):
+    """K times a power of two divides the solution by it: to the refinement's tolerance, for
+    scales at which s K w is no FP32 pair (below 2^-74 such a pair has 24 bits)."""
+    mesh = _bar_mesh((6, 8, 7), h=(0.2, 0.1, 0.15))
+    f = _source(mesh, 3)
+    A, b = _dense(mesh, f)
+    ref = torch.linalg.solve(A, b)
+    for e in (-90, -75, -60, 0, 60):
+        m = fem3.Mesh(mesh.verts, mesh.tets)
+        m.assemble(ALPHA, [k * 2.0 ** e for k in K], precision)
+        u = m.solve(f, tol=1e-12).reshape(ref.shape) * 2.0 ** e
+        m.free()
+        assert float((u - ref).norm() / ref.norm()) <= 1e-10, e
+
+
+@pytest.mark.parametrize("precision", ["tf32x3", "fp64"])
+def test_batch_replay_after_another_scale(precision):
+    """A replayed graph writes the operator of the run it was captured from, whatever operator the
+    mesh's handle was used with since."""
+    import ctypes as C
+    mesh = _bar_mesh((6, 8, 7), h=(0.2, 0.1, 0.15))
+    f = _source(mesh, 2)
+    A, b = _dense(mesh, f)
+    ref = torch.linalg.solve(A, b)
+    batch = fem3.Batch([(mesh.verts, mesh.tets)])
+    h = C.c_void_p()
+    fem3._check(fem3._lib.fem3_batch_mesh(batch.h, 0, C.byref(h)))
+    fc, u1 = f.T.contiguous(), torch.empty((2, batch.n_dof[0]), dtype=torch.float64, device="cuda")
+    for _ in range(4):   # eager, captured, replayed twice
+        u = batch.run([ALPHA], [K], [f], precision)[0]
+        assert float((u - ref).norm() / ref.norm()) <= 1e-8
+        fem3.solve(h, fc, 2, u1)   # the run's factor and operator
+        assert float((u1.T - ref).norm() / ref.norm()) <= 1e-8
+        fem3.assemble(h, (1.7, 1.2, 1.5), [k * 2.0 ** 40 for k in K], "tf32x3")
+        fem3.solve(h, fc, 2, u1)
+    batch.free()
