@@ -509,15 +509,9 @@ __global__ void __launch_bounds__(256) k_join_dinv(const double *__restrict__ A,
 int chol_f64(double *A, int64_t n, double *dinv, const int *first_col, int *flags, int32_t *err,
              cudaStream_t s, int *launches) {
     if (n <= 0) return FEM3_OK;
-    static int sms = 0;
-    if (sms == 0) {
-        int dev = 0, v = 0;
-        FEM3_CUDA(cudaGetDevice(&dev));
-        FEM3_CUDA(cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev));
-        FEM3_CUDA(cudaFuncSetAttribute(k_chol_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kSmemBytes));
-        sms = v;
-    }
+    int sms = 0;
+    FEM3_CUDA(device_sms(&sms));
+    FEM3_CUDA(device_smem((const void *)k_chol_f64, kSmemBytes));
     const int nblk = (int)((n + kT - 1) / kT);
     const int ntask = nblk * (nblk + 1) / 2;
     FEM3_CUDA(cudaMemsetAsync(flags, 0, sizeof(int) * chol_f64_flags(n), s));

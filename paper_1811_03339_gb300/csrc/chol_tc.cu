@@ -597,24 +597,12 @@ int chol_tc(Mesh *m, SideCtx *cx, float *A, int64_t n) {
     CUtensorMap maps[2][2];
     for (int b = 0; b < 2; b++)
         for (int h = 0; h < 2; h++) FEM3_TRY(make_w_map(&maps[b][h], W[b][h], wrows));
-    static bool attr = false;
-    if (!attr) {
-        FEM3_CUDA(cudaFuncSetAttribute(k_cholp_diag, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(sizeof(float) * kDiagSmemFloats)));
-        FEM3_CUDA(cudaFuncSetAttribute(k_cholp_panel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)panel_smem<32>()));
-        FEM3_CUDA(cudaFuncSetAttribute(k_cholp_panel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)panel_smem<64>()));
-        FEM3_CUDA(cudaFuncSetAttribute(k_cholp_trail, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kTrailSmem));
-        attr = true;
-    }
-    static int sms = 0;
-    if (sms == 0) {
-        int dev = 0;
-        FEM3_CUDA(cudaGetDevice(&dev));
-        FEM3_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    }
+    FEM3_CUDA(device_smem((const void *)k_cholp_diag, sizeof(float) * kDiagSmemFloats));
+    FEM3_CUDA(device_smem((const void *)k_cholp_panel<32>, panel_smem<32>()));
+    FEM3_CUDA(device_smem((const void *)k_cholp_panel<64>, panel_smem<64>()));
+    FEM3_CUDA(device_smem((const void *)k_cholp_trail, kTrailSmem));
+    int sms = 0;
+    FEM3_CUDA(device_sms(&sms));
     const int npan = (int)((n + kP - 1) / kP);
     while ((int)cx->ev.size() < 4 * npan) {
         cudaEvent_t e;

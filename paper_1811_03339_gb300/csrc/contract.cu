@@ -385,16 +385,9 @@ static int launch_rows(Mesh *m, const RowsAxes &P, typename Arith<TA>::Out *A,
                        sizeof(int) * (2 * (size_t)max_gp + 1 + max_dof) +
                        sizeof(uint16_t) * cap + 15) &
                       ~size_t(15);
-    static bool attr = false;
-    if (!attr) {
-        FEM3_CUDA(cudaFuncSetAttribute(k_contract_rows<TA, OUT, true>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kRowsSmemMax));
-        FEM3_CUDA(cudaFuncSetAttribute(k_contract_rows<TA, OUT, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kRowsSmemMax));
-        attr = true;
-    }
+    FEM3_CUDA(device_smem(half ? (const void *)k_contract_rows<TA, OUT, true>
+                               : (const void *)k_contract_rows<TA, OUT, false>,
+                          kRowsSmemMax));
     kc_begin(m, KC_CONTRACT);
     if (half)
         k_contract_rows<TA, OUT, true><<<(unsigned)nw, kRowsThreads, sh, m->stream>>>(

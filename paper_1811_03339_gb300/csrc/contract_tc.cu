@@ -335,22 +335,10 @@ static int tc_prepare(Mesh *m) {
                                           cudaMemcpyHostToDevice, s));
         }
     }
-    static bool attr = false;
-    if (!attr) {
-        FEM3_CUDA(cudaFuncSetAttribute(k_contract_tc<false, 256>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)TcCfg<256>::kSmemBytes));
-        FEM3_CUDA(cudaFuncSetAttribute(k_contract_tc<true, 256>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)TcCfg<256>::kSmemBytes));
-        FEM3_CUDA(cudaFuncSetAttribute(k_contract_tc<false, 128>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)TcCfg<128>::kSmemBytes));
-        FEM3_CUDA(cudaFuncSetAttribute(k_contract_tc<true, 128>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)TcCfg<128>::kSmemBytes));
-        attr = true;
-    }
+    FEM3_CUDA(device_smem((const void *)k_contract_tc<false, 256>, TcCfg<256>::kSmemBytes));
+    FEM3_CUDA(device_smem((const void *)k_contract_tc<true, 256>, TcCfg<256>::kSmemBytes));
+    FEM3_CUDA(device_smem((const void *)k_contract_tc<false, 128>, TcCfg<128>::kSmemBytes));
+    FEM3_CUDA(device_smem((const void *)k_contract_tc<true, 128>, TcCfg<128>::kSmemBytes));
     m->tc_ready = true;
     return FEM3_OK;
 }

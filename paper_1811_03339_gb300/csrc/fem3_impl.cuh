@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/fem3.h"
+#include "per_device.h"
 
 namespace fem3 {
 

@@ -376,21 +376,12 @@ int chol_tiles(float *A, int64_t n, cudaStream_t s, Mesh *m) {
     if (n <= 0) return FEM3_OK;
     const int nblk = (int)((n + NB - 1) / NB);
     const int ntask = nblk * (nblk + 1) / 2;
-    static int sms = 0;
-    if (sms == 0) {
-        int dev = 0;
-        FEM3_CUDA(cudaGetDevice(&dev));
-        FEM3_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    }
+    int sms = 0;
+    FEM3_CUDA(device_sms(&sms));
     FEM3_CUDA(cudaMemsetAsync(m->chol_flags, 0, sizeof(int32_t) * (2 * ntask + 2), s));
     // one CTA per SM: the chain CTA gets an SM of its own
     const int grid = std::min(ntask + 1, std::max(sms, 2));
-    static bool attr = false;
-    if (!attr) {
-        FEM3_CUDA(cudaFuncSetAttribute(k_chol_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(kCholTilesSmem * sizeof(float))));
-        attr = true;
-    }
+    FEM3_CUDA(device_smem((const void *)k_chol_tiles, kCholTilesSmem * sizeof(float)));
     kc_begin(m, KC_FACTOR);
     k_chol_tiles<<<grid, 512, kCholTilesSmem * sizeof(float), s>>>(
         A, n, nblk, reinterpret_cast<float *>(m->dinv), m->chol_flags, m->err);
@@ -695,12 +686,7 @@ int factor(Mesh *m) {
 
 int axis_forms(Mesh *m, const double *u_d, const double *lam_d, double out[3]) {
     cudaStream_t s = m->stream;
-    static bool attr = false;
-    if (!attr) {
-        FEM3_CUDA(cudaFuncSetAttribute(k_axis_form, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(sizeof(double2) * kMaxBinItems)));
-        attr = true;
-    }
+    FEM3_CUDA(device_smem((const void *)k_axis_form, sizeof(double2) * kMaxBinItems));
     FEM3_CUDA(cudaMemsetAsync(m->norms, 0, sizeof(double) * 3, s));
     for (int axis = 0; axis < 3; axis++) {
         AxisBins &B = m->bins[axis];

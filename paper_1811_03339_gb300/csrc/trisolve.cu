@@ -409,12 +409,7 @@ template <class TF, int NR, bool TRI>
 int launch_cols(const TF *M, int64_t ldm, int rows, int64_t cols, const TF *x, int64_t n, int nrhs,
                 TF *out, cudaStream_t s) {
     constexpr size_t sh = ColCfg<TF, NR>::kSmem;
-    static bool attr = false;
-    if (sh > 48 * 1024 && !attr) {
-        FEM3_CUDA(cudaFuncSetAttribute(k_tri_cols<TF, NR, TRI>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
-        attr = true;
-    }
+    if (sh > 48 * 1024) FEM3_CUDA(device_smem((const void *)k_tri_cols<TF, NR, TRI>, sh));
     return launch_chained(false, k_tri_cols<TF, NR, TRI>, (cols + 31) / 32, kColThreads, sh, s, M, ldm,
                           rows, cols, x, n, nrhs, out);
 }
