@@ -205,6 +205,8 @@ int fem3_batch_run(fem3_batch hb, const double *alpha, const double *K, int prec
         m->precision = precision;
         m->factored = false;
         m->op_ready = false;
+        m->integer_order = false;   // of an earlier assembly through the mesh's handle
+        m->nonsym = false;
     }
     // the operators' block patterns and storage (the first run's; one wait for all of them)
     for (Mesh *m : b->ms)

@@ -1,5 +1,7 @@
 """Batched assembly and solve (fem3_batch_*): every mesh of a batch gives the result of
 the single-mesh path, which is itself pinned to the oracle."""
+import ctypes as C
+
 import numpy as np
 import pytest
 
@@ -100,4 +102,40 @@ def test_batch_assembly_replays_as_one_graph(precision):
             u = us[i].cpu().numpy()
             assert np.linalg.norm(u - ref2[i]) <= tol * np.linalg.norm(ref2[i]), (rep, i)
     assert b.graph_launches() == 5
+    b.free()
+
+
+def _handle(b, i):
+    h = C.c_void_p()
+    fem3._check(fem3._lib.fem3_batch_mesh(b.h, i, C.byref(h)))
+    return h
+
+
+@pytest.mark.parametrize("precision", ["fp64", "tf32x3"])
+def test_run_after_other_assemblies_of_a_mesh(precision):
+    """A batch's run is one of the fractional operator whatever its meshes' handles last held: the
+    integer order (its FP64 factorisation follows a profile) or the divergence form."""
+    meshes = [inputs.cube_mesh(n, 0.1, n) for n in (9, 10)]
+    alpha, K = np.tile((1.3, 1.6, 1.8), (2, 1)), np.ones((2, 3))
+    fs = [np.random.default_rng(i).standard_normal((m.n_nodes, 2)) for i, m in enumerate(meshes)]
+    ref = []
+    for i, m in enumerate(meshes):
+        one = fem3.Mesh(m.verts, m.tets)
+        one.assemble(alpha[i], K[i], "fp64")
+        ref.append(one.solve(fs[i]))
+        n_gp = one.n_gp
+        one.free()
+    b = fem3.Batch([(m.verts, m.tets) for m in meshes])
+    p = np.ones((3, n_gp))
+    for _ in range(3):   # eager, captured, replayed
+        fem3.assemble_integer(_handle(b, 0), K[0])
+        fem3.assemble_divergence(_handle(b, 1), (0.6, 0.7, 0.8), p, p, "fp64")
+        us = b.run(alpha, K, fs, precision)
+        for u, r in zip(us, ref):
+            assert float((u - r).norm() / r.norm()) <= 1e-8
+        # and the handle then solves with the run's operator
+        u = torch.empty((2, b.n_dof[1]), dtype=torch.float64, device="cuda")
+        f = torch.from_numpy(np.ascontiguousarray(fs[1].T)).cuda()
+        fem3.solve(_handle(b, 1), f, 2, u)
+        assert float((u.T - ref[1]).norm() / ref[1].norm()) <= 1e-8
     b.free()
