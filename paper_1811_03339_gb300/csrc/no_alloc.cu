@@ -29,8 +29,9 @@ namespace {
 constexpr int kNaMaxN = 512;   // largest system this entry point accepts
 constexpr int NBS = 64;
 
-// factor [kNaMaxN^2] | diagonal-block inverses [8][64 * 64] | flags of the factorisation, then
-// of the substitutions (2 kNaBlocks, a ticket, an abort word) | ERR_COUNT error words
+// factor [kNaMaxN^2] | diagonal-block inverses [8][64 * 64] | y, then z | flags of the
+// factorisation, then of the substitutions (2 kNaBlocks, a ticket, an abort word) | ERR_COUNT error
+// words | exponents of the rows' scales
 constexpr int kNaBlocks = kNaMaxN / NBS;
 constexpr size_t kNaFactor = (size_t)kNaMaxN * kNaMaxN;
 constexpr size_t kNaInv = (size_t)kNaBlocks * NBS * NBS;
@@ -38,7 +39,7 @@ constexpr int kNaCholTiles = kNaMaxN / kChol64Tile;
 constexpr size_t kNaCholFlags = (size_t)kNaCholTiles * (kNaCholTiles + 1) + 2;
 constexpr size_t kNaSolveFlags = 2 * kNaBlocks + 2;
 constexpr size_t kNaElems =
-    kNaFactor + kNaInv + (kNaCholFlags + kNaSolveFlags + ERR_COUNT + 1) / 2;
+    kNaFactor + kNaInv + kNaMaxN + (kNaCholFlags + kNaSolveFlags + ERR_COUNT + kNaMaxN + 1) / 2;
 static __device__ __align__(256) double g_na_scratch[kNaElems];
 
 #include "chol_smem.cuh"
@@ -46,11 +47,24 @@ static __device__ __align__(256) double g_na_scratch[kNaElems];
 std::mutex g_na_mutex;
 void *g_na_ptr[256];   // per device: device address of g_na_scratch (host-side table)
 
-// F = the lower triangle of A (row-major n x n); flags and error words cleared
+// e with d 2^(2 e) in [1, 4) for a positive finite d, else 0
+__device__ __forceinline__ int scale_exponent(double d) {
+    if (!(d > 0.0) || isinf(d)) return 0;
+    const int x = ilogb(d);
+    return -((x - (x & 1)) / 2);
+}
+
+// F = S A S (the lower triangle, row-major n x n), S = diag(2^e) so that F's diagonal lies in [1, 4):
+// an exact step, F's factor is A's with its rows scaled alike, but the factorisation's
+// reciprocals of pivots stay finite where a pivot of A is subnormal.  Flags and error words cleared.
 __global__ void __launch_bounds__(256) k_na_copy(const double *__restrict__ A, int n, double *F,
-                                                 int *flags, int n_flags) {
+                                                 int *scale, int *flags, int n_flags) {
     const int i = blockIdx.x;
-    for (int c = threadIdx.x; c <= i; c += blockDim.x) F[(int64_t)i * n + c] = A[(int64_t)i * n + c];
+    const int ei = scale_exponent(A[(int64_t)i * n + i]);
+    for (int c = threadIdx.x; c <= i; c += blockDim.x)
+        F[(int64_t)i * n + c] =
+            scalbn(A[(int64_t)i * n + c], ei + scale_exponent(A[(int64_t)c * n + c]));
+    if (threadIdx.x == 0) scale[i] = ei;
     if (i == 0)
         for (int q = threadIdx.x; q < n_flags; q += blockDim.x) flags[q] = 0;
 }
@@ -63,8 +77,8 @@ __device__ __forceinline__ double dot16(const double m[16], const double *v, int
     return s;
 }
 
-// Both substitutions in one launch: L y = b, then L^T x = y, in blocks of 64 rows.  A CTA takes
-// roles from a ticket: role s < nb is the forward step of block s, role nb + s the backward
+// Both substitutions in one launch: L y = S b, then L^T z = y (z in y's place) and x = S z, in
+// blocks of 64 rows.  A CTA takes roles from a ticket: role s < nb is the forward step of block s, role nb + s the backward
 // step of block nb - 1 - s.  A step reads the tiles of its block row (column) into registers
 // one ahead, adds each solved block as its flag appears, multiplies by the diagonal inverse
 // and publishes the block.  A role waits only for earlier tickets, so the launch needs no
@@ -72,7 +86,8 @@ __device__ __forceinline__ double dot16(const double m[16], const double *v, int
 // 256 threads, thread (row r = t & 63, quarter q = t >> 6 of the columns).
 __global__ void __launch_bounds__(256) k_na_solve(const double *__restrict__ F,
                                                   const double *__restrict__ dinv, int n, int nb,
-                                                  const double *__restrict__ b, double *y,
+                                                  const double *__restrict__ b,
+                                                  const int *__restrict__ scale, double *y,
                                                   double *x, int *flags, int *err) {
     __shared__ double v[NBS], red[4][NBS];
     __shared__ int s_role, s_ok;
@@ -115,7 +130,7 @@ __global__ void __launch_bounds__(256) k_na_solve(const double *__restrict__ F,
             }
             __syncthreads();
             if (!s_ok) return;
-            if (t < NBS) v[t] = jd * NBS + t < n ? __ldcg((bw ? x : y) + jd * NBS + t) : 0.0;
+            if (t < NBS) v[t] = jd * NBS + t < n ? __ldcg(y + jd * NBS + t) : 0.0;
             if (d + 1 < nd) tile(d + 1, mn);
             __syncthreads();
             acc += dot16(mt, v, q);
@@ -147,15 +162,19 @@ __global__ void __launch_bounds__(256) k_na_solve(const double *__restrict__ F,
         __syncthreads();
         if (!s_ok) return;
         if (t < NBS) {
-            const double rhs = blk * NBS + t < n ? (bw ? __ldcg(y + blk * NBS + t) : b[blk * NBS + t])
-                                                 : 0.0;
+            const int i = blk * NBS + t;
+            const double rhs = i < n ? (bw ? __ldcg(y + i) : scalbn(b[i], scale[i])) : 0.0;
             v[t] = rhs - ((red[0][t] + red[1][t]) + (red[2][t] + red[3][t]));
         }
         __syncthreads();
         red[q][r] = dot16(mt, v, q);
         __syncthreads();
-        if (t < NBS && blk * NBS + t < n)
-            (bw ? x : y)[blk * NBS + t] = (red[0][t] + red[1][t]) + (red[2][t] + red[3][t]);
+        if (t < NBS && blk * NBS + t < n) {
+            const int i = blk * NBS + t;
+            const double z = (red[0][t] + red[1][t]) + (red[2][t] + red[3][t]);
+            y[i] = z;   // (only this step reads this block of y)
+            if (bw) x[i] = scalbn(z, scale[i]);
+        }
         __syncthreads();   // the block's stores are issued before the (cumulative) release
         if (t == 0) st_release_gpu(&done[role], 1);
     }
@@ -214,15 +233,16 @@ extern "C" int fem3_spd_solve_static(const double *A, int64_t n, const double *b
     FEM3_TRY(na_scratch(&scratch));
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const int nn = (int)n, nb = (nn + NBS - 1) / NBS;
-    double *F = scratch, *dinv = F + kNaFactor;
-    int *chol_flags = reinterpret_cast<int *>(dinv + kNaInv);
+    double *F = scratch, *dinv = F + kNaFactor, *y = dinv + kNaInv;
+    int *chol_flags = reinterpret_cast<int *>(y + kNaMaxN);
     int *flags = chol_flags + kNaCholFlags;
     int *err = flags + kNaSolveFlags;   // cleared with the substitutions' flags
+    int *scale = err + ERR_COUNT;
     int launches = 0;
-    k_na_copy<<<(unsigned)nn, 256, 0, s>>>(A, nn, F, flags, (int)(kNaSolveFlags + ERR_COUNT));
+    k_na_copy<<<(unsigned)nn, 256, 0, s>>>(A, nn, F, scale, flags,
+                                                 (int)(kNaSolveFlags + ERR_COUNT));
     FEM3_TRY(chol_f64(F, n, dinv, nullptr, chol_flags, err, s, &launches));
-    // y shares x: a backward step reads its block of y before it writes that block of x
-    k_na_solve<<<(unsigned)nb, 256, 0, s>>>(F, dinv, nn, nb, b, x, x, flags, err);
+    k_na_solve<<<(unsigned)nb, 256, 0, s>>>(F, dinv, nn, nb, b, scale, y, x, flags, err);
     FEM3_CUDA(cudaGetLastError());
     int h_err[ERR_COUNT];
     FEM3_CUDA(cudaMemcpyAsync(h_err, err, sizeof(h_err), cudaMemcpyDeviceToHost, s));

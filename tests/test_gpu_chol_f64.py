@@ -2,6 +2,8 @@
 the 64-column diagonal inverses that the solves use: integer-order problems of chosen order
 against the oracle's matrix, solved by numpy; and the allocation-free solve, which shares it, on dense
 systems of the same kind of sizes."""
+from fractions import Fraction
+
 import numpy as np
 import pytest
 
@@ -73,4 +75,77 @@ def test_f64_factor_band(cells):
         m.assemble_integer((1.0, 2.0, 0.5))
         u = m.solve(f)
         assert float((u - first).norm() / first.norm()) <= 1e-11
+    m.free()
+
+
+def _pairs(d, c):
+    """block-diagonal matrix of [[d, c], [c, d]] for arrays d, c"""
+    n = 2 * len(d)
+    A = np.zeros((n, n))
+    i = np.arange(0, n, 2)
+    A[i, i] = A[i + 1, i + 1] = d
+    A[i, i + 1] = A[i + 1, i] = c
+    return A
+
+
+def _static(A, b):
+    x = torch.empty(len(b), dtype=torch.float64, device="cuda")
+    fem3.spd_solve_static(torch.from_numpy(A).cuda(), torch.from_numpy(b).cuda(), x)
+    return x.cpu().numpy()
+
+
+# exponents of the pivots: subnormal, the ends of the range in which a reciprocal is normal (biased 8
+# and 2,038: -1,015 and 1,015), one and the largest
+@pytest.mark.parametrize("e", [-1074, -1060, -1030, -1025, -1024, -1023, -1022, -1017, -1016, -1015,
+                               -1014, -500, 0, 500, 1013, 1014, 1015, 1016, 1017, 1020])
+def test_pivots_of_any_exponent(e):
+    """[[d, d/2], [d/2, d]] x = d (2, 2.5) and, for the smallest numbers, diag(d, d) x = d (1, 2):
+    every step is exact in binary but the square roots, so 64 of them give (1, 2) to a few 2^-53"""
+    d = np.ldexp(np.ones(32), e)
+    tiny = e < -1060
+    A = _pairs(d, 0.0 * d if tiny else d / 2)
+    x = _static(A, np.ldexp(np.tile((1.0, 2.0) if tiny else (2.0, 2.5), 32), e))
+    assert np.abs(x - np.tile((1.0, 2.0), 32)).max() <= 16 * 2.0 ** -53
+
+
+def test_pivot_reciprocals():
+    """x / d to a unit or two in the last place for pivots of random significands, against exact
+    fractions: 256 systems [[d, c], [c, d]] of condition 3 at most per call"""
+    rng = np.random.default_rng(11)
+    for e in (-900, -1, 0, 1, 900):
+        d = np.ldexp(1.0 + rng.random(256), e)
+        c = d * rng.uniform(-0.5, 0.5, 256)
+        b = np.ldexp(rng.standard_normal(512), e)
+        x = _static(_pairs(d, c), b)
+        for i in range(256):
+            D, Cc, p, q = (Fraction(float(v)) for v in (d[i], c[i], b[2 * i], b[2 * i + 1]))
+            det = D * D - Cc * Cc
+            ref = np.array([float((D * p - Cc * q) / det), float((D * q - Cc * p) / det)])
+            assert np.abs(x[2 * i:2 * i + 2] - ref).max() <= 32 * 2.0 ** -53 * np.abs(ref).max()
+
+
+def test_rows_of_any_scale():
+    """D M D x = D c for a diagonal D of powers of two from 2^-500 to 2^500: x is D^{-1} M^{-1} c, row by
+    row to the accuracy of M (condition below 5)"""
+    n = 130
+    rng = np.random.default_rng(4)
+    B = rng.standard_normal((n, n))
+    M, c, e = B @ B.T + n * np.eye(n), rng.standard_normal(n), rng.integers(-500, 501, n)
+    x = np.ldexp(_static(np.ldexp(np.ldexp(M, e[:, None]), e[None, :]), np.ldexp(c, e)), e)
+    ref = np.linalg.solve(M, c)
+    assert np.linalg.norm(x - ref) <= 1e-12 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("e", [-1013, -1008, 1008, 1013])
+def test_integer_order_at_the_range_ends(e):
+    """K times 2^e: pivots on both sides of the exponents from which their reciprocal is taken by
+    division"""
+    mesh = _bar_mesh((5, 6, 7))
+    f = np.random.default_rng(2).standard_normal(mesh.n_nodes)
+    m = fem3.Mesh(mesh.verts, mesh.tets)
+    m.assemble_integer((1.0, 2.0, 0.5))
+    ref = m.solve(f)
+    m.assemble_integer([k * 2.0 ** e for k in (1.0, 2.0, 0.5)])
+    u = m.solve(f) * 2.0 ** (e // 2) * 2.0 ** (e - e // 2)
+    assert float((u - ref).norm() / ref.norm()) <= 1e-11
     m.free()
