@@ -9,7 +9,7 @@
 // and there are twice as many.  The other SMs do not mind: a 32^3 product is 8 us of one SM's
 // FP64 pipe, enough to hide the next tiles' loads and flags.  Narrower (16) tiles would not be.
 //
-// CTA 0 runs the diagonal chain: for each block column j it applies the last update
+// The first CTA to start runs the diagonal chain: for each block column j it applies the last update
 // (k = j - 1) to the diagonal tile, factors and inverts it, solves the tile below it,
 // L_{j+1,j} = A_{j+1,j} L_jj^{-T}, and keeps that tile in shared memory for the next
 // diagonal update, so the critical path never leaves one SM.  The other CTAs take tasks
@@ -19,11 +19,16 @@
 // ("updated" flag U), every other tile is solved with L_jj^{-1} once the chain has published
 // it and stored as final (flag F).  Every task depends only on tiles of earlier columns (or,
 // for the solve, on the chain's step j), and tickets are taken in column order, so the
-// earliest unfinished claimed task always proceeds and the launch needs no co-residency.
+// earliest unfinished claimed task always proceeds.  The chain itself waits for tasks, which no CTA
+// may have claimed yet when other work holds the rest of the chip: a chain that has waited
+// kHelpSpins then takes tickets up to the tile it needs and does them itself.  So every wait is
+// for a CTA that is running, and the launch needs no co-residency: one CTA alone finishes it (with
+// all SMs but one held by other work, the allocation-free solve of 384 unknowns takes 21 ms, 16 of
+// them before the chain first helps; 0.42 ms undisturbed, as without this provision).
 // Waits are bounded; one that expires sets the abort word, which every other wait also
 // watches, and records ERR_CHOL.
-// flags: F [0, ntask), U [ntask, 2 ntask), ticket [2 ntask], abort word [2 ntask + 1];
-// all zero at launch.
+// flags: F [0, ntask), U [ntask, 2 ntask), ticket [2 ntask], abort word [2 ntask + 1], CTAs that
+// have started [2 ntask + 2]; all zero at launch.
 //
 // Work split.  Warp w of 16 owns the 8 x 8 outputs (block row w / 4, block column w % 4) of a
 // tile product, two neighbouring columns per lane.  With whole 8 x 8 blocks per warp the
@@ -76,6 +81,19 @@ __device__ __forceinline__ bool wait_tile(const int *f, int *abort_w, int32_t *e
         if (spins > 64) __nanosleep(128);   // 150 pollers on one L2 line slow its owner
     }
     return true;
+}
+
+// polls of the chain before it helps, and once it had to: 16 ms, above the chain's waits in an
+// undisturbed launch up to some 30,000 columns, and some 20 us
+constexpr int kHelpSpins = 1 << 15, kHungrySpins = 32;
+// the chain's look at a flag: 1 set, 0 another wait gave up, 2 not set after `limit` polls
+__device__ __forceinline__ int poll_tile(const int *f, const int *abort_w, int limit) {
+    for (int spins = 0; ld_acquire_gpu(f) == 0; spins++) {
+        if (ld_acquire_gpu(abort_w) != 0) return 0;
+        if (spins >= limit) return 2;
+        if (spins > 64) __nanosleep(128);
+    }
+    return 1;
 }
 
 // rows 2w, 2w + 1 of a tile for warp w, lane = column (L2 loads: the tile was written by
@@ -139,7 +157,7 @@ __device__ __forceinline__ int64_t dinv_at(int j) {
 }
 
 // ---------------------------------------------------------------------------------
-// The diagonal chain (CTA 0).  One FP64 instruction of a warp holds its SM sub-partition's
+// The diagonal chain (one CTA).  One FP64 instruction of a warp holds its SM sub-partition's
 // FP64 pipe for 64 clocks whatever its lanes do (measured), so the chain is counted in
 // those slots.  Warps 0-11 compute; warps 12-15 load the tiles of the coming step and publish
 // the finished ones, so no compute warp waits for a flag, a load or a release.
@@ -161,6 +179,116 @@ struct ChainSmem {
     int ok_diag, ok_sub;   // the waits for the step's two tiles (written by the loading warps)
 };
 static_assert(sizeof(ChainSmem) <= kSmemBytes, "chain shared memory");
+
+constexpr size_t kTaskAt = (sizeof(ChainSmem) + 15) / 16 * 16;   // shared memory of a task
+static_assert(kTaskAt + sizeof(double) * 4 * kT * kLd <= kSmemBytes, "shared memory");
+
+// Task W(i, j), all threads; false if a wait gave up.  Not inlined: the workers and the chain's help
+// share one copy, and shared memory is named here so that it is addressed as such.
+__device__ __noinline__ bool tile_task(double *A, int64_t n, int nblk, double *dinv,
+                                       const int *__restrict__ first_col, int i, int j, int *F, int *U,
+                                       int *abort_w, int32_t *err) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double(*b0)[kLd] = reinterpret_cast<double(*)[kLd]>(smem_raw + kTaskAt);   // two pairs of tiles
+    __shared__ int s_ok, s_fa, s_fb, s_pa[2], s_pb[2];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rb = warp >> 2, cb = warp & 3;
+    const int r = rb * 8 + (lane >> 2), c = cb * 8 + (lane & 3) * 2;
+    const int64_t r0 = (int64_t)i * kT, c0 = (int64_t)j * kT;
+    const int kmax = i == j ? max(j - 1, 0) : j;   // the chain applies k = j - 1 to (j, j)
+    int kmin = 0;
+    if (first_col) kmin = max(first_col[i], first_col[j]);
+    double2 acc = load_acc(A, n, r0, c0, false, r, c);
+    // Updates k = 0 .. kmax-1, pipelined: the tiles L_ik, L_jk of update k + 1 are
+    // loaded into registers while update k's product runs (when their flags are
+    // already set; otherwise after it, with a blocking wait), and stored into the other
+    // pair of shared tiles.  Threads 0 and 32 read the two flags at the same time.
+    double2 va, vb;
+    bool have = false;   // va / vb hold the tiles of update k
+    for (int k = kmin; k < kmax; k++) {
+        double(*ta)[kLd] = b0 + (k & 1) * 2 * kT;
+        double(*tb)[kLd] = ta + kT;
+        if (!have) {
+            if (tid == 0) s_fa = wait_tile(&F[tile_id(i, k)], abort_w, err);
+            if (tid == 32) s_fb = wait_tile(&F[tile_id(j, k)], abort_w, err);
+            __syncthreads();
+            if (!(s_fa && s_fb)) return false;
+            va = tile_rows(A + r0 * n + (int64_t)k * kT, n, n - r0);
+            if (i != j) vb = tile_rows(A + c0 * n + (int64_t)k * kT, n, n - c0);
+        }
+        tile_store_T(va, ta);
+        if (i != j) tile_store_T(vb, tb);
+        const int q = (k + 1) & 1;
+        if (k + 1 < kmax) {   // a look at update k + 1's flags, without waiting
+            if (tid == 0) s_pa[q] = ld_acquire_gpu(&F[tile_id(i, k + 1)]) != 0;
+            if (tid == 32) s_pb[q] = ld_acquire_gpu(&F[tile_id(j, k + 1)]) != 0;
+        }
+        __syncthreads();   // update k's tiles stored (the pair written two updates ago
+                           // is no longer read); update k + 1's flags seen
+        have = k + 1 < kmax && s_pa[q] && s_pb[q];
+        if (have) {
+            va = tile_rows(A + r0 * n + (int64_t)(k + 1) * kT, n, n - r0);
+            if (i != j) vb = tile_rows(A + c0 * n + (int64_t)(k + 1) * kT, n, n - c0);
+        }
+        if (i != j || rb >= cb) {
+            const double2 s = dot2(ta, i == j ? ta : tb, kT, r, c);
+            acc.x -= s.x;
+            acc.y -= s.y;
+        }
+    }
+    __syncthreads();   // the last product is done before the shared tiles are reused
+    if (i <= j + 1) {
+        // diagonal or sub-diagonal tile: the chain finishes it
+        store_acc(A, n, r0, c0, acc, r, c);
+        publish(&U[tile_id(i, j)]);
+        return true;
+    }
+    // L_ij = A_ij L_jj^{-T}: column c of the product ends at the inverse's row c
+    double(*at)[kLd] = b0, (*lt)[kLd] = b0 + kT;   // A_ij^T, (L_jj^{-1})^T
+    at[c][r] = acc.x;
+    at[c + 1][r] = acc.y;
+    if (tid == 0) s_ok = wait_tile(&F[tile_id(j, j)], abort_w, err);
+    __syncthreads();
+    if (!s_ok) return false;
+    tile_store_T(tile_rows(dinv + dinv_at(j), 64, kT), lt);
+    __syncthreads();
+    const double2 o = dot2(at, lt, 8 * (cb + 1), r, c);
+    store_acc(A, n, r0, c0, o, r, c);
+    publish(&F[tile_id(i, j)]);
+    return true;
+}
+
+// first ticket of a column
+__device__ __forceinline__ int ticket_of(int nblk, int i, int j) {
+    return j * nblk - j * (j - 1) / 2 + (i - j);
+}
+
+// The chain's CTA, all threads: one ticket up to `last`, if there is one that nobody has claimed;
+// false if not.  Ends with a barrier.
+__device__ bool help(double *A, int64_t n, int nblk, double *dinv, const int *__restrict__ first_col,
+                     int last, int *F, int *U, int *ticket, int *abort_w, int32_t *err) {
+    __shared__ int s_claim;
+    if (threadIdx.x == 0) {
+        int t = ld_acquire_gpu(ticket);
+        while (t <= last) {
+            const int seen = atomicCAS(ticket, t, t + 1);
+            if (seen == t) break;
+            t = seen;
+        }
+        s_claim = t <= last ? t : -1;
+    }
+    __syncthreads();
+    const int t = s_claim;
+    if (t >= 0) {
+        int j = 0;
+        while (t >= ticket_of(nblk, j + 1, j + 1)) j++;
+        const int i = j + (t - ticket_of(nblk, j, j));
+        if (!first_col || i <= j + 1 || j >= first_col[i])
+            tile_task(A, n, nblk, dinv, first_col, i, j, F, U, abort_w, err);
+    }
+    __syncthreads();   // also after a task whose wait gave up (the chain's next poll sees that)
+    return t >= 0;
+}
 
 // Panel p (columns 8p .. 8p + 7) of the augmented rows [A; I] by one warp: lanes 0-7 the
 // pivot rows, lanes 8-31 the rows in `row` (-1: none).  Step j: f = x_j / d_j,
@@ -262,45 +390,64 @@ __device__ __forceinline__ void diag_factor_inv(ChainSmem &S, int nb, int64_t k0
     bar_sync_n(kBarMain, kMainThreads);
 }
 
-__device__ void chain64(double *A, int64_t n, int nblk, double *dinv, int *F, int *U, int *abort_w,
-                        int32_t *err, unsigned char *smem_raw) {
+__device__ void chain64(double *A, int64_t n, int nblk, double *dinv,
+                        const int *__restrict__ first_col, int *F, int *U, int *ticket, int *abort_w,
+                        int32_t *err) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     ChainSmem &S = *reinterpret_cast<ChainSmem *>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (warp >= kMainWarps) {
         // ---- loads and publication (four warps, eight rows of a tile each) ----
         const int iw = warp - kMainWarps;
         const bool lead = tid == kMainThreads;
+        int limit = kHelpSpins;
+        // `wait`: the flag of tile (i, j) into ok and, once it is set, load(); the chain's other
+        // warps stand at barrier `bar`.  While it is not set and its ticket or an earlier one is
+        // unclaimed, all of them help.
+        const auto wait = [&](int *ok, int i, int j, int bar, auto load) {
+            bool claimed = false;   // by a CTA that is running: no more to help with
+            for (;;) {
+                if (lead) {
+                    int got = poll_tile(&U[tile_id(i, j)], abort_w, claimed ? kSpinLimit : limit);
+                    if (got == 2 && claimed) {
+                        atomicAdd(&err[ERR_CHOL], 1);
+                        atomicExch(abort_w, 1);
+                        got = 0;
+                    }
+                    *ok = got;
+                }
+                bar_sync_n(kBarIo, 128);
+                if (*ok == 1) load();
+                bar_sync_n(bar, kThreads);
+                if (*ok != 2) return *ok == 1;
+                claimed = !help(A, n, nblk, dinv, first_col, ticket_of(nblk, i, j), F, U, ticket,
+                                abort_w, err);
+                limit = kHungrySpins;
+            }
+        };
         for (int j = 0; j < nblk; j++) {
             const int64_t c0 = (int64_t)j * kT, r0 = c0 + kT;
             const bool next = j + 1 < nblk;
-            if (lead) S.ok_diag = wait_tile(&U[tile_id(j, j)], abort_w, err);
-            bar_sync_n(kBarIo, 128);
-            if (S.ok_diag) {
+            const auto load_d = [&] {
 #pragma unroll
                 for (int k = 0; k < 8; k++) {
                     const int64_t i = 8 * iw + k;
                     S.d[i][lane] = c0 + i < n && c0 + lane < n ? __ldcg(A + (c0 + i) * n + c0 + lane)
                                                               : (i == lane ? 1.0 : 0.0);
                 }
-            }
-            bar_sync_n(kBarDiag, kThreads);
-            if (!S.ok_diag) return;
-            if (next) {
-                if (lead) S.ok_sub = wait_tile(&U[tile_id(j + 1, j)], abort_w, err);
-                bar_sync_n(kBarIo, 128);
-                if (S.ok_sub) {
+            };
+            if (!wait(&S.ok_diag, j, j, kBarDiag, load_d)) return;
+            const auto load_at = [&] {
 #pragma unroll
-                    for (int k = 0; k < 8; k += 2) {
-                        const int i = 8 * iw + k;
-                        const double *src = A + (r0 + i) * n + c0 + lane;
-                        *reinterpret_cast<double2 *>(&S.at[lane][i]) =
-                            make_double2(r0 + i < n ? __ldcg(src) : 0.0,
-                                         r0 + i + 1 < n ? __ldcg(src + n) : 0.0);
-                    }
+                for (int k = 0; k < 8; k += 2) {
+                    const int i = 8 * iw + k;
+                    const double *src = A + (r0 + i) * n + c0 + lane;
+                    *reinterpret_cast<double2 *>(&S.at[lane][i]) =
+                        make_double2(r0 + i < n ? __ldcg(src) : 0.0,
+                                     r0 + i + 1 < n ? __ldcg(src + n) : 0.0);
                 }
-                bar_sync_n(kBarSub, kThreads);
-                if (!S.ok_sub) return;
-            }
+            };
+            if (next && !wait(&S.ok_sub, j + 1, j, kBarSub, load_at)) return;
             bar_sync_n(kBarDone, kThreads);
             double *Lj = dinv + dinv_at(j);
             const double(*xt)[kLd] = S.xt[j & 1];
@@ -319,6 +466,13 @@ __device__ void chain64(double *A, int64_t n, int nblk, double *dinv, int *F, in
         return;
     }
     // ---- compute ----
+    const auto wait = [&](const int *ok, int i, int j, int bar) {   // as above
+        for (;;) {
+            bar_sync_n(bar, kThreads);
+            if (*ok != 2) return *ok == 1;
+            help(A, n, nblk, dinv, first_col, ticket_of(nblk, i, j), F, U, ticket, abort_w, err);
+        }
+    };
     for (int j = 0; j < nblk; j++) {
         const bool next = j + 1 < nblk;
         // the update k = j - 1 on and below the diagonal: 20 half blocks of 8 x 4 outputs,
@@ -338,8 +492,7 @@ __device__ void chain64(double *A, int64_t n, int nblk, double *dinv, int *F, in
                 for (int k = 0; k < kT; k++) t[h] = fma(xp[k][tr[h]], xp[k][tc[h]], t[h]);
             }
         }
-        bar_sync_n(kBarDiag, kThreads);
-        if (!S.ok_diag) return;
+        if (!wait(&S.ok_diag, j, j, kBarDiag)) return;
 #pragma unroll
         for (int h = 0; h < 2; h++)
             if (warp + kMainWarps * h < 20) S.u[tr[h]][tc[h]] = S.d[tr[h]][tc[h]] - t[h];
@@ -347,8 +500,7 @@ __device__ void chain64(double *A, int64_t n, int nblk, double *dinv, int *F, in
         bar_sync_n(kBarMain, kMainThreads);
         diag_factor_inv(S, (int)min((int64_t)kT, n - (int64_t)j * kT), (int64_t)j * kT, err);
         if (next) {
-            bar_sync_n(kBarSub, kThreads);
-            if (!S.ok_sub) return;
+            if (!wait(&S.ok_sub, j + 1, j, kBarSub)) return;
             // xt = L_jj^{-1} A_{j+1,j}^T: row r of the inverse ends at column r
             double(*xt)[kLd] = S.xt[j & 1];
             const int cb = warp & 3;
@@ -373,18 +525,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_chol_f64(double *A, int64_t n, 
                                                           double *dinv,
                                                           const int *__restrict__ first_col,
                                                           int *flags, int32_t *err) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double(*b0)[kLd] = reinterpret_cast<double(*)[kLd]>(smem_raw);   // two pairs of tiles
-    __shared__ int s_task, s_ok, s_fa, s_fb, s_pa[2], s_pb[2];
+    __shared__ int s_task;
     const int ntask = nblk * (nblk + 1) / 2;
     int *F = flags, *U = flags + ntask, *ticket = flags + 2 * ntask, *abort_w = ticket + 1;
-    if (blockIdx.x == 0) {
-        chain64(A, n, nblk, dinv, F, U, abort_w, err, smem_raw);
+    const int tid = threadIdx.x;
+    if (tid == 0) s_task = atomicAdd(ticket + 2, 1);
+    __syncthreads();
+    if (s_task == 0) {
+        chain64(A, n, nblk, dinv, first_col, F, U, ticket, abort_w, err);
         return;
     }
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int rb = warp >> 2, cb = warp & 3;
-    const int r = rb * 8 + (lane >> 2), c = cb * 8 + (lane & 3) * 2;
+    __syncthreads();   // s_task is read before the first ticket is stored in it
     int j = 0, first = 0;   // column of the last ticket and the first ticket of that column
     const auto row_of = [&](int t) {   // (t in column j from here on)
         while (t - first >= nblk - j) first += nblk - j++;
@@ -407,67 +558,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_chol_f64(double *A, int64_t n, 
         const int t = s_task;
         if (t >= ntask) return;
         const int i = row_of(t);
-        const int64_t r0 = (int64_t)i * kT, c0 = (int64_t)j * kT;
-        const int kmax = i == j ? max(j - 1, 0) : j;   // the chain applies k = j - 1 to (j, j)
-        int kmin = 0;
-        if (first_col) kmin = max(first_col[i], first_col[j]);
-        double2 acc = load_acc(A, n, r0, c0, false, r, c);
-        // Updates k = 0 .. kmax-1, pipelined: the tiles L_ik, L_jk of update k + 1 are
-        // loaded into registers while update k's product runs (when their flags are
-        // already set; otherwise after it, with a blocking wait), and stored into the other
-        // pair of shared tiles.  Threads 0 and 32 read the two flags at the same time.
-        double2 va, vb;
-        bool have = false;   // va / vb hold the tiles of update k
-        for (int k = kmin; k < kmax; k++) {
-            double(*ta)[kLd] = b0 + (k & 1) * 2 * kT;
-            double(*tb)[kLd] = ta + kT;
-            if (!have) {
-                if (tid == 0) s_fa = wait_tile(&F[tile_id(i, k)], abort_w, err);
-                if (tid == 32) s_fb = wait_tile(&F[tile_id(j, k)], abort_w, err);
-                __syncthreads();
-                if (!(s_fa && s_fb)) return;
-                va = tile_rows(A + r0 * n + (int64_t)k * kT, n, n - r0);
-                if (i != j) vb = tile_rows(A + c0 * n + (int64_t)k * kT, n, n - c0);
-            }
-            tile_store_T(va, ta);
-            if (i != j) tile_store_T(vb, tb);
-            const int q = (k + 1) & 1;
-            if (k + 1 < kmax) {   // a look at update k + 1's flags, without waiting
-                if (tid == 0) s_pa[q] = ld_acquire_gpu(&F[tile_id(i, k + 1)]) != 0;
-                if (tid == 32) s_pb[q] = ld_acquire_gpu(&F[tile_id(j, k + 1)]) != 0;
-            }
-            __syncthreads();   // update k's tiles stored (the pair written two updates ago
-                               // is no longer read); update k + 1's flags seen
-            have = k + 1 < kmax && s_pa[q] && s_pb[q];
-            if (have) {
-                va = tile_rows(A + r0 * n + (int64_t)(k + 1) * kT, n, n - r0);
-                if (i != j) vb = tile_rows(A + c0 * n + (int64_t)(k + 1) * kT, n, n - c0);
-            }
-            if (i != j || rb >= cb) {
-                const double2 s = dot2(ta, i == j ? ta : tb, kT, r, c);
-                acc.x -= s.x;
-                acc.y -= s.y;
-            }
-        }
-        __syncthreads();   // the last product is done before the shared tiles are reused
-        if (i <= j + 1) {
-            // diagonal or sub-diagonal tile: the chain finishes it
-            store_acc(A, n, r0, c0, acc, r, c);
-            publish(&U[tile_id(i, j)]);
-            continue;
-        }
-        // L_ij = A_ij L_jj^{-T}: column c of the product ends at the inverse's row c
-        double(*at)[kLd] = b0, (*lt)[kLd] = b0 + kT;   // A_ij^T, (L_jj^{-1})^T
-        at[c][r] = acc.x;
-        at[c + 1][r] = acc.y;
-        if (tid == 0) s_ok = wait_tile(&F[tile_id(j, j)], abort_w, err);
-        __syncthreads();
-        if (!s_ok) return;
-        tile_store_T(tile_rows(dinv + dinv_at(j), 64, kT), lt);
-        __syncthreads();
-        const double2 o = dot2(at, lt, 8 * (cb + 1), r, c);
-        store_acc(A, n, r0, c0, o, r, c);
-        publish(&F[tile_id(i, j)]);
+        if (!tile_task(A, n, nblk, dinv, first_col, i, j, F, U, abort_w, err)) return;
     }
 }
 

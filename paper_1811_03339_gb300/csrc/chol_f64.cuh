@@ -10,7 +10,7 @@ constexpr int kChol64Tile = 32;
 // flag words of a factorisation of order n (zeroed by the call)
 inline int64_t chol_f64_flags(int64_t n) {
     const int64_t nblk = (n + kChol64Tile - 1) / kChol64Tile;
-    return nblk * (nblk + 1) + 2;
+    return nblk * (nblk + 1) + 3;
 }
 
 // A = L L^T (row-major n x n, lower triangle read) in place below the diagonal tiles, and the

@@ -36,7 +36,7 @@ constexpr int kNaBlocks = kNaMaxN / NBS;
 constexpr size_t kNaFactor = (size_t)kNaMaxN * kNaMaxN;
 constexpr size_t kNaInv = (size_t)kNaBlocks * NBS * NBS;
 constexpr int kNaCholTiles = kNaMaxN / kChol64Tile;
-constexpr size_t kNaCholFlags = (size_t)kNaCholTiles * (kNaCholTiles + 1) + 2;
+constexpr size_t kNaCholFlags = (size_t)kNaCholTiles * (kNaCholTiles + 1) + 3;
 constexpr size_t kNaSolveFlags = 2 * kNaBlocks + 2;
 constexpr size_t kNaElems =
     kNaFactor + kNaInv + kNaMaxN + (kNaCholFlags + kNaSolveFlags + ERR_COUNT + kNaMaxN + 1) / 2;

@@ -4,6 +4,10 @@ against the oracle's matrix, solved by numpy; and the allocation-free solve, whi
 systems of the same kind of sizes."""
 from fractions import Fraction
 
+import ctypes as C
+import subprocess
+import time
+
 import numpy as np
 import pytest
 
@@ -16,7 +20,7 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("needs a CUDA device", allow_module_level=True)
 
-from paper_1811_03339_gb300 import fem3  # noqa: E402
+from paper_1811_03339_gb300 import _build_lib, fem3  # noqa: E402
 
 # interior dofs of a box of cells: (a - 1)(b - 1)(c - 1)
 SIZES = {1: (2, 2, 2), 8: (3, 3, 3), 9: (10, 2, 2), 31: (32, 2, 2), 32: (3, 5, 5), 33: (4, 12, 2),
@@ -149,3 +153,55 @@ def test_integer_order_at_the_range_ends(e):
     u = m.solve(f) * 2.0 ** (e // 2) * 2.0 ** (e - e // 2)
     assert float((u - ref).norm() / ref.norm()) <= 1e-11
     m.free()
+
+
+HOLD = r"""
+#include <cuda_runtime.h>
+__global__ void k_hold(long long ns) {
+    long long t0, t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
+    for (int i = 0; i < 1 << 27; i++) {
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+        if (t - t0 >= ns) break;
+        __nanosleep(1000);
+    }
+}
+extern "C" int hold(int ctas, int smem, long long ns, void *stream) {
+    cudaFuncSetAttribute(k_hold, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    k_hold<<<ctas, 1, smem, (cudaStream_t)stream>>>(ns);
+    return (int)cudaGetLastError();
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def hold(tmp_path_factory):
+    d = tmp_path_factory.mktemp("hold")
+    (d / "hold.cu").write_text(HOLD)
+    subprocess.run(["nvcc", *_build_lib.ARCH, "-shared", "-Xcompiler", "-fPIC", str(d / "hold.cu"),
+                    "-o", str(d / "hold.so")], check=True)
+    f = C.CDLL(str(d / "hold.so")).hold
+    f.argtypes = [C.c_int, C.c_int, C.c_longlong, C.c_void_p]
+    return f
+
+
+@pytest.mark.parametrize("n,free", [(384, 1), (512, 1), (384, 2)])
+def test_static_solve_beside_other_work(hold, n, free):
+    """All SMs but `free` are held for a second by blocks that leave no room for one of the
+    factorisation's: it finishes there, before they do."""
+    rng = np.random.default_rng(n)
+    B = rng.standard_normal((n, n))
+    A, b = torch.from_numpy(B @ B.T + n * np.eye(n)).cuda(), torch.from_numpy(rng.standard_normal(n)).cuda()
+    x, ref = torch.empty_like(b), torch.empty_like(b)
+    fem3.spd_solve_static(A, b, ref)
+    assert hold(1, 1 << 17, 1000, None) == 0   # loads the kernel
+    torch.cuda.synchronize()
+    side, done = torch.cuda.Stream(), torch.cuda.Event()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert hold(sms - free, 200 << 10, 1_000_000_000, side.cuda_stream) == 0
+    done.record(side)
+    time.sleep(0.05)
+    fem3.spd_solve_static(A, b, x)
+    assert not done.query()
+    assert torch.equal(x, ref)
+    torch.cuda.synchronize()
