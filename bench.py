@@ -123,19 +123,19 @@ def kernel_rooflines(kms: dict, cnt: dict, n_dof: int, precision: str, peaks: di
     walk_tables  HBM: 160 B (one tet record) per walked segment; FP64 side: 25 flops per
                  segment against the FP64 rate
     split        HBM: per table element 16 B read (L and R pairs) and the four operand halves
-                 written (2 B each for BF16, 4 B for TF32); the class's time also holds the
-                 transposition of the refinement operator's blocks, whose bytes are not counted
+                 written (2 B each for BF16, 4 B for TF32)
     contract     tensor: algorithmic flops sum_g 4 nnz(L[g]) nnz(R[g]) per axis (when
-                 counted) and the executed split-product MMA flops (3 x 2 D_b^2 G_b); the
-                 mixed forms' time also holds the contraction that builds the refinement's
-                 operator (k_contract_rows), whose flops are not counted
+                 counted) and the executed split-product MMA flops (3 x 2 D_b^2 G_b)
+    operator     FP32 issue: the build of the refinement's operator, one double-float multiply-add
+                 (13 FP32 instructions) per pair of nonzeros: a quarter of the algorithmic flops
     factor       FP32 pipe: n^3 / 3 flops
     chain        HBM: the factor's lower triangle once per direction (4 n^2 B for FP32) and
                  solve of a group of columns
-    apply        FP32 issue: the matrix-free work the block-sparse operator replaces, 2
-                 double-float multiply-adds (13 FP32 instructions each) per nonzero table entry
-                 (of L and of R) and vector, when the nonzeros are counted (else 4 per dense
-                 bin-table element pair)
+    apply        the block-sparse operator (block_operator): time per launch only, as its sweeps run
+                 in three arithmetics (FP64, double-float, FP32) on three pipes.  An apply from the
+                 tables: FP32 issue, 2 double-float multiply-adds (13 FP32 instructions each) per
+                 nonzero table entry (of L and of R) and vector, when the nonzeros are counted (else
+                 4 per dense bin-table element pair)
     """
     out = {}
     hbm = float(peaks["hbm_gbs"])
@@ -160,7 +160,7 @@ def kernel_rooflines(kms: dict, cnt: dict, n_dof: int, precision: str, peaks: di
         lists = bool(snz) and cnt.get("apply_lists", True)
         tail = 0 if cnt.get("block_operator") else (2 * 10 * snz if lists else 8 * elems)
         gbs = (per * elems + tail) / (s[0] * 1e-3) / 1e9
-        out["split"] = {"kernel": "k_split_ops (+ k_op_mirror)", "bound": "hbm", "unit": "GB/s",
+        out["split"] = {"kernel": "k_split_ops", "bound": "hbm", "unit": "GB/s",
                         "achieved": gbs, "peak": hbm, "frac": gbs / hbm, "launches": s[1],
                         "launch_ms": s[0] / s[1], "traffic": None,
                         "algorithmic": f"{per} B per table element x {elems:.0f} elements"
@@ -172,7 +172,7 @@ def kernel_rooflines(kms: dict, cnt: dict, n_dof: int, precision: str, peaks: di
         if ratio is not None:
             peak = float(peaks.get("bf16_tflops", 1900.0)) * ratio
             ach = executed / (c[0] * 1e-3) / 1e12
-            rec = {"kernel": "k_contract_tc (+ k_contract_rows)", "bound": "tensor", "unit": "TFLOP/s",
+            rec = {"kernel": "k_contract_tc", "bound": "tensor", "unit": "TFLOP/s",
                    "achieved": ach, "peak": peak, "frac": ach / peak,
                    "basis": "executed split-product MMA flops (3 x 2 D_b^2 G_b over the bins)"}
         else:
@@ -190,6 +190,15 @@ def kernel_rooflines(kms: dict, cnt: dict, n_dof: int, precision: str, peaks: di
                 rec["executed_over_algorithmic"] = executed / alg
         rec.update(launches=c[1], launch_ms=c[0] / c[1], traffic=None)
         out["contract"] = rec
+    o = kms.get("operator", (0, 0))
+    if o[0] > 0 and cnt.get("algorithmic_flops"):
+        ach = DF_OPS_PER_PRODUCT * cnt["algorithmic_flops"] / 4 / (o[0] * 1e-3) / 1e12
+        out["operator"] = {"kernel": "k_contract_rows, k_op_mirror", "bound": "alu",
+                           "unit": "T FP32 instr/s", "achieved": ach, "peak": FP32_ISSUE_TOPS,
+                           "frac": ach / FP32_ISSUE_TOPS, "launches": o[1], "launch_ms": o[0] / o[1],
+                           "traffic": None,
+                           "algorithmic": f"{DF_OPS_PER_PRODUCT} FP32 instructions per pair of "
+                                          "nonzeros of L and R at a Gauss point"}
     f = kms.get("factor", (0, 0))
     if f[0] > 0:
         fl = n_dof ** 3 / 3.0
@@ -225,7 +234,11 @@ def kernel_rooflines(kms: dict, cnt: dict, n_dof: int, precision: str, peaks: di
                         "launch_ms": ch[0] / ch[1], "traffic": None,
                         "algorithmic": "the factor's lower triangle twice per solve"}
     a = kms.get("apply", (0, 0))
-    if a[0] > 0 and cnt.get("apply_vectors"):
+    if a[0] > 0 and cnt.get("block_operator"):
+        out["apply"] = {"kernel": "k_op_apply", "bound": "the FP64 pipe, then FP32 issue or hbm",
+                        "launches": a[1], "launch_ms": a[0] / a[1], "traffic": None,
+                        "vector_applies": cnt.get("apply_vectors")}
+    elif a[0] > 0 and cnt.get("apply_vectors"):
         nnz = cnt.get("table_nnz")
         if nnz:
             ops = 2 * DF_OPS_PER_PRODUCT * nnz * cnt["apply_vectors"]
@@ -238,10 +251,11 @@ def kernel_rooflines(kms: dict, cnt: dict, n_dof: int, precision: str, peaks: di
                    f"per table element and vector, {elems:.0f} elements, "
                    f"{cnt['apply_vectors']} vector-applies")
         ach = ops / (a[0] * 1e-3) / 1e12
-        out["apply"] = {"kernel": "k_op_apply", "bound": "alu", "unit": "T FP32 instr/s",
+        out["apply"] = {"kernel": "an apply from the tables", "bound": "alu",
+                        "unit": "T FP32 instr/s",
                         "achieved": ach, "peak": FP32_ISSUE_TOPS, "frac": ach / FP32_ISSUE_TOPS,
                         "launches": a[1], "launch_ms": a[0] / a[1], "traffic": None,
-                        "algorithmic": alg + " (matrix-free equivalent)"}
+                        "algorithmic": alg}
         if nnz:
             out["apply"]["nonzero_fraction_of_bin_tables"] = nnz / (2.0 * elems)
     return out

@@ -318,8 +318,9 @@ int fem3_table_nnz(fem3_mesh m, int64_t *nnz, void *stream);
  * CUDA events on the launch stream around every launch of the class, summed over the
  * launches since the last fem3_assemble and collected by the next synchronising call
  * (fem3_solve, fem3_sync).  Classes: 0 walk + derivative tables (one launch, three axes),
- * 1 operand split of the tables, 2 contraction GEMMs, 3 Cholesky factorisation,
- * 4 triangular-solve chains, 5 refinement operator apply.  Any output pointer may be NULL. */
+ * 1 operand split of the tables, 2 contraction of the matrix, 3 Cholesky factorisation,
+ * 4 triangular solves (one entry per solve of a group of columns), 5 refinement operator apply,
+ * 6 build of the refinement's operator.  Any output pointer may be NULL. */
 int fem3_kernel_ms(fem3_mesh m, int kclass, float *ms, int32_t *launches);
 
 /* Transverse bins of one axis (Section 2.3 template, per axis): number of bins, template

@@ -388,14 +388,15 @@ static int launch_rows(Mesh *m, const RowsAxes &P, typename Arith<TA>::Out *A,
     FEM3_CUDA(device_smem(half ? (const void *)k_contract_rows<TA, OUT, true>
                                : (const void *)k_contract_rows<TA, OUT, false>,
                           kRowsSmemMax));
-    kc_begin(m, KC_CONTRACT);
+    const int kc = OUT == kBlocks ? KC_OPERATOR : KC_CONTRACT;
+    kc_begin(m, kc);
     if (half)
         k_contract_rows<TA, OUT, true><<<(unsigned)nw, kRowsThreads, sh, m->stream>>>(
             P, cap, win, max_gp, max_dof, A, m->n_dof, map);
     else
         k_contract_rows<TA, OUT, false><<<(unsigned)nw, kRowsThreads, sh, m->stream>>>(
             P, cap, win, max_gp, max_dof, A, m->n_dof, map);
-    kc_end(m, KC_CONTRACT);
+    kc_end(m, kc);
     note_launch(m);
     FEM3_CUDA(cudaGetLastError());
     return FEM3_OK;

@@ -246,12 +246,13 @@ void stage_collect(Mesh *m);
 // CUDA events on the launch stream around every launch of the class.
 enum KernelClass {
     KC_WALK = 0,      // k_walk_tables: walk + derivative tables, three axes in one launch
-    KC_SPLIT = 1,     // operand splits: the tables' (k_split_ops), the operator's (k_op_mirror)
-    KC_CONTRACT = 2,  // contraction GEMMs (tensor-core or CUDA-core)
+    KC_SPLIT = 1,     // the tensor-core contraction's operand split (k_split_ops)
+    KC_CONTRACT = 2,  // contraction of the matrix (tensor-core or CUDA-core)
     KC_FACTOR = 3,    // Cholesky factorisation
     KC_CHAIN = 4,     // triangular solves (both directions of a group of columns)
     KC_APPLY = 5,     // operator apply of the refinement residual
-    KC_COUNT = 6
+    KC_OPERATOR = 6,  // build of the refinement's operator (k_contract_rows, k_op_mirror)
+    KC_COUNT = 7
 };
 void kc_begin(Mesh *m, int cls);
 void kc_end(Mesh *m, int cls);

@@ -495,9 +495,9 @@ int op_build(Mesh *m) {
                               m->stream));
     FEM3_TRY(contract_blocks(m, O));
     if (O.n_full > 0) {
-        kc_begin(m, KC_SPLIT);
+        kc_begin(m, KC_OPERATOR);
         k_op_mirror<<<(unsigned)O.n_full, 256, 0, m->stream>>>(O.low, O.src, O.row_of, O.col, O.full);
-        kc_end(m, KC_SPLIT);
+        kc_end(m, KC_OPERATOR);
         note_launch(m);
     }
     FEM3_CUDA(cudaGetLastError());

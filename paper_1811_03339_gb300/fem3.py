@@ -247,7 +247,8 @@ def table_nnz(h, stream=None):
     return v.value
 
 
-KERNEL_CLASSES = ("walk_tables", "split", "contract", "factor", "chain", "apply")
+KERNEL_CLASSES = ("walk_tables", "split", "contract", "factor", "chain", "apply",
+                  "operator")
 
 
 def kernel_ms(h):
@@ -447,8 +448,7 @@ class Mesh:
         return tc_tile(self.h)
 
     def apply_lists(self):
-        """whether the refinement's operator apply runs from the tables' nonzero lists (else
-        from the dense table blocks of the bins)"""
+        """whether the bins are narrow (see fem3_apply_lists; it selects nothing)"""
         return apply_lists(self.h)
 
     def free(self):
