@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(512, 1) k_cholp_diag(float *A, int64_t n, int6
         at[c][i] = v21[q];
     }
     __syncthreads();
-    potrf_inv_smem<float, NB>(a_s, x_s, nb1, j0, err);
+    potrf_inv_smem(a_s, x_s, nb1, j0, err);
     float *d1 = dinv + (j0 / NB) * (int64_t)NB * NB;
     for (int e = tid; e < NB * NB; e += 512) {
         const int i = e >> 6, c = e & 63;
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(512, 1) k_cholp_diag(float *A, int64_t n, int6
 #pragma unroll 8
     for (int k = 0; k < NB; k++) {
         float v[4];
-        lds4<float>(&at[k][4 * tx], v);
+        lds4(&at[k][4 * tx], v);
         const float u0 = x_s[2 * ty][k], u1 = x_s[2 * ty + 1][k];
 #pragma unroll
         for (int q = 0; q < 4; q++) {
@@ -130,8 +130,8 @@ __global__ void __launch_bounds__(512, 1) k_cholp_diag(float *A, int64_t n, int6
 #pragma unroll 8
     for (int k = 0; k < NB; k++) {
         float u[2], v[4];
-        lds2<float>(&lt[k][2 * ty], u);
-        lds4<float>(&lt[k][4 * tx], v);
+        lds2(&lt[k][2 * ty], u);
+        lds4(&lt[k][4 * tx], v);
 #pragma unroll
         for (int p = 0; p < 2; p++)
 #pragma unroll
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(512, 1) k_cholp_diag(float *A, int64_t n, int6
         Pinv[2 * NB * NB + e] = lt[i][c];
     }
     __syncthreads();
-    potrf_inv_smem<float, NB>(a_s, x_s, nb2, j0 + NB, err);    // x_s = X22
+    potrf_inv_smem(a_s, x_s, nb2, j0 + NB, err);    // x_s = X22
     float *d2 = d1 + (int64_t)NB * NB;
     for (int e = tid; e < NB * NB; e += 512) {
         const int i = e >> 6, c = e & 63;
@@ -180,11 +180,11 @@ __device__ __forceinline__ void panel_gemm(const float (*a)[kQ], const float (*b
     for (int k = 0; k < 64; k += 4) {
         float av[R][4];
 #pragma unroll
-        for (int p = 0; p < R; p++) lds4<float>(&a[R * ty + p][k], av[p]);
+        for (int p = 0; p < R; p++) lds4(&a[R * ty + p][k], av[p]);
 #pragma unroll
         for (int kk = 0; kk < 4; kk++) {
             float bv[4];
-            lds4<float>(&bt[k + kk][4 * tx], bv);
+            lds4(&bt[k + kk][4 * tx], bv);
 #pragma unroll
             for (int p = 0; p < R; p++)
 #pragma unroll
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(256) k_cholp_panel(float *A, int64_t n, int64_
 #pragma unroll
     for (int p = 0; p < R; p++) {
         float v[4];
-        lds4<float>(&a2[R * ty + p][4 * tx], v);
+        lds4(&a2[R * ty + p][4 * tx], v);
 #pragma unroll
         for (int q = 0; q < 4; q++) acc[p][q] = v[q] - acc[p][q];
     }

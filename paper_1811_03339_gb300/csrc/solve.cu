@@ -141,8 +141,8 @@ __device__ __forceinline__ void tile_gemm_T(float acc[2][4], const float (*bi)[k
 #pragma unroll 8
     for (int c = 0; c < NB; c++) {
         float u[2], v[4];
-        lds2<float>(&bi[c][ty * 2], u);
-        lds4<float>(&bj[c][tx * 4], v);
+        lds2(&bi[c][ty * 2], u);
+        lds4(&bj[c][tx * 4], v);
 #pragma unroll
         for (int p = 0; p < 2; p++)
 #pragma unroll
@@ -210,7 +210,7 @@ __device__ void chol_chain(float *A, int64_t n, int nblk, float *dinv, int *F, i
 #pragma unroll
             for (int q = 0; q < 4; q++) a_s[ty * 2 + p][tx * 4 + q] = acc[p][q];
         __syncthreads();
-        potrf_inv_smem<float, NB>(a_s, x_s, (int)min((int64_t)NB, n - c0), c0, err);
+        potrf_inv_smem(a_s, x_s, (int)min((int64_t)NB, n - c0), c0, err);
         if (next) {
             // L_{j+1,j} = A~_{j+1,j} L_jj^{-T}, computed transposed: xt = L_jj^{-1} A~_{j+1,j}^T
             // the next diagonal tile's flag is looked at now, beside this wait, and once more
@@ -229,7 +229,7 @@ __device__ void chol_chain(float *A, int64_t n, int nblk, float *dinv, int *F, i
 #pragma unroll 8
             for (int k = 0; k < NB; k++) {
                 float v[4];
-                lds4<float>(&at[k][tx * 4], v);
+                lds4(&at[k][tx * 4], v);
                 const float u0 = x_s[ty * 2][k], u1 = x_s[ty * 2 + 1][k];
 #pragma unroll
                 for (int q = 0; q < 4; q++) {
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(512, 1) k_chol_tiles(float *A, int64_t n, int 
 #pragma unroll 8
         for (int c = 0; c < NB; c++) {
             float v[4];
-            lds4<float>(&b1[c][tx * 4], v);
+            lds4(&b1[c][tx * 4], v);
             const float u0 = a[ty * 2][c], u1 = a[ty * 2 + 1][c];
 #pragma unroll
             for (int q = 0; q < 4; q++) {

@@ -18,7 +18,8 @@
 // 0.49 -> 0.32 ms, FP64 four columns at n = 1,000 0.31 -> 0.16 ms, one at n = 343 47 -> 14 us.
 // Chaining the launches (launch_chained) then took the eight-column refined solve at n = 6,859 from
 // 1.77 to 1.62 ms and the 16^3 TF32 x 3 step from 4.31 to 4.16 ms (24^3: 28.1 ms either way, the
-// updates are bound by HBM there); without the fetches into L2 the former is 1.70 ms.
+// updates take about eight rounds of loads and products one after another there, on 350 CTAs or
+// fewer: 0.8 TB/s, an eighth of HBM's rate); without the fetches into L2 the former is 1.70 ms.
 #include <algorithm>
 
 #include "fem3_impl.cuh"
@@ -392,17 +393,18 @@ template <class TF> int tri_width(int64_t n) {
     return (int)B;
 }
 
-// rows of a launch: one per warp until that fills the chip (about eight warps per SM), then four
-// (NR sums each), which share the reads of x
+// rows of a launch: one per warp until that fills the chip (about eight warps per SM; a triangular
+// block's 1,024 rows never do), then four (NR sums each), which share the reads of x
 template <class TF, int NR, bool TRI>
 int launch_rows(const TF *M, int64_t ldm, int64_t rows, int K, const TF *x, int64_t n, int nrhs,
                 TF *out, cudaStream_t s, bool first = false) {
-    if (rows <= 4 * 1216)
-        return launch_chained(first, k_tri_rows<TF, NR, 1, TRI>, (rows + kTriWarps - 1) / kTriWarps,
-                              kTriThreads, 0, s, M, ldm, rows, K, x, n, nrhs, out);
-    return launch_chained(first, k_tri_rows<TF, NR, 4, TRI>,
-                          (rows + 4 * kTriWarps - 1) / (4 * kTriWarps), kTriThreads, 0, s, M, ldm,
-                          rows, K, x, n, nrhs, out);
+    if constexpr (!TRI)
+        if (rows > 4 * 1216)
+            return launch_chained(first, k_tri_rows<TF, NR, 4, TRI>,
+                                  (rows + 4 * kTriWarps - 1) / (4 * kTriWarps), kTriThreads, 0, s, M,
+                                  ldm, rows, K, x, n, nrhs, out);
+    return launch_chained(first, k_tri_rows<TF, NR, 1, TRI>, (rows + kTriWarps - 1) / kTriWarps,
+                          kTriThreads, 0, s, M, ldm, rows, K, x, n, nrhs, out);
 }
 
 template <class TF, int NR, bool TRI>

@@ -54,3 +54,19 @@ def test_f32_solve_sizes(n, nrhs):
     res = np.linalg.norm(b - A @ u, axis=0) / np.linalg.norm(b, axis=0)
     assert res.max() <= 1e-3, res
     m.free()
+
+
+@pytest.mark.parametrize("chol_tc", [-1, 1])
+@pytest.mark.parametrize("nrhs", [1, 8, 17])
+def test_f32_solve_of_wide_blocks(nrhs, chol_tc):
+    """Above 4,096 unknowns the FP32 blocks are 1,024 wide, and one column's updates of more than 4,864
+    rows take four rows a warp: 6,156 unknowns, a ragged last block.  One sweep's residual is formed in
+    FP64; a backward-stable FP32 solve leaves 2^-24 sqrt(n) of |A| |u| (tens of b): below 1e-4."""
+    mesh = _bar_mesh((19, 19, 20))
+    m = fem3.Mesh(mesh.verts, mesh.tets, chol_tc=chol_tc)
+    assert m.n_dof == 6156
+    m.assemble((1.3, 1.6, 1.8), (1.0, 2.0, 0.5), "fp32")
+    f = np.random.default_rng(nrhs).standard_normal((mesh.n_nodes, nrhs))
+    m.solve(f, tol=1e-4, max_iter=1)
+    assert m.iters == 1 and m.resid <= 1e-4
+    m.free()
