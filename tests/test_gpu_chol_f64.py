@@ -2,11 +2,11 @@
 the 64-column diagonal inverses that the solves use: integer-order problems of chosen order
 against the oracle's matrix, solved by numpy; and the allocation-free solve, which shares it, on dense
 systems of the same kind of sizes."""
-from fractions import Fraction
-
 import ctypes as C
+import os
 import subprocess
 import time
+from fractions import Fraction
 
 import numpy as np
 import pytest
@@ -178,8 +178,8 @@ extern "C" int hold(int ctas, int smem, long long ns, void *stream) {
 def hold(tmp_path_factory):
     d = tmp_path_factory.mktemp("hold")
     (d / "hold.cu").write_text(HOLD)
-    subprocess.run(["nvcc", *_build_lib.ARCH, "-shared", "-Xcompiler", "-fPIC", str(d / "hold.cu"),
-                    "-o", str(d / "hold.so")], check=True)
+    subprocess.run([os.environ.get("NVCC", "nvcc"), *_build_lib.ARCH, "-shared", "-Xcompiler", "-fPIC",
+                    str(d / "hold.cu"), "-o", str(d / "hold.so")], check=True)
     f = C.CDLL(str(d / "hold.so")).hold
     f.argtypes = [C.c_int, C.c_int, C.c_longlong, C.c_void_p]
     return f
