@@ -9,7 +9,7 @@
 // right-hand side and the output.  Each call ends by reading the error words back and
 // synchronising its stream.
 //
-// Three steps: copy A (the factorisation works in place), the FP64 tile factorisation of
+// Three steps: copy A, scaled (the factorisation works in place), the FP64 tile factorisation of
 // chol_f64.cu, and one launch for both substitutions (k_na_solve).  What bounds it is the
 // factorisation's diagonal chain (12 steps of 28 us at n = 384) and, for the substitutions,
 // a hand-over between SMs per 64-row block.  Measured at n = 384 (GB300): 2.58 ms as one

@@ -15,7 +15,8 @@
 //                by the solve);
 //     kOpUpdate  double-float FP32 (11 instructions per multiply-add against 64 clocks of the
 //                FP64 pipe): the update r -= A d of a correction d, 1e-3 of u or less;
-//     kOpLate    FP32: the update of the last sweeps (about 1e-6 relative).
+//     kOpLate    FP32: the update of the single-mesh solve's last sweeps, and A times the carries
+//                (about 1e-6 relative).
 //
 // Bound: the FP64 pipe in kOpFull with many vectors, FP32 issue in the others, HBM for one
 // vector (8 bytes per entry of a nonzero block, a tenth to a half of n^2).  Applying the
